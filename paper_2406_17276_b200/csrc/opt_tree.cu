@@ -575,14 +575,14 @@ struct BuildSink {
 
 // Algorithm 1 for a whole batch in one launch: persistent CTAs take rows from their mailboxes; layers
 // of different sequences overlap freely because sequences never exchange data.
-template <bool kPrune, int NCAP>
+template <bool kPrune, int NCAP, bool kAligned>
 __global__ void __launch_bounds__(kThreads)
 build_kernel(Workspace w, Params p, const uint16_t* __restrict__ draft, opt_tree_out out) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     CtaSmemT<NCAP>& s = *reinterpret_cast<CtaSmemT<NCAP>*>(smem_raw);
     BuildSource<kPrune> src{w, p, draft};
     BuildSink<kPrune> sink{w, p, out};
-    run_pipeline(s, src, sink, p.V, p.k, p.aligned != 0, w.status);
+    run_pipeline<kAligned>(s, src, sink, p.V, p.k, draft, draft + (size_t)p.H * p.V, w.status);
 }
 
 // The row step alone over a list of rows (static round-robin over the CTAs).
@@ -612,6 +612,7 @@ struct ListSink {
         }
     }
 };
+template <bool kAligned>
 __global__ void __launch_bounds__(kThreads)
 row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __restrict__ rows, int nrows,
                 int32_t* tok_out, double* prob_out, int* status) {
@@ -619,7 +620,7 @@ row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __
     CtaSmem& s = *reinterpret_cast<CtaSmem*>(smem_raw);
     ListSource src{logits, rows, nrows, p.V, p.H, (int)blockIdx.x, (int)gridDim.x, status};
     ListSink sink{tok_out, prob_out, p.k};
-    run_pipeline(s, src, sink, p.V, p.k, p.aligned != 0, status);
+    run_pipeline<kAligned>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.H * p.V, status);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1260,38 +1261,49 @@ bool bad_tree(const opt_tree_out* t) {
 }
 int check_launch() { return cudaGetLastError() == cudaSuccess ? OPT_TREE_OK : OPT_TREE_ERR_CUDA; }
 
-}  // namespace
+// Shared memory of a CTA of the persistent kernels for node budget n (one of two layouts).
+bool small_n(int n) { return n <= ot::kSmallN; }
+size_t cta_smem_bytes(int n) { return small_n(n) ? sizeof(ot::CtaSmemT<ot::kSmallN>) : sizeof(ot::CtaSmemT<ot::kMaxN>); }
+size_t layer_smem_bytes(int n) { return small_n(n) ? sizeof(ot::LayerScratchT<ot::kSmallN>) : sizeof(ot::LayerScratchT<ot::kMaxN>); }
 
-extern "C" {
+using BuildKernel = void (*)(ot::Workspace, ot::Params, const uint16_t*, opt_tree_out);
+template <int NCAP> BuildKernel build_variant(bool prune, bool aligned) {
+    return prune ? (aligned ? ot::build_kernel<true, NCAP, true> : ot::build_kernel<true, NCAP, false>)
+                 : (aligned ? ot::build_kernel<false, NCAP, true> : ot::build_kernel<false, NCAP, false>);
+}
+BuildKernel build_kernel_for(int n, bool prune, bool aligned) {
+    return small_n(n) ? build_variant<ot::kSmallN>(prune, aligned) : build_variant<ot::kMaxN>(prune, aligned);
+}
+template <class F> bool allow_smem(F* kernel, size_t bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+}
 
 // CTAs of the persistent kernels on the current device (one CTA of kThreads per SM as long as its
 // shared memory fits); 0 if there is no usable device.
-// Shared memory of a CTA of the persistent kernels for node budget n (one of two layouts).
-static bool small_n(int n) { return n <= ot::kSmallN; }
-static size_t cta_smem_bytes(int n) { return small_n(n) ? sizeof(ot::CtaSmemT<ot::kSmallN>) : sizeof(ot::CtaSmemT<ot::kMaxN>); }
-static size_t layer_smem_bytes(int n) { return small_n(n) ? sizeof(ot::LayerScratchT<ot::kSmallN>) : sizeof(ot::LayerScratchT<ot::kMaxN>); }
-
-static int persistent_grid(int n) {
+int persistent_grid(int n) {
     int dev = 0, per_sm = 0, sms = 0;
     constexpr int S = ot::kSmallN, L = ot::kMaxN;
-    const auto dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
-    if (cudaFuncSetAttribute(ot::build_kernel<false, S>, dyn, (int)sizeof(ot::CtaSmemT<S>)) != cudaSuccess ||
-        cudaFuncSetAttribute(ot::build_kernel<true, S>, dyn, (int)sizeof(ot::CtaSmemT<S>)) != cudaSuccess ||
-        cudaFuncSetAttribute(ot::build_kernel<false, L>, dyn, (int)sizeof(ot::CtaSmemT<L>)) != cudaSuccess ||
-        cudaFuncSetAttribute(ot::build_kernel<true, L>, dyn, (int)sizeof(ot::CtaSmemT<L>)) != cudaSuccess ||
-        cudaFuncSetAttribute(ot::row_topk_kernel, dyn, (int)sizeof(ot::CtaSmem)) != cudaSuccess ||
-        cudaFuncSetAttribute(ot::layer_step_kernel<S>, dyn, (int)sizeof(ot::LayerScratchT<S>)) != cudaSuccess ||
-        cudaFuncSetAttribute(ot::layer_step_kernel<L>, dyn, (int)sizeof(ot::LayerScratchT<L>)) != cudaSuccess ||
-        (small_n(n) ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ot::build_kernel<true, S>, ot::kThreads, sizeof(ot::CtaSmemT<S>))
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ot::build_kernel<true, L>, ot::kThreads, sizeof(ot::CtaSmemT<L>))) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    bool ok = allow_smem(ot::row_topk_kernel<true>, sizeof(ot::CtaSmem)) && allow_smem(ot::row_topk_kernel<false>, sizeof(ot::CtaSmem)) &&
+              allow_smem(ot::layer_step_kernel<S>, sizeof(ot::LayerScratchT<S>)) && allow_smem(ot::layer_step_kernel<L>, sizeof(ot::LayerScratchT<L>));
+    for (int v = 0; v < 4; ++v)
+        ok = ok && allow_smem(build_variant<S>(v & 1, v & 2), sizeof(ot::CtaSmemT<S>)) && allow_smem(build_variant<L>(v & 1, v & 2), sizeof(ot::CtaSmemT<L>));
+    int least = 1 << 30;                             // the variants share one grid: the smallest occupancy counts
+    for (int v = 0; v < 4 && ok; ++v) {
+        ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_kernel_for(n, v & 1, v & 2), ot::kThreads, cta_smem_bytes(n)) == cudaSuccess;
+        least = per_sm < least ? per_sm : least;
+    }
+    if (!ok || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
-    const int grid = per_sm * sms;
+    const int grid = least * sms;
     return grid >= 1 && grid <= ot::kMaxGrid ? grid : 0;
 }
+
+}  // namespace
+
+extern "C" {
 
 size_t opt_tree_workspace_bytes(const opt_tree_config* cfg) {
     if (!valid_cfg(cfg) || supported_cfg(cfg) != OPT_TREE_OK) return 0;
@@ -1355,9 +1367,7 @@ static int build_common(opt_tree_ctx* ctx, const void* draft, const int32_t* roo
     p.prune = prune;
     const long long init_threads = (long long)ctx->grid * ctx->mcap > B ? (long long)ctx->grid * ctx->mcap : B;
     launch_after(ot::init_build_kernel, dim3((unsigned)((init_threads + 255) / 256)), dim3(256), 0, st, ctx->ws, p, root_token);
-    auto kernel = small_n(ctx->cfg.n) ? (prune ? ot::build_kernel<true, ot::kSmallN> : ot::build_kernel<false, ot::kSmallN>)
-                                      : (prune ? ot::build_kernel<true, ot::kMaxN> : ot::build_kernel<false, ot::kMaxN>);
-    launch_after(kernel, dim3(ctx->grid), dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(draft), *out);
+    launch_after(build_kernel_for(ctx->cfg.n, prune != 0, p.aligned != 0), dim3(ctx->grid), dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(draft), *out);
     ctx->launches += 2;
     int rc = check_launch();
     if (rc == OPT_TREE_OK && rows_read &&
@@ -1446,7 +1456,7 @@ int opt_tree_layers_step(opt_tree_ctx* ctx, const void* frontier_logits, int32_t
     ot::Params pr = p;
     pr.H = nrows;                                            // the dense buffer is the "table" of the row step
     const int grid = nrows < ctx->grid ? nrows : ctx->grid;
-    launch_after(ot::row_topk_kernel, dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem), st,
+    launch_after(p.aligned ? ot::row_topk_kernel<true> : ot::row_topk_kernel<false>, dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem), st,
                  pr, static_cast<const uint16_t*>(frontier_logits), static_cast<const int32_t*>(nullptr), nrows, ctx->ws.rtok,
                  ctx->ws.rprob, ctx->ws.status);
     launch_after(small_n(ctx->cfg.n) ? ot::layer_step_kernel<ot::kSmallN> : ot::layer_step_kernel<ot::kMaxN>, dim3(B), dim3(ot::kTeam),
@@ -1462,8 +1472,8 @@ int opt_tree_row_softmax_topk(opt_tree_ctx* ctx, const void* logits, const int32
     if (nrows == 0) return OPT_TREE_OK;
     const ot::Params p = make_params(ctx, logits, 0.0f);
     const int grid = nrows < ctx->grid ? nrows : ctx->grid;
-    ot::row_topk_kernel<<<grid, ot::kThreads, sizeof(ot::CtaSmem), static_cast<cudaStream_t>(stream)>>>(
-        p, static_cast<const uint16_t*>(logits), rows, nrows, tok_out, prob_out, ctx->ws.status);
+    launch_after(p.aligned ? ot::row_topk_kernel<true> : ot::row_topk_kernel<false>, dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem),
+        static_cast<cudaStream_t>(stream), p, static_cast<const uint16_t*>(logits), rows, nrows, tok_out, prob_out, ctx->ws.status);
     ctx->launches++;
     return check_launch();
 }

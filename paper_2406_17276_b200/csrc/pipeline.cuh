@@ -108,17 +108,43 @@ __device__ void fetcher_role(CtaCore& s, Source& src, int* status, long long lim
 }
 
 // ---- issuer warp -------------------------------------------------------------------------------
-// A chunk of a row that bulk copies cannot take (see issuer_role), by the whole warp; rare, out of line.
-__device__ __noinline__ void copy_chunk_plain(uint16_t* stage, const uint16_t* src, int ne) {
+// A chunk of a row that does not start on a 16-byte boundary: the 16-byte granules that cover it are copied
+// whole (they may hold the end or the start of a neighbouring row), except for those that reach beyond the
+// table's logits [lo, hi): what is left of the chunk there, at most seven halves at either end of the table, the warp
+// copies with ordinary loads.  The chunk starts at half vec_offset(row) of the stage.
+// Measured (1999 rows of 50257 logits, B200): 2591 us with two-byte loads by the issuer warp, whose round trips
+// were the bound; 71.5 us with granule copies (2.8 TB/s), bound by the consumers' instructions.
+__device__ __noinline__ void copy_chunk_unaligned(uint16_t* stage, const uint16_t* src, int ne, const uint16_t* lo, const uint16_t* hi,
+                                                  unsigned long long* bar) {
     const int lane = threadIdx.x & 31;
-    const int padded = (ne + 7) & ~7;
-    for (int i = lane; i < padded; i += 32) stage[i] = i < ne ? __ldg(src + i) : (uint16_t)0xFF80u;
+    const uintptr_t lo16 = (reinterpret_cast<uintptr_t>(lo) + 15u) & ~(uintptr_t)15u, hi16 = reinterpret_cast<uintptr_t>(hi) & ~(uintptr_t)15u;
+    const uintptr_t first = reinterpret_cast<uintptr_t>(src), last = reinterpret_cast<uintptr_t>(src + ne);
+    const uintptr_t base = first & ~(uintptr_t)15u;                        // address of the stage's first half
+    const uintptr_t b0 = base < lo16 ? lo16 : base;
+    const uintptr_t up = (last + 15u) & ~(uintptr_t)15u, b1 = up > hi16 ? hi16 : up;
+    const bool bulk = b0 < b1;
+    const uintptr_t head_end = bulk ? (b0 > first ? b0 : first) : last;    // [first, head_end) and [tail, last) by ordinary loads
+    const uintptr_t tail = bulk ? b1 : last;
+    if (head_end > first || last > tail) {
+        for (uintptr_t a = first + 2u * lane; a < head_end; a += 64u) stage[(a - base) >> 1] = __ldg(reinterpret_cast<const uint16_t*>(a));
+        for (uintptr_t a = tail + 2u * lane; a < last; a += 64u) stage[(a - base) >> 1] = __ldg(reinterpret_cast<const uint16_t*>(a));
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // before a later bulk copy overwrites these bytes
+        __syncwarp();
+    }
+    if (lane == 0) {
+        if (bulk) {
+            mbar_expect_tx(bar, (uint32_t)(b1 - b0));
+            bulk_load(stage + ((b0 - base) >> 1), reinterpret_cast<const void*>(b0), (uint32_t)(b1 - b0), bar);
+        } else {
+            mbar_arrive(bar);
+        }
+    }
     __syncwarp();
 }
 
-// With `aligned` false (table base or row pitch not 16-byte aligned) the whole warp copies the
-// chunk with ordinary loads instead of a bulk copy.
-__device__ void issuer_role(CtaCore& s, int V, bool aligned, int* status) {
+// lo / hi: the first logit of the table and the one past its last (looked at when rows are not aligned).
+template <bool kAligned>
+__device__ void issuer_role(CtaCore& s, int V, const uint16_t* lo, const uint16_t* hi, int* status) {
     const int lane = threadIdx.x & 31;
     const int nchunks = (V + kChunkElems - 1) / kChunkElems;
     long long g = 0;
@@ -136,14 +162,13 @@ __device__ void issuer_role(CtaCore& s, int V, bool aligned, int* status) {
                 return;
             }
             const int ne = chunk_elems(V, c);
-            if (aligned) {
+            if (kAligned) {
                 if (lane == 0) {
                     mbar_expect_tx(&s.full_bar[st], (uint32_t)ne * 2u);
                     bulk_load(&s.stage[st][0], row + (size_t)c * kChunkElems, (uint32_t)ne * 2u, &s.full_bar[st]);
                 }
             } else {
-                copy_chunk_plain(&s.stage[st][0], row + (size_t)c * kChunkElems, ne);
-                if (lane == 0) mbar_arrive(&s.full_bar[st]);
+                copy_chunk_unaligned(&s.stage[st][0], row + (size_t)c * kChunkElems, ne, lo, hi, &s.full_bar[st]);
             }
         }
     }
@@ -153,12 +178,14 @@ __device__ void issuer_role(CtaCore& s, int V, bool aligned, int* status) {
 // A warp takes its share of a chunk out of the ring into registers and hands the stage back at once
 // (so the issuer can refill it while the exponentials run); a row's descriptor is only looked at for
 // its stop flag.
+template <bool kAligned>
 __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
     const int lane = threadIdx.x & 31, tid = cwarp * 32 + lane;     // index among the consumer threads
     const int nchunks = (V + kChunkElems - 1) / kChunkElems;
     ThreadAcc acc;
     acc.reset();
     ChunkRegs ch;
+    int off = 0;                                               // half of the stage at which the row in hand starts
     long long g = 0;
     for (int r = 0;; ++r) {
         for (int c = 0; c < nchunks; ++c, ++g) {
@@ -169,10 +196,12 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
                     if (tid == 0) s.stop_row = r;                  // the finishers poll this
                     return;
                 }
+                if (!kAligned) off = vec_offset(s.desc[r % kDescRing].row);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&s.desc_empty[r % kDesc]);      // this warp has looked at the descriptor
             }
-            chunk_take(ch, reinterpret_cast<const uint4*>(&s.stage[st][0]), (chunk_elems(V, c) + 7) >> 3, tid);
+            if (kAligned) chunk_take(ch, reinterpret_cast<const uint4*>(&s.stage[st][0]), chunk_elems(V, c) >> 3, tid);
+            else chunk_take_shifted(ch, reinterpret_cast<const uint4*>(&s.stage[st][0]), chunk_elems(V, c), off, tid);
             __syncwarp();
             if (lane == 0) mbar_arrive(&s.empty_bar[st]);          // the data is in registers: the stage is free
             chunk_chain(ch);
@@ -191,8 +220,8 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
 
 // ---- finisher warps ----------------------------------------------------------------------------
 // Sink::row_done(const RowDesc&, const RowOut&, FinScratch&) is called by the whole warp.
-template <class Sink>
-__device__ void finisher_role(CtaCore& s, Sink& sink, int fidx, int V, int k, bool aligned, int* status) {
+template <bool kAligned, class Sink>
+__device__ void finisher_role(CtaCore& s, Sink& sink, int fidx, int V, int k, int* status) {
     const int lane = threadIdx.x & 31;
     FinScratch& f = s.fin[fidx];
     for (int r = fidx;; r += kFinishers) {
@@ -215,26 +244,28 @@ __device__ void finisher_role(CtaCore& s, Sink& sink, int fidx, int V, int k, bo
         const RowSlot& slot = s.slot[sl];
         const RowDesc dsc = s.desc[r % kDescRing];
         RowOut out;
-        finish_row_warp(f, slot, dsc.row, V, k, aligned, out);
+        finish_row_warp<kAligned>(f, slot, dsc.row, V, k, out);
         __syncwarp();
         if (lane == 0) mbar_arrive(&s.free_bar[sl]);                              // the slot can be refilled
         sink.row_done(dsc, out, f);
     }
 }
 
-template <class Smem, class Source, class Sink>
-__device__ __forceinline__ void run_pipeline(Smem& sm, Source& src, Sink& sink, int V, int k, bool aligned, int* status) {
+// kAligned: the table's base and row pitch are multiples of 16 bytes (a compile-time choice, so that the code of the
+// common case carries nothing of the other).  lo / hi bound the table.
+template <bool kAligned, class Smem, class Source, class Sink>
+__device__ __forceinline__ void run_pipeline(Smem& sm, Source& src, Sink& sink, int V, int k, const uint16_t* lo, const uint16_t* hi, int* status) {
     CtaCore& s = sm.core;
     pipeline_init(s, sm.layer);
     grid_dependency_wait();                                // shared memory is set up; global memory from here on
     const int warp = threadIdx.x >> 5;
-    if (warp < kConsumerWarps) { consumer_role(s, warp, V, status); return; }
+    if (warp < kConsumerWarps) { consumer_role<kAligned>(s, warp, V, status); return; }
     const int helper = warp - kConsumerWarps;
-    if (helper == kHelperIssuer) issuer_role(s, V, aligned, status);
+    if (helper == kHelperIssuer) issuer_role<kAligned>(s, V, lo, hi, status);
     else if (helper == kHelperFetcher) fetcher_role(s, src, status);
     else if (helper == kHelperLayer) sink.layer_loop(sm.layer);
     else if (helper < kHelperFirstFinisher) sink.layer_assist(sm.layer, helper - kHelperLayer);
-    else finisher_role(s, sink, helper - kHelperFirstFinisher, V, k, aligned, status);
+    else finisher_role<kAligned>(s, sink, helper - kHelperFirstFinisher, V, k, status);
 }
 
 }  // namespace ot

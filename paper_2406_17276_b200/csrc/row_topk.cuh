@@ -32,6 +32,7 @@ constexpr int kVecPerThread = 4;                   // 16-byte vectors per consum
 constexpr int kChunkVecs = kConsumers * kVecPerThread;   // 2048
 constexpr int kChunkElems = kChunkVecs * 8;        // 16384 bf16 elements per stage (32 KB)
 constexpr int kStages = 4;                         // ring depth (128 KB)
+constexpr int kStageElems = kChunkElems + 8;       // a chunk that starts off a 16-byte boundary lies in one vector more
 constexpr int kSlots = kFinishers + 2;             // finished rows waiting for / held by finishers
 constexpr int kCandCap = 128;                      // candidate list capacity per row
 constexpr int kMaxFlag = 64;                       // flagged threads the fast finisher accepts
@@ -107,6 +108,7 @@ struct alignas(16) LayerScratchT {
     int cache_b, cache_d;                      // rsel / vals hold the top-n of this sequence after this layer (-1: nothing)
 };
 
+static_assert((kStageElems * 2) % 16 == 0, "bulk copies start on 16-byte boundaries");
 static_assert(sizeof(RowSlot) % 16 == 0, "slots must keep 16-byte alignment in an array");
 static_assert(sizeof(FinScratch) % 16 == 0 && offsetof(FinScratch, hist) % 16 == 0, "hist must be 16-byte aligned in every finisher's scratch");
 // rows between "descriptor written" and "finisher has its copy": kDesc known + 1 streaming + kSlots handed on
@@ -114,7 +116,7 @@ static_assert(kDescRing >= kDesc + 1 + kSlots + 1, "descriptor ring too short");
 
 // The row pipeline's part of a CTA's shared memory (the same for every node budget) ...
 struct alignas(128) CtaCore {
-    uint16_t stage[kStages][kChunkElems];
+    uint16_t stage[kStages][kStageElems];
     RowSlot slot[kSlots];
     FinScratch fin[kFinishers];
     RowDesc desc[kDescRing];                   // row r in entry r % kDescRing
@@ -161,6 +163,49 @@ struct ChunkRegs {
     uint32_t m2;
     float Ec;
 };
+
+// ---- rows that do not start on a 16-byte boundary (a vocabulary that is no multiple of 8, or an odd base) ----
+// The 16-byte granules that cover a chunk are copied whole and the logits are shifted into place on the way
+// into the registers, so that a thread holds the same logits, and a row's sums are formed in the same
+// order, wherever the row lies.  (Treating the granules themselves as the vectors would save the shift but make a
+// row's last bits depend on its address.)
+
+// Halves by which an address lies beyond a 16-byte boundary.
+__device__ __forceinline__ int vec_offset(const uint16_t* p) { return (int)((reinterpret_cast<uintptr_t>(p) & 15u) >> 1); }
+
+// Halves o .. o+7 of the sixteen in (a, b).
+__device__ __forceinline__ uint4 shift_halves(const uint4& a, const uint4& b, int o) {
+    uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y, w6 = b.z;
+    if (o & 4) { w0 = w2; w1 = w3; w2 = w4; w3 = w5; w4 = w6; w5 = b.w; }
+    if (o & 2) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
+    if (o & 1) {
+        w0 = __funnelshift_r(w0, w1, 16); w1 = __funnelshift_r(w1, w2, 16);
+        w2 = __funnelshift_r(w2, w3, 16); w3 = __funnelshift_r(w3, w4, 16);
+    }
+    return make_uint4(w0, w1, w2, w3);
+}
+// The first `cnt` (0 .. 8) halves of a vector; the rest read as -inf.
+__device__ __noinline__ uint4 mask_tail(uint4 v, int cnt) {
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (2 * i + 1 >= cnt) w[i] = (w[i] & 0xFFFFu) | 0xFF800000u;
+        if (2 * i >= cnt) w[i] = 0xFF80FF80u;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// chunk_take for a chunk of ne logits that starts at half o (the same for the whole warp) of its stage.
+__device__ __forceinline__ void chunk_take_shifted(ChunkRegs& c, const uint4* vec, int ne, int o, int tid) {
+#pragma unroll
+    for (int u = 0; u < kVecPerThread; ++u) {
+        const int v = tid + u * kConsumers;
+        c.w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+        if (v * 8 < ne) {
+            c.w[u] = shift_halves(vec[v], vec[v + 1], o);
+            if (v * 8 + 8 > ne) c.w[u] = mask_tail(c.w[u], ne - v * 8);
+        }
+    }
+}
 
 __device__ __forceinline__ void chunk_take(ChunkRegs& c, const uint4* vec, int nv, int tid) {
 #pragma unroll
@@ -423,20 +468,29 @@ __device__ __noinline__ void row_exact_warp(FinScratch& f, const uint16_t* row, 
 }
 
 // One 16-byte vector of the row (8 logits starting at token 8*vi) as four packed words; logits at or
-// beyond V read as -inf.  `aligned` rows take one vector load, others eight scalar loads.
-__device__ __noinline__ uint4 load_row_vec_scalar(const uint16_t* row, int vi, int V) {
+// beyond V read as -inf.  Aligned rows take one vector load, others the two granules that hold the vector, or, at
+// either end of the row, where those may reach beyond the table, eight scalar loads.
+__device__ __noinline__ uint4 load_row_vec_unaligned(const uint16_t* row, int vi, int V) {
+    const uint16_t* p = row + (size_t)vi * 8;
+    if (vi >= 1 && vi * 8 + 16 <= V) {
+        const int o = vec_offset(p);
+        const uint4* q = reinterpret_cast<const uint4*>(p - o);
+        const uint4 a = __ldg(q), b = __ldg(q + 1);
+        return shift_halves(a, b, o);
+    }
     uint32_t h[8];
-    for (int e = 0; e < 8; ++e) h[e] = (vi * 8 + e < V) ? (uint32_t)__ldg(row + vi * 8 + e) : 0xFF80u;
+    for (int e = 0; e < 8; ++e) h[e] = (vi * 8 + e < V) ? (uint32_t)__ldg(p + e) : 0xFF80u;
     return make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
 }
-__device__ __forceinline__ uint4 load_row_vec(const uint16_t* row, int vi, int V, bool aligned) {
-    if (aligned) {
+template <bool kAligned>
+__device__ __forceinline__ uint4 load_row_vec(const uint16_t* row, int vi, int V) {
+    if (kAligned) {
         uint4 v;
         asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
                      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(reinterpret_cast<const uint4*>(row) + vi));
         return v;
     }
-    return load_row_vec_scalar(row, vi, V);
+    return load_row_vec_unaligned(row, vi, V);
 }
 
 __device__ __noinline__ double exp_f64(double x) { return exp(x); }    // one copy of the routine for all its callers
@@ -462,7 +516,8 @@ __device__ __noinline__ void finish_many(FinScratch& f, int M, int kk, double m,
 }
 
 // Turns a finished slot into the row's k winners.  Whole finisher warp; f is its private scratch.
-__device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& slot, const uint16_t* row, int V, int k, bool aligned, RowOut& out) {
+template <bool kAligned>
+__device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& slot, const uint16_t* row, int V, int k, RowOut& out) {
     const int lane = threadIdx.x & 31;
     const int kk = k < V ? k : V;
     const int nvec = (V + 7) >> 3;
@@ -566,7 +621,7 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
                 w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
                 if (idx < total && fi < nflag) {
                     const int vi = (j / kVecPerThread) * kChunkVecs + (j % kVecPerThread) * kConsumers + f.flist[fi];
-                    if (vi < nvec) { vis[u] = vi; w[u] = load_row_vec(row, vi, V, aligned); }
+                    if (vi < nvec) { vis[u] = vi; w[u] = load_row_vec<kAligned>(row, vi, V); }
                 }
             }
             if (i0 == 0) {
