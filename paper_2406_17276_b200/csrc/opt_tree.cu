@@ -15,10 +15,12 @@ namespace ot {
 
 constexpr int kRowMul = 31;                 // row of (token t, depth d) = (t*31 + d) mod H
 constexpr int kSmallThreads = 256;          // block size of the mask / init kernels
-// Verify: one CTA per target row.  With 128 threads sixteen CTAs fit an SM, so the n + 1 rows of 32
-// sequences (c4: 2080 CTAs) are all resident at once instead of in two uneven waves; a thread keeps
-// eight 16-byte loads in flight.
-constexpr int kVerifyThreads = 128;
+// Verify: one CTA per target row, a thread keeps eight 16-byte loads in flight.  With 128 threads sixteen CTAs fit an
+// SM, so the n + 1 rows of 32 sequences (c4: 2080 CTAs) are all resident at once instead of in two uneven waves.  When
+// three CTAs of 512 threads per SM hold all rows (444 of them), a row is spread over four times the threads: few
+// rows are bound by the round trips of a CTA's loop (32000 logits: four of them with 128 threads, one with 512).
+// Measured (B200): 65 rows of 128256 logits 24.9 us with 128 threads, 12.8 with 512.
+constexpr int kVerifyThreads = 128, kVerifyThreadsFew = 512;
 
 __device__ __forceinline__ int row_of(int token, int depth, int H) {
     return (int)(((long long)token * kRowMul + depth) % H);
@@ -774,64 +776,87 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
     return v;
 }
 
+template <int T>
 struct VerifySmem {
-    unsigned long long red_u64[kVerifyThreads / 32];
+    unsigned long long red_u64[T / 32];
     int flag;
-    int hit;
 };
 
-// The end of a verification CTA: position j's token y is recorded; the CTA that records a sequence's
-// last token walks the tree: accept the child that carries the recorded token, until none does.
-__device__ void verify_tail(VerifySmem& s, const Workspace& w, const Params& p, int b, int j, int ns, int y,
+// The end of a verification CTA: position j's token y (thread 0's) is recorded; the CTA that records a sequence's
+// last token walks the tree: accept the child that carries the recorded token, until none does.  The tree and the
+// tokens go to shared memory first and one warp walks (a step is a few shared loads and a ballot per 32 nodes; with
+// the arrays read from L2 at every step by the whole block it took about a microsecond: 32 sequences, 2080 rows of 32000
+// logits, 26.5 us then, 20.4 now, 6.5 TB/s).
+// walk: 3 n + 1 ints of dynamic shared memory.
+template <int T>
+__device__ void verify_tail(VerifySmem<T>& s, int* walk, const Workspace& w, const Params& p, int b, int j, int ns, int y,
                             const int32_t* tok, const int32_t* par, int32_t* accept_len, int32_t* accept_tokens,
                             int32_t* accept_nodes, int32_t* next_root) {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31;
     int32_t* g = w.g + (size_t)b * (p.n + 1);
     if (tid == 0) {
         g[j] = y;
         __threadfence();
         s.flag = (atomicAdd(&w.vdone[b], 1) == ns);
+        __threadfence();
     }
     __syncthreads();
     if (!s.flag) return;
-    __threadfence();
 
-    // acceptance walk (block-wide child search; children of one node carry distinct tokens)
+    int *wtok = walk, *wpar = walk + p.n, *wg = walk + 2 * p.n;
+    for (int i = tid; i < ns; i += T) { wtok[i] = tok[i]; wpar[i] = par[i]; }
+    for (int i = tid; i <= ns; i += T) wg[i] = __ldcg(&g[i]);
+    __syncthreads();
+    if (tid >= 32) return;
     int32_t* at = accept_tokens + (size_t)b * (p.max_depth + 1);
     int32_t* an = accept_nodes + (size_t)b * p.max_depth;
-    for (int i = tid; i <= p.max_depth; i += kVerifyThreads) at[i] = -1;
-    for (int i = tid; i < p.max_depth; i += kVerifyThreads) an[i] = -1;
-    __syncthreads();
-    int cur = -1, A = 0;
-    for (int step = 0; step <= p.max_depth; ++step) {
-        const int yy = __ldcg(&g[cur + 1]);
-        if (tid == 0) { at[A] = yy; s.hit = -1; }
-        ++A;
-        __syncthreads();
-        if (A > p.max_depth) break;
-        for (int i = tid; i < ns; i += kVerifyThreads)
-            if (par[i] == cur && tok[i] == yy) s.hit = i;
-        __syncthreads();
-        const int hit = s.hit;
-        __syncthreads();
+    int cur = -1, A = 0, yy;
+    for (;;) {
+        yy = wg[cur + 1];
+        if (lane == 0) at[A] = yy;
+        if (++A > p.max_depth) break;
+        int hit = -1;                                        // (a child is packed behind its parent; siblings carry distinct tokens)
+        for (int i0 = (cur + 1) & ~31; i0 < ns && hit < 0; i0 += 32) {
+            const int i = i0 + lane;
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, i < ns && wpar[i] == cur && wtok[i] == yy);
+            if (m) hit = i0 + __ffs(m) - 1;
+        }
         if (hit < 0) break;
-        if (tid == 0) an[A - 1] = hit;
+        if (lane == 0) an[A - 1] = hit;
         cur = hit;
     }
-    if (tid == 0) {
+    for (int i = A + lane; i <= p.max_depth; i += 32) at[i] = -1;
+    for (int i = A - 1 + lane; i < p.max_depth; i += 32) an[i] = -1;
+    if (lane == 0) {
         accept_len[b] = A;
-        next_root[b] = __ldcg(&g[cur + 1]);
+        next_root[b] = yy;
         w.vdone[b] = 0;
     }
+}
+
+// Keys of the halves [0, h0) and [h1, V) of a row, at most seven at either end, that lie outside its whole 16-byte
+// granules: the best of those this thread takes.  (With the whole of an unaligned row read in single logits the
+// verification of 784 rows of 32003 logits took 31 us; 13.8 now.)
+__device__ __noinline__ unsigned long long best_of_ends(const uint16_t* row, int V, int h0, int h1) {
+    const int tid = threadIdx.x;
+    unsigned long long best = 0ull;
+    if (tid < h0) best = cand_key(__ldg(row + tid), (uint32_t)tid);
+    if (tid < V - h1) {
+        const unsigned long long key = cand_key(__ldg(row + h1 + tid), (uint32_t)(h1 + tid));
+        best = key > best ? key : best;
+    }
+    return best;
 }
 
 // Greedy verification.  CTA (j, b): j = 0 takes the target row after the root, j >= 1 the row after
 // kept node j-1; each finds the row's argmax (lowest token on ties).  The last CTA of a sequence
 // then walks the tree: accept the child that carries the target's token, until none does.
-__global__ void __launch_bounds__(kVerifyThreads)
+template <int T>
+__global__ void __launch_bounds__(T)
 verify_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const int32_t* __restrict__ root_token,
               opt_tree_out tree, int32_t* accept_len, int32_t* accept_tokens, int32_t* accept_nodes, int32_t* next_root) {
-    __shared__ VerifySmem s;
+    extern __shared__ int verify_walk[];
+    __shared__ VerifySmem<T> s;
     grid_dependency_wait();
     const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x;
     const int ns = tree.n_sel[b];
@@ -843,47 +868,45 @@ verify_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const 
     if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
     const uint16_t* row = target + (size_t)row_of(token, depth, p.H) * p.V;
 
-    unsigned long long best_key = 0ull;
-    if (p.aligned) {
-        const uint4* vec = reinterpret_cast<const uint4*>(row);
-        const int nv = p.V >> 3;
-        float best = -INFINITY;
-        int best_v = -1;
+    // the row's whole granules, from half h0 on (a row may start anywhere: unaligned rows only differ by their ends)
+    const int h0 = min((8 - vec_offset(row)) & 7, p.V);
+    const uint4* vec = reinterpret_cast<const uint4*>(row + h0);
+    const int nv = (p.V - h0) >> 3;
+    float best = -INFINITY;
+    int best_v = -1;
 #pragma unroll 1
-        for (int v0 = tid; v0 < nv; v0 += 8 * kVerifyThreads) {
-            uint4 q[8];
+    for (int v0 = tid; v0 < nv; v0 += 8 * T) {
+        uint4 q[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                q[u] = v0 + u * kVerifyThreads < nv ? ld_nc_v4(vec + v0 + u * kVerifyThreads)
-                                                    : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+        for (int u = 0; u < 8; ++u)
+            q[u] = v0 + u * T < nv ? ld_nc_v4(vec + v0 + u * T) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint32_t m2 = max_bf16x2(max_bf16x2(q[u].x, q[u].y), max_bf16x2(q[u].z, q[u].w));
-                const float f = fmaxf(__uint_as_float(m2 << 16), __uint_as_float(m2 & 0xFFFF0000u));
-                if (v0 + u * kVerifyThreads < nv && (f > best || best_v < 0)) { best = f; best_v = v0 + u * kVerifyThreads; }
-            }
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t m2 = max_bf16x2(max_bf16x2(q[u].x, q[u].y), max_bf16x2(q[u].z, q[u].w));
+            const float f = fmaxf(__uint_as_float(m2 << 16), __uint_as_float(m2 & 0xFFFF0000u));
+            if (v0 + u * T < nv && (f > best || best_v < 0)) { best = f; best_v = v0 + u * T; }
         }
-        if (best_v >= 0) {
-            const uint4 q = vec[best_v];
-            const uint32_t ww[4] = {q.x, q.y, q.z, q.w};
+    }
+    unsigned long long best_key = 0ull;
+    if (best_v >= 0) {
+        const uint4 q = vec[best_v];
+        const uint32_t ww[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-            for (int e = 7; e >= 0; --e) {
-                const uint32_t bits = (e & 1) ? (ww[e >> 1] >> 16) : (ww[e >> 1] & 0xFFFFu);
-                if (bf16_bits_to_float(bits) == best) best_key = cand_key(bits, (uint32_t)(best_v * 8 + e));
-            }
+        for (int e = 7; e >= 0; --e) {
+            const uint32_t bits = (e & 1) ? (ww[e >> 1] >> 16) : (ww[e >> 1] & 0xFFFFu);
+            if (bf16_bits_to_float(bits) == best) best_key = cand_key(bits, (uint32_t)(h0 + best_v * 8 + e));
         }
-    } else {
-        for (int v = tid; v < p.V; v += kVerifyThreads) {
-            const unsigned long long key = cand_key(__ldg(row + v), (uint32_t)v);
-            best_key = key > best_key ? key : best_key;
-        }
+    }
+    if (h0 + nv * 8 < p.V || h0 > 0) {
+        const unsigned long long key = best_of_ends(row, p.V, h0, h0 + nv * 8);
+        best_key = key > best_key ? key : best_key;
     }
     best_key = warp_max_u64(best_key);
     if ((tid & 31) == 0) s.red_u64[tid >> 5] = best_key;
     __syncthreads();
     if (tid == 0)
-        for (int q = 1; q < kVerifyThreads / 32; ++q) best_key = s.red_u64[q] > best_key ? s.red_u64[q] : best_key;
-    verify_tail(s, w, p, b, j, ns, (int32_t)cand_token(best_key), tok, par, accept_len, accept_tokens, accept_nodes, next_root);
+        for (int q = 1; q < T / 32; ++q) best_key = s.red_u64[q] > best_key ? s.red_u64[q] : best_key;
+    verify_tail<T>(s, verify_walk, w, p, b, j, ns, (int32_t)cand_token(best_key), tok, par, accept_len, accept_tokens, accept_nodes, next_root);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -918,22 +941,23 @@ constexpr int kSegTokens = kSegVecs * 8;
 constexpr int kMaxSeg = 640;                 // rows of up to 327 680 logits take the one-pass path
 constexpr int kSampleExpLimit = 1 << 22;     // |exponent| beyond which the single-precision pass cannot scale
 struct alignas(8) SegPart { float sum; int E; };       // a segment's sum of 2^(x*c - E), E an integer
+template <int T>
 struct SampleSmem {
     union { SegPart part[kMaxSeg]; double cum[kMaxSeg]; };   // per segment: its partial sum, then the running sum up to and including it
-    double wsum[kVerifyThreads / 32];
+    double wsum[T / 32];
     double S;
-    float wmax[kVerifyThreads / 32];
-    int wE[kVerifyThreads / 32];
+    float wmax[T / 32];
+    int wE[T / 32];
     int chosen, last_live, seg, live_seg;
 };
 
-// The plain way, for rows the one-pass path does not take (unaligned rows, very long rows, extreme
-// magnitudes): thread t owns the tokens [t*L, (t+1)*L); the row's maximum, then every thread's sum of
+// The plain way, for rows the one-pass path does not take (very long rows, extreme magnitudes): thread t owns the tokens [t*L, (t+1)*L); the row's maximum, then every thread's sum of
 // double-precision exponentials in token order, a scan over the threads, and the thread in whose stretch
 // u*S falls walks it once more.  Returns the drawn token to every thread.
-__device__ __noinline__ int sample_row_plain(SampleSmem& q, const uint16_t* row, int V, bool vec, double tau, double u) {
+template <int T>
+__device__ __noinline__ int sample_row_plain(SampleSmem<T>& q, const uint16_t* row, int V, bool vec, double tau, double u) {
     const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
-    const int L = (((V + kVerifyThreads - 1) / kVerifyThreads) + 7) & ~7;       // tokens per thread, a multiple of 8
+    const int L = (((V + T - 1) / T) + 7) & ~7;       // tokens per thread, a multiple of 8
     const int lo = min(tid * L, V), hi = min(lo + L, V);
     auto logit = [&](int v) -> float { return bf16_bits_to_float(__ldg(row + v)); };
     const uint4* rv = reinterpret_cast<const uint4*>(row);
@@ -954,7 +978,7 @@ __device__ __noinline__ int sample_row_plain(SampleSmem& q, const uint16_t* row,
     __syncthreads();
     mx = q.wmax[0];
 #pragma unroll
-    for (int i = 1; i < kVerifyThreads / 32; ++i) mx = fmaxf(mx, q.wmax[i]);
+    for (int i = 1; i < T / 32; ++i) mx = fmaxf(mx, q.wmax[i]);
     const double m = (double)mx;
     double mine = 0.0;
     int live = -1;                                           // last token of the stretch with a positive term
@@ -973,7 +997,7 @@ __device__ __noinline__ int sample_row_plain(SampleSmem& q, const uint16_t* row,
     __syncthreads();
     double base = 0.0, S = 0.0;                              // running sums before this warp / of the row, added up in one fixed order
 #pragma unroll
-    for (int i = 0; i < kVerifyThreads / 32; ++i) { if (i == wp) base = S; S += q.wsum[i]; }
+    for (int i = 0; i < T / 32; ++i) { if (i == wp) base = S; S += q.wsum[i]; }
     // a thread's stretch begins exactly where the previous thread's ends: the same expression on both sides
     double prev = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
     if (lane == 0) prev = 0.0;
@@ -995,21 +1019,41 @@ __device__ __noinline__ int sample_row_plain(SampleSmem& q, const uint16_t* row,
     return y;
 }
 
-// CTA (j, b) as in verify_kernel.  One pass over the row: warp w takes the segments w, w + 4, ...; a
-// segment's terms 2^(x*c - E) (c = log2(e) / tau, E an integer just above the segment's largest exponent)
+// Sum of the terms of the at most seven logits [t0, t1) at either end of a row, by one warp: a segment of its own.
+__device__ __noinline__ SegPart edge_part(const uint16_t* row, int t0, int t1, float c32, float c_hi, float c_lo) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t bits = t0 + lane < t1 ? (uint32_t)__ldg(row + t0 + lane) : 0xFF80u;
+    const uint32_t wkey = __reduce_max_sync(0xFFFFFFFFu, ord16(bits));
+    SegPart part;
+    part.sum = 0.0f; part.E = 0;
+    if (wkey > kOrdNegInf) {
+        const float Ef = rintf(fminf(fmaxf(fmaf(bf16_bits_to_float(ord16_inv(wkey)), c32, 1.0f), -1e9f), 1e9f));
+        const float x = fmaxf(bf16_bits_to_float(bits), -1e30f);
+        float sum = ex2_approx(fmaf(x, c_lo, fmaf(x, c_hi, -Ef)));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        part.sum = sum; part.E = (int)Ef;
+    }
+    return part;
+}
+
+// CTA (j, b) as in verify_kernel.  One pass over the row's whole granules: warp w takes the segments w, w + T/32, ...
+// of them (an unaligned row has two more segments, its ends before and after them); a segment's terms 2^(x*c - E) (c = log2(e) / tau, E an integer just above the segment's largest exponent)
 // are summed in single precision with ex2.approx and kept per segment, so the running sum is known in
 // token order at segment granularity.  The exponent x*c is formed with c split into a 16-bit head and a
 // tail: x is bf16, so x * head is exact, and the rounding of c does not grow with |x*c| (low temperatures).
 // Then: a double-precision scan over the segments, the segment in which u*S falls, and inside that segment
-// (512 logits, four per thread) double-precision exponentials and an exact scan.  What can differ from a
+// (512 logits, 512 / T per thread) double-precision exponentials and an exact scan.  What can differ from a
 // double-precision inverse CDF over the whole row is the placement of u*S relative to a segment's start, by
 // the rounding of the single-precision sums (a few 1e-7 of S).
-__global__ void __launch_bounds__(kVerifyThreads)
+template <int T>
+__global__ void __launch_bounds__(T, T == kVerifyThreads ? 16 : 3)
 verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const int32_t* __restrict__ root_token,
                       opt_tree_out tree, double tau, unsigned long long seed, unsigned long long step, int32_t* accept_len,
                       int32_t* accept_tokens, int32_t* accept_nodes, int32_t* next_root) {
-    __shared__ VerifySmem s;
-    __shared__ SampleSmem q;
+    extern __shared__ int verify_walk[];
+    __shared__ VerifySmem<T> s;
+    __shared__ SampleSmem<T> q;
     grid_dependency_wait();
     const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
     const int ns = tree.n_sel[b];
@@ -1021,21 +1065,28 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
     if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
     const uint16_t* row = target + (size_t)row_of(token, depth, p.H) * p.V;
     const double u = uniform53(seed, step, b, j);
-    const int nv = p.V >> 3, nseg = (nv + kSegVecs - 1) / kSegVecs;
+    const int h0 = min((8 - vec_offset(row)) & 7, p.V), nv = (p.V - h0) >> 3, h1 = h0 + nv * 8;
+    const int ngs = (nv + kSegVecs - 1) / kSegVecs, nseg = ngs + 2;    // segment 0: [0, h0); 1 ... ngs: 512 logits each; ngs + 1: [h1, V)
     const double c64 = kLog2eD / tau;
-    bool fast = p.aligned != 0 && nseg <= kMaxSeg && c64 < 1e30;
+    bool fast = nseg <= kMaxSeg && c64 < 1e30;
     int y = 0;
     if (fast) {
         const float c32 = (float)c64;
         const float c_hi = __uint_as_float(__float_as_uint(c32) & 0xFFFFFF00u);      // 16 significant bits
         const float c_lo = (float)(c64 - (double)c_hi);
-        const uint4* rv = reinterpret_cast<const uint4*>(row);
+        const uint4* rv = reinterpret_cast<const uint4*>(row + h0);
         if (tid == 0) { q.chosen = -1; q.last_live = -1; q.seg = 0x7FFFFFFF; q.live_seg = -1; }
         // two segments per turn: four 16-byte loads in flight per lane
         const unsigned long long chi2 = pack2(c_hi, c_hi), clo2 = pack2(c_lo, c_lo);
-        constexpr int kStep = kVerifyThreads / 32;
+        constexpr int kStep = T / 32;
+        if (wp == 0) {                                        // the ends (empty for aligned rows)
+            const SegPart zero = {0.0f, 0};
+            const SegPart head = h0 > 0 ? edge_part(row, 0, h0, c32, c_hi, c_lo) : zero;
+            const SegPart tail = h1 < p.V ? edge_part(row, h1, p.V, c32, c_hi, c_lo) : zero;
+            if (lane == 0) { q.part[0] = head; q.part[ngs + 1] = tail; }
+        }
 #pragma unroll 1
-        for (int sg0 = wp; sg0 < nseg; sg0 += 2 * kStep) {
+        for (int sg0 = wp; sg0 < ngs; sg0 += 2 * kStep) {
             const uint4 pad = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
             uint4 qq[2][2];
 #pragma unroll
@@ -1047,7 +1098,7 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int sg = sg0 + h * kStep;
-                if (sg >= nseg) break;                            // (warp-uniform)
+                if (sg >= ngs) break;                            // (warp-uniform)
                 const uint32_t ww[8] = {qq[h][0].x, qq[h][0].y, qq[h][0].z, qq[h][0].w, qq[h][1].x, qq[h][1].y, qq[h][1].z, qq[h][1].w};
                 uint32_t m2 = ww[0];
 #pragma unroll
@@ -1073,18 +1124,18 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
                 }
-                if (lane == 0) { q.part[sg].sum = sum; q.part[sg].E = (int)Ef; }
+                if (lane == 0) { q.part[sg + 1].sum = sum; q.part[sg + 1].E = (int)Ef; }
             }
         }
         __syncthreads();
         int e = -0x7FFFFFFF;
-        for (int sg = tid; sg < nseg; sg += kVerifyThreads) if (q.part[sg].sum > 0.0f) e = max(e, q.part[sg].E);
+        for (int sg = tid; sg < nseg; sg += T) if (q.part[sg].sum > 0.0f) e = max(e, q.part[sg].E);
         e = __reduce_max_sync(0xFFFFFFFFu, e);
         if (lane == 0) q.wE[wp] = e;
         __syncthreads();
         int Eg = q.wE[0];
 #pragma unroll
-        for (int i = 1; i < kVerifyThreads / 32; ++i) Eg = max(Eg, q.wE[i]);
+        for (int i = 1; i < T / 32; ++i) Eg = max(Eg, q.wE[i]);
         fast = Eg > -kSampleExpLimit && Eg < kSampleExpLimit;                     // the same for every thread
         if (fast) {
             if (wp == 0) {                                    // running sums over the segments, in token order
@@ -1108,7 +1159,7 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
             }
             __syncthreads();
             const double t = u * q.S;
-            for (int sg = tid; sg < nseg; sg += kVerifyThreads) {
+            for (int sg = tid; sg < nseg; sg += T) {
                 const double c = q.cum[sg];
                 if (c > t) atomicMin(&q.seg, sg);
                 if (c > (sg > 0 ? q.cum[sg - 1] : 0.0)) atomicMax(&q.live_seg, sg);
@@ -1117,21 +1168,23 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
             int sg = q.seg;
             if (sg == 0x7FFFFFFF) sg = q.live_seg < 0 ? 0 : q.live_seg;          // u*S rounded up to S: the last segment with a positive sum
             const double before = sg > 0 ? q.cum[sg - 1] : 0.0;
-            // inside the segment: four logits per thread, double precision
-            const int t0 = sg * kSegTokens + 4 * tid;
-            double ev[4] = {0.0, 0.0, 0.0, 0.0};
+            // inside the segment: kPer logits per thread, double precision
+            constexpr int kPer = kSegTokens / T;
+            const int seg0 = sg == 0 ? 0 : min(h0 + (sg - 1) * kSegTokens, h1);
+            const int seg1 = sg == 0 ? h0 : (sg > ngs ? p.V : min(seg0 + kSegTokens, h1));
+            const int t0 = seg0 + kPer * tid;
+            double ev[kPer];
             int live = -1;
-            if (t0 < p.V) {                                   // V is a multiple of 8, so all four exist
-                const uint2 x = *reinterpret_cast<const uint2*>(row + t0);
-                const uint32_t h[4] = {x.x & 0xFFFFu, x.x >> 16, x.y & 0xFFFFu, x.y >> 16};
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float xf = bf16_bits_to_float(h[i]);
-                    ev[i] = xf == -INFINITY ? 0.0 : exp2((double)xf * c64 - (double)Eg);
-                    if (ev[i] > 0.0) live = t0 + i;
-                }
+            for (int i = 0; i < kPer; ++i) {
+                const int tk = t0 + i;
+                const float xf = tk < seg1 ? bf16_bits_to_float(__ldg(row + tk)) : -INFINITY;
+                ev[i] = xf == -INFINITY ? 0.0 : exp2((double)xf * c64 - (double)Eg);
+                if (ev[i] > 0.0) live = tk;
             }
-            const double mine = ((ev[0] + ev[1]) + ev[2]) + ev[3];
+            double mine = ev[0];
+#pragma unroll
+            for (int i = 1; i < kPer; ++i) mine += ev[i];
             double incl = mine;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -1146,11 +1199,11 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
             if (lane == 0) prev = 0.0;
             const double excl_t = base + prev, incl_t = base + incl;
             atomicMax(&q.last_live, live);
-            if (incl_t > t && !(excl_t > t)) {                // this thread's four logits: one thread
+            if (incl_t > t && !(excl_t > t)) {                // this thread's logits: one thread
                 double run = excl_t;
                 int yy = live;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < kPer; ++i) {
                     run += ev[i];
                     if (run > t && ev[i] > 0.0) { yy = t0 + i; break; }
                 }
@@ -1158,11 +1211,11 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
             }
             __syncthreads();
             y = q.chosen;
-            if (y < 0) y = q.last_live < 0 ? min(sg * kSegTokens, p.V - 1) : q.last_live;   // the exact sums end just below u*S: the segment's last live token
+            if (y < 0) y = q.last_live < 0 ? min(seg0, p.V - 1) : q.last_live;   // the exact sums end just below u*S: the segment's last live token
         }
     }
-    if (!fast) y = sample_row_plain(q, row, p.V, p.aligned != 0, tau, u);
-    verify_tail(s, w, p, b, j, ns, y, tok, par, accept_len, accept_tokens, accept_nodes, next_root);
+    if (!fast) y = sample_row_plain<T>(q, row, p.V, p.aligned != 0, tau, u);
+    verify_tail<T>(s, verify_walk, w, p, b, j, ns, y, tok, par, accept_len, accept_tokens, accept_nodes, next_root);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1207,6 +1260,7 @@ struct opt_tree_ctx {
     void* base;
     size_t bytes;
     int device;
+    int sms;
     int grid;              // resident CTAs of the persistent kernels (SMs x occupancy)
     size_t smem;           // dynamic shared memory of one such CTA (cta_smem_bytes(cfg.n))
     int mcap;
@@ -1256,6 +1310,9 @@ void launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, 
     cfg.attrs = attr; cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+// Whether the verification's rows are so few that CTAs of kVerifyThreadsFew threads are all resident at once.
+bool few_rows(int n, int B, int sms) { return (long long)(n + 1) * B <= (long long)sms * 3; }
+size_t walk_smem(int n) { return (size_t)(3 * n + 1) * sizeof(int); }
 bool bad_tree(const opt_tree_out* t) {
     return !t || !t->token || !t->parent || !t->depth || !t->phat || !t->n_sel || !t->depth_reached || !t->expected_len;
 }
@@ -1328,7 +1385,8 @@ int opt_tree_create(opt_tree_ctx** out, const opt_tree_config* cfg) {
     ctx->mcap = (int)ot::mailbox_capacity(*cfg, ctx->grid);
     ctx->bytes = ot::carve(*cfg, ctx->grid, nullptr, nullptr);
     if ((long long)ctx->mcap * ctx->grid > 0x7FFFFFFFLL) { delete ctx; return OPT_TREE_ERR_UNSUPPORTED; }
-    if (cudaGetDevice(&ctx->device) != cudaSuccess || cudaMalloc(&ctx->base, ctx->bytes) != cudaSuccess) {
+    if (cudaGetDevice(&ctx->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || cudaMalloc(&ctx->base, ctx->bytes) != cudaSuccess) {
         cudaGetLastError();
         delete ctx;
         return OPT_TREE_ERR_CUDA;
@@ -1402,7 +1460,9 @@ int opt_tree_verify(opt_tree_ctx* ctx, const opt_tree_out* tree, const void* tar
         B < 1 || B > ctx->cfg.max_batch)
         return OPT_TREE_ERR_INVALID_ARG;
     const ot::Params p = make_params(ctx, target, 0.0f);
-    launch_after(ot::verify_kernel, dim3(ctx->cfg.n + 1, B), dim3(ot::kVerifyThreads), 0, static_cast<cudaStream_t>(stream),
+    const bool few = few_rows(ctx->cfg.n, B, ctx->sms);
+    launch_after(few ? ot::verify_kernel<ot::kVerifyThreadsFew> : ot::verify_kernel<ot::kVerifyThreads>, dim3(ctx->cfg.n + 1, B),
+                 dim3(few ? ot::kVerifyThreadsFew : ot::kVerifyThreads), walk_smem(ctx->cfg.n), static_cast<cudaStream_t>(stream),
                  ctx->ws, p, static_cast<const uint16_t*>(target), root_token, *tree, accept_len, accept_tokens, accept_nodes, next_root);
     ctx->launches++;
     return check_launch();
@@ -1415,7 +1475,9 @@ int opt_tree_verify_sampled(opt_tree_ctx* ctx, const opt_tree_out* tree, const v
         B < 1 || B > ctx->cfg.max_batch || !(tau > 0.0))
         return OPT_TREE_ERR_INVALID_ARG;
     const ot::Params p = make_params(ctx, target, 0.0f);
-    launch_after(ot::verify_sampled_kernel, dim3(ctx->cfg.n + 1, B), dim3(ot::kVerifyThreads), 0, static_cast<cudaStream_t>(stream),
+    const bool few = few_rows(ctx->cfg.n, B, ctx->sms);
+    launch_after(few ? ot::verify_sampled_kernel<ot::kVerifyThreadsFew> : ot::verify_sampled_kernel<ot::kVerifyThreads>, dim3(ctx->cfg.n + 1, B),
+                 dim3(few ? ot::kVerifyThreadsFew : ot::kVerifyThreads), walk_smem(ctx->cfg.n), static_cast<cudaStream_t>(stream),
                  ctx->ws, p, static_cast<const uint16_t*>(target), root_token, *tree, tau, (unsigned long long)seed,
                  (unsigned long long)step, accept_len, accept_tokens, accept_nodes, next_root);
     ctx->launches++;
@@ -1614,7 +1676,7 @@ extern "C" int opt_tree_verify_static(const opt_tree_config* cfg, const opt_tree
     p.V = cfg->V; p.H = cfg->H; p.n = cfg->n; p.k = cfg->k; p.kk = cfg->k < cfg->V ? cfg->k : cfg->V;
     p.max_depth = cfg->max_depth; p.Dcap = cfg->max_depth < cfg->n ? cfg->max_depth : cfg->n;
     p.aligned = ((reinterpret_cast<uintptr_t>(target) & 15u) == 0 && (cfg->V % 8) == 0) ? 1 : 0;
-    ot::verify_kernel<<<dim3(cfg->n + 1, B), ot::kVerifyThreads, 0, st>>>(
+    ot::verify_kernel<ot::kVerifyThreads><<<dim3(cfg->n + 1, B), ot::kVerifyThreads, walk_smem(cfg->n), st>>>(
         ws, p, static_cast<const uint16_t*>(target), root_token, *tree, accept_len, accept_tokens, accept_nodes, next_root);
     if (cudaGetLastError() != cudaSuccess) return OPT_TREE_ERR_CUDA;
     if (device_status && cudaMemcpyAsync(device_status, ws.status, sizeof(int32_t), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
