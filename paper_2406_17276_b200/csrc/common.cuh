@@ -30,6 +30,12 @@ enum { kHelperIssuer = 0, kHelperFetcher = 1, kHelperLayer = 2, kHelperFirstAssi
 constexpr int kMaxK = 32;
 constexpr int kMaxN = 1024;
 
+// The kernels' dynamic shared memory.  Functions that are not inlined get the offset of what they work on and not a
+// reference: through a generic pointer every access to it would be a generic load, store or atomic.
+extern __shared__ __align__(128) unsigned char ot_smem[];
+template <class S> __device__ __forceinline__ S& smem_at(int offset) { return *reinterpret_cast<S*>(ot_smem + offset); }
+__device__ __forceinline__ int smem_offset(const void* p);
+
 // Device status codes mirror opt_tree_status.
 constexpr int kErrTimeout = -4;
 constexpr int kErrInternal = -5;
@@ -74,6 +80,8 @@ constexpr uint32_t kOrdNegInf = 0x007Fu;    // ord16(0xFF80)
 // Small PTX wrappers.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ int smem_offset(const void* p) { return (int)(smem_u32(p) - smem_u32(ot_smem)); }
 
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;

@@ -256,7 +256,7 @@ struct BuildSink {
     __device__ bool first_layer_direct(const RowDesc& d, const RowOut& r, const SeqWork& sw) {
         const int lane = threadIdx.x & 31;
         const double ph = lane < r.kk ? d.pphat * r.p : 0.0;              // Eq. 2
-        const double esub = warp_sum(ph);                                  // (the order update_running_warp sums in)
+        const double esub = warp_sum(ph);                                  // (the order update_running_team sums in)
         const bool more = 1 < p.Dcap && (esub > (double)p.delta);          // loop test of Algorithm 1 with E = 0
         if (r.kk > p.n || !more) return false;
         const TreeOut to = tree_out(out, p, d.b);
@@ -386,15 +386,12 @@ struct BuildSink {
         cp_async_wait_all();
         __syncwarp();
         team_sync();
-        const LayerJob j = ls.job;
-        const int nR = select_running_team(ls, j, lane, w.status);
+        const int nR = select_running_team<LS>(smem_offset(&ls), lane, w.status);
         int kept_old = 0;
 #pragma unroll
         for (int q = 0; q < kTeamWarps; ++q) kept_old += ls.scan_c[q];
         const int cnt = nR - kept_old;                      // new members = the rows of the next layer
-        double part = 0.0;
-        for (int i = lane; i < nR; i += 32) part += ls.vals[i];
-        const double esub = warp_sum(part);
+        const double esub = running_esub(ls, nR);
         const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
         bool more = d < p.Dcap && (esub - eprev > (double)p.delta);
         const TreeOut to = tree_out(out, p, b);
@@ -419,8 +416,27 @@ struct BuildSink {
             if (to.esub_trace) for (int i = d + lane; i < d_end; i += 32) to.esub_trace[i] = esub;
             __syncwarp();
         }
-        pack_tree_warp(ls, sw, to, d_end, nR, p.n, p.max_depth, esub, w.status);
+        pack(ls, sw, to, b, d_end, nR, esub);
         return -1;
+    }
+    // The tree of sequence b from the running top-n in the scratch.  A tree of up to two nodes per lane of the layer warp is
+    // packed by that warp: with the team's barriers one sequence of n = 10 takes 83.2 us a step, without 81.9; at n = 512 the
+    // team's four warps save about 10 us.
+    static constexpr int kPackAlone = 64;
+    template <class LS>
+    __device__ void pack(LS& ls, const SeqWork& sw, const TreeOut& to, int b, int d, int nR, double esub) {
+        if ((threadIdx.x & 31) == 0) {
+            LayerJob& j = ls.job;
+            j.kind = 4; j.d = d; j.n = p.n; j.nR_old = nR; j.b = b; j.max_depth = p.max_depth;
+            j.T_tok = sw.T_tok; j.T_par = sw.T_par;
+            ls.last_esub = esub;
+        }
+        __syncwarp();
+        const bool alone = p.n <= kPackAlone;
+        if (!alone) team_sync();
+        pack_tree<LS>(smem_offset(&ls), to, (int)(threadIdx.x & 31), alone ? 32 : kTeam, w.status);
+        if (!alone) team_sync();                            // the scratch may be written again
+        __syncwarp();
     }
     // The layer warp follows its sequences (layer_follow); whenever a layer is complete it hands the
     // selection to the whole team: the job goes into shared memory, the team barrier starts it.  The
@@ -437,11 +453,13 @@ struct BuildSink {
         const int tt = tw * 32 + (int)(threadIdx.x & 31);
         for (;;) {
             team_sync();
-            const LayerJob j = ls.job;
-            if (j.kind == 0) return;
-            if (j.kind == 2) select_running_team(ls, j, tt, w.status);
-            else if (j.fsize * j.k <= kStageCap) select_layer_team<kPrune>(ls, j, tt, w.status);
-            else select_layer_team_big<kPrune>(ls, j, tt, w.status);
+            const int kind = ls.job.kind, at = smem_offset(&ls);
+            if (kind == 0) return;
+            if (kind == 2) select_running_team<LS>(at, tt, w.status);
+            else if (kind == 3) update_running_team<LS>(at, tt, w.status);
+            else if (kind == 4) { pack_tree<LS>(at, tree_out(out, p, ls.job.b), tt, kTeam, w.status); team_sync(); }
+            else if (ls.job.fsize * ls.job.k <= kStageCap) select_layer_team<kPrune, LS>(at, tt, w.status);
+            else select_layer_team_big<kPrune, LS>(at, tt, w.status);
         }
     }
     template <class LS>
@@ -520,21 +538,42 @@ struct BuildSink {
                         if (small) cp_async_wait_all();       // the staged candidates are in shared memory
                         __syncwarp();
                         team_sync();                          // ... and, with the job, visible to the assistants
-                        const LayerJob j = ls.job;
-                        if (small) select_layer_team<kPrune>(ls, j, lane, w.status);
-                        else select_layer_team_big<kPrune>(ls, j, lane, w.status);
+                        if (small) select_layer_team<kPrune, LS>(smem_offset(&ls), lane, w.status);
+                        else select_layer_team_big<kPrune, LS>(smem_offset(&ls), lane, w.status);
                     }
                     if (early) publish_layer(ls, b, d, nl, g0);
-                    bool more = update_running_warp(ls, sw, tree_out(out, p, b), d, nl, p.n, p.Dcap, p.max_depth, p.delta,
-                                                    w.status);
-                    if (lane == 0) { ls.cache_b = b; ls.cache_d = d; }                // rsel / vals now hold this top-n
+                    double esub;
+                    int nR;
+                    {
+                        const bool cached = ls.cache_b == b && ls.cache_d == d - 1;   // rsel / vals hold the top-n before this layer
+                        const int nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
+                        __syncwarp();
+                        if (lane == 0) {
+                            LayerJob& j = ls.job;
+                            j.kind = 3; j.fsize = nl; j.nR_old = nR_old; j.off = cached ? 1 : 0;
+                            j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
+                            ls.cache_b = b; ls.cache_d = d;
+                        }
+                        __syncwarp();
+                        team_sync();
+                        nR = update_running_team<LS>(smem_offset(&ls), lane, w.status);
+                        esub = running_esub(ls, nR);
+                    }
+                    const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
+                    bool more = d < p.Dcap && (esub - eprev > (double)p.delta);       // loop test of Algorithm 1
+                    const TreeOut to = tree_out(out, p, b);
+                    if (lane == 0) {
+                        if (to.esub_trace) to.esub_trace[d - 1] = esub;
+                        sw.st[kStNR] = nR;
+                        *sw.E_prev = esub;
+                    }
+                    __syncwarp();
+                    if (!more) pack(ls, sw, to, b, d, nR, esub);
                     int sent = nl;                             // rows of the next layer
                     if (kPrune && more) {
                         // The new layer's nodes among the n largest are the tail of the ascending list rsel
                         // (their gids are the largest); only they are drafted from.
                         const int gid0 = (d - 1) * p.n;
-                        const int nR = ls.last_nR;
-                        const double esub = ls.last_esub;
                         int mine = 0;
                         for (int i = lane; i < nR; i += 32) mine += ls.rsel[i] >= gid0 ? 1 : 0;
                         sent = __reduce_add_sync(0xFFFFFFFFu, mine);
@@ -547,10 +586,9 @@ struct BuildSink {
                             // of Algorithm 1 would go on testing a gain of zero: to the depth limit if the
                             // threshold is negative, else for one more layer.
                             const int d_end = p.delta < 0.0f ? p.Dcap : d + 1;
-                            const TreeOut to = tree_out(out, p, b);
                             if (to.esub_trace) for (int i = d + lane; i < d_end; i += 32) to.esub_trace[i] = esub;
                             __syncwarp();
-                            pack_tree_warp(ls, sw, to, d_end, nR, p.n, p.max_depth, esub, w.status);
+                            pack(ls, sw, to, b, d_end, nR, esub);
                             more = false;
                         }
                     } else if (more && !early) {
@@ -580,8 +618,7 @@ struct BuildSink {
 template <bool kPrune, int NCAP, bool kAligned>
 __global__ void __launch_bounds__(kThreads)
 build_kernel(Workspace w, Params p, const uint16_t* __restrict__ draft, opt_tree_out out) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    CtaSmemT<NCAP>& s = *reinterpret_cast<CtaSmemT<NCAP>*>(smem_raw);
+    CtaSmemT<NCAP>& s = *reinterpret_cast<CtaSmemT<NCAP>*>(ot_smem);
     BuildSource<kPrune> src{w, p, draft};
     BuildSink<kPrune> sink{w, p, out};
     run_pipeline<kAligned>(s, src, sink, p.V, p.k, draft, draft + (size_t)p.H * p.V, w.status);
@@ -618,8 +655,7 @@ template <bool kAligned>
 __global__ void __launch_bounds__(kThreads)
 row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __restrict__ rows, int nrows,
                 int32_t* tok_out, double* prob_out, int* status) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    CtaSmem& s = *reinterpret_cast<CtaSmem*>(smem_raw);
+    CtaSmem& s = *reinterpret_cast<CtaSmem*>(ot_smem);
     ListSource src{logits, rows, nrows, p.V, p.H, (int)blockIdx.x, (int)gridDim.x, status};
     ListSink sink{tok_out, prob_out, p.k};
     run_pipeline<kAligned>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.H * p.V, status);
@@ -647,11 +683,10 @@ template <int NCAP>
 __global__ void __launch_bounds__(kTeam)
 layer_step_kernel(Workspace w, Params p, int fstride, opt_tree_out out, int32_t* next_tokens, int32_t* next_parent,
                   int32_t* next_count) {
-    extern __shared__ __align__(16) unsigned char ls_raw[];
-    LayerScratchT<NCAP>& ls = *reinterpret_cast<LayerScratchT<NCAP>*>(ls_raw);
+    LayerScratchT<NCAP>& ls = *reinterpret_cast<LayerScratchT<NCAP>*>(ot_smem);
     grid_dependency_wait();
-    const int b = blockIdx.x, tt = threadIdx.x, lane = tt & 31;
-    for (int i = tt; i < 3 * 256; i += kTeam) (&ls.thist[0][0])[i] = 0;
+    const int b = blockIdx.x, tt = threadIdx.x;
+    for (int i = tt; i < 4 * 256; i += kTeam) (&ls.thist[0][0])[i] = 0;
     const SeqWork sw = seq_work(w, p, b);
     const int d = sw.st[kStDepth], fsize = sw.st[kStFsize];
     if (d == 0) {                                            // this sequence stopped at an earlier layer
@@ -681,20 +716,35 @@ layer_step_kernel(Workspace w, Params p, int fstride, opt_tree_out out, int32_t*
         j.fmap = nullptr; j.nR_old = 0; j.off = 0; j.Rnew = nullptr;
     }
     __syncthreads();
-    const LayerJob j = ls.job;
-    const int nl = small ? select_layer_team<false>(ls, j, tt, w.status) : select_layer_team_big<false>(ls, j, tt, w.status);
-    if (tt >= 32) return;                                    // the rest is one warp's work
-    const bool more = update_running_warp(ls, sw, tree_out(out, p, b), d, nl, p.n, p.Dcap, p.max_depth, p.delta, w.status);
+    using LS = LayerScratchT<NCAP>;
+    const int at = smem_offset(&ls);
+    const int nl = small ? select_layer_team<false, LS>(at, tt, w.status) : select_layer_team_big<false, LS>(at, tt, w.status);
+    if (tt == 0) {
+        LayerJob& j = ls.job;
+        j.fsize = nl; j.nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]); j.off = 0;
+        j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
+    }
+    team_sync();
+    const int nR = update_running_team<LS>(at, tt, w.status);
+    const double esub = running_esub(ls, nR);
+    const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
+    const bool more = d < p.Dcap && (esub - eprev > (double)p.delta);     // loop test of Algorithm 1
+    const TreeOut to = tree_out(out, p, b);
+    if (to.esub_trace && tt == 0) to.esub_trace[d - 1] = esub;
     if (more) {
         const int gid0 = (d - 1) * p.n;
-        for (int i = lane; i < nl; i += 32) {
+        for (int i = tt; i < nl; i += kTeam) {
             next_tokens[(size_t)b * p.n + i] = ls.ltok[i];
             next_parent[(size_t)b * p.n + i] = __ldcg(&sw.T_par[gid0 + i]);
             w.front_phat[(size_t)b * p.n + i] = __longlong_as_double((long long)(ls.lkeys[i] - 1ull));
         }
-        if (lane == 0) { sw.st[kStDepth] = d + 1; sw.st[kStFsize] = nl; next_count[b] = nl; }
-    } else if (lane == 0) {
-        sw.st[kStDepth] = 0; next_count[b] = 0;
+        team_sync();                                         // (everyone has read E and |R|)
+        if (tt == 0) { sw.st[kStNR] = nR; *sw.E_prev = esub; sw.st[kStDepth] = d + 1; sw.st[kStFsize] = nl; next_count[b] = nl; }
+    } else {
+        if (tt == 0) { ls.last_esub = esub; ls.job.nR_old = nR; ls.job.max_depth = p.max_depth; }
+        team_sync();
+        pack_tree<LS>(at, to, tt, kTeam, w.status);
+        if (tt == 0) { sw.st[kStDepth] = 0; next_count[b] = 0; }
     }
 }
 
@@ -855,7 +905,7 @@ template <int T>
 __global__ void __launch_bounds__(T)
 verify_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const int32_t* __restrict__ root_token,
               opt_tree_out tree, int32_t* accept_len, int32_t* accept_tokens, int32_t* accept_nodes, int32_t* next_root) {
-    extern __shared__ int verify_walk[];
+    int* verify_walk = reinterpret_cast<int*>(ot_smem);
     __shared__ VerifySmem<T> s;
     grid_dependency_wait();
     const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x;
@@ -1051,7 +1101,7 @@ __global__ void __launch_bounds__(T, T == kVerifyThreads ? 16 : 3)
 verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const int32_t* __restrict__ root_token,
                       opt_tree_out tree, double tau, unsigned long long seed, unsigned long long step, int32_t* accept_len,
                       int32_t* accept_tokens, int32_t* accept_nodes, int32_t* next_root) {
-    extern __shared__ int verify_walk[];
+    int* verify_walk = reinterpret_cast<int*>(ot_smem);
     __shared__ VerifySmem<T> s;
     __shared__ SampleSmem<T> q;
     grid_dependency_wait();
@@ -1231,8 +1281,7 @@ struct NeverSource {
 };
 __global__ void __launch_bounds__(kThreads)
 wait_probe_kernel(int* result, const unsigned long long* zero_words, long long limit, int polls) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    CtaSmem& s = *reinterpret_cast<CtaSmem*>(smem_raw);
+    CtaSmem& s = *reinterpret_cast<CtaSmem*>(ot_smem);
     pipeline_init(s.core, s.layer);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) {

@@ -37,7 +37,7 @@ __device__ __forceinline__ void pipeline_init(CtaCore& s, LS& layer) {
         s.stop_row = 0x7FFFFFFF;
         mbar_fence_init();
     }
-    for (int i = threadIdx.x; i < 3 * 256; i += kThreads) (&layer.thist[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < 4 * 256; i += kThreads) (&layer.thist[0][0])[i] = 0;
     if (threadIdx.x == 0) { layer.cache_b = -1; layer.cache_d = -1; }
     __syncthreads();
 }

@@ -79,6 +79,10 @@ struct LayerJob {                  // what the layer warp hands its assistants (
     // kind 2 (pruned draft, one selection over the running top-n and the candidates together):
     int nR_old, off;               // old top-n in keys[0..nR_old), candidates from keys[off] (off even, >= nR_old)
     int32_t* Rnew;                 // the new top-n's gids, ascending
+    // kind 3 (running top-n after a layer of fsize nodes): off: the old one is still in rsel / vals, else in Rold
+    const int32_t* Rold;
+    // kind 4 (pack the running top-n in rsel / vals, nR_old nodes, as the tree of sequence b)
+    int b, max_depth;
 };
 
 constexpr int kStageCap = 1024;                    // candidates of a layer that the shared-memory staging holds
@@ -89,7 +93,9 @@ constexpr int kSmallN = 256;                       // node budgets up to this us
 // CTA's shared memory (and with it the SM's L1) where it is best for them.
 template <int NCAP>
 struct alignas(16) LayerScratchT {
-    static constexpr int kKeys = (2 * NCAP > kStageCap ? 2 * NCAP : kStageCap) + 2;
+    static constexpr int kSurvivors = 2 * NCAP > kStageCap ? 2 * NCAP : kStageCap;   // candidates that keys can hold
+    static constexpr bool kWideGids = 2 * NCAP > kStageCap;    // gids holds as many as keys
+    static constexpr int kKeys = kSurvivors + 2;
     unsigned long long keys[kKeys];            // staged candidate keys, then the keys of R + layer
     unsigned long long lkeys[NCAP];            // keys of the new layer, slot order
     double vals[NCAP];                         // path values of the new running top-n
@@ -97,13 +103,11 @@ struct alignas(16) LayerScratchT {
     int gids[2 * NCAP];
     int rsel[NCAP];                            // gids of the new running top-n, ascending
     int ltok[NCAP];                            // tokens of the new layer, slot order
-    int hist[256];
-    int thist[3][256];                         // the team's digit counts, rotating (all zero between selections)
+    int thist[4][256];                         // the team's digit counts, rotating (all zero between selections); all four: coarse counts
     unsigned long long red_or[kTeamWarps], red_and[kTeamWarps];
     int scan_a[kTeamWarps], scan_b[kTeamWarps];
     LayerJob job;
-    double last_esub;                          // E_sub and |R| of the last update of the running top-n
-    int last_nR;
+    double last_esub;                          // E_sub of the tree that is to be packed
     int scan_c[kTeamWarps];
     int cache_b, cache_d;                      // rsel / vals hold the top-n of this sequence after this layer (-1: nothing)
 };

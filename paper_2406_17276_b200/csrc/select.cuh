@@ -1,7 +1,7 @@
-// K2 / K3: layer selection (the n candidates of largest path value) by the layer team, running
-// E_sub(T, n), the loop test of Algorithm 1 and the scan-based tree packer by the layer warp.
+// K2 / K3: layer selection (the n candidates of largest path value), running E_sub(T, n) and the
+// tree packer by the layer team.
 //
-// Selection never sorts: an 8-pass radix select on the 64-bit keys finds the threshold of the
+// Selection never sorts: a radix select of at most 8 passes on the 64-bit keys finds the threshold of the
 // "need" largest, then an ordered compaction (ballot scans) emits the kept elements in index
 // order, which is exactly the storage order the method wants (candidate-index order for a layer;
 // (depth, slot) order for the running top-n, which is also the packed order of the final tree).
@@ -21,91 +21,6 @@ __device__ __forceinline__ unsigned long long warp_or_u64(unsigned long long v) 
 __device__ __forceinline__ unsigned long long warp_and_u64(unsigned long long v) {
     const uint32_t lo = __reduce_and_sync(0xFFFFFFFFu, (uint32_t)v), hi = __reduce_and_sync(0xFFFFFFFFu, (uint32_t)(v >> 32));
     return ((unsigned long long)hi << 32) | lo;
-}
-
-// Threshold of the `need` largest keys among keyf(0..N); key 0 means "not an element".
-// key_or / key_and are the bitwise OR / AND over all non-zero keys (the caller folds them into the
-// sweep that stages the keys): the bits on which all keys agree need no pass, and a pass whose
-// threshold bin holds exactly the elements still needed ends the search.  On return the selection
-// is {key > thr} plus the first need_eq elements (lowest indices) with key == thr.
-// Requires 1 <= need <= number of non-zero keys.  Whole warp; hist has 256 ints.
-template <class KeyFn>
-__device__ void warp_radix_select(KeyFn keyf, int N, int need, int* hist, unsigned long long key_or,
-                                  unsigned long long key_and, unsigned long long& thr, int& need_eq) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long diff = key_or ^ key_and;
-    if (diff == 0ull) { thr = key_or; need_eq = need; return; }          // all elements equal
-    int top = 64 - __clzll((long long)diff);                             // the low `top` bits vary
-    unsigned long long prefix = top == 64 ? 0ull : ((key_or >> top) << top);
-    while (top > 0) {
-        const int wbits = top < 8 ? top : 8, shift = top - wbits;
-        const unsigned int dmask = (1u << wbits) - 1u;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) hist[lane * 8 + j] = 0;
-        __syncwarp();
-        #pragma unroll 1
-        for (int i = lane; i < N; i += 32) {
-            const unsigned long long key = keyf(i);
-            const bool match = key != 0ull && (top == 64 || (key >> top) == (prefix >> top));
-            if (match) atomicAdd(&hist[(int)((unsigned int)(key >> shift) & dmask)], 1);
-        }
-        __syncwarp();
-        int c[8], mine = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { c[j] = hist[lane * 8 + j]; mine += c[j]; }
-        int incl = mine;                                   // suffix sums over lanes from the top
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int u = __shfl_down_sync(0xFFFFFFFFu, incl, o);
-            if (lane + o < 32) incl += u;
-        }
-        const int above = incl - mine;
-        const bool here = above < need && need <= incl;
-        int bin = 0, nd = 0, cb = 0;
-        if (here) {
-            int a = above;
-            bin = lane * 8;
-#pragma unroll
-            for (int b = 7; b >= 0; --b) {                 // highest bin whose suffix count reaches need
-                if (nd == 0) {
-                    if (a + c[b] >= need) { bin = lane * 8 + b; nd = need - a; cb = c[b]; }
-                    else a += c[b];
-                }
-            }
-        }
-        const int src = __ffs(__ballot_sync(0xFFFFFFFFu, here)) - 1;
-        bin = __shfl_sync(0xFFFFFFFFu, bin, src);
-        need = __shfl_sync(0xFFFFFFFFu, nd, src);
-        cb = __shfl_sync(0xFFFFFFFFu, cb, src);
-        prefix |= (unsigned long long)bin << shift;
-        top = shift;
-        __syncwarp();
-        if (cb == need && prefix != 0ull) { thr = prefix - 1ull; need_eq = 0; return; }   // the whole bin belongs
-    }
-    thr = prefix;
-    need_eq = need;
-}
-
-// Emits, in index order, the elements with key > thr and the first need_eq with key == thr.
-// emit(pos, i) is called once per kept element; returns the number kept.  Whole warp.
-template <class KeyFn, class EmitFn>
-__device__ int warp_compact_selected(KeyFn keyf, int N, unsigned long long thr, int need_eq, EmitFn emit) {
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
-    int eq_seen = 0, taken = 0;
-    #pragma unroll 1
-    for (int i0 = 0; i0 < N; i0 += 32) {
-        const int i = i0 + lane;
-        const unsigned long long key = i < N ? keyf(i) : 0ull;
-        const bool eq = i < N && key == thr;
-        const unsigned eqm = __ballot_sync(0xFFFFFFFFu, eq);
-        const bool take = i < N && (key > thr || (eq && eq_seen + __popc(eqm & below) < need_eq));
-        const unsigned tm = __ballot_sync(0xFFFFFFFFu, take);
-        if (take) emit(taken + __popc(tm & below), i);
-        eq_seen += __popc(eqm);
-        taken += __popc(tm);
-    }
-    return taken;
 }
 
 // Per-sequence state and arrays in the workspace (device pointers already offset to the sequence).
@@ -180,19 +95,20 @@ __device__ __forceinline__ int team_excl_scan(int v, int* wtot, int tw, int& tot
     return base + before;
 }
 
-// Threshold of the `need` largest keys among s.keys[0..N) (0 = not an element); see
-// warp_radix_select for the result and the shortcuts.  The digit counts rotate through three
+// Threshold of the `need` largest keys among s.keys[0..N); key 0 means "not an element".  key_or / key_and
+// are the bitwise OR / AND over all non-zero keys (the caller folds them into the sweep that stages the keys): the
+// bits on which all keys agree need no pass, and a pass whose threshold bin holds exactly the elements still needed
+// ends the search.  On return the selection is {key > thr} plus the first need_eq elements (lowest indices) with
+// key == thr.  Requires 1 <= need <= number of non-zero keys.  The digit counts rotate through three
 // arrays that are all zero on entry: pass p counts into array p % 3 and clears the one pass p-1
 // read, so one barrier per pass is enough.  Returns the array that is left non-zero (the caller
 // clears it after its next barrier), or -1.
-// kGlobal: the keys are not staged; they are read from the candidate words gw[0..N) in global memory
-// (all written: the caller has looked at every one), eight loads in flight per thread.
 __device__ __forceinline__ unsigned long long key_of_word(unsigned long long x) {
     return x == ~0ull ? 0ull : (x & 0x7FFFFFFFFFFFFFFFull) + 1ull;
 }
-template <bool kGlobal, class LS>
-__device__ int team_radix_select(LS& s, const unsigned long long* gw, int N, int need, int tt, unsigned long long key_or,
-                                 unsigned long long key_and, unsigned long long& thr, int& need_eq) {
+template <class LS>
+__device__ int team_radix_select(LS& s, int N, int need, int tt, unsigned long long key_or, unsigned long long key_and,
+                                 unsigned long long& thr, int& need_eq) {
     const int lane = threadIdx.x & 31;
     const unsigned long long diff = key_or ^ key_and;
     if (diff == 0ull) { thr = key_or; need_eq = need; return -1; }       // all elements equal
@@ -203,26 +119,11 @@ __device__ int team_radix_select(LS& s, const unsigned long long* gw, int N, int
         const int wbits = top < 8 ? top : 8, shift = top - wbits;
         const unsigned int dmask = (1u << wbits) - 1u;
         int* hist = s.thist[pass % 3];
-        if (!kGlobal) {
-            #pragma unroll 1
-            for (int i = tt; i < N; i += kTeam) {
-                const unsigned long long key = s.keys[i];
-                const bool match = key != 0ull && (top == 64 || (key >> top) == (prefix >> top));
-                if (match) atomicAdd(&hist[(int)((unsigned int)(key >> shift) & dmask)], 1);
-            }
-        } else {
-            #pragma unroll 1
-            for (int i0 = tt; i0 < N; i0 += 8 * kTeam) {
-                unsigned long long x[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) x[u] = i0 + u * kTeam < N ? ld_relaxed_u64(&gw[i0 + u * kTeam]) : ~0ull;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const unsigned long long key = key_of_word(x[u]);
-                    const bool match = key != 0ull && (top == 64 || (key >> top) == (prefix >> top));
-                    if (match) atomicAdd(&hist[(int)((unsigned int)(key >> shift) & dmask)], 1);
-                }
-            }
+        #pragma unroll 1
+        for (int i = tt; i < N; i += kTeam) {
+            const unsigned long long key = s.keys[i];
+            const bool match = key != 0ull && (top == 64 || (key >> top) == (prefix >> top));
+            if (match) atomicAdd(&hist[(int)((unsigned int)(key >> shift) & dmask)], 1);
         }
         team_sync();
         int c[8], mine = 0;
@@ -270,14 +171,22 @@ __device__ int team_radix_select(LS& s, const unsigned long long* gw, int N, int
 // by the layer warp).  On return (after a last barrier) the new layer's nodes are in T and its
 // tokens and keys in s.ltok / s.lkeys.  Returns nl.
 template <bool kPrune, class LS>
-__device__ __noinline__ int select_layer_team(LS& s, const LayerJob& j, int tt, int* status) {
+__device__ __noinline__ int select_layer_team(int at, int tt, int* status) {
+    LS& s = smem_at<LS>(at);
+    const LayerJob& j = s.job;
+    const int k = j.k;
+    int32_t *const T_tok = j.T_tok, *const T_par = j.T_par;
+    double* const T_phat = j.T_phat;
+    const int32_t* const fmap = j.fmap;
     const int lane = threadIdx.x & 31, tw = tt >> 5;
-    const int N = j.fsize * j.k;
+    const int N = j.fsize * k;
     const int nvalid = j.fsize * j.kk;
     const int nl = nvalid < j.n ? nvalid : j.n;
     const int gid0 = (j.d - 1) * j.n;
-    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(j.cand_phat);
-    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(j.cand_tok);
+    double* const cand_phat = j.cand_phat;
+    int32_t* const cand_tok = j.cand_tok;
+    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(cand_phat);
+    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(cand_tok);
     unsigned long long ko = 0ull, ka = ~0ull;
     #pragma unroll 1
     for (int i = tt; i < N; i += kTeam) {
@@ -298,12 +207,12 @@ __device__ __noinline__ int select_layer_team(LS& s, const LayerJob& j, int tt, 
     for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
     // every candidate has been read: the arrays are free for the next layer's rows once they are zero again
     #pragma unroll 1
-    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(&j.cand_phat[i]) = make_uint4(0, 0, 0, 0);
+    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
     #pragma unroll 1
-    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(&j.cand_tok[i]) = make_uint4(0, 0, 0, 0);
+    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
     unsigned long long thr = 0ull;                         // with no more candidates than wanted, all of them (key > 0) are taken
     int need_eq = 0, dirty = -1;
-    if (nl < nvalid) dirty = team_radix_select<false>(s, nullptr, N, nl, tt, ko, ka, thr, need_eq);
+    if (nl < nvalid) dirty = team_radix_select(s, N, nl, tt, ko, ka, thr, need_eq);
     // ordered compaction: thread tt owns a contiguous stretch of candidates
     const int per = (N + kTeam - 1) / kTeam;
     const int lo = min(tt * per, N), hi = min(lo + per, N);
@@ -323,7 +232,7 @@ __device__ __noinline__ int select_layer_team(LS& s, const LayerJob& j, int tt, 
     }
     int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
     if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }     // everyone is past the last pass
-    int frow = lo / j.k, frank = lo - frow * j.k;          // frontier row and sibling rank of candidate i, carried along
+    int frow = lo / k, frank = lo - frow * k;          // frontier row and sibling rank of candidate i, carried along
     #pragma unroll 1
     for (int i = lo; i < hi; ++i) {
         const unsigned long long key = s.keys[i];
@@ -332,14 +241,14 @@ __device__ __noinline__ int select_layer_team(LS& s, const LayerJob& j, int tt, 
         if (take) {
             const unsigned int t32 = (unsigned int)s.toks[i];
             const int tok = t32 == ~0u ? -1 : (int)(t32 & 0x7FFFFFFFu);
-            j.T_tok[gid0 + pos] = tok;
+            T_tok[gid0 + pos] = tok;
             s.ltok[pos] = tok;
-            j.T_par[gid0 + pos] = kPrune ? __ldcg(&j.fmap[frow]) : frow;
-            j.T_phat[gid0 + pos] = __longlong_as_double((long long)(key - 1ull));
+            T_par[gid0 + pos] = kPrune ? __ldcg(&fmap[frow]) : frow;
+            T_phat[gid0 + pos] = __longlong_as_double((long long)(key - 1ull));
             s.lkeys[pos] = key;
             ++pos;
         }
-        if (++frank == j.k) { frank = 0; ++frow; }
+        if (++frank == k) { frank = 0; ++frow; }
     }
     if (total != nl) set_status(status, kErrInternal);
     team_sync();
@@ -355,14 +264,22 @@ __device__ __noinline__ int select_layer_team(LS& s, const LayerJob& j, int tt, 
 // gid0 .. gid0+cnt in candidate order with tokens and keys in s.ltok / s.lkeys, and s.scan_c sums
 // to the number of old members kept.  Returns |new top-n|.
 template <class LS>
-__device__ __noinline__ int select_running_team(LS& s, const LayerJob& j, int tt, int* status) {
+__device__ __noinline__ int select_running_team(int at, int tt, int* status) {
+    LS& s = smem_at<LS>(at);
+    const LayerJob& j = s.job;
+    const int k = j.k;
+    int32_t *const T_tok = j.T_tok, *const T_par = j.T_par, *const Rnew = j.Rnew;
+    double* const T_phat = j.T_phat;
+    const int32_t* const fmap = j.fmap;
     const int lane = threadIdx.x & 31, tw = tt >> 5;
-    const int N = j.fsize * j.k, nRo = j.nR_old, off = j.off, M = off + N;
+    const int N = j.fsize * k, nRo = j.nR_old, off = j.off, M = off + N;
     const int nvalid = j.fsize * j.kk;
     const int need = nRo + nvalid < j.n ? nRo + nvalid : j.n;
     const int gid0 = (j.d - 1) * j.n;
-    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(j.cand_phat);
-    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(j.cand_tok);
+    double* const cand_phat = j.cand_phat;
+    int32_t* const cand_tok = j.cand_tok;
+    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(cand_phat);
+    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(cand_tok);
     unsigned long long ko = 0ull, ka = ~0ull;
     #pragma unroll 1
     for (int i = tt; i < M; i += kTeam) {
@@ -387,12 +304,12 @@ __device__ __noinline__ int select_running_team(LS& s, const LayerJob& j, int tt
 #pragma unroll
     for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
     #pragma unroll 1
-    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(&j.cand_phat[i]) = make_uint4(0, 0, 0, 0);
+    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
     #pragma unroll 1
-    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(&j.cand_tok[i]) = make_uint4(0, 0, 0, 0);
+    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
     unsigned long long thr = 0ull;
     int need_eq = 0, dirty = -1;
-    if (need < nRo + nvalid) dirty = team_radix_select<false>(s, nullptr, M, need, tt, ko, ka, thr, need_eq);
+    if (need < nRo + nvalid) dirty = team_radix_select(s, M, need, tt, ko, ka, thr, need_eq);
     const int per = (M + kTeam - 1) / kTeam;
     const int lo = min(tt * per, M), hi = min(lo + per, M);
     int gt = 0, eq = 0;
@@ -442,15 +359,15 @@ __device__ __noinline__ int select_running_team(LS& s, const LayerJob& j, int tt
             const unsigned int t32 = (unsigned int)s.toks[c];
             const int tok = t32 == ~0u ? -1 : (int)(t32 & 0x7FFFFFFFu);
             gid = gid0 + slot;
-            j.T_tok[gid] = tok;
-            j.T_par[gid] = __ldcg(&j.fmap[c / j.k]);      // layer slot of the node behind the candidate's frontier row
-            j.T_phat[gid] = __longlong_as_double((long long)(key - 1ull));
+            T_tok[gid] = tok;
+            T_par[gid] = __ldcg(&fmap[c / k]);      // layer slot of the node behind the candidate's frontier row
+            T_phat[gid] = __longlong_as_double((long long)(key - 1ull));
             s.ltok[slot] = tok;
             s.lkeys[slot] = key;
         }
         s.rsel[pos] = gid;
         s.vals[pos] = __longlong_as_double((long long)(key - 1ull));
-        j.Rnew[pos] = gid;
+        Rnew[pos] = gid;
         ++pos;
     }
     if (total != need) set_status(status, kErrInternal);
@@ -458,19 +375,143 @@ __device__ __noinline__ int select_running_team(LS& s, const LayerJob& j, int tt
     return need;
 }
 
+// Ordered compaction of the elements i in [0, M) with keys[i] > thr, and the first need_eq with keys[i] == thr: their keys
+// go to s.lkeys and idx[i] to s.ltok.  `dirty`: digit counts to clear.  Returns their number (two barriers at most).
+template <class LS>
+__device__ __forceinline__ int team_compact_layer(LS& s, const unsigned long long* keys, const int* idx, int M, unsigned long long thr,
+                                                  int need_eq, int dirty, int tt) {
+    const int tw = tt >> 5;
+    const int per = (M + kTeam - 1) / kTeam, lo = min(tt * per, M), hi = min(lo + per, M);
+    int gt = 0, eq = 0;
+    #pragma unroll 1
+    for (int i = lo; i < hi; ++i) { gt += keys[i] > thr ? 1 : 0; eq += keys[i] == thr ? 1 : 0; }
+    int total_eq, total, eq_take = 0;
+    if (need_eq > 0) {
+        const int eq_before = team_excl_scan(eq, s.scan_a, tw, total_eq);
+        eq_take = need_eq - eq_before;
+        eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
+    }
+    int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
+    if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }
+    #pragma unroll 1
+    for (int i = lo; i < hi; ++i) {
+        bool take = keys[i] > thr;
+        if (keys[i] == thr && eq_take > 0) { take = true; --eq_take; }
+        if (take) { s.lkeys[pos] = keys[i]; s.ltok[pos] = idx[i]; ++pos; }
+    }
+    return total;
+}
+
+// The same selection with every sweep over the candidate words in global memory (rare, see select_layer_team_big).
+template <class LS>
+__device__ __noinline__ int team_select_global(int at, const unsigned long long* gph, int N, int need, int tt) {
+    LS& s = smem_at<LS>(at);
+    const int tw = tt >> 5;
+    unsigned long long prefix = 0ull;
+    int left = need;
+    team_sync();                                           // (the counts have been cleared)
+    for (int shift = 56; shift >= 0; shift -= 8) {         // one digit per sweep; the counts go to s.thist[0]
+        #pragma unroll 4
+        for (int i = tt; i < N; i += kTeam) {
+            const unsigned long long key = key_of_word(ld_relaxed_u64(&gph[i]));
+            if (key != 0ull && (shift == 56 || (key >> (shift + 8)) == (prefix >> (shift + 8))))
+                atomicAdd(&s.thist[0][(int)((key >> shift) & 255ull)], 1);
+        }
+        team_sync();
+        int a = 0, b = 255;
+        while (b > 0 && a + s.thist[0][b] < left) { a += s.thist[0][b]; --b; }
+        left -= a;
+        prefix |= (unsigned long long)b << shift;
+        team_sync();
+        s.thist[0][tt] = 0; s.thist[0][tt + kTeam] = 0;
+        team_sync();
+    }
+    const unsigned long long thr = prefix;                 // the need-th largest key; `left` of its copies belong
+    const int per = (N + kTeam - 1) / kTeam, lo = min(tt * per, N), hi = min(lo + per, N);
+    int gt = 0, eq = 0;
+    #pragma unroll 4
+    for (int i = lo; i < hi; ++i) {
+        const unsigned long long key = key_of_word(ld_relaxed_u64(&gph[i]));
+        gt += key > thr ? 1 : 0;
+        eq += key == thr && key != 0ull ? 1 : 0;
+    }
+    int total_eq, total;
+    const int eq_before = team_excl_scan(eq, s.scan_a, tw, total_eq);
+    int eq_take = left - eq_before;
+    eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
+    int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
+    #pragma unroll 1
+    for (int i = lo; i < hi; ++i) {
+        const unsigned long long key = key_of_word(ld_relaxed_u64(&gph[i]));
+        bool take = key > thr;
+        if (key == thr && key != 0ull && eq_take > 0) { take = true; --eq_take; }
+        if (take) { s.lkeys[pos] = key; s.ltok[pos] = i; ++pos; }
+    }
+    return total;
+}
+
+// The largest bin of the 1024 counts in s.thist at which at least `need` elements lie at or above; `at_or_above` is their
+// number (the elements must be that many).  Every warp for itself.
+template <class LS>
+__device__ __forceinline__ int warp_coarse_bin(const LS& s, int need, int& at_or_above) {
+    const int lane = threadIdx.x & 31;
+    const int* h = &s.thist[0][0];
+    int mine = 0;
+#pragma unroll 8
+    for (int q = 0; q < 32; ++q) mine += h[lane * 32 + ((q + lane) & 31)];     // (rotated: no bank conflicts)
+    auto find = [&](int v, int want, int& above) -> int {                       // the lane in which the want-th from the top lies
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_down_sync(0xFFFFFFFFu, incl, o);
+            if (lane + o < 32) incl += u;
+        }
+        const unsigned hm = __ballot_sync(0xFFFFFFFFu, incl - v < want && want <= incl);
+        const int src = hm ? __ffs(hm) - 1 : 0;
+        above = __shfl_sync(0xFFFFFFFFu, incl - v, src);
+        return src;
+    };
+    int a0, a1;
+    const int l0 = find(mine, need, a0);
+    const int c = h[l0 * 32 + lane];
+    const int l1 = find(c, need - a0, a1);
+    at_or_above = a0 + a1 + __shfl_sync(0xFFFFFFFFu, c, l1);
+    return l0 * 32 + l1;
+}
+// Coarse bin of a path-value key: sixteen bins per factor of two, 1 at the top, everything below 2^-63 at the bottom.
+constexpr int kCoarseShift = 48, kCoarseBase = 16 * 0x3FF - 1023, kFineShift = kCoarseShift - 10;
+__device__ __forceinline__ int coarse_bin(unsigned long long key) {
+    const int e = (int)(key >> kCoarseShift) - kCoarseBase;
+    return e < 0 ? 0 : (e > 1023 ? 1023 : e);
+}
+
 // The team's selection for layers with more candidates than the shared-memory staging holds
-// (1024 < N <= n*k): the same steps, but every sweep reads the candidate words from global memory
-// (they sit in L2), a thread's loads eight at a time.  The candidate arrays are cleared at the end.
+// (kStageCap < N <= n*k).  Bound by the round trips of 128 threads to the candidate words in L2 (a sweep over
+// 8192 of them takes about 4 us), so there are two sweeps and no more: the first counts the candidates into coarse
+// bins of their path values, the second marks those at or above the bin in which the threshold lies, usually few
+// more than n (if there are too many, one more sweep splits that bin in 1024).  Only these are brought into shared
+// memory, in index order, where the exact selection is the ordinary one.  If they still do not fit (over a thousand
+// ties, or a threshold below 2^-63) further sweeps read global memory once per digit.
+// Measured (two sequences, n = 512, k = 16, B200): 980 us per build with a sweep per digit, tokens fetched one after
+// the other in the emission and the running top-n by one warp; 440 us with both by the team.
 template <bool kPrune, class LS>
-__device__ __noinline__ int select_layer_team_big(LS& s, const LayerJob& j, int tt, int* status) {
+__device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
+    LS& s = smem_at<LS>(at);
+    const LayerJob& j = s.job;
+    const int k = j.k;
+    int32_t *const T_tok = j.T_tok, *const T_par = j.T_par;
+    double* const T_phat = j.T_phat;
+    const int32_t* const fmap = j.fmap;
     const int lane = threadIdx.x & 31, tw = tt >> 5;
-    const int N = j.fsize * j.k;
+    const int N = j.fsize * k;
     const int nvalid = j.fsize * j.kk;
     const int nl = nvalid < j.n ? nvalid : j.n;
     const int gid0 = (j.d - 1) * j.n;
-    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(j.cand_phat);
-    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(j.cand_tok);
-    unsigned long long ko = 0ull, ka = ~0ull;
+    double* const cand_phat = j.cand_phat;
+    int32_t* const cand_tok = j.cand_tok;
+    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(cand_phat);
+    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(cand_tok);
+    int* coarse = &s.thist[0][0];
     #pragma unroll 1
     for (int i0 = tt; i0 < N; i0 += 8 * kTeam) {
         unsigned long long x[8];
@@ -480,90 +521,144 @@ __device__ __noinline__ int select_layer_team_big(LS& s, const LayerJob& j, int 
         for (int u = 0; u < 8; ++u) {
             if (!(x[u] >> 63)) x[u] = poll_phat_word(&gph[i0 + u * kTeam], status);      // not written yet: read again
             const unsigned long long key = key_of_word(x[u]);
-            if (key) { ko |= key; ka &= key; }
+            if (key) atomicAdd(&coarse[coarse_bin(key)], 1);
         }
     }
-    ko = warp_or_u64(ko); ka = warp_and_u64(ka);
-    if (lane == 0) { s.red_or[tw] = ko; s.red_and[tw] = ka; }
     team_sync();
-    ko = 0ull; ka = ~0ull;
+    int S;
+    const int bin = warp_coarse_bin(s, nl, S);
+    unsigned long long low = bin > 0 ? (unsigned long long)(bin + kCoarseBase) << kCoarseShift : 1ull;      // what counts is at or above this key
+    if (S > LS::kSurvivors && bin > 0) {
+        const int over = S - coarse[bin];                  // elements in the bins above
+        team_sync();
+        #pragma unroll
+        for (int q = 0; q < 1024 / kTeam; ++q) coarse[q * kTeam + tt] = 0;
+        team_sync();
+        #pragma unroll 1
+        for (int i0 = tt; i0 < N; i0 += 8 * kTeam) {
+            unsigned long long x[8];
 #pragma unroll
-    for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
-    unsigned long long thr = 0ull;
-    int need_eq = 0, dirty = -1;
-    if (nl < nvalid) dirty = team_radix_select<true>(s, gph, N, nl, tt, ko, ka, thr, need_eq);
-    // ordered compaction: thread tt owns a contiguous stretch of candidates (a multiple of 8 long)
-    const int per = (((N + kTeam - 1) / kTeam) + 7) & ~7;
-    const int lo = min(tt * per, N), hi = min(lo + per, N);
-    int gt = 0, eq = 0;
+            for (int u = 0; u < 8; ++u) x[u] = i0 + u * kTeam < N ? ld_relaxed_u64(&gph[i0 + u * kTeam]) : ~0ull;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const unsigned long long key = key_of_word(x[u]);
+                if (key && coarse_bin(key) == bin) atomicAdd(&coarse[(int)((key >> kFineShift) & 1023ull)], 1);
+            }
+        }
+        team_sync();
+        const int sub = warp_coarse_bin(s, nl - over, S);
+        S += over;
+        low |= (unsigned long long)sub << kFineShift;
+    }
+    // second sweep: marks (one bit per candidate, kept where the new layer's keys will go) and their number
+    unsigned int* marks = reinterpret_cast<unsigned int*>(s.lkeys);
+    const int per = (((N + kTeamWarps - 1) / kTeamWarps) + 255) & ~255;        // candidates per warp
+    const int lo = min(tw * per, N), hi = min(lo + per, N);
+    int mine = 0;
     #pragma unroll 1
-    for (int i0 = lo; i0 < hi; i0 += 8) {
+    for (int i0 = lo; i0 < hi; i0 += 256) {
         unsigned long long x[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = i0 + u < hi ? ld_relaxed_u64(&gph[i0 + u]) : ~0ull;
+        for (int u = 0; u < 8; ++u) x[u] = i0 + u * 32 + lane < hi ? ld_relaxed_u64(&gph[i0 + u * 32 + lane]) : ~0ull;
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const unsigned long long key = key_of_word(x[u]);
-            gt += key > thr ? 1 : 0;
-            eq += (key == thr && key != 0ull) ? 1 : 0;
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, key >= low);
+            if (lane == u && i0 + u * 32 < hi) marks[(i0 >> 5) + u] = m;
+            mine += __popc(m);
         }
     }
-    int total_eq, total;
-    int eq_take = 0;
-    if (need_eq > 0) {
-        const int eq_before = team_excl_scan(eq, s.scan_a, tw, total_eq);
-        eq_take = need_eq - eq_before;
-        eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
-    }
-    int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
-    if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }
-    if (gt + eq_take > 0) {
+    if (lane == 0) s.scan_a[tw] = mine;
+    team_sync();
+    #pragma unroll
+    for (int q = 0; q < 1024 / kTeam; ++q) coarse[q * kTeam + tt] = 0;         // (every warp has its bin)
+    constexpr int kCap = LS::kSurvivors;
+    int* idx = LS::kWideGids ? s.gids : s.toks;
+    int total = 0;
+    if (S <= kCap) {
+        int pos = 0;
+        for (int q = 0; q < tw; ++q) pos += s.scan_a[q];
         #pragma unroll 1
-        for (int i = lo; i < hi; ++i) {
-            const unsigned long long key = key_of_word(ld_relaxed_u64(&gph[i]));
-            bool take = key > thr;
-            if (key == thr && key != 0ull && eq_take > 0) { take = true; --eq_take; }
-            if (take) {
-                unsigned int t32 = ld_relaxed_u32(&gtk[i]);
-                if (!(t32 >> 31)) t32 = poll_tok_word(&gtk[i], status);
-                const int tok = t32 == ~0u ? -1 : (int)(t32 & 0x7FFFFFFFu);
-                j.T_tok[gid0 + pos] = tok;
-                s.ltok[pos] = tok;
-                j.T_par[gid0 + pos] = kPrune ? __ldcg(&j.fmap[i / j.k]) : i / j.k;
-                j.T_phat[gid0 + pos] = __longlong_as_double((long long)(key - 1ull));
-                s.lkeys[pos] = key;
-                ++pos;
-            }
+        for (int i0 = lo; i0 < hi; i0 += 1024) {
+            const int c0 = i0 + lane * 32;
+            unsigned m = c0 < hi ? marks[c0 >> 5] : 0u;
+            int tot;
+            int p = pos + warp_excl_scan(__popc(m), tot);
+            for (; m; m &= m - 1) { if (p < kCap) idx[p] = c0 + __ffs(m) - 1; ++p; }
+            pos += tot;
         }
+        team_sync();
+        unsigned long long ko = 0ull, ka = ~0ull;
+        #pragma unroll 1
+        for (int i0 = tt; i0 < S; i0 += 4 * kTeam) {
+            unsigned long long x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = i0 + u * kTeam < S ? ld_relaxed_u64(&gph[idx[i0 + u * kTeam]]) : ~0ull;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i0 + u * kTeam < S) {
+                    const unsigned long long key = key_of_word(x[u]);
+                    s.keys[i0 + u * kTeam] = key;
+                    ko |= key; ka &= key;
+                }
+        }
+        ko = warp_or_u64(ko); ka = warp_and_u64(ka);
+        if (lane == 0) { s.red_or[tw] = ko; s.red_and[tw] = ka; }
+        team_sync();
+        ko = 0ull; ka = ~0ull;
+#pragma unroll
+        for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
+        unsigned long long thr = 0ull;
+        int need_eq = 0, dirty = -1;
+        if (nl < S) dirty = team_radix_select(s, S, nl, tt, ko, ka, thr, need_eq);
+        total = team_compact_layer(s, s.keys, idx, S, thr, need_eq, dirty, tt);
+    } else {
+        total = team_select_global<LS>(at, gph, N, nl, tt);
+    }
+    team_sync();                                           // s.ltok[i] is the candidate index of the new layer's node i, s.lkeys[i] its key
+    #pragma unroll 1
+    for (int i = tt; i < nl && i < total; i += kTeam) {
+        const int c = s.ltok[i];
+        unsigned int t32 = ld_relaxed_u32(&gtk[c]);
+        if (!(t32 >> 31)) t32 = poll_tok_word(&gtk[c], status);
+        const int tok = t32 == ~0u ? -1 : (int)(t32 & 0x7FFFFFFFu);
+        const int frow = c / k;
+        T_tok[gid0 + i] = tok;
+        T_par[gid0 + i] = kPrune ? __ldcg(&fmap[frow]) : frow;
+        T_phat[gid0 + i] = __longlong_as_double((long long)(s.lkeys[i] - 1ull));
+        s.ltok[i] = tok;
     }
     if (total != nl) set_status(status, kErrInternal);
     team_sync();                                           // everyone has read what it needs: the arrays can be cleared
     #pragma unroll 1
-    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(&j.cand_phat[i]) = make_uint4(0, 0, 0, 0);
+    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
     #pragma unroll 1
-    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(&j.cand_tok[i]) = make_uint4(0, 0, 0, 0);
+    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
     team_sync();
     return nl;
 }
 
 // Once per sequence, when it is finished: T_opt = the running top-n (s.rsel / s.vals, already in
-// (depth, parent's index, sibling rank) order), packed with parent indices.
+// (depth, parent's index, sibling rank) order), packed with parent indices.  By `stride` threads, this
+// one the tt-th: the team, or the layer warp alone for trees so small that handing them over costs more (see kPackAlone).
 template <class LS>
-__device__ __noinline__ void pack_tree_warp(LS& s, const SeqWork& w, const TreeOut& out, int d, int nR, int n, int max_depth,
-                                            double esub, int* status) {
-    const int lane = threadIdx.x & 31;
-    if (out.esub_trace) for (int i = d + lane; i < max_depth; i += 32) out.esub_trace[i] = 0.0;
+__device__ __noinline__ void pack_tree(int at, TreeOut out, int tt, int stride, int* status) {
+    LS& s = smem_at<LS>(at);
+    const LayerJob& j = s.job;
+    const int d = j.d, nR = j.nR_old, n = j.n, max_depth = j.max_depth;
+    const int32_t *const T_tok = j.T_tok, *const T_par = j.T_par;
+    if (out.esub_trace) for (int i = d + tt; i < max_depth; i += stride) out.esub_trace[i] = 0.0;
     #pragma unroll 1
-    for (int i = lane; i < n; i += 32) {
+    for (int i = tt; i < n; i += stride) {
         int32_t tok = -1, par = -1, dep = 0;
         double ph = 0.0;
         if (i < nR) {
             const int gid = s.rsel[i];
             dep = gid / n + 1;
-            tok = __ldcg(&w.T_tok[gid]);
+            tok = __ldcg(&T_tok[gid]);
             ph = s.vals[i];
             if (dep > 1) {
-                const int pg = (dep - 2) * n + __ldcg(&w.T_par[gid]);
+                const int pg = (dep - 2) * n + __ldcg(&T_par[gid]);
                 int lo = 0, hi = i;                        // the parent is packed before its child
                 while (lo < hi) {
                     const int mid = (lo + hi) >> 1;
@@ -575,65 +670,79 @@ __device__ __noinline__ void pack_tree_warp(LS& s, const SeqWork& w, const TreeO
         }
         out.token[i] = tok; out.parent[i] = par; out.depth[i] = dep; out.phat[i] = ph;
     }
-    if (lane == 0) { *out.n_sel = nR; *out.depth_reached = d; *out.expected_len = esub; }
+    if (tt == 0) { *out.n_sel = nR; *out.depth_reached = d; *out.expected_len = s.last_esub; }
 }
 
-// Layer job, second half: the running top-n and E_sub(T, n) with the new layer (left in s by
-// the selection), the loop test of Algorithm 1, and the packed tree if the sequence is
-// finished.  All layers of a sequence are handled by the same warp, in order.  Returns true if the
-// sequence continues with layer d+1, false if it is finished (outputs written).
+// E_sub(T, n) from the running top-n in the scratch, in one fixed order (lanes stride the packed order); whole warp.
 template <class LS>
-__device__ __noinline__ bool update_running_warp(LS& s, const SeqWork& w, const TreeOut& out, int d, int nl, int n, int Dcap,
-                                    int max_depth, float delta, int* status) {
-    const int lane = threadIdx.x & 31;
-    int* hist = s.hist;
-    const int gid0 = (d - 1) * n;
-    unsigned long long thr;
-    int need_eq;
-    const int nR_old = d == 1 ? 0 : __ldcg(&w.st[kStNR]);
-    const double eprev = d == 1 ? 0.0 : __ldcg(w.E_prev);
+__device__ __forceinline__ double running_esub(const LS& s, int nR) {
+    double part = 0.0;
+    #pragma unroll 1
+    for (int i = threadIdx.x & 31; i < nR; i += 32) part += s.vals[i];
+    return warp_sum(part);
+}
 
-    // --- E_sub(T, n): the n largest path values among the previous top-n and the new layer ---
-    const int32_t* Rold = w.R + ((d - 1) & 1) * n;
-    int32_t* Rnew = w.R + (d & 1) * n;
-    const int NR = nR_old + nl;                           // <= 2n
-    const int nR = NR < n ? NR : n;
+// Layer job, second half: the running top-n and E_sub(T, n) with the new layer (j.fsize nodes, left in s by the
+// selection), by the team: a radix select over the keys of the old top-n and the layer.  j.off: s.rsel / s.vals still
+// hold the old one (else it is read from j.Rold).  On return s.rsel / s.vals hold the new one (ascending gids; also
+// written to j.Rnew); returns |R|.
+template <class LS>
+__device__ __noinline__ int update_running_team(int at, int tt, int* status) {
+    LS& s = smem_at<LS>(at);
+    const LayerJob& j = s.job;
+    const bool cached = j.off != 0;
+    const int32_t* const Rold = j.Rold;
+    const double* const T_phat = j.T_phat;
+    int32_t* const Rnew = j.Rnew;
+    const int lane = tt & 31, tw = tt >> 5;
+    const int nRo = j.nR_old, NR = nRo + j.fsize, need = NR < j.n ? NR : j.n, gid0 = (j.d - 1) * j.n;
     unsigned long long ko = 0ull, ka = ~0ull;
     #pragma unroll 1
-    for (int i = lane; i < NR; i += 32) {
+    for (int i = tt; i < NR; i += kTeam) {
         int gid;
         unsigned long long key;
-        if (i < nR_old) { gid = __ldcg(&Rold[i]); key = phat_key(__ldcg(&w.T_phat[gid])); }
-        else { gid = gid0 + (i - nR_old); key = s.lkeys[i - nR_old]; }
+        if (i >= nRo) { gid = gid0 + (i - nRo); key = s.lkeys[i - nRo]; }
+        else if (cached) { gid = s.rsel[i]; key = phat_key(s.vals[i]); }
+        else { gid = __ldcg(&Rold[i]); key = phat_key(__ldcg(&T_phat[gid])); }
         s.gids[i] = gid;
         s.keys[i] = key;
         ko |= key; ka &= key;
     }
-    __syncwarp();
-    auto rkey = [&](int i) -> unsigned long long { return s.keys[i]; };
-    warp_radix_select(rkey, NR, nR, hist, warp_or_u64(ko), warp_and_u64(ka), thr, need_eq);
-    warp_compact_selected(rkey, NR, thr, need_eq, [&](int pos, int i) {
+    ko = warp_or_u64(ko); ka = warp_and_u64(ka);
+    if (lane == 0) { s.red_or[tw] = ko; s.red_and[tw] = ka; }
+    team_sync();
+    ko = 0ull; ka = ~0ull;
+#pragma unroll
+    for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
+    unsigned long long thr = 0ull;                         // (keys are never 0: all are taken when nothing has to be left out)
+    int need_eq = 0, dirty = -1;
+    if (need < NR) dirty = team_radix_select(s, NR, need, tt, ko, ka, thr, need_eq);
+    const int per = (NR + kTeam - 1) / kTeam, lo = min(tt * per, NR), hi = min(lo + per, NR);
+    int gt = 0, eq = 0;
+    #pragma unroll 1
+    for (int i = lo; i < hi; ++i) { const unsigned long long key = s.keys[i]; gt += key > thr ? 1 : 0; eq += key == thr ? 1 : 0; }
+    int total_eq, total, eq_take = 0;
+    if (need_eq > 0) {
+        const int eq_before = team_excl_scan(eq, s.scan_a, tw, total_eq);
+        eq_take = need_eq - eq_before;
+        eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
+    }
+    int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
+    if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }
+    #pragma unroll 1
+    for (int i = lo; i < hi; ++i) {
+        const unsigned long long key = s.keys[i];
+        bool take = key > thr;
+        if (key == thr && eq_take > 0) { take = true; --eq_take; }
+        if (!take) continue;
         Rnew[pos] = s.gids[i];
         s.rsel[pos] = s.gids[i];
-        s.vals[pos] = __longlong_as_double((long long)(s.keys[i] - 1ull));
-    });
-    __syncwarp();
-    double part = 0.0;
-    #pragma unroll 1
-    for (int i = lane; i < nR; i += 32) part += s.vals[i];
-    const double esub = warp_sum(part);                   // fixed order: lanes stride the packed order
-    const bool more = d < Dcap && (esub - eprev > (double)delta);     // loop test of Algorithm 1
-    if (out.esub_trace && lane == 0) out.esub_trace[d - 1] = esub;
-    if (lane == 0) {
-        w.st[kStNR] = nR;
-        *w.E_prev = esub;
+        s.vals[pos] = __longlong_as_double((long long)(key - 1ull));
+        ++pos;
     }
-    __syncwarp();
-    if (lane == 0) { s.last_nR = nR; s.last_esub = esub; }
-    __syncwarp();
-    if (more) return true;
-    pack_tree_warp(s, w, out, d, nR, n, max_depth, esub, status);
-    return false;
+    if (total != need) set_status(status, kErrInternal);
+    team_sync();
+    return need;
 }
 
 }  // namespace ot
