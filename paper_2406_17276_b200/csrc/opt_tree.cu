@@ -606,7 +606,7 @@ struct BuildSink {
                 if (progressed) t0 = clock64();
                 else {
                     if (clock64() - t0 > kWaitCycles) { set_status(w.status, kErrTimeout); return; }
-                    __nanosleep(100);
+                    __nanosleep(kPollPauseNs);
                 }
             }
         }
@@ -749,7 +749,7 @@ layer_step_kernel(Workspace w, Params p, int fstride, opt_tree_out out, int32_t*
 }
 
 // Tree attention mask + position ids: one CTA per sequence, a thread per node (in rounds of the block
-// size when n is larger): the node's ancestor chain is walked and its bits gathered in registers.
+// size when n is larger): the node's ancestor chain is walked, in shared memory, and its bits gathered in registers.
 __global__ void __launch_bounds__(kSmallThreads)
 mask_kernel(const int32_t* __restrict__ parent, const int32_t* __restrict__ depth, const int32_t* __restrict__ n_sel,
             const int32_t* __restrict__ base_pos, int n, uint64_t* mask, int32_t* position_ids, int* status) {
@@ -757,7 +757,9 @@ mask_kernel(const int32_t* __restrict__ parent, const int32_t* __restrict__ dept
     const int b = blockIdx.x;
     const int W = (n + 63) >> 6;
     const int ns = n_sel[b];
-    const int32_t* par = parent + (size_t)b * n;
+    int* par = reinterpret_cast<int*>(ot_smem);
+    for (int i = threadIdx.x; i < n; i += kSmallThreads) par[i] = parent[(size_t)b * n + i];
+    __syncthreads();
     for (int i = threadIdx.x; i < n; i += kSmallThreads) {
         uint64_t bits[kMaxN / 64];
 #pragma unroll
@@ -1497,7 +1499,7 @@ int opt_tree_build_pruned(opt_tree_ctx* ctx, const void* draft, const int32_t* r
 int opt_tree_mask(opt_tree_ctx* ctx, const opt_tree_out* tree, int32_t B, const int32_t* base_pos, uint64_t* mask,
                   int32_t* position_ids, void* stream) {
     if (!ctx || bad_tree(tree) || !mask || !position_ids || B < 1 || B > ctx->cfg.max_batch) return OPT_TREE_ERR_INVALID_ARG;
-    launch_after(ot::mask_kernel, dim3(B), dim3(ot::kSmallThreads), 0, static_cast<cudaStream_t>(stream),
+    launch_after(ot::mask_kernel, dim3(B), dim3(ot::kSmallThreads), ctx->cfg.n * sizeof(int), static_cast<cudaStream_t>(stream),
                  tree->parent, tree->depth, tree->n_sel, base_pos, ctx->cfg.n, mask, position_ids, ctx->ws.status);
     ctx->launches++;
     return check_launch();

@@ -102,7 +102,7 @@ __device__ void fetcher_role(CtaCore& s, Source& src, int* status, long long lim
         if (rm) t0 = clock64();
         else {
             if ((turn & 63) == 63 && clock64() - t0 > limit) { set_status(status, kErrTimeout); return; }
-            __nanosleep(100);
+            __nanosleep(kPollPauseNs);
         }
     }
 }

@@ -543,7 +543,8 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
     // tau: the kk-th largest of the 32 lanes' maxima (each the largest of 16 per-thread maxima).  That
     // is at most the kk-th largest per-thread maximum, hence at most the row's kk-th largest logit, so
     // every winner still lives in a thread whose maximum is >= tau; a few more threads than kk get
-    // flagged, and in exchange tau takes sixteen ballots instead of a histogram over 512 keys.
+    // flagged, and in exchange tau takes 32 independent shuffles instead of a histogram over 512 keys (sixteen dependent
+    // ballots took 1.3 % longer over a whole build of 32 sequences).
     // With fewer than kk finite lane maxima tau is -inf and the row goes the exact way.  The bound gets
     // loose as kk approaches the 32 lanes (about 32 ln(32 / (32 - kk)) threads are flagged), so beyond
     // kLaneTauMaxK the exact kk-th largest per-thread maximum is used instead.
@@ -552,15 +553,11 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
         tau_key = tau_from_histogram(f, slot.tkey, mk, kk);
     } else {
         const uint32_t lane_max = max(lane_mk & 0xFFFFu, lane_mk >> 16);
-        unsigned cand = 0xFFFFFFFFu;                       // lanes whose maximum matches tau's bits so far
-        int need = kk;
-#pragma unroll 1
-        for (int bit = 15; bit >= 0; --bit) {
-            const unsigned ones = __ballot_sync(0xFFFFFFFFu, (lane_max >> bit) & 1u) & cand;
-            const int c = __popc(ones);
-            if (c >= need) { tau_key |= 1u << bit; cand = ones; }
-            else { need -= c; cand &= ~ones; }
-        }
+        const uint32_t mine = (lane_max << 5) | (uint32_t)lane;        // (distinct)
+        int above = 0;
+#pragma unroll 4
+        for (int q = 0; q < 32; ++q) above += __shfl_sync(0xFFFFFFFFu, mine, q) > mine ? 1 : 0;
+        tau_key = __shfl_sync(0xFFFFFFFFu, lane_max, __ffs(__ballot_sync(0xFFFFFFFFu, above == kk - 1)) - 1);
     }
     bool exact = tau_key <= kOrdNegInf || emax >= kExpLimit || emax <= -kExpLimit;
 
