@@ -615,13 +615,13 @@ struct BuildSink {
 
 // Algorithm 1 for a whole batch in one launch: persistent CTAs take rows from their mailboxes; layers
 // of different sequences overlap freely because sequences never exchange data.
-template <bool kPrune, int NCAP, bool kAligned>
+template <bool kPrune, int NCAP, bool kAligned, bool kLong>
 __global__ void __launch_bounds__(kThreads)
 build_kernel(Workspace w, Params p, const uint16_t* __restrict__ draft, opt_tree_out out) {
     CtaSmemT<NCAP>& s = *reinterpret_cast<CtaSmemT<NCAP>*>(ot_smem);
     BuildSource<kPrune> src{w, p, draft};
     BuildSink<kPrune> sink{w, p, out};
-    run_pipeline<kAligned>(s, src, sink, p.V, p.k, draft, draft + (size_t)p.H * p.V, w.status);
+    run_pipeline<kAligned, kLong>(s, src, sink, p.V, p.k, draft, draft + (size_t)p.H * p.V, w.status);
 }
 
 // The row step alone over a list of rows (static round-robin over the CTAs).
@@ -651,14 +651,14 @@ struct ListSink {
         }
     }
 };
-template <bool kAligned>
+template <bool kAligned, bool kLong>
 __global__ void __launch_bounds__(kThreads)
 row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __restrict__ rows, int nrows,
                 int32_t* tok_out, double* prob_out, int* status) {
     CtaSmem& s = *reinterpret_cast<CtaSmem*>(ot_smem);
     ListSource src{logits, rows, nrows, p.V, p.H, (int)blockIdx.x, (int)gridDim.x, status};
     ListSink sink{tok_out, prob_out, p.k};
-    run_pipeline<kAligned>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.H * p.V, status);
+    run_pipeline<kAligned, kLong>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.H * p.V, status);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1375,13 +1375,23 @@ size_t cta_smem_bytes(int n) { return small_n(n) ? sizeof(ot::CtaSmemT<ot::kSmal
 size_t layer_smem_bytes(int n) { return small_n(n) ? sizeof(ot::LayerScratchT<ot::kSmallN>) : sizeof(ot::LayerScratchT<ot::kMaxN>); }
 
 using BuildKernel = void (*)(ot::Workspace, ot::Params, const uint16_t*, opt_tree_out);
-template <int NCAP> BuildKernel build_variant(bool prune, bool aligned) {
-    return prune ? (aligned ? ot::build_kernel<true, NCAP, true> : ot::build_kernel<true, NCAP, false>)
-                 : (aligned ? ot::build_kernel<false, NCAP, true> : ot::build_kernel<false, NCAP, false>);
+using RowKernel = void (*)(ot::Params, const uint16_t*, const int32_t*, int, int32_t*, double*, int*);
+// Variants: bit 0 pruned draft, bit 1 aligned rows, bit 2 long rows.
+constexpr int kPrunedBit = 1, kAlignedBit = 2, kLongBit = 4, kVariants = 8;
+template <int NCAP> BuildKernel build_variant(int v) {
+    static const BuildKernel kernels[kVariants] = {
+        ot::build_kernel<false, NCAP, false, false>, ot::build_kernel<true, NCAP, false, false>,
+        ot::build_kernel<false, NCAP, true, false>,  ot::build_kernel<true, NCAP, true, false>,
+        ot::build_kernel<false, NCAP, false, true>,  ot::build_kernel<true, NCAP, false, true>,
+        ot::build_kernel<false, NCAP, true, true>,   ot::build_kernel<true, NCAP, true, true>};
+    return kernels[v];
 }
-BuildKernel build_kernel_for(int n, bool prune, bool aligned) {
-    return small_n(n) ? build_variant<ot::kSmallN>(prune, aligned) : build_variant<ot::kMaxN>(prune, aligned);
+BuildKernel build_kernel_for(int n, int v) { return small_n(n) ? build_variant<ot::kSmallN>(v) : build_variant<ot::kMaxN>(v); }
+RowKernel row_variant(int v) {
+    return (v & kLongBit) ? ((v & kAlignedBit) ? ot::row_topk_kernel<true, true> : ot::row_topk_kernel<false, true>)
+                          : ((v & kAlignedBit) ? ot::row_topk_kernel<true, false> : ot::row_topk_kernel<false, false>);
 }
+int variant_of(const ot::Params& p) { return (p.prune ? kPrunedBit : 0) | (p.aligned ? kAlignedBit : 0) | (p.V > ot::kLongRow ? kLongBit : 0); }
 template <class F> bool allow_smem(F* kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
 }
@@ -1392,13 +1402,13 @@ int persistent_grid(int n) {
     int dev = 0, per_sm = 0, sms = 0;
     constexpr int S = ot::kSmallN, L = ot::kMaxN;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
-    bool ok = allow_smem(ot::row_topk_kernel<true>, sizeof(ot::CtaSmem)) && allow_smem(ot::row_topk_kernel<false>, sizeof(ot::CtaSmem)) &&
-              allow_smem(ot::layer_step_kernel<S>, sizeof(ot::LayerScratchT<S>)) && allow_smem(ot::layer_step_kernel<L>, sizeof(ot::LayerScratchT<L>));
-    for (int v = 0; v < 4; ++v)
-        ok = ok && allow_smem(build_variant<S>(v & 1, v & 2), sizeof(ot::CtaSmemT<S>)) && allow_smem(build_variant<L>(v & 1, v & 2), sizeof(ot::CtaSmemT<L>));
+    bool ok = allow_smem(ot::layer_step_kernel<S>, sizeof(ot::LayerScratchT<S>)) && allow_smem(ot::layer_step_kernel<L>, sizeof(ot::LayerScratchT<L>));
+    for (int v = 0; v < kVariants; ++v)
+        ok = ok && allow_smem(build_variant<S>(v), sizeof(ot::CtaSmemT<S>)) && allow_smem(build_variant<L>(v), sizeof(ot::CtaSmemT<L>)) &&
+             allow_smem(row_variant(v), sizeof(ot::CtaSmem));
     int least = 1 << 30;                             // the variants share one grid: the smallest occupancy counts
-    for (int v = 0; v < 4 && ok; ++v) {
-        ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_kernel_for(n, v & 1, v & 2), ot::kThreads, cta_smem_bytes(n)) == cudaSuccess;
+    for (int v = 0; v < kVariants && ok; ++v) {
+        ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_kernel_for(n, v), ot::kThreads, cta_smem_bytes(n)) == cudaSuccess;
         least = per_sm < least ? per_sm : least;
     }
     if (!ok || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -1476,7 +1486,7 @@ static int build_common(opt_tree_ctx* ctx, const void* draft, const int32_t* roo
     p.prune = prune;
     const long long init_threads = (long long)ctx->grid * ctx->mcap > B ? (long long)ctx->grid * ctx->mcap : B;
     launch_after(ot::init_build_kernel, dim3((unsigned)((init_threads + 255) / 256)), dim3(256), 0, st, ctx->ws, p, root_token);
-    launch_after(build_kernel_for(ctx->cfg.n, prune != 0, p.aligned != 0), dim3(ctx->grid), dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(draft), *out);
+    launch_after(build_kernel_for(ctx->cfg.n, variant_of(p)), dim3(ctx->grid), dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(draft), *out);
     ctx->launches += 2;
     int rc = check_launch();
     if (rc == OPT_TREE_OK && rows_read &&
@@ -1569,7 +1579,7 @@ int opt_tree_layers_step(opt_tree_ctx* ctx, const void* frontier_logits, int32_t
     ot::Params pr = p;
     pr.H = nrows;                                            // the dense buffer is the "table" of the row step
     const int grid = nrows < ctx->grid ? nrows : ctx->grid;
-    launch_after(p.aligned ? ot::row_topk_kernel<true> : ot::row_topk_kernel<false>, dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem), st,
+    launch_after(row_variant(variant_of(p)), dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem), st,
                  pr, static_cast<const uint16_t*>(frontier_logits), static_cast<const int32_t*>(nullptr), nrows, ctx->ws.rtok,
                  ctx->ws.rprob, ctx->ws.status);
     launch_after(small_n(ctx->cfg.n) ? ot::layer_step_kernel<ot::kSmallN> : ot::layer_step_kernel<ot::kMaxN>, dim3(B), dim3(ot::kTeam),
@@ -1585,7 +1595,7 @@ int opt_tree_row_softmax_topk(opt_tree_ctx* ctx, const void* logits, const int32
     if (nrows == 0) return OPT_TREE_OK;
     const ot::Params p = make_params(ctx, logits, 0.0f);
     const int grid = nrows < ctx->grid ? nrows : ctx->grid;
-    launch_after(p.aligned ? ot::row_topk_kernel<true> : ot::row_topk_kernel<false>, dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem),
+    launch_after(row_variant(variant_of(p)), dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem),
         static_cast<cudaStream_t>(stream), p, static_cast<const uint16_t*>(logits), rows, nrows, tok_out, prob_out, ctx->ws.status);
     ctx->launches++;
     return check_launch();

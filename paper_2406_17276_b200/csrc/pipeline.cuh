@@ -178,7 +178,7 @@ __device__ void issuer_role(CtaCore& s, int V, const uint16_t* lo, const uint16_
 // A warp takes its share of a chunk out of the ring into registers and hands the stage back at once
 // (so the issuer can refill it while the exponentials run); a row's descriptor is only looked at for
 // its stop flag.
-template <bool kAligned>
+template <bool kAligned, bool kLong>
 __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
     const int lane = threadIdx.x & 31, tid = cwarp * 32 + lane;     // index among the consumer threads
     const int nchunks = (V + kChunkElems - 1) / kChunkElems;
@@ -200,13 +200,14 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&s.desc_empty[r % kDesc]);      // this warp has looked at the descriptor
             }
-            if (kAligned) chunk_take(ch, reinterpret_cast<const uint4*>(&s.stage[st][0]), chunk_elems(V, c) >> 3, tid);
-            else chunk_take_shifted(ch, reinterpret_cast<const uint4*>(&s.stage[st][0]), chunk_elems(V, c), off, tid);
+            const int ne = chunk_elems(V, c);
+            if (kAligned) chunk_take(ch, reinterpret_cast<const uint4*>(&s.stage[st][0]), ne >> 3, tid);
+            else chunk_take_shifted(ch, reinterpret_cast<const uint4*>(&s.stage[st][0]), ne, off, tid);
             __syncwarp();
             if (lane == 0) mbar_arrive(&s.empty_bar[st]);          // the data is in registers: the stage is free
             chunk_chain(ch);
             const unsigned long long C2 = chunk_apply(acc, ch);
-            chunk_exps(acc, ch, C2);
+            chunk_exps<kLong>(acc, ch, C2, (ne + 7) >> 3);
         }
         // hand the row to its finisher
         const int sl = r % kSlots;
@@ -220,7 +221,7 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
 
 // ---- finisher warps ----------------------------------------------------------------------------
 // Sink::row_done(const RowDesc&, const RowOut&, FinScratch&) is called by the whole warp.
-template <bool kAligned, class Sink>
+template <bool kAligned, bool kLong, class Sink>
 __device__ void finisher_role(CtaCore& s, Sink& sink, int fidx, int V, int k, int* status) {
     const int lane = threadIdx.x & 31;
     FinScratch& f = s.fin[fidx];
@@ -244,7 +245,7 @@ __device__ void finisher_role(CtaCore& s, Sink& sink, int fidx, int V, int k, in
         const RowSlot& slot = s.slot[sl];
         const RowDesc dsc = s.desc[r % kDescRing];
         RowOut out;
-        finish_row_warp<kAligned>(f, slot, dsc.row, V, k, out);
+        finish_row_warp<kAligned, kLong>(f, slot, dsc.row, V, k, out);
         __syncwarp();
         if (lane == 0) mbar_arrive(&s.free_bar[sl]);                              // the slot can be refilled
         sink.row_done(dsc, out, f);
@@ -252,20 +253,20 @@ __device__ void finisher_role(CtaCore& s, Sink& sink, int fidx, int V, int k, in
 }
 
 // kAligned: the table's base and row pitch are multiples of 16 bytes (a compile-time choice, so that the code of the
-// common case carries nothing of the other).  lo / hi bound the table.
-template <bool kAligned, class Smem, class Source, class Sink>
+// common case carries nothing of the other); kLong: more than kLongRow logits.  lo / hi bound the table.
+template <bool kAligned, bool kLong, class Smem, class Source, class Sink>
 __device__ __forceinline__ void run_pipeline(Smem& sm, Source& src, Sink& sink, int V, int k, const uint16_t* lo, const uint16_t* hi, int* status) {
     CtaCore& s = sm.core;
     pipeline_init(s, sm.layer);
     grid_dependency_wait();                                // shared memory is set up; global memory from here on
     const int warp = threadIdx.x >> 5;
-    if (warp < kConsumerWarps) { consumer_role<kAligned>(s, warp, V, status); return; }
+    if (warp < kConsumerWarps) { consumer_role<kAligned, kLong>(s, warp, V, status); return; }
     const int helper = warp - kConsumerWarps;
     if (helper == kHelperIssuer) issuer_role<kAligned>(s, V, lo, hi, status);
     else if (helper == kHelperFetcher) fetcher_role(s, src, status);
     else if (helper == kHelperLayer) sink.layer_loop(sm.layer);
     else if (helper < kHelperFirstFinisher) sink.layer_assist(sm.layer, helper - kHelperLayer);
-    else finisher_role<kAligned>(s, sink, helper - kHelperFirstFinisher, V, k, status);
+    else finisher_role<kAligned, kLong>(s, sink, helper - kHelperFirstFinisher, V, k, status);
 }
 
 }  // namespace ot

@@ -38,6 +38,12 @@ constexpr int kCandCap = 128;                      // candidate list capacity pe
 constexpr int kMaxFlag = 64;                       // flagged threads the fast finisher accepts
 constexpr int kDesc = 4;                           // rows a CTA may hold between ticket and descriptor read
 constexpr int kDescRing = 16;                      // descriptors kept: a row's lives until its finisher has copied it
+// Rows of more than two chunks take kernels of their own (kLong): their last chunk may be mostly padding, and a finisher
+// has many vectors to look at again per flagged thread.  Both cost code in the two hottest loops, which the kernels for
+// short rows do without (in one kernel for all, the row step on 32000 logits was 3 to 7 % slower, a build of 32
+// sequences 4 %).
+constexpr int kLongRow = 2 * kChunkElems;          // rows up to this many logits are short
+constexpr int kFinLoads = 8;                       // long rows: vectors a finisher lane has in flight
 constexpr int kLaneTauMaxK = 16;                   // largest k for which the finisher's threshold comes from the lane maxima
 constexpr int kPerLane = kConsumers / 32;          // per-thread results one finisher lane handles (16)
 
@@ -246,21 +252,33 @@ __device__ __forceinline__ unsigned long long chunk_apply(ThreadAcc& a, const Ch
     return pack2(-En, -En);
 }
 
-// The 32 exponentials of a chunk: 2^(x*log2e - E) in packed fp32x2 FMA + ex2.approx.
-__device__ __forceinline__ void chunk_exps(ThreadAcc& a, const ChunkRegs& c, unsigned long long C2) {
+// The eight exponentials of a vector: 2^(x*log2e - E) in packed fp32x2 FMA + ex2.approx.
+__device__ __forceinline__ void vector_exps(ThreadAcc& a, const uint4& w, unsigned long long C2) {
     const unsigned long long L2 = pack2(kLog2e, kLog2e);
+    const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-    for (int u = 0; u < kVecPerThread; ++u) {
-        const uint32_t ww[4] = {c.w[u].x, c.w[u].y, c.w[u].z, c.w[u].w};
+    for (int i = 0; i < 4; ++i) {
+        const float lo = __uint_as_float(ww[i] << 16), hi = __uint_as_float(ww[i] & 0xFFFF0000u);
+        float a0, a1;
+        unpack2(fma2(pack2(lo, hi), L2, C2), a0, a1);            // x*log2e - E
+        const unsigned long long e2 = pack2(ex2_approx(a0), ex2_approx(a1));
+        if (i & 1) a.acc1 = add2(a.acc1, e2);
+        else       a.acc0 = add2(a.acc0, e2);
+    }
+}
+// A chunk's exponentials.  A long row's last chunk ends after nv vectors, and those that lie behind its end for all threads
+// are left out, since exponentials of padding cost as much as others.  (A test per vector in the common case would keep
+// the compiler from interleaving the vectors.)
+template <bool kLong>
+__device__ __forceinline__ void chunk_exps(ThreadAcc& a, const ChunkRegs& c, unsigned long long C2, int nv) {
+    static_assert(kVecPerThread == 4, "the short case is written out");
+    if (!kLong || nv > 3 * kConsumers) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float lo = __uint_as_float(ww[i] << 16), hi = __uint_as_float(ww[i] & 0xFFFF0000u);
-            float a0, a1;
-            unpack2(fma2(pack2(lo, hi), L2, C2), a0, a1);            // x*log2e - E
-            const unsigned long long e2 = pack2(ex2_approx(a0), ex2_approx(a1));
-            if (i & 1) a.acc1 = add2(a.acc1, e2);
-            else       a.acc0 = add2(a.acc0, e2);
-        }
+        for (int u = 0; u < kVecPerThread; ++u) vector_exps(a, c.w[u], C2);
+    } else {
+        vector_exps(a, c.w[0], C2);
+        if (nv > kConsumers) vector_exps(a, c.w[1], C2);
+        if (nv > 2 * kConsumers) vector_exps(a, c.w[2], C2);
     }
 }
 
@@ -519,8 +537,86 @@ __device__ __noinline__ void finish_many(FinScratch& f, int M, int kk, double m,
     if (lane < kk) { out.tok = (int32_t)cand_token(x0); out.p = e0 / S; }
 }
 
-// Turns a finished slot into the row's k winners.  Whole finisher warp; f is its private scratch.
+// The search of finish_row_warp in long rows: the flagged threads' vectors are read again for the logits >= tau.  The list is
+// first cut down to the threads at or above the exact kk-th largest per-thread maximum (for kk > kLaneTauMaxK tau is that
+// already), kFinLoads vectors per lane are in flight, and a vector that holds a candidate (few do) is read once more for
+// its logits.  Leaves the candidates in f.cand / f.cand_count, raises tau_key and returns the sum of the lane's candidates'
+// approximate terms.
+// Measured with the skipped padding (B200): one sequence, V = 128256, k = 16: 325 -> 297 us a step; row step on 128256
+// logits, k = 16: 5.5 -> 6.0 TB/s, on 152064, k = 10: 6.0 -> 6.15, 1999 unaligned rows of 50257: 71.6 -> 68.0 us.
 template <bool kAligned>
+__device__ __forceinline__ float find_candidates_long(FinScratch& f, const uint16_t* tkey, const uint16_t* row, int V, int kk, int nflag, float negE,
+                                                      uint32_t& tau_key) {
+    const int lane = threadIdx.x & 31;
+    const int nvec = (V + 7) >> 3, nchunks = (V + kChunkElems - 1) / kChunkElems, vpt = nchunks * kVecPerThread;
+    if (kk <= kLaneTauMaxK && nflag > kk) {
+        const int t0 = lane < nflag ? f.flist[lane] : 0, t1 = lane + 32 < nflag ? f.flist[lane + 32] : 0;
+        const uint32_t a = lane < nflag ? tkey[t0] : 0u, b = lane + 32 < nflag ? tkey[t1] : 0u;
+        int ra = 0, rb = 0;
+#pragma unroll 4
+        for (int q = 0; q < nflag; ++q) {
+            const uint32_t x = tkey[f.flist[q]];
+            ra += x > a ? 1 : 0;
+            rb += x > b ? 1 : 0;
+        }
+        const bool ka = a != 0u && ra < kk, kb = b != 0u && rb < kk;
+        const unsigned am = __ballot_sync(0xFFFFFFFFu, ka), bm = __ballot_sync(0xFFFFFFFFu, kb), below = (1u << lane) - 1u;
+        tau_key = __reduce_min_sync(0xFFFFFFFFu, min(ka ? a : 0xFFFFu, kb ? b : 0xFFFFu));
+        __syncwarp();
+        if (ka) f.flist[__popc(am & below)] = t0;
+        if (kb) f.flist[__popc(am) + __popc(bm & below)] = t1;
+        nflag = __popc(am) + __popc(bm);
+        __syncwarp();
+    }
+    const uint32_t tau_bits = ord16_inv(tau_key), tau_b2 = tau_bits | (tau_bits << 16);
+    // Work item i: flagged thread i mod nflag, vector i / nflag = umulhi(i, magic) (exact: i * nflag stays below 2^32).
+    const int total = vpt * nflag;
+    const unsigned magic = 0xFFFFFFFFu / (unsigned)nflag + 1u;
+    auto vector_of = [&](int i) -> int {
+        const int j = nflag > 1 ? (int)__umulhi((unsigned)i, magic) : i;
+        return (j / kVecPerThread) * kChunkVecs + (j % kVecPerThread) * kConsumers + f.flist[i - j * nflag];
+    };
+    float sub = 0.0f;
+#pragma unroll 1
+    for (int i0 = lane; i0 - lane < total; i0 += 32 * kFinLoads) {
+        uint4 w[kFinLoads];
+#pragma unroll
+        for (int u = 0; u < kFinLoads; ++u) {
+            const int idx = i0 + u * 32;
+            w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+            if (idx < total) {
+                const int vi = vector_of(idx);
+                if (vi < nvec) w[u] = load_row_vec<kAligned>(row, vi, V);
+            }
+        }
+        uint32_t hits = 0;                                  // bit u: vector u holds a candidate
+#pragma unroll
+        for (int u = 0; u < kFinLoads; ++u)
+            hits |= (ge_bf16x2(max_bf16x2(max_bf16x2(w[u].x, w[u].y), max_bf16x2(w[u].z, w[u].w)), tau_b2) ? 1u : 0u) << u;
+#pragma unroll 1
+        for (; hits; hits &= hits - 1) {
+            const int vi = vector_of(i0 + (__ffs(hits) - 1) * 32);
+            const uint4 x = load_row_vec<kAligned>(row, vi, V);
+            const uint32_t gx = ge_bf16x2(x.x, tau_b2), gy = ge_bf16x2(x.y, tau_b2);
+            const uint32_t gz = ge_bf16x2(x.z, tau_b2), gw = ge_bf16x2(x.w, tau_b2);
+            uint32_t m8 = ((gx & 1u) | ((gx >> 15) & 2u)) | (((gy & 1u) | ((gy >> 15) & 2u)) << 2) |
+                          (((gz & 1u) | ((gz >> 15) & 2u)) << 4) | (((gw & 1u) | ((gw >> 15) & 2u)) << 6);
+#pragma unroll 1
+            for (; m8; m8 &= m8 - 1) {
+                const int h = __ffs(m8) - 1;
+                const uint32_t word = h < 4 ? (h < 2 ? x.x : x.y) : (h < 6 ? x.z : x.w);
+                const uint32_t bits = (h & 1) ? (word >> 16) : (word & 0xFFFFu);
+                const int pos = atomicAdd(&f.cand_count, 1);
+                if (pos < kCandCap) f.cand[pos] = cand_key(bits, (uint32_t)(vi * 8 + h));
+                sub += ex2_approx(fmaf(bf16_bits_to_float(bits), kLog2e, negE));
+            }
+        }
+    }
+    return sub;
+}
+
+// Turns a finished slot into the row's k winners.  Whole finisher warp; f is its private scratch.
+template <bool kAligned, bool kLong>
 __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& slot, const uint16_t* row, int V, int k, RowOut& out) {
     const int lane = threadIdx.x & 31;
     const int kk = k < V ? k : V;
@@ -600,6 +696,9 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
         // approximate term is taken out again here (the two differ by rounding of the exponent, a
         // few 1e-8 of the term), and the candidate comes back below with an exact exponential.
         // Work item i: flagged thread i mod P (P = nflag rounded up to a power of two), vector i / P.
+        const float negE = -(float)emax;
+        float sub = 0.0f;
+        if (kLong) sub = find_candidates_long<kAligned>(f, slot.tkey, row, V, kk, nflag, negE, tau_key);
         const uint32_t tau_bits = ord16_inv(tau_key);
         const float tau_f = bf16_bits_to_float(tau_bits);
         const uint32_t tau_b2 = tau_bits | (tau_bits << 16);
@@ -607,11 +706,16 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
         const int vpt = nchunks * kVecPerThread;
         const int lg = nflag > 1 ? 32 - __clz(nflag - 1) : 0;
         const int total = vpt << lg;
-        const float negE = -(float)emax;
-        float sub = 0.0f;
         double corr = 1.0;                                  // e^gap, see below; computed while the first loads are in flight
+        // Bulk terms are 2^(fl(x*L32) - E) with L32 the fp32 log2(e); wanted e^(x-m) = 2^((x-m)*L).
+        // The exponent gap E - m*L + x*(L - L32) is evaluated at a typical bulk logit x = tau - 2.
+        auto scale_factor = [&]() {
+            const double gap = (double)emax - m * kLog2eD + ((double)tau_f - 2.0) * (kLog2eD - (double)kLog2e);
+            corr = exp_f64(gap * 0.693147180559945309417);
+        };
+        if (kLong) scale_factor();
 #pragma unroll 1
-        for (int i0 = 0; i0 < total; i0 += 32 * 4) {
+        for (int i0 = 0; !kLong && i0 < total; i0 += 32 * 4) {
             uint4 w[4];
             int vis[4];
 #pragma unroll
@@ -625,12 +729,7 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
                     if (vi < nvec) { vis[u] = vi; w[u] = load_row_vec<kAligned>(row, vi, V); }
                 }
             }
-            if (i0 == 0) {
-                // Bulk terms are 2^(fl(x*L32) - E) with L32 the fp32 log2(e); wanted e^(x-m) = 2^((x-m)*L).
-                // The exponent gap E - m*L + x*(L - L32) is evaluated at a typical bulk logit x = tau - 2.
-                const double gap = (double)emax - m * kLog2eD + ((double)tau_f - 2.0) * (kLog2eD - (double)kLog2e);
-                corr = exp_f64(gap * 0.693147180559945309417);
-            }
+            if (i0 == 0) scale_factor();
             // bit 8u+e of m32: element e of vector u is a candidate (most vectors hold none)
             uint32_t m32 = 0;
 #pragma unroll
