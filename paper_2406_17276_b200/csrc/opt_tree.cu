@@ -23,7 +23,7 @@ constexpr int kSmallThreads = 256;          // block size of the mask / init ker
 constexpr int kVerifyThreads = 128, kVerifyThreadsFew = 512;
 
 __device__ __forceinline__ int row_of(int token, int depth, int H) {
-    return (int)(((long long)token * kRowMul + depth) % H);
+    return (int)(((unsigned)token * (unsigned)kRowMul + (unsigned)depth) % (unsigned)H);     // below 2^31 (supported_cfg); in 64 bits this is 1 % of a build
 }
 
 // ------------------------------------------------------------------------------------------------

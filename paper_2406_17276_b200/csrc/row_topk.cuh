@@ -113,6 +113,9 @@ struct alignas(16) LayerScratchT {
     unsigned long long red_or[kTeamWarps], red_and[kTeamWarps];
     int scan_a[kTeamWarps], scan_b[kTeamWarps];
     LayerJob job;
+    static constexpr int kList = 64;
+    unsigned long long list[kList];            // large layers: keys of the threshold's bin
+    int listn;
     double last_esub;                          // E_sub of the tree that is to be packed
     int scan_c[kTeamWarps];
     int cache_b, cache_d;                      // rsel / vals hold the top-n of this sequence after this layer (-1: nothing)

@@ -95,7 +95,7 @@ __device__ __forceinline__ int team_excl_scan(int v, int* wtot, int tw, int& tot
     return base + before;
 }
 
-// Threshold of the `need` largest keys among s.keys[0..N); key 0 means "not an element".  key_or / key_and
+// Threshold of the `need` largest keys among keyf(0..N); key 0 means "not an element".  key_or / key_and
 // are the bitwise OR / AND over all non-zero keys (the caller folds them into the sweep that stages the keys): the
 // bits on which all keys agree need no pass, and a pass whose threshold bin holds exactly the elements still needed
 // ends the search.  On return the selection is {key > thr} plus the first need_eq elements (lowest indices) with
@@ -106,8 +106,8 @@ __device__ __forceinline__ int team_excl_scan(int v, int* wtot, int tw, int& tot
 __device__ __forceinline__ unsigned long long key_of_word(unsigned long long x) {
     return x == ~0ull ? 0ull : (x & 0x7FFFFFFFFFFFFFFFull) + 1ull;
 }
-template <class LS>
-__device__ int team_radix_select(LS& s, int N, int need, int tt, unsigned long long key_or, unsigned long long key_and,
+template <class LS, class KeyFn>
+__device__ int team_radix_select(LS& s, KeyFn keyf, int N, int need, int tt, unsigned long long key_or, unsigned long long key_and,
                                  unsigned long long& thr, int& need_eq) {
     const int lane = threadIdx.x & 31;
     const unsigned long long diff = key_or ^ key_and;
@@ -121,7 +121,7 @@ __device__ int team_radix_select(LS& s, int N, int need, int tt, unsigned long l
         int* hist = s.thist[pass % 3];
         #pragma unroll 1
         for (int i = tt; i < N; i += kTeam) {
-            const unsigned long long key = s.keys[i];
+            const unsigned long long key = keyf(i);
             const bool match = key != 0ull && (top == 64 || (key >> top) == (prefix >> top));
             if (match) atomicAdd(&hist[(int)((unsigned int)(key >> shift) & dmask)], 1);
         }
@@ -212,7 +212,8 @@ __device__ __noinline__ int select_layer_team(int at, int tt, int* status) {
     for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
     unsigned long long thr = 0ull;                         // with no more candidates than wanted, all of them (key > 0) are taken
     int need_eq = 0, dirty = -1;
-    if (nl < nvalid) dirty = team_radix_select(s, N, nl, tt, ko, ka, thr, need_eq);
+    auto staged = [&](int i) { return s.keys[i]; };
+    if (nl < nvalid) dirty = team_radix_select(s, staged, N, nl, tt, ko, ka, thr, need_eq);
     // ordered compaction: thread tt owns a contiguous stretch of candidates
     const int per = (N + kTeam - 1) / kTeam;
     const int lo = min(tt * per, N), hi = min(lo + per, N);
@@ -309,7 +310,8 @@ __device__ __noinline__ int select_running_team(int at, int tt, int* status) {
     for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
     unsigned long long thr = 0ull;
     int need_eq = 0, dirty = -1;
-    if (need < nRo + nvalid) dirty = team_radix_select(s, M, need, tt, ko, ka, thr, need_eq);
+    auto staged = [&](int i) { return s.keys[i]; };
+    if (need < nRo + nvalid) dirty = team_radix_select(s, staged, M, need, tt, ko, ka, thr, need_eq);
     const int per = (M + kTeam - 1) / kTeam;
     const int lo = min(tt * per, M), hi = min(lo + per, M);
     int gt = 0, eq = 0;
@@ -373,33 +375,6 @@ __device__ __noinline__ int select_running_team(int at, int tt, int* status) {
     if (total != need) set_status(status, kErrInternal);
     team_sync();
     return need;
-}
-
-// Ordered compaction of the elements i in [0, M) with keys[i] > thr, and the first need_eq with keys[i] == thr: their keys
-// go to s.lkeys and idx[i] to s.ltok.  `dirty`: digit counts to clear.  Returns their number (two barriers at most).
-template <class LS>
-__device__ __forceinline__ int team_compact_layer(LS& s, const unsigned long long* keys, const int* idx, int M, unsigned long long thr,
-                                                  int need_eq, int dirty, int tt) {
-    const int tw = tt >> 5;
-    const int per = (M + kTeam - 1) / kTeam, lo = min(tt * per, M), hi = min(lo + per, M);
-    int gt = 0, eq = 0;
-    #pragma unroll 1
-    for (int i = lo; i < hi; ++i) { gt += keys[i] > thr ? 1 : 0; eq += keys[i] == thr ? 1 : 0; }
-    int total_eq, total, eq_take = 0;
-    if (need_eq > 0) {
-        const int eq_before = team_excl_scan(eq, s.scan_a, tw, total_eq);
-        eq_take = need_eq - eq_before;
-        eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
-    }
-    int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
-    if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }
-    #pragma unroll 1
-    for (int i = lo; i < hi; ++i) {
-        bool take = keys[i] > thr;
-        if (keys[i] == thr && eq_take > 0) { take = true; --eq_take; }
-        if (take) { s.lkeys[pos] = keys[i]; s.ltok[pos] = idx[i]; ++pos; }
-    }
-    return total;
 }
 
 // The same selection with every sweep over the candidate words in global memory (rare, see select_layer_team_big).
@@ -486,14 +461,14 @@ __device__ __forceinline__ int coarse_bin(unsigned long long key) {
 }
 
 // The team's selection for layers with more candidates than the shared-memory staging holds
-// (kStageCap < N <= n*k).  Bound by the round trips of 128 threads to the candidate words in L2 (a sweep over
-// 8192 of them takes about 4 us), so there are two sweeps and no more: the first counts the candidates into coarse
-// bins of their path values, the second marks those at or above the bin in which the threshold lies, usually few
-// more than n (if there are too many, one more sweep splits that bin in 1024).  Only these are brought into shared
-// memory, in index order, where the exact selection is the ordinary one.  If they still do not fit (over a thousand
-// ties, or a threshold below 2^-63) further sweeps read global memory once per digit.
-// Measured (two sequences, n = 512, k = 16, B200): 980 us per build with a sweep per digit, tokens fetched one after
-// the other in the emission and the running top-n by one warp; 440 us with both by the team.
+// (kStageCap < N <= n*k).  Bound by the round trips of 128 threads to the candidate words in L2 (8192 of them take 3 us,
+// 6 with their counting), so there are two sweeps and no more: the first counts the candidates into coarse bins of their path
+// values, the second brings those at or above the bin in which the threshold lies, usually few more than n, into shared
+// memory, each warp into a segment of its own; the keys of that bin are listed and the threshold is found by ranking
+// them.  (If the bin is too full one more sweep splits it in 1024; if over a thousand ties or a threshold below
+// 2^-63 make that useless too, or a warp's segment overflows, further sweeps read global memory once per digit.)
+// Measured (two sequences, n = 512, k = 16, B200): 1059 us per step with a sweep per digit and tokens fetched one by one, 452
+// with bit marks, a gather and a radix select after the second sweep, 431 with the segments.
 template <bool kPrune, class LS>
 __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
     LS& s = smem_at<LS>(at);
@@ -512,14 +487,29 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
     const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(cand_phat);
     const unsigned int* gtk = reinterpret_cast<const unsigned int*>(cand_tok);
     int* coarse = &s.thist[0][0];
+    if (tt == 0) s.listn = 0;
     #pragma unroll 1
-    for (int i0 = tt; i0 < N; i0 += 8 * kTeam) {
+    for (int i0 = tt; i0 - tt < N; i0 += 8 * kTeam) {
         unsigned long long x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) x[u] = i0 + u * kTeam < N ? ld_relaxed_u64(&gph[i0 + u * kTeam]) : ~0ull;
+        // what is not written yet is read again, all of it at once (bounded)
+        #pragma unroll 1
+        for (int t = 0;; ++t) {
+            bool missing = false;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (!(x[u] >> 63)) { x[u] = ld_relaxed_u64(&gph[i0 + u * kTeam]); missing = missing || !(x[u] >> 63); }
+            if (!__any_sync(0xFFFFFFFFu, missing)) break;
+            if (t >= kWaitPolls) {
+                set_status(status, kErrTimeout);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) if (!(x[u] >> 63)) x[u] = ~0ull;
+                break;
+            }
+        }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            if (!(x[u] >> 63)) x[u] = poll_phat_word(&gph[i0 + u * kTeam], status);      // not written yet: read again
             const unsigned long long key = key_of_word(x[u]);
             if (key) atomicAdd(&coarse[coarse_bin(key)], 1);
         }
@@ -528,8 +518,9 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
     int S;
     const int bin = warp_coarse_bin(s, nl, S);
     unsigned long long low = bin > 0 ? (unsigned long long)(bin + kCoarseBase) << kCoarseShift : 1ull;      // what counts is at or above this key
+    unsigned long long high = bin < 1023 ? (unsigned long long)(bin + 1 + kCoarseBase) << kCoarseShift : ~0ull;
+    int over = S - coarse[bin];                            // candidates at or above `high`
     if (S > LS::kSurvivors && bin > 0) {
-        const int over = S - coarse[bin];                  // elements in the bins above
         team_sync();
         #pragma unroll
         for (int q = 0; q < 1024 / kTeam; ++q) coarse[q * kTeam + tt] = 0;
@@ -548,10 +539,14 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
         team_sync();
         const int sub = warp_coarse_bin(s, nl - over, S);
         S += over;
+        over = S - coarse[sub];
         low |= (unsigned long long)sub << kFineShift;
+        high = low + (1ull << kFineShift);
     }
-    // second sweep: marks (one bit per candidate, kept where the new layer's keys will go) and their number
-    unsigned int* marks = reinterpret_cast<unsigned int*>(s.lkeys);
+    // second sweep
+    constexpr int kSeg = LS::kSurvivors / kTeamWarps;
+    int* idx = LS::kWideGids ? s.gids : s.toks;
+    const unsigned below = (1u << lane) - 1u;
     const int per = (((N + kTeamWarps - 1) / kTeamWarps) + 255) & ~255;        // candidates per warp
     const int lo = min(tw * per, N), hi = min(lo + per, N);
     int mine = 0;
@@ -564,69 +559,108 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
         for (int u = 0; u < 8; ++u) {
             const unsigned long long key = key_of_word(x[u]);
             const unsigned m = __ballot_sync(0xFFFFFFFFu, key >= low);
-            if (lane == u && i0 + u * 32 < hi) marks[(i0 >> 5) + u] = m;
+            const int pos = mine + __popc(m & below);
+            if (key >= low && pos < kSeg) {
+                s.keys[tw * kSeg + pos] = key;
+                idx[tw * kSeg + pos] = i0 + u * 32 + lane;
+            }
             mine += __popc(m);
         }
     }
-    if (lane == 0) s.scan_a[tw] = mine;
+    if (lane == 0) s.scan_c[tw] = mine;
     team_sync();
     #pragma unroll
     for (int q = 0; q < 1024 / kTeam; ++q) coarse[q * kTeam + tt] = 0;         // (every warp has its bin)
-    constexpr int kCap = LS::kSurvivors;
-    int* idx = LS::kWideGids ? s.gids : s.toks;
+    int start[kTeamWarps];                                 // survivors before each warp's segment
+    bool fits = true;
+    S = 0;
+#pragma unroll
+    for (int q = 0; q < kTeamWarps; ++q) { start[q] = S; const int c = s.scan_c[q]; fits = fits && c <= kSeg; S += c; }
     int total = 0;
-    if (S <= kCap) {
-        int pos = 0;
-        for (int q = 0; q < tw; ++q) pos += s.scan_a[q];
-        #pragma unroll 1
-        for (int i0 = lo; i0 < hi; i0 += 1024) {
-            const int c0 = i0 + lane * 32;
-            unsigned m = c0 < hi ? marks[c0 >> 5] : 0u;
-            int tot;
-            int p = pos + warp_excl_scan(__popc(m), tot);
-            for (; m; m &= m - 1) { if (p < kCap) idx[p] = c0 + __ffs(m) - 1; ++p; }
-            pos += tot;
+    if (fits) {
+        auto at_of = [&](int v) -> int {                   // survivor v, in index order: its place
+            int q = 0;
+#pragma unroll
+            for (int e = 1; e < kTeamWarps; ++e) q = v >= start[e] ? e : q;
+            int st = start[0];
+#pragma unroll
+            for (int e = 1; e < kTeamWarps; ++e) st = q == e ? start[e] : st;
+            return q * kSeg + v - st;
+        };
+        const int mper = (S + kTeam - 1) / kTeam, v0 = min(tt * mper, S), v1 = min(v0 + mper, S);
+        unsigned long long thr = low - 1ull;               // all of them
+        int need_eq = 0, dirty = -1, L = 0;
+        if (nl < S) {
+            #pragma unroll 1
+            for (int v = v0; v < v1; ++v) {
+                const unsigned long long key = s.keys[at_of(v)];
+                if (key < high) { const int q = atomicAdd(&s.listn, 1); if (q < LS::kList) s.list[q] = key; }
+            }
+            team_sync();
+            L = s.listn;
         }
-        team_sync();
-        unsigned long long ko = 0ull, ka = ~0ull;
-        #pragma unroll 1
-        for (int i0 = tt; i0 < S; i0 += 4 * kTeam) {
-            unsigned long long x[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = i0 + u * kTeam < S ? ld_relaxed_u64(&gph[idx[i0 + u * kTeam]]) : ~0ull;
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (i0 + u * kTeam < S) {
-                    const unsigned long long key = key_of_word(x[u]);
-                    s.keys[i0 + u * kTeam] = key;
-                    ko |= key; ka &= key;
-                }
+        if (nl < S && L <= LS::kList) {
+            const int need = nl - over;
+            const unsigned long long a = lane < L ? s.list[lane] : 0ull, b = lane + 32 < L ? s.list[lane + 32] : 0ull;
+            int ga = 0, gb = 0, ea = 0, eb = 0;            // keys above / equal to this lane's two
+            #pragma unroll 2
+            for (int e = 0; e < L; ++e) {
+                const unsigned long long x = s.list[e];
+                ga += x > a ? 1 : 0; ea += x == a ? 1 : 0;
+                gb += x > b ? 1 : 0; eb += x == b ? 1 : 0;
+            }
+            const bool ha = a != 0ull && ga < need && need <= ga + ea, hb = b != 0ull && gb < need && need <= gb + eb;
+            const unsigned hm = __ballot_sync(0xFFFFFFFFu, ha || hb);
+            const int src = hm ? __ffs(hm) - 1 : 0;
+            thr = __shfl_sync(0xFFFFFFFFu, ha ? a : b, src);
+            need_eq = __shfl_sync(0xFFFFFFFFu, need - (ha ? ga : gb), src);
+        } else if (nl < S) {
+            dirty = team_radix_select(s, [&](int v) { return s.keys[at_of(v)]; }, S, nl, tt, ~0ull, 0ull, thr, need_eq);
         }
-        ko = warp_or_u64(ko); ka = warp_and_u64(ka);
-        if (lane == 0) { s.red_or[tw] = ko; s.red_and[tw] = ka; }
-        team_sync();
-        ko = 0ull; ka = ~0ull;
-#pragma unroll
-        for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
-        unsigned long long thr = 0ull;
-        int need_eq = 0, dirty = -1;
-        if (nl < S) dirty = team_radix_select(s, S, nl, tt, ko, ka, thr, need_eq);
-        total = team_compact_layer(s, s.keys, idx, S, thr, need_eq, dirty, tt);
+        int gt = 0, eq = 0;
+        #pragma unroll 1
+        for (int v = v0; v < v1; ++v) { const unsigned long long key = s.keys[at_of(v)]; gt += key > thr ? 1 : 0; eq += key == thr ? 1 : 0; }
+        int total_eq, eq_take = 0;
+        if (need_eq > 0) {
+            const int eq_before = team_excl_scan(eq, s.scan_a, tw, total_eq);
+            eq_take = need_eq - eq_before;
+            eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
+        }
+        int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
+        if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }
+        #pragma unroll 1
+        for (int v = v0; v < v1; ++v) {
+            const int at_v = at_of(v);
+            const unsigned long long key = s.keys[at_v];
+            bool take = key > thr;
+            if (key == thr && eq_take > 0) { take = true; --eq_take; }
+            if (take) { s.lkeys[pos] = key; s.ltok[pos] = idx[at_v]; ++pos; }
+        }
     } else {
         total = team_select_global<LS>(at, gph, N, nl, tt);
     }
     team_sync();                                           // s.ltok[i] is the candidate index of the new layer's node i, s.lkeys[i] its key
     #pragma unroll 1
-    for (int i = tt; i < nl && i < total; i += kTeam) {
-        const int c = s.ltok[i];
-        unsigned int t32 = ld_relaxed_u32(&gtk[c]);
-        if (!(t32 >> 31)) t32 = poll_tok_word(&gtk[c], status);
-        const int tok = t32 == ~0u ? -1 : (int)(t32 & 0x7FFFFFFFu);
-        const int frow = c / k;
-        T_tok[gid0 + i] = tok;
-        T_par[gid0 + i] = kPrune ? __ldcg(&fmap[frow]) : frow;
-        T_phat[gid0 + i] = __longlong_as_double((long long)(s.lkeys[i] - 1ull));
-        s.ltok[i] = tok;
+    for (int i0 = tt; i0 < nl; i0 += 4 * kTeam) {
+        int c[4];
+        unsigned int t32[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            c[u] = i0 + u * kTeam < nl ? s.ltok[i0 + u * kTeam] : 0;
+            t32[u] = ld_relaxed_u32(&gtk[c[u]]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * kTeam;
+            if (i >= nl) break;
+            if (!(t32[u] >> 31)) t32[u] = poll_tok_word(&gtk[c[u]], status);
+            const int tok = t32[u] == ~0u ? -1 : (int)(t32[u] & 0x7FFFFFFFu);
+            const int frow = c[u] / k;
+            T_tok[gid0 + i] = tok;
+            T_par[gid0 + i] = kPrune ? __ldcg(&fmap[frow]) : frow;
+            T_phat[gid0 + i] = __longlong_as_double((long long)(s.lkeys[i] - 1ull));
+            s.ltok[i] = tok;
+        }
     }
     if (total != nl) set_status(status, kErrInternal);
     team_sync();                                           // everyone has read what it needs: the arrays can be cleared
@@ -716,7 +750,8 @@ __device__ __noinline__ int update_running_team(int at, int tt, int* status) {
     for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
     unsigned long long thr = 0ull;                         // (keys are never 0: all are taken when nothing has to be left out)
     int need_eq = 0, dirty = -1;
-    if (need < NR) dirty = team_radix_select(s, NR, need, tt, ko, ka, thr, need_eq);
+    auto staged = [&](int i) { return s.keys[i]; };
+    if (need < NR) dirty = team_radix_select(s, staged, NR, need, tt, ko, ka, thr, need_eq);
     const int per = (NR + kTeam - 1) / kTeam, lo = min(tt * per, NR), hi = min(lo + per, NR);
     int gt = 0, eq = 0;
     #pragma unroll 1
