@@ -41,9 +41,7 @@ struct Workspace {
     int32_t* st;           // [B][8]
     int32_t* fmap;         // [B][n]   pruned draft: layer slot behind each frontier row
     // layer-by-layer build (logits handed in per layer)
-    double* front_phat;    // [B][n]   path values of the nodes whose logits come next
-    int32_t* rtok;         // [B*n][k] row results of the layer in hand
-    double* rprob;         // [B*n][k]
+    double* front_phat;    // [B][2][n]   path values of the nodes whose logits come next (even and odd layers)
     // row mailboxes of the build: one per CTA, filled by the layer warps, never wrapped within a build.
     // The rows of a build are numbered by one running count (q_ctl[kQCursor]): row g goes to CTA
     // g % grid, entry g / grid of its mailbox.
@@ -61,7 +59,7 @@ struct Workspace {
     uint64_t* o_mask; int32_t* o_pos;
     int32_t *o_alen, *o_atok, *o_anode, *o_next;
 };
-enum { kQFinished = 2, kQDone = 3, kQCursor = 4 };
+enum { kQFinished = 2, kQDone = 3, kQCursor = 4, kQLayer = 5, kQLeft = 6 };   // 5, 6: layer-by-layer build: layers done, CTAs that have left this one
 
 constexpr int kMaxGrid = 4096;              // CTAs of the persistent kernels (SMs x occupancy) this layout supports
 
@@ -101,9 +99,7 @@ static size_t carve(const opt_tree_config& c, int grid, char* base, Workspace* w
     OT_TAKE(E_prev, double, B)
     OT_TAKE(st, int32_t, B * 8)
     OT_TAKE(fmap, int32_t, B * n)
-    OT_TAKE(front_phat, double, B * n)
-    OT_TAKE(rtok, int32_t, B * n * (size_t)c.k)
-    OT_TAKE(rprob, double, B * n * (size_t)c.k)
+    OT_TAKE(front_phat, double, 2 * B * n)
     OT_TAKE(mb_items, unsigned long long, mailbox_capacity(c, grid) * grid)
     OT_TAKE(mb_phat, unsigned long long, mailbox_capacity(c, grid) * grid)
     OT_TAKE(q_ctl, int32_t, 8)
@@ -672,90 +668,198 @@ row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __
 }
 
 // ------------------------------------------------------------------------------------------------
-// Layer-by-layer build: the caller (a real draft model) hands in the logits of one layer's nodes at
-// a time.  Per layer one launch of the row kernel over the dense buffer and one of layer_step_kernel:
-// a CTA of kTeam threads per sequence forms the candidates (Eq. 2), selects the layer with the same
-// team selection as the persistent build, updates the running top-n / E_sub, applies the loop test
-// and hands back the next layer's tokens; a sequence that stops is packed on the spot.
+// Layer-by-layer build: the caller (a real draft model) hands in the logits of one layer's nodes at a time.  One launch
+// per layer: the row pipeline over the dense buffer, its finishers leave the candidates (Eq. 2) as they do in the
+// persistent build, and the CTA whose finisher completes a sequence's last row has its layer team select the layer, update
+// the running top-n / E_sub, apply the loop test and hand back the next layer's tokens; a sequence that stops is packed on
+// the spot.  No CTA waits for another one, so nothing is assumed about which of them run together.
+// Two launches per layer (rows, then a CTA per sequence that formed the candidates) took 31 us a layer for 8 sequences of n = 50,
+// V = 32000, this 26.
 // ------------------------------------------------------------------------------------------------
 __global__ void layers_begin_kernel(Workspace w, Params p) {
     grid_dependency_wait();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= p.B) return;
-    int32_t* st = w.st + (size_t)b * 8;
-    st[kStDone] = 0; st[kStNR] = 0; st[kStRows] = 0; st[kStDepth] = 1; st[kStFsize] = 1;
-    w.E_prev[b] = 0.0;
-    w.front_phat[(size_t)b * p.n] = 1.0;                       // the root counts as factor 1
-    w.fmap[(size_t)b * p.n] = 0;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    for (long long j = i; j < (long long)p.B * p.cstride; j += (long long)gridDim.x * blockDim.x) {
+        reinterpret_cast<unsigned long long*>(w.cand_phat)[j] = 0ull;
+        w.cand_tok[j] = 0;
+    }
+    if (i == 0) { w.q_ctl[kQLayer] = 0; w.q_ctl[kQLeft] = 0; }
+    if (i >= p.B) return;
+    int32_t* st = w.st + (size_t)i * 8;
+    st[kStDone] = 0; st[kStNR] = 0; st[kStRows] = 0; st[kStFront] = 1; st[kStFront + 1] = 0;
+    w.E_prev[i] = 0.0;
+    w.front_phat[(size_t)i * 2 * p.n] = 1.0;                       // the root counts as factor 1
 }
 
-template <int NCAP>
-__global__ void __launch_bounds__(kTeam)
-layer_step_kernel(Workspace w, Params p, int fstride, opt_tree_out out, int32_t* next_tokens, int32_t* next_parent,
-                  int32_t* next_count) {
-    LayerScratchT<NCAP>& ls = *reinterpret_cast<LayerScratchT<NCAP>*>(ot_smem);
-    grid_dependency_wait();
-    const int b = blockIdx.x, tt = threadIdx.x;
-    for (int i = tt; i < 4 * 256; i += kTeam) (&ls.thist[0][0])[i] = 0;
-    const SeqWork sw = seq_work(w, p, b);
-    const int d = sw.st[kStDepth], fsize = sw.st[kStFsize];
-    if (d == 0) {                                            // this sequence stopped at an earlier layer
-        if (tt == 0) next_count[b] = 0;
-        return;
+// Rows of the dense buffer [B][fstride][V]; rows at or beyond a sequence's count are not read.
+struct LayersSource {
+    static constexpr bool kHasEmpty = true;
+    Workspace w; Params p;
+    const uint16_t* logits;
+    int fstride, layer;                                    // layers done before this one
+    __device__ long long claim(int i) {
+        const long long idx = (long long)blockIdx.x + (long long)i * gridDim.x;
+        return idx < (long long)p.B * fstride ? idx : -1;
     }
-    if (fsize < 1 || fsize > fstride || fsize > p.n) { if (tt == 0) { set_status(w.status, kErrInternal); next_count[b] = 0; } return; }
-    // candidates of the layer (Eq. 2), left the way the finishers of the persistent build leave them
-    const int N = fsize * p.k;
-    const double* fph = w.front_phat + (size_t)b * p.n;
-    for (int i = tt; i < N; i += kTeam) {
-        const int f = i / p.k, r = i - f * p.k;
-        const size_t src = ((size_t)b * fstride + f) * p.k + r;
-        const int tok = w.rtok[src];
-        const bool valid = r < p.kk && tok >= 0;
-        reinterpret_cast<unsigned long long*>(sw.cand_phat)[i] = valid ? phat_word(fph[f] * w.rprob[src]) : ~0ull;
-        reinterpret_cast<unsigned int*>(sw.cand_tok)[i] = valid ? (0x80000000u | (unsigned int)tok) : ~0u;
+    __device__ int poll(long long idx, RowDesc& d, bool) {
+        const int b = (int)(idx / fstride), f = (int)(idx - (long long)b * fstride);
+        const int fs = __ldcg(&w.st[(size_t)b * 8 + kStFront + (layer & 1)]);
+        if (f >= fs || fs > fstride) return 2;
+        d.row = logits + (size_t)idx * p.V;
+        d.b = b; d.d = layer + 1; d.slot = f; d.fsize = fs;
+        d.pphat = __ldcg(&w.front_phat[((size_t)b * 2 + (layer & 1)) * p.n + f]);
+        return 1;
     }
-    __syncthreads();
-    const bool small = N <= kStageCap;
-    if (tt < 32 && small) { stage_layer_candidates(ls, sw, fsize, p.k); cp_async_wait_all(); }
-    if (tt == 0) {
-        LayerJob& j = ls.job;
-        j.kind = 1; j.d = d; j.fsize = fsize; j.n = p.n; j.k = p.k; j.kk = p.kk;
-        j.cand_phat = sw.cand_phat; j.cand_tok = sw.cand_tok;
-        j.T_tok = sw.T_tok; j.T_par = sw.T_par; j.T_phat = sw.T_phat;
-        j.fmap = nullptr; j.nR_old = 0; j.off = 0; j.Rnew = nullptr;
+};
+template <class LS>
+struct LayersSink {
+    Workspace w; Params p; opt_tree_out out;
+    int fstride, layer, at;                                // at: offset of the layer scratch in shared memory
+    int32_t *next_tokens, *next_parent, *next_count;
+    __device__ void row_done(const RowDesc& d, const RowOut& r, FinScratch&) {
+        const int lane = threadIdx.x & 31;
+        const SeqWork sw = seq_work(w, p, d.b);
+        if (lane < p.k) {
+            unsigned long long* ph = reinterpret_cast<unsigned long long*>(sw.cand_phat) + d.slot * p.k + lane;
+            unsigned int* tk = reinterpret_cast<unsigned int*>(sw.cand_tok) + d.slot * p.k + lane;
+            *ph = lane < r.kk ? phat_word(d.pphat * r.p) : ~0ull;
+            *tk = lane < r.kk ? (0x80000000u | (unsigned int)r.tok) : ~0u;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            LS& ls = smem_at<LS>(at);
+            if (atomicAdd(&sw.st[kStDone], 1) + 1 == d.fsize) {            // (the words validate themselves: no fence)
+                const int pos = atomicAdd(&ls.todo_tail, 1);
+                const long long t0 = clock64();
+                while (pos - ls.todo_head >= LS::kTodo)
+                    if (clock64() - t0 > kWaitCycles) { set_status(w.status, kErrTimeout); break; }
+                ls.todo[pos % LS::kTodo] = d.b + 1;
+            }
+            __threadfence_block();
+            atomicAdd(&ls.rows_done, 1);
+        }
+        __syncwarp();
     }
-    __syncthreads();
-    using LS = LayerScratchT<NCAP>;
-    const int at = smem_offset(&ls);
-    const int nl = small ? select_layer_team<false, LS>(at, tt, w.status) : select_layer_team_big<false, LS>(at, tt, w.status);
-    if (tt == 0) {
-        LayerJob& j = ls.job;
-        j.fsize = nl; j.nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]); j.off = 0;
-        j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
+    __device__ void layer_loop(LS& ls) {
+        const int lane = threadIdx.x & 31;
+        // sequences that stopped at an earlier layer, or whose layer does not fit the buffer
+        for (int b = (int)blockIdx.x + lane * (int)gridDim.x; b < p.B; b += 32 * (int)gridDim.x) {
+            const int fs = __ldcg(&w.st[(size_t)b * 8 + kStFront + (layer & 1)]);
+            if (fs >= 1 && fs <= fstride) continue;
+            if (fs > fstride) set_status(w.status, kErrInternal);
+            next_count[b] = 0;
+            w.st[(size_t)b * 8 + kStFront + ((layer + 1) & 1)] = 0;
+        }
+        __syncwarp();
+        const CtaCore& core = smem_at<CtaCore>(0);
+        int head = 0, seen = 0;
+        long long t0 = clock64();
+        for (;;) {
+            const int v = __shfl_sync(0xFFFFFFFFu, ls.todo[head % LS::kTodo], 0);
+            if (v) {
+                __syncwarp();
+                if (lane == 0) { ls.todo[head % LS::kTodo] = 0; __threadfence_block(); ls.todo_head = head + 1; }
+                ++head;
+                step(ls, v - 1);
+                t0 = clock64();
+                continue;
+            }
+            // every row of this CTA finished, and (pushed before it was counted) every sequence taken
+            const int done = *reinterpret_cast<volatile int*>(&ls.rows_done);
+            if (__any_sync(0xFFFFFFFFu, done >= core.stop_row && head == *reinterpret_cast<volatile int*>(&ls.todo_tail))) break;
+            if (done != seen) { seen = done; t0 = clock64(); }
+            else if (__any_sync(0xFFFFFFFFu, clock64() - t0 > kWaitCycles)) { set_status(w.status, kErrTimeout); break; }
+            __nanosleep(kPollPauseNs);
+            __syncwarp();
+        }
+        if (lane == 0) {
+            ls.job.kind = 0;
+            __threadfence();
+            if (atomicAdd(&w.q_ctl[kQLeft], 1) == (int)gridDim.x - 1) { w.q_ctl[kQLeft] = 0; w.q_ctl[kQLayer] = layer + 1; }
+        }
+        __syncwarp();
+        team_sync();
     }
-    team_sync();
-    const int nR = update_running_team<LS>(at, tt, w.status);
-    const double esub = running_esub(ls, nR);
-    const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
-    const bool more = d < p.Dcap && (esub - eprev > (double)p.delta);     // loop test of Algorithm 1
-    const TreeOut to = tree_out(out, p, b);
-    if (to.esub_trace && tt == 0) to.esub_trace[d - 1] = esub;
-    if (more) {
-        const int gid0 = (d - 1) * p.n;
+    __device__ void layer_assist(LS& ls, int tw) {
+        const int tt = tw * 32 + (int)(threadIdx.x & 31);
+        for (;;) {
+            team_sync();
+            const int kind = ls.job.kind;
+            if (kind == 0) return;
+            work(ls, kind, tt);
+        }
+    }
+    // The team's part of a job; ends with a barrier.
+    __device__ void work(LS& ls, int kind, int tt) {
+        if (kind == 3) update_running_team<LS>(at, tt, w.status);
+        else if (kind == 4) { pack_tree<LS>(at, tree_out(out, p, ls.job.b), tt, kTeam, w.status); team_sync(); }
+        else if (kind == 6) { hand_back(ls, tt); team_sync(); }
+        else if (ls.job.fsize * ls.job.k <= kStageCap) select_layer_team<false, LS>(at, tt, w.status);
+        else select_layer_team_big<false, LS>(at, tt, w.status);
+    }
+    __device__ void hand_back(LS& ls, int tt) {
+        const int b = ls.job.b, nl = ls.job.fsize, gid0 = (ls.job.d - 1) * p.n;
+        const int32_t* T_par = ls.job.T_par;
+        double* front = w.front_phat + ((size_t)b * 2 + ((layer + 1) & 1)) * p.n;
         for (int i = tt; i < nl; i += kTeam) {
             next_tokens[(size_t)b * p.n + i] = ls.ltok[i];
-            next_parent[(size_t)b * p.n + i] = __ldcg(&sw.T_par[gid0 + i]);
-            w.front_phat[(size_t)b * p.n + i] = __longlong_as_double((long long)(ls.lkeys[i] - 1ull));
+            next_parent[(size_t)b * p.n + i] = __ldcg(&T_par[gid0 + i]);
+            front[i] = __longlong_as_double((long long)(ls.lkeys[i] - 1ull));
         }
-        team_sync();                                         // (everyone has read E and |R|)
-        if (tt == 0) { sw.st[kStNR] = nR; *sw.E_prev = esub; sw.st[kStDepth] = d + 1; sw.st[kStFsize] = nl; next_count[b] = nl; }
-    } else {
-        if (tt == 0) { ls.last_esub = esub; ls.job.nR_old = nR; ls.job.max_depth = p.max_depth; }
-        team_sync();
-        pack_tree<LS>(at, to, tt, kTeam, w.status);
-        if (tt == 0) { sw.st[kStDepth] = 0; next_count[b] = 0; }
     }
+    __device__ void do_job(LS& ls, int kind) {               // the job's fields are set by lane 0
+        const int lane = threadIdx.x & 31;
+        if (lane == 0) ls.job.kind = kind;
+        __syncwarp();
+        team_sync();
+        work(ls, kind, lane);
+    }
+    // One layer of one sequence.
+    __device__ void step(LS& ls, int b) {
+        const int lane = threadIdx.x & 31, d = layer + 1;
+        const SeqWork sw = seq_work(w, p, b);
+        const int fsize = __ldcg(&sw.st[kStFront + (layer & 1)]), nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
+        const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
+        const int nvalid = fsize * p.kk, nl = nvalid < p.n ? nvalid : p.n;
+        stage_layer_candidates(ls, sw, fsize, p.k);
+        if (lane == 0) {
+            LayerJob& j = ls.job;
+            j.b = b; j.d = d; j.fsize = fsize; j.n = p.n; j.k = p.k; j.kk = p.kk;
+            j.cand_phat = sw.cand_phat; j.cand_tok = sw.cand_tok;
+            j.T_tok = sw.T_tok; j.T_par = sw.T_par; j.T_phat = sw.T_phat; j.fmap = nullptr;
+            j.nR_old = nR_old; j.off = 0; j.max_depth = p.max_depth;
+            j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
+        }
+        cp_async_wait_all();
+        do_job(ls, 1);
+        if (lane == 0) ls.job.fsize = nl;
+        do_job(ls, 3);
+        const int NR = nR_old + nl, nR = NR < p.n ? NR : p.n;
+        const double esub = running_esub(ls, nR);
+        const bool more = d < p.Dcap && (esub - eprev > (double)p.delta);     // loop test of Algorithm 1
+        const TreeOut to = tree_out(out, p, b);
+        __syncwarp();
+        if (lane == 0) {
+            if (to.esub_trace) to.esub_trace[d - 1] = esub;
+            sw.st[kStNR] = nR; *sw.E_prev = esub;
+            sw.st[kStDone] = 0;
+            sw.st[kStFront + ((layer + 1) & 1)] = more ? nl : 0;
+            next_count[b] = more ? nl : 0;
+            ls.job.nR_old = nR; ls.last_esub = esub;
+        }
+        do_job(ls, more ? 6 : 4);
+    }
+};
+template <int NCAP, bool kAligned, bool kLong>
+__global__ void __launch_bounds__(kThreads)
+layers_kernel(Workspace w, Params p, const uint16_t* __restrict__ logits, int fstride, opt_tree_out out, int32_t* next_tokens,
+              int32_t* next_parent, int32_t* next_count) {
+    CtaSmemT<NCAP>& s = *reinterpret_cast<CtaSmemT<NCAP>*>(ot_smem);
+    grid_dependency_wait();
+    const int layer = __ldcg(&w.q_ctl[kQLayer]);             // (every thread has it before any CTA can leave: see run_pipeline's barrier)
+    LayersSource src{w, p, logits, fstride, layer};
+    LayersSink<LayerScratchT<NCAP>> sink{w, p, out, fstride, layer, smem_offset(&s.layer), next_tokens, next_parent, next_count};
+    run_pipeline<kAligned, kLong>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.B * fstride * p.V, w.status);
 }
 
 // Tree attention mask + position ids: one CTA per sequence, a thread per node (in rounds of the block
@@ -1382,7 +1486,6 @@ int check_launch() { return cudaGetLastError() == cudaSuccess ? OPT_TREE_OK : OP
 // Shared memory of a CTA of the persistent kernels for node budget n (one of two layouts).
 bool small_n(int n) { return n <= ot::kSmallN; }
 size_t cta_smem_bytes(int n) { return small_n(n) ? sizeof(ot::CtaSmemT<ot::kSmallN>) : sizeof(ot::CtaSmemT<ot::kMaxN>); }
-size_t layer_smem_bytes(int n) { return small_n(n) ? sizeof(ot::LayerScratchT<ot::kSmallN>) : sizeof(ot::LayerScratchT<ot::kMaxN>); }
 
 using BuildKernel = void (*)(ot::Workspace, ot::Params, const uint16_t*, opt_tree_out);
 using RowKernel = void (*)(ot::Params, const uint16_t*, const int32_t*, int, int32_t*, double*, int*);
@@ -1401,6 +1504,11 @@ RowKernel row_variant(int v) {
     return (v & kLongBit) ? ((v & kAlignedBit) ? ot::row_topk_kernel<true, true> : ot::row_topk_kernel<false, true>)
                           : ((v & kAlignedBit) ? ot::row_topk_kernel<true, false> : ot::row_topk_kernel<false, false>);
 }
+using LayersKernel = void (*)(ot::Workspace, ot::Params, const uint16_t*, int, opt_tree_out, int32_t*, int32_t*, int32_t*);
+template <int NCAP> LayersKernel layers_variant(int v) {
+    return (v & kLongBit) ? ((v & kAlignedBit) ? ot::layers_kernel<NCAP, true, true> : ot::layers_kernel<NCAP, false, true>)
+                          : ((v & kAlignedBit) ? ot::layers_kernel<NCAP, true, false> : ot::layers_kernel<NCAP, false, false>);
+}
 int variant_of(const ot::Params& p) { return (p.prune ? kPrunedBit : 0) | (p.aligned ? kAlignedBit : 0) | (p.V > ot::kLongRow ? kLongBit : 0); }
 template <class F> bool allow_smem(F* kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
@@ -1412,10 +1520,11 @@ int persistent_grid(int n) {
     int dev = 0, per_sm = 0, sms = 0;
     constexpr int S = ot::kSmallN, L = ot::kMaxN;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
-    bool ok = allow_smem(ot::layer_step_kernel<S>, sizeof(ot::LayerScratchT<S>)) && allow_smem(ot::layer_step_kernel<L>, sizeof(ot::LayerScratchT<L>));
+    bool ok = true;
     for (int v = 0; v < kVariants; ++v)
         ok = ok && allow_smem(build_variant<S>(v), sizeof(ot::CtaSmemT<S>)) && allow_smem(build_variant<L>(v), sizeof(ot::CtaSmemT<L>)) &&
-             allow_smem(row_variant(v), sizeof(ot::CtaSmem));
+             allow_smem(row_variant(v), sizeof(ot::CtaSmem)) && allow_smem(layers_variant<S>(v), sizeof(ot::CtaSmemT<S>)) &&
+             allow_smem(layers_variant<L>(v), sizeof(ot::CtaSmemT<L>));
     int least = 1 << 30;                             // the variants share one grid: the smallest occupancy counts
     for (int v = 0; v < kVariants && ok; ++v) {
         ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_kernel_for(n, v), ot::kThreads, cta_smem_bytes(n)) == cudaSuccess;
@@ -1572,7 +1681,8 @@ int opt_tree_layers_begin(opt_tree_ctx* ctx, int32_t B, void* stream) {
     if (!ctx || B < 1 || B > ctx->cfg.max_batch) return OPT_TREE_ERR_INVALID_ARG;
     ot::Params p = make_params(ctx, nullptr, 0.0f);
     p.B = B;
-    launch_after(ot::layers_begin_kernel, dim3((unsigned)((B + 127) / 128)), dim3(128), 0, static_cast<cudaStream_t>(stream), ctx->ws, p);
+    const long long blocks = ((long long)B * p.cstride + 255) / 256;
+    launch_after(ot::layers_begin_kernel, dim3((unsigned)(blocks < 1024 ? blocks : 1024)), dim3(256), 0, static_cast<cudaStream_t>(stream), ctx->ws, p);
     ctx->launches++;
     return check_launch();
 }
@@ -1585,17 +1695,11 @@ int opt_tree_layers_step(opt_tree_ctx* ctx, const void* frontier_logits, int32_t
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     ot::Params p = make_params(ctx, frontier_logits, delta);
     p.B = B;
-    const int nrows = B * frontier_stride;
-    ot::Params pr = p;
-    pr.H = nrows;                                            // the dense buffer is the "table" of the row step
-    const int grid = nrows < ctx->grid ? nrows : ctx->grid;
-    launch_after(row_variant(variant_of(p)), dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem), st,
-                 pr, static_cast<const uint16_t*>(frontier_logits), static_cast<const int32_t*>(nullptr), nrows, ctx->ws.rtok,
-                 ctx->ws.rprob, ctx->ws.status);
-    launch_after(small_n(ctx->cfg.n) ? ot::layer_step_kernel<ot::kSmallN> : ot::layer_step_kernel<ot::kMaxN>, dim3(B), dim3(ot::kTeam),
-                 layer_smem_bytes(ctx->cfg.n), st, ctx->ws, p, frontier_stride, *out, next_tokens,
-                 next_parent, next_count);
-    ctx->launches += 2;
+    const int nrows = B * frontier_stride, v = variant_of(p);
+    launch_after(small_n(ctx->cfg.n) ? layers_variant<ot::kSmallN>(v) : layers_variant<ot::kMaxN>(v), dim3(nrows < ctx->grid ? nrows : ctx->grid),
+                 dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(frontier_logits), frontier_stride, *out,
+                 next_tokens, next_parent, next_count);
+    ctx->launches++;
     return check_launch();
 }
 
@@ -1649,12 +1753,12 @@ int opt_tree_selftest_waits(opt_tree_ctx* ctx, int32_t* result, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (cudaFuncSetAttribute(ot::wait_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ot::CtaSmem)) != cudaSuccess ||
         cudaMemsetAsync(result, 0, OPT_TREE_SELFTEST_WAITS * sizeof(int32_t), st) != cudaSuccess ||
-        cudaMemsetAsync(ctx->ws.rprob, 0, 2 * sizeof(unsigned long long), st) != cudaSuccess) {     // two words nobody writes
+        cudaMemsetAsync(ctx->ws.o_mask, 0, 2 * sizeof(unsigned long long), st) != cudaSuccess) {    // two words nobody writes meanwhile
         cudaGetLastError();
         return OPT_TREE_ERR_CUDA;
     }
     ot::wait_probe_kernel<<<1, ot::kThreads, sizeof(ot::CtaSmem), st>>>(
-        result, reinterpret_cast<const unsigned long long*>(ctx->ws.rprob), 1ll << 16, 1 << 10);
+        result, reinterpret_cast<const unsigned long long*>(ctx->ws.o_mask), 1ll << 16, 1 << 10);
     ctx->launches++;
     return check_launch();
 }
