@@ -16,11 +16,13 @@ namespace ot {
 constexpr int kRowMul = 31;                 // row of (token t, depth d) = (t*31 + d) mod H
 constexpr int kSmallThreads = 256;          // block size of the mask / init kernels
 // Verify: one CTA per target row, a thread keeps eight 16-byte loads in flight.  With 128 threads sixteen CTAs fit an
-// SM, so the n + 1 rows of 32 sequences (c4: 2080 CTAs) are all resident at once instead of in two uneven waves.  When
-// three CTAs of 512 threads per SM hold all rows (444 of them), a row is spread over four times the threads: few
-// rows are bound by the round trips of a CTA's loop (32000 logits: four of them with 128 threads, one with 512).
-// Measured (B200): 65 rows of 128256 logits 24.9 us with 128 threads, 12.8 with 512.
-constexpr int kVerifyThreads = 128, kVerifyThreadsFew = 512;
+// SM, so the n + 1 rows of 32 sequences (c4: 2080 CTAs) are all resident at once instead of in two uneven waves.  Fewer
+// rows are bound by the round trips of a CTA's loop (32000 logits: four of them with 128 threads, one with 512) and take
+// wider CTAs as long as all are resident: 512 threads up to three rows per SM, 256 up to eight (sampled: six).
+// Measured (B200, us with 128 / 256 / 512 threads): 65 rows of 128256 logits greedy 24.9 / 15.5 / 12.5; 244 rows of 32000
+// greedy - / 9.4 / 8.6, sampled - / 13.4 / 12.3; 488 rows 12.2 / 10.5 / 13.1 and 20.2 / 17.0 / 18.7; 784 rows 14.0 / 12.1 / - and
+// 22.4 / 20.8 / -; 1026 rows 15.9 / 14.6 / - and 26.2 / 27.9 / -.
+constexpr int kVerifyMany = 128, kVerifySome = 256, kVerifyFew = 512;
 
 __device__ __forceinline__ int row_of(int token, int depth, int H) {
     return (int)(((unsigned)token * (unsigned)kRowMul + (unsigned)depth) % (unsigned)H);     // below 2^31 (supported_cfg); in 64 bits this is 1 % of a build
@@ -1018,19 +1020,19 @@ __device__ __noinline__ unsigned long long best_of_ends(const uint16_t* row, int
 // kept node j-1; each finds the row's argmax (lowest token on ties).  The last CTA of a sequence
 // then walks the tree: accept the child that carries the target's token, until none does.
 template <int T>
-__global__ void __launch_bounds__(T)
+__global__ void __launch_bounds__(T, T == kVerifyFew ? 3 : 2048 / T)
 verify_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const int32_t* __restrict__ root_token,
               opt_tree_out tree, int32_t* accept_len, int32_t* accept_tokens, int32_t* accept_nodes, int32_t* next_root) {
     int* verify_walk = reinterpret_cast<int*>(ot_smem);
     __shared__ VerifySmem<T> s;
     grid_dependency_wait();
     const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x;
-    const int ns = tree.n_sel[b];
-    if (j > ns) return;
     const int32_t* tok = tree.token + (size_t)b * p.n;
     const int32_t* par = tree.parent + (size_t)b * p.n;
+    const int ns = tree.n_sel[b];                            // (all three loads at once: an unused slot's token is never looked at)
     int token = j == 0 ? root_token[b] : tok[j - 1];
     const int depth = j == 0 ? 0 : tree.depth[(size_t)b * p.n + j - 1];
+    if (j > ns) return;
     if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
     const uint16_t* row = target + (size_t)row_of(token, depth, p.H) * p.V;
 
@@ -1213,7 +1215,7 @@ __device__ __noinline__ SegPart edge_part(const uint16_t* row, int t0, int t1, f
 // double-precision inverse CDF over the whole row is the placement of u*S relative to a segment's start, by
 // the rounding of the single-precision sums (a few 1e-7 of S).
 template <int T>
-__global__ void __launch_bounds__(T, T == kVerifyThreads ? 16 : 3)
+__global__ void __launch_bounds__(T, T == kVerifyMany ? 16 : (T == kVerifySome ? 6 : 3))
 verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const int32_t* __restrict__ root_token,
                       opt_tree_out tree, double tau, unsigned long long seed, unsigned long long step, int32_t* accept_len,
                       int32_t* accept_tokens, int32_t* accept_nodes, int32_t* next_root) {
@@ -1222,12 +1224,12 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
     __shared__ SampleSmem<T> q;
     grid_dependency_wait();
     const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
-    const int ns = tree.n_sel[b];
-    if (j > ns) return;
     const int32_t* tok = tree.token + (size_t)b * p.n;
     const int32_t* par = tree.parent + (size_t)b * p.n;
+    const int ns = tree.n_sel[b];                            // (all three loads at once: an unused slot's token is never looked at)
     int token = j == 0 ? root_token[b] : tok[j - 1];
     const int depth = j == 0 ? 0 : tree.depth[(size_t)b * p.n + j - 1];
+    if (j > ns) return;
     if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
     const uint16_t* row = target + (size_t)row_of(token, depth, p.H) * p.V;
     const double u = uniform53(seed, step, b, j);
@@ -1475,8 +1477,11 @@ void launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, 
     cfg.attrs = attr; cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
-// Whether the verification's rows are so few that CTAs of kVerifyThreadsFew threads are all resident at once.
-bool few_rows(int n, int B, int sms) { return (long long)(n + 1) * B <= (long long)sms * 3; }
+// Threads of a verification CTA for (n + 1) * B rows (see kVerifyMany); `some`: rows per SM up to which CTAs of 256 are taken.
+int verify_threads(int n, int B, int sms, int some) {
+    const long long rows = (long long)(n + 1) * B;
+    return rows <= 3ll * sms ? ot::kVerifyFew : (rows <= (long long)some * sms ? ot::kVerifySome : ot::kVerifyMany);
+}
 size_t walk_smem(int n) { return (size_t)(3 * n + 1) * sizeof(int); }
 bool bad_tree(const opt_tree_out* t) {
     return !t || !t->token || !t->parent || !t->depth || !t->phat || !t->n_sel || !t->depth_reached || !t->expected_len;
@@ -1640,9 +1645,10 @@ int opt_tree_verify(opt_tree_ctx* ctx, const opt_tree_out* tree, const void* tar
         B < 1 || B > ctx->cfg.max_batch)
         return OPT_TREE_ERR_INVALID_ARG;
     const ot::Params p = make_params(ctx, target, 0.0f);
-    const bool few = few_rows(ctx->cfg.n, B, ctx->sms);
-    launch_after(few ? ot::verify_kernel<ot::kVerifyThreadsFew> : ot::verify_kernel<ot::kVerifyThreads>, dim3(ctx->cfg.n + 1, B),
-                 dim3(few ? ot::kVerifyThreadsFew : ot::kVerifyThreads), walk_smem(ctx->cfg.n), static_cast<cudaStream_t>(stream),
+    const int threads = verify_threads(ctx->cfg.n, B, ctx->sms, 8);
+    launch_after(threads == ot::kVerifyFew ? ot::verify_kernel<ot::kVerifyFew>
+                                           : (threads == ot::kVerifySome ? ot::verify_kernel<ot::kVerifySome> : ot::verify_kernel<ot::kVerifyMany>),
+                 dim3(ctx->cfg.n + 1, B), dim3(threads), walk_smem(ctx->cfg.n), static_cast<cudaStream_t>(stream),
                  ctx->ws, p, static_cast<const uint16_t*>(target), root_token, *tree, accept_len, accept_tokens, accept_nodes, next_root);
     ctx->launches++;
     return check_launch();
@@ -1655,9 +1661,10 @@ int opt_tree_verify_sampled(opt_tree_ctx* ctx, const opt_tree_out* tree, const v
         B < 1 || B > ctx->cfg.max_batch || !(tau > 0.0))
         return OPT_TREE_ERR_INVALID_ARG;
     const ot::Params p = make_params(ctx, target, 0.0f);
-    const bool few = few_rows(ctx->cfg.n, B, ctx->sms);
-    launch_after(few ? ot::verify_sampled_kernel<ot::kVerifyThreadsFew> : ot::verify_sampled_kernel<ot::kVerifyThreads>, dim3(ctx->cfg.n + 1, B),
-                 dim3(few ? ot::kVerifyThreadsFew : ot::kVerifyThreads), walk_smem(ctx->cfg.n), static_cast<cudaStream_t>(stream),
+    const int threads = verify_threads(ctx->cfg.n, B, ctx->sms, 6);
+    launch_after(threads == ot::kVerifyFew ? ot::verify_sampled_kernel<ot::kVerifyFew>
+                                           : (threads == ot::kVerifySome ? ot::verify_sampled_kernel<ot::kVerifySome> : ot::verify_sampled_kernel<ot::kVerifyMany>),
+                 dim3(ctx->cfg.n + 1, B), dim3(threads), walk_smem(ctx->cfg.n), static_cast<cudaStream_t>(stream),
                  ctx->ws, p, static_cast<const uint16_t*>(target), root_token, *tree, tau, (unsigned long long)seed,
                  (unsigned long long)step, accept_len, accept_tokens, accept_nodes, next_root);
     ctx->launches++;
@@ -1851,7 +1858,7 @@ extern "C" int opt_tree_verify_static(const opt_tree_config* cfg, const opt_tree
     p.V = cfg->V; p.H = cfg->H; p.n = cfg->n; p.k = cfg->k; p.kk = cfg->k < cfg->V ? cfg->k : cfg->V;
     p.max_depth = cfg->max_depth; p.Dcap = cfg->max_depth < cfg->n ? cfg->max_depth : cfg->n;
     p.aligned = ((reinterpret_cast<uintptr_t>(target) & 15u) == 0 && (cfg->V % 8) == 0) ? 1 : 0;
-    ot::verify_kernel<ot::kVerifyThreads><<<dim3(cfg->n + 1, B), ot::kVerifyThreads, walk_smem(cfg->n), st>>>(
+    ot::verify_kernel<ot::kVerifyMany><<<dim3(cfg->n + 1, B), ot::kVerifyMany, walk_smem(cfg->n), st>>>(
         ws, p, static_cast<const uint16_t*>(target), root_token, *tree, accept_len, accept_tokens, accept_nodes, next_root);
     if (cudaGetLastError() != cudaSuccess) return OPT_TREE_ERR_CUDA;
     if (device_status && cudaMemcpyAsync(device_status, ws.status, sizeof(int32_t), cudaMemcpyDeviceToDevice, st) != cudaSuccess)

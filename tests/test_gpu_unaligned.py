@@ -49,7 +49,7 @@ def test_a_row_gives_the_same_bits_at_every_offset():
 
 
 @pytest.mark.parametrize("V", [1, 5, 9, 513, 4103, 33013])
-@pytest.mark.parametrize("B", [1, 64])                       # 9 rows take wide blocks, 576 the narrow ones
+@pytest.mark.parametrize("B", [1, 64, 130])                  # 9 rows take blocks of 512 threads, 576 of 256, 1170 of 128 (148 SMs)
 @pytest.mark.parametrize("shift", [0, 1, 7])
 def test_verification_at_any_offset(V, B, shift):
     n, k, D, H = 8, min(4, V), 5, 17
