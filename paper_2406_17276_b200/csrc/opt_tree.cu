@@ -1019,8 +1019,10 @@ __device__ __noinline__ unsigned long long best_of_ends(const uint16_t* row, int
 // Greedy verification.  CTA (j, b): j = 0 takes the target row after the root, j >= 1 the row after
 // kept node j-1; each finds the row's argmax (lowest token on ties).  The last CTA of a sequence
 // then walks the tree: accept the child that carries the target's token, until none does.
+// (0: no minimum of resident CTAs is asked for.  The narrow forms then take 32 registers and read 6.5 TB/s; asked for 16 or 8
+// CTAs they do so with worse scheduling, 22.1 us instead of 20.4 on 2080 rows, and asked for one they take 56 registers, 24.3 us.)
 template <int T>
-__global__ void __launch_bounds__(T, T == kVerifyFew ? 3 : 2048 / T)
+__global__ void __launch_bounds__(T, T == kVerifyFew ? 3 : 0)
 verify_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const int32_t* __restrict__ root_token,
               opt_tree_out tree, int32_t* accept_len, int32_t* accept_tokens, int32_t* accept_nodes, int32_t* next_root) {
     int* verify_walk = reinterpret_cast<int*>(ot_smem);
