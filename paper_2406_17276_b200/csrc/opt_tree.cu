@@ -464,14 +464,15 @@ struct BuildSink {
             else select_layer_team_big<kPrune, LS>(at, tt, w.status);
         }
     }
-    // Rows of a layer of f rows that may still be missing when the team starts on it.  Candidate words validate themselves,
+    // Rows of layer d, of f rows, that may still be missing when the team starts on it.  Candidate words validate themselves,
     // so the job's hand-over, the staging and most of the sweep go on while the last rows are finished, and only what
-    // is missing then is waited for.  Sixteen rows, or a quarter of a large layer: one sequence of n = 50 126.7 us per
-    // build with none, 125.8 with 2, 124.2 with 8, 123.5 with 16; n = 512 429 with none, 422 with 16, 413 with a quarter
-    // or a half; n = 64, V = 128256 281 with none, 272 with 16, 276 with half; 32 sequences 221.5, 219.7, 220.7.
+    // is missing then is waited for.  As long as a layer's rows of all sequences take the SMs at most four times round, all
+    // but the first may be missing (see sweep_candidates); otherwise, and in the selections that stage their
+    // candidates (pruned draft, depth limit), sixteen rows or a quarter of a large layer: 32 sequences 221.5 us per build with
+    // none, 219.7 with 16, 220.7 with half; n = 512 429 with none, 413 with a quarter or a half.
     // A warp that follows several sequences must not wait for one of them.
-    __device__ int rows_ahead(int f) const {
-        const int a = max(16, f >> 2);
+    __device__ int rows_ahead(int f, int d) const {
+        const int a = !kPrune && d < p.Dcap && p.B * f <= 4 * (int)gridDim.x ? f - 1 : max(16, f >> 2);
         return p.B <= (int)gridDim.x ? min(a, f - 1) : 0;
     }
     template <class LS>
@@ -498,7 +499,7 @@ struct BuildSink {
                     int done = 0;
                     if (lane == 0) done = ld_acquire_s32(&sw.st[kStDone]);
                     done = __shfl_sync(0xFFFFFFFFu, done, 0);
-                    if (done < cur_tot[q] - (cur_d[q] > 1 ? rows_ahead(cur_f[q]) : 0)) continue;
+                    if (done < cur_tot[q] - (cur_d[q] > 1 ? rows_ahead(cur_f[q], cur_d[q]) : 0)) continue;
                     progressed = true;
                     if (cur_d[q] == 1) {
                         // the finisher of the root's row says whether it grew layer 1 itself (then layer 2 is on its way)
@@ -535,7 +536,7 @@ struct BuildSink {
                         }
                     }
                     const bool early = !kPrune && d < p.Dcap && p.delta == -INFINITY;
-                    stage_layer_candidates(ls, sw, fsize, p.k);
+                    if (fsize * p.k <= kTeam) stage_layer_candidates(ls, sw, fsize, p.k);
                     unsigned g0 = 0;
                     if (early) g0 = reserve_layer(nl);        // the rows' numbers, while the candidates load
                     {
@@ -547,7 +548,7 @@ struct BuildSink {
                             j.T_tok = sw.T_tok; j.T_par = sw.T_par; j.T_phat = sw.T_phat;
                             j.fmap = kPrune ? sw.fmap : nullptr;
                         }
-                        if (small) cp_async_wait_all();       // the staged candidates are in shared memory
+                        if (fsize * p.k <= kTeam) cp_async_wait_all();       // the staged candidates are in shared memory
                         __syncwarp();
                         team_sync();                          // ... and, with the job, visible to the assistants
                         if (small) select_layer_team<kPrune, LS>(smem_offset(&ls), lane, w.status);
@@ -827,7 +828,6 @@ struct LayersSink {
         const int fsize = __ldcg(&sw.st[kStFront + (layer & 1)]), nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
         const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
         const int nvalid = fsize * p.kk, nl = nvalid < p.n ? nvalid : p.n;
-        stage_layer_candidates(ls, sw, fsize, p.k);
         if (lane == 0) {
             LayerJob& j = ls.job;
             j.b = b; j.d = d; j.fsize = fsize; j.n = p.n; j.k = p.k; j.kk = p.kk;
@@ -836,7 +836,7 @@ struct LayersSink {
             j.nR_old = nR_old; j.off = 0; j.max_depth = p.max_depth;
             j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
         }
-        cp_async_wait_all();
+        if (fsize * p.k <= kTeam) { stage_layer_candidates(ls, sw, fsize, p.k); cp_async_wait_all(); }
         do_job(ls, 1);
         if (lane == 0) ls.job.fsize = nl;
         do_job(ls, 3);
