@@ -309,45 +309,6 @@ struct RowOut {        // lane j < kk holds the j-th most probable token and its
     double p;
 };
 
-// 64 keys, two per lane (element i = lane + 32*q is x[q]), sorted descending by element index.
-__device__ __forceinline__ void warp_sort64_desc(unsigned long long& x0, unsigned long long& x1) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int size = 2; size <= 64; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride == 32) {
-                // partner of element lane is element lane+32; in the last merge all pairs keep the maximum low
-                const unsigned long long hi = x0 > x1 ? x0 : x1, lo = x0 > x1 ? x1 : x0;
-                x0 = hi; x1 = lo;
-            } else {
-                const unsigned long long p0 = __shfl_xor_sync(0xFFFFFFFFu, x0, stride);
-                const unsigned long long p1 = __shfl_xor_sync(0xFFFFFFFFu, x1, stride);
-                const bool lower = (lane & stride) == 0;
-                const bool desc0 = (lane & size) == 0;                   // block of element lane
-                const bool desc1 = ((lane + 32) & size) == 0;            // block of element lane+32
-                x0 = (lower == desc0) ? (x0 > p0 ? x0 : p0) : (x0 < p0 ? x0 : p0);
-                x1 = (lower == desc1) ? (x1 > p1 ? x1 : p1) : (x1 < p1 ? x1 : p1);
-            }
-        }
-    }
-}
-
-// 32 keys, one per lane, sorted descending across lanes.
-__device__ __forceinline__ unsigned long long warp_sort32_desc(unsigned long long v) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const unsigned long long p = __shfl_xor_sync(0xFFFFFFFFu, v, stride);
-            const bool keep_max = ((lane & stride) == 0) == ((lane & size) == 0);
-            v = keep_max ? (v > p ? v : p) : (v < p ? v : p);
-        }
-    }
-    return v;
-}
-
 // The finisher's code is walked once per row, by several warps at different places at once, next to
 // the consumers' loop: its size decides how often instructions have to be fetched again.  So its
 // common path is kept short (packed 16-bit operations, loops instead of unrolled sequences), and
@@ -532,16 +493,28 @@ __device__ __forceinline__ uint32_t ge_bf16x2(uint32_t a, uint32_t b) {
 }
 
 // Ranks M <= 64 candidates (f.cand[0..M), distinct keys) and gives lane j < kk the j-th largest with
-// its probability.  S is the row's sum without the candidates unless `exact`.  The common case, up
-// to one candidate per lane, ranks by counting; more than 32 are sorted (rare).
+// its probability.  S is the row's sum without the candidates unless `exact`.  Every row with kk near 32 comes here (up to 32
+// candidates finish_row_warp ranks itself).  By counting, two candidates per lane: a bitonic sort of 64 keys had as many
+// instructions, but 22 KB of them in a row, which a finisher had to fetch again for every row (20000 rows of 32000 logits, k = 32: 243 -> 235 us).
 __device__ __noinline__ void finish_many(FinScratch& f, int M, int kk, double m, double S, bool exact, RowOut& out) {
     const int lane = threadIdx.x & 31;
-    unsigned long long x0 = f.cand[lane], x1 = lane + 32 < M ? f.cand[lane + 32] : 0ull;
-    warp_sort64_desc(x0, x1);
+    const unsigned long long x0 = f.cand[lane], x1 = lane + 32 < M ? f.cand[lane + 32] : 0ull;
     const double e0 = exp_f64((double)cand_logit(x0) - m);
     const double e1 = x1 ? exp_f64((double)cand_logit(x1) - m) : 0.0;
     if (!exact) S += (double)warp_sum_u64(__double2ull_rn(e0 * kFixScale) + __double2ull_rn(e1 * kFixScale)) / kFixScale;
-    if (lane < kk) { out.tok = (int32_t)cand_token(x0); out.p = e0 / S; }
+    int r0 = 0, r1 = 0;
+#pragma unroll 2
+    for (int j = 0; j < M; ++j) {
+        const unsigned long long x = f.cand[j];
+        r0 += x > x0 ? 1 : 0;
+        r1 += x > x1 ? 1 : 0;
+    }
+    __syncwarp();
+    if (r0 < kk) { f.cand[r0] = x0; f.cand[64 + r0] = (unsigned long long)__double_as_longlong(e0); }
+    if (x1 && r1 < kk) { f.cand[r1] = x1; f.cand[64 + r1] = (unsigned long long)__double_as_longlong(e1); }
+    __syncwarp();
+    if (lane < kk) { out.tok = (int32_t)cand_token(f.cand[lane]); out.p = __longlong_as_double((long long)f.cand[64 + lane]) / S; }
+    __syncwarp();
 }
 
 // The search of finish_row_warp in long rows: the flagged threads' vectors are read again for the logits >= tau.  The list is
