@@ -114,7 +114,7 @@ __device__ void fetcher_role(CtaCore& s, Source& src, int* status, long long lim
 // table's logits [lo, hi): what is left of the chunk there, at most seven halves at either end of the table, the warp
 // copies with ordinary loads.  The chunk starts at half vec_offset(row) of the stage.
 // Measured (1999 rows of 50257 logits, B200): 2591 us with two-byte loads by the issuer warp, whose round trips
-// were the bound; 71.5 us with granule copies (2.8 TB/s), bound by the consumers' instructions.
+// were the bound; 71.5 us with granule copies, bound by the consumers' instructions, 61.9 (3.2 TB/s) since these were cut.
 __device__ __noinline__ void copy_chunk_unaligned(uint16_t* stage, const uint16_t* src, int ne, const uint16_t* lo, const uint16_t* hi,
                                                   unsigned long long* bar) {
     const int lane = threadIdx.x & 31;
