@@ -61,7 +61,8 @@ struct Workspace {
     uint64_t* o_mask; int32_t* o_pos;
     int32_t *o_alen, *o_atok, *o_anode, *o_next;
 };
-enum { kQFinished = 2, kQDone = 3, kQCursor = 4, kQLayer = 5, kQLeft = 6 };   // 5, 6: layer-by-layer build: layers done, CTAs that have left this one
+enum { kQFinished = 2, kQDone = 3, kQCursor = 4, kQLayer = 5, kQLeft = 6,    // 5, 6: layer-by-layer build: layers done, CTAs that have left this one
+       kQTail = 0, kQHead = 1 };    // and sequences put into / taken from the queue of those whose rows are all in
 
 constexpr int kMaxGrid = 4096;              // CTAs of the persistent kernels (SMs x occupancy) this layout supports
 
@@ -679,9 +680,12 @@ row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __
 // per layer: the row pipeline over the dense buffer, its finishers leave the candidates (Eq. 2) as they do in the
 // persistent build, and the CTA whose finisher completes a sequence's last row has its layer team select the layer, update
 // the running top-n / E_sub, apply the loop test and hand back the next layer's tokens; a sequence that stops is packed on
-// the spot.  No CTA waits for another one, so nothing is assumed about which of them run together.
-// Two launches per layer (rows, then a CTA per sequence that formed the candidates) took 31 us a layer for 8 sequences of n = 50,
-// V = 32000, this 26.
+// the spot.  A CTA whose team is at work finishes its rows later than others and so tends to complete the next sequences too:
+// what it completes meanwhile goes to a queue that every idle team looks at, and that a CTA leaves only empty.  No CTA waits
+// for another one's rows, so nothing is assumed about which of them run together.
+// Ten layers, V = 32000 (us): two launches per layer (rows, then a CTA per sequence that formed the candidates) / the CTA that
+// completes a sequence takes it / with the queue: 8 sequences of n = 50 354 / 268 / 237; 32 of n = 64 519 / 739 / 375; 64 of n = 24
+// 436 / 672 / 347; 8 of n = 256, k = 16 969 / 622 / 463.
 // ------------------------------------------------------------------------------------------------
 __global__ void layers_begin_kernel(Workspace w, Params p) {
     grid_dependency_wait();
@@ -690,9 +694,10 @@ __global__ void layers_begin_kernel(Workspace w, Params p) {
         reinterpret_cast<unsigned long long*>(w.cand_phat)[j] = 0ull;
         w.cand_tok[j] = 0;
     }
-    if (i == 0) { w.q_ctl[kQLayer] = 0; w.q_ctl[kQLeft] = 0; }
+    if (i == 0) { w.q_ctl[kQLayer] = 0; w.q_ctl[kQLeft] = 0; w.q_ctl[kQTail] = 0; w.q_ctl[kQHead] = 0; }
     if (i >= p.B) return;
     int32_t* st = w.st + (size_t)i * 8;
+    st[kStQueue] = 0;
     st[kStDone] = 0; st[kStNR] = 0; st[kStFront] = 1; st[kStFront + 1] = 0;
     w.E_prev[i] = 0.0;
     w.front_phat[(size_t)i * 2 * p.n] = 1.0;                       // the root counts as factor 1
@@ -736,16 +741,26 @@ struct LayersSink {
         if (lane == 0) {
             LS& ls = smem_at<LS>(at);
             if (atomicAdd(&sw.st[kStDone], 1) + 1 == d.fsize) {            // (the words validate themselves: no fence)
-                const int pos = atomicAdd(&ls.todo_tail, 1);
-                const long long t0 = clock64();
-                while (pos - ls.todo_head >= LS::kTodo)
-                    if (clock64() - t0 > kWaitCycles) { set_status(w.status, kErrTimeout); break; }
-                ls.todo[pos % LS::kTodo] = d.b + 1;
+                // this CTA's team, or, if that has a sequence already, the team that comes first
+                if (atomicCAS(const_cast<int*>(&ls.todo), 0, d.b + 1) != 0) {
+                    const int pos = atomicAdd(&w.q_ctl[kQTail], 1);
+                    st_release_s32(&w.st[(size_t)pos * 8 + kStQueue], d.b + 1);
+                }
             }
             __threadfence_block();
             atomicAdd(&ls.rows_done, 1);
         }
         __syncwarp();
+    }
+    static constexpr int kClaimed = 0x7FFFFFFF;
+    // 1 + the sequence in place h of the queue, whose number was given out before the entry was written; the place is free again.
+    __device__ __noinline__ int take_queued(int h) {
+        int32_t* e = &w.st[(size_t)h * 8 + kStQueue];
+        int v = ld_acquire_s32(e);
+        for (int t = 0; v == 0 && t < kWaitPolls; ++t) v = ld_acquire_s32(e);
+        if (v == 0) set_status(w.status, kErrTimeout);
+        *e = 0;
+        return v;
     }
     __device__ void layer_loop(LS& ls) {
         const int lane = threadIdx.x & 31;
@@ -759,21 +774,44 @@ struct LayersSink {
         }
         __syncwarp();
         const CtaCore& core = smem_at<CtaCore>(0);
-        int head = 0, seen = 0;
+        int seen = 0;
         long long t0 = clock64();
-        for (;;) {
-            const int v = __shfl_sync(0xFFFFFFFFu, ls.todo[head % LS::kTodo], 0);
+        for (int turn = 0;; ++turn) {
+            const int v = __shfl_sync(0xFFFFFFFFu, ls.todo, 0);
             if (v) {
-                __syncwarp();
-                if (lane == 0) { ls.todo[head % LS::kTodo] = 0; __threadfence_block(); ls.todo_head = head + 1; }
-                ++head;
                 step(ls, v - 1);
+                if (lane == 0) ls.todo = 0;
+                __syncwarp();
                 t0 = clock64();
                 continue;
             }
-            // every row of this CTA finished, and (pushed before it was counted) every sequence taken
-            const int done = *reinterpret_cast<volatile int*>(&ls.rows_done);
-            if (__any_sync(0xFFFFFFFFu, done >= core.stop_row && head == *reinterpret_cast<volatile int*>(&ls.todo_tail))) break;
+            // Every row of this CTA finished: it leaves when it finds the queue empty (what its own finishers put there came before
+            // they counted the row).
+            const int done = __shfl_sync(0xFFFFFFFFu, *reinterpret_cast<volatile int*>(&ls.rows_done), 0);
+            const bool last = __any_sync(0xFFFFFFFFu, lane == 0 && done >= core.stop_row);
+            if (last || (turn & 7) == 7) {
+                int got = 0;                               // lane 0: 1 + the sequence taken, -1: the queue is empty
+                if (lane == 0) {
+                    __threadfence_block();
+                    // (the team is claimed first, so that the finishers send what they complete to the queue)
+                    if (atomicCAS(const_cast<int*>(&ls.todo), 0, kClaimed) == 0) {
+                        const unsigned int* q = reinterpret_cast<const unsigned int*>(w.q_ctl);
+                        const int h = (int)ld_relaxed_u32(&q[kQHead]), t = (int)ld_relaxed_u32(&q[kQTail]);
+                        if (h >= t) got = -1;
+                        else if (atomicCAS(&w.q_ctl[kQHead], h, h + 1) == h) got = take_queued(h);
+                        if (got <= 0) ls.todo = 0;
+                    }
+                }
+                got = __shfl_sync(0xFFFFFFFFu, got, 0);
+                if (got > 0) {
+                    step(ls, got - 1);
+                    if (lane == 0) ls.todo = 0;
+                    __syncwarp();
+                    t0 = clock64();
+                    continue;
+                }
+                if (last && got < 0) break;
+            }
             if (done != seen) { seen = done; t0 = clock64(); }
             else if (__any_sync(0xFFFFFFFFu, clock64() - t0 > kWaitCycles)) { set_status(w.status, kErrTimeout); break; }
             __nanosleep(kPollPauseNs);
@@ -782,7 +820,9 @@ struct LayersSink {
         if (lane == 0) {
             ls.job.kind = 0;
             __threadfence();
-            if (atomicAdd(&w.q_ctl[kQLeft], 1) == (int)gridDim.x - 1) { w.q_ctl[kQLeft] = 0; w.q_ctl[kQLayer] = layer + 1; }
+            if (atomicAdd(&w.q_ctl[kQLeft], 1) == (int)gridDim.x - 1) {
+                w.q_ctl[kQLeft] = 0; w.q_ctl[kQTail] = 0; w.q_ctl[kQHead] = 0; w.q_ctl[kQLayer] = layer + 1;
+            }
         }
         __syncwarp();
         team_sync();

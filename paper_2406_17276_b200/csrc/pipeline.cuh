@@ -38,8 +38,7 @@ __device__ __forceinline__ void pipeline_init(CtaCore& s, LS& layer) {
         mbar_fence_init();
     }
     for (int i = threadIdx.x; i < 4 * 256; i += kThreads) (&layer.thist[0][0])[i] = 0;
-    if (threadIdx.x < LS::kTodo) layer.todo[threadIdx.x] = 0;
-    if (threadIdx.x == 0) { layer.cache_b = -1; layer.cache_d = -1; layer.todo_head = 0; layer.todo_tail = 0; layer.rows_done = 0; }
+    if (threadIdx.x == 0) { layer.cache_b = -1; layer.cache_d = -1; layer.todo = 0; layer.rows_done = 0; }
     __syncthreads();
 }
 

@@ -116,10 +116,8 @@ struct alignas(16) LayerScratchT {
     static constexpr int kList = 64;
     unsigned long long list[kList];            // large layers: keys of the threshold's bin
     int listn;
-    static constexpr int kTodo = 64;
-    volatile int todo[kTodo];                  // layer-by-layer build: sequences whose rows are all in (index + 1), a ring
-    volatile int todo_head;
-    int todo_tail, rows_done;
+    volatile int todo;                         // layer-by-layer build: the sequence the team has (index + 1), 0: it is idle
+    int rows_done;
     double last_esub;                          // E_sub of the tree that is to be packed
     int scan_c[kTeamWarps];
     int cache_b, cache_d;                      // rsel / vals hold the top-n of this sequence after this layer (-1: nothing)

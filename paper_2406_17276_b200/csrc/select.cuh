@@ -35,8 +35,9 @@ struct SeqWork {
     int32_t* st;           // [8]      1: rows finished since the build began, 2: |R|
     int32_t* fmap;         // [n]      pruned draft: layer slot of the node behind each frontier row
 };
-enum { kStDone = 1, kStNR = 2, kStFront = 4, kStL1 = 6 };   // 4, 5: layer-by-layer build: rows of an even / odd layer (0: finished)
+enum { kStDone = 1, kStNR = 2, kStFront = 4, kStL1 = 6, kStQueue = 7 };   // 4, 5: layer-by-layer build: rows of an even / odd layer (0: finished)
 // 6: how the root's row was handled (top bit: decided; the rest: rows of layer 2 if its finisher grew layer 1 itself, else 0)
+// 7: layer-by-layer build: entry of the queue of sequences whose rows are all in (sequence + 1)
 
 struct TreeOut {           // mirrors opt_tree_out, pointers offset to the sequence
     int32_t *token, *parent, *depth;
