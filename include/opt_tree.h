@@ -181,6 +181,8 @@ int opt_tree_build_pruned(opt_tree_ctx *ctx, const void *draft_logits_bf16, cons
  *   next_tokens     (dev) [B][n] int32  tokens of the new layer's nodes (to be expanded next)
  *   next_parent     (dev) [B][n] int32  for each, the index of its parent in the previous layer
  *   next_count      (dev) [B]   int32  nodes in the new layer; 0: this tree is finished
+ * A step may be asked of the first B sequences of the batch only; the others stay where they are, and every sequence goes
+ * on from its own layer.
  * One context builds one batch of trees at a time this way (the state lives in its workspace).
  * Both calls only enqueue work on `stream`; errors as opt_tree_build. */
 int opt_tree_layers_begin(opt_tree_ctx *ctx, int32_t B, void *stream);

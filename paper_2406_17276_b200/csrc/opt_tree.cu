@@ -61,7 +61,7 @@ struct Workspace {
     uint64_t* o_mask; int32_t* o_pos;
     int32_t *o_alen, *o_atok, *o_anode, *o_next;
 };
-enum { kQFinished = 2, kQDone = 3, kQCursor = 4, kQLayer = 5, kQLeft = 6,    // 5, 6: layer-by-layer build: layers done, CTAs that have left this one
+enum { kQFinished = 2, kQDone = 3, kQCursor = 4, kQCall = 5, kQLeft = 6,    // 5, 6: layer-by-layer build: steps since the beginning, CTAs that have left this one
        kQTail = 0, kQHead = 1 };    // and sequences put into / taken from the queue of those whose rows are all in
 
 constexpr int kMaxGrid = 4096;              // CTAs of the persistent kernels (SMs x occupancy) this layout supports
@@ -687,6 +687,27 @@ row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __
 // completes a sequence takes it / with the queue: 8 sequences of n = 50 354 / 268 / 237; 32 of n = 64 519 / 739 / 375; 64 of n = 24
 // 436 / 672 / 347; 8 of n = 256, k = 16 969 / 622 / 463.
 // ------------------------------------------------------------------------------------------------
+// Where a sequence's tree stands: `rows` nodes of layer `layer` are to be expanded next (0: the tree is finished).  A step may
+// be asked of fewer sequences than the one before, so every sequence counts its own layers.  While a step runs, its CTAs
+// must all see the state from before it: a sequence's even and odd layers have a word each, with the number of the
+// step from which on it holds, and the newest that holds already counts.
+struct Front { int layer, rows; };
+constexpr int kNever = 0x7FFFFFFF;
+__device__ __forceinline__ unsigned long long front_word(int call, int layer, int rows) {
+    return ((unsigned long long)(unsigned)call << 32) | ((unsigned)layer << 16) | (unsigned)rows;
+}
+__device__ __forceinline__ unsigned long long* front_words(const Workspace& w, int b) {
+    return reinterpret_cast<unsigned long long*>(w.st + (size_t)b * 8 + kStFront);
+}
+__device__ __forceinline__ Front front_at(const Workspace& w, int b, int call) {
+    const unsigned long long* f = front_words(w, b);
+    unsigned long long e = ld_relaxed_u64(f), o = ld_relaxed_u64(f + 1);
+    if ((int)(e >> 32) > call) e = 0ull;
+    if ((int)(o >> 32) > call) o = 0ull;
+    const unsigned long long v = (e >> 32) >= (o >> 32) ? e : o;
+    return Front{(int)((v >> 16) & 0xFFFFu), (int)(v & 0xFFFFu)};
+}
+
 __global__ void layers_begin_kernel(Workspace w, Params p) {
     grid_dependency_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -694,11 +715,13 @@ __global__ void layers_begin_kernel(Workspace w, Params p) {
         reinterpret_cast<unsigned long long*>(w.cand_phat)[j] = 0ull;
         w.cand_tok[j] = 0;
     }
-    if (i == 0) { w.q_ctl[kQLayer] = 0; w.q_ctl[kQLeft] = 0; w.q_ctl[kQTail] = 0; w.q_ctl[kQHead] = 0; }
+    if (i == 0) { w.q_ctl[kQCall] = 0; w.q_ctl[kQLeft] = 0; w.q_ctl[kQTail] = 0; w.q_ctl[kQHead] = 0; }
     if (i >= p.B) return;
     int32_t* st = w.st + (size_t)i * 8;
     st[kStQueue] = 0;
-    st[kStDone] = 0; st[kStNR] = 0; st[kStFront] = 1; st[kStFront + 1] = 0;
+    st[kStDone] = 0; st[kStNR] = 0;
+    front_words(w, (int)i)[0] = front_word(0, 0, 1);               // the root
+    front_words(w, (int)i)[1] = front_word(kNever, 0, 0);
     w.E_prev[i] = 0.0;
     w.front_phat[(size_t)i * 2 * p.n] = 1.0;                       // the root counts as factor 1
 }
@@ -708,25 +731,25 @@ struct LayersSource {
     static constexpr bool kHasEmpty = true;
     Workspace w; Params p;
     const uint16_t* logits;
-    int fstride, layer;                                    // layers done before this one
+    int fstride, call;                                     // steps before this one
     __device__ long long claim(int i) {
         const long long idx = (long long)blockIdx.x + (long long)i * gridDim.x;
         return idx < (long long)p.B * fstride ? idx : -1;
     }
     __device__ int poll(long long idx, RowDesc& d, bool) {
         const int b = (int)(idx / fstride), f = (int)(idx - (long long)b * fstride);
-        const int fs = __ldcg(&w.st[(size_t)b * 8 + kStFront + (layer & 1)]);
-        if (f >= fs || fs > fstride) return 2;
+        const Front at = front_at(w, b, call);
+        if (f >= at.rows || at.rows > fstride) return 2;
         d.row = logits + (size_t)idx * p.V;
-        d.b = b; d.d = layer + 1; d.slot = f; d.fsize = fs;
-        d.pphat = __ldcg(&w.front_phat[((size_t)b * 2 + (layer & 1)) * p.n + f]);
+        d.b = b; d.d = at.layer + 1; d.slot = f; d.fsize = at.rows;
+        d.pphat = __ldcg(&w.front_phat[((size_t)b * 2 + (at.layer & 1)) * p.n + f]);
         return 1;
     }
 };
 template <class LS>
 struct LayersSink {
     Workspace w; Params p; opt_tree_out out;
-    int fstride, layer, at;                                // at: offset of the layer scratch in shared memory
+    int fstride, call, at;                                 // at: offset of the layer scratch in shared memory
     int32_t *next_tokens, *next_parent, *next_count;
     __device__ void row_done(const RowDesc& d, const RowOut& r, FinScratch&) {
         const int lane = threadIdx.x & 31;
@@ -766,11 +789,13 @@ struct LayersSink {
         const int lane = threadIdx.x & 31;
         // sequences that stopped at an earlier layer, or whose layer does not fit the buffer
         for (int b = (int)blockIdx.x + lane * (int)gridDim.x; b < p.B; b += 32 * (int)gridDim.x) {
-            const int fs = __ldcg(&w.st[(size_t)b * 8 + kStFront + (layer & 1)]);
-            if (fs >= 1 && fs <= fstride) continue;
-            if (fs > fstride) set_status(w.status, kErrInternal);
+            const Front now = front_at(w, b, call);
+            if (now.rows >= 1 && now.rows <= fstride) continue;
             next_count[b] = 0;
-            w.st[(size_t)b * 8 + kStFront + ((layer + 1) & 1)] = 0;
+            if (now.rows > fstride) {
+                set_status(w.status, kErrInternal);
+                st_relaxed_u64(front_words(w, b) + ((now.layer + 1) & 1), front_word(call + 1, now.layer + 1, 0));
+            }
         }
         __syncwarp();
         const CtaCore& core = smem_at<CtaCore>(0);
@@ -821,7 +846,7 @@ struct LayersSink {
             ls.job.kind = 0;
             __threadfence();
             if (atomicAdd(&w.q_ctl[kQLeft], 1) == (int)gridDim.x - 1) {
-                w.q_ctl[kQLeft] = 0; w.q_ctl[kQTail] = 0; w.q_ctl[kQHead] = 0; w.q_ctl[kQLayer] = layer + 1;
+                w.q_ctl[kQLeft] = 0; w.q_ctl[kQTail] = 0; w.q_ctl[kQHead] = 0; w.q_ctl[kQCall] = call + 1;
             }
         }
         __syncwarp();
@@ -847,7 +872,7 @@ struct LayersSink {
     __device__ void hand_back(LS& ls, int tt) {
         const int b = ls.job.b, nl = ls.job.fsize, gid0 = (ls.job.d - 1) * p.n;
         const int32_t* T_par = ls.job.T_par;
-        double* front = w.front_phat + ((size_t)b * 2 + ((layer + 1) & 1)) * p.n;
+        double* front = w.front_phat + ((size_t)b * 2 + (ls.job.d & 1)) * p.n;
         for (int i = tt; i < nl; i += kTeam) {
             next_tokens[(size_t)b * p.n + i] = ls.ltok[i];
             next_parent[(size_t)b * p.n + i] = __ldcg(&T_par[gid0 + i]);
@@ -863,9 +888,10 @@ struct LayersSink {
     }
     // One layer of one sequence.
     __device__ void step(LS& ls, int b) {
-        const int lane = threadIdx.x & 31, d = layer + 1;
+        const Front now = front_at(w, b, call);
+        const int lane = threadIdx.x & 31, d = now.layer + 1, fsize = now.rows;
         const SeqWork sw = seq_work(w, p, b);
-        const int fsize = __ldcg(&sw.st[kStFront + (layer & 1)]), nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
+        const int nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
         const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
         const int nvalid = fsize * p.kk, nl = nvalid < p.n ? nvalid : p.n;
         if (lane == 0) {
@@ -889,7 +915,7 @@ struct LayersSink {
             if (to.esub_trace) to.esub_trace[d - 1] = esub;
             sw.st[kStNR] = nR; *sw.E_prev = esub;
             sw.st[kStDone] = 0;
-            sw.st[kStFront + ((layer + 1) & 1)] = more ? nl : 0;
+            st_relaxed_u64(front_words(w, b) + (d & 1), front_word(call + 1, d, more ? nl : 0));
             next_count[b] = more ? nl : 0;
             ls.job.nR_old = nR; ls.last_esub = esub;
         }
@@ -902,9 +928,9 @@ layers_kernel(Workspace w, Params p, const uint16_t* __restrict__ logits, int fs
               int32_t* next_parent, int32_t* next_count) {
     CtaSmemT<NCAP>& s = *reinterpret_cast<CtaSmemT<NCAP>*>(ot_smem);
     grid_dependency_wait();
-    const int layer = __ldcg(&w.q_ctl[kQLayer]);             // (every thread has it before any CTA can leave: see run_pipeline's barrier)
-    LayersSource src{w, p, logits, fstride, layer};
-    LayersSink<LayerScratchT<NCAP>> sink{w, p, out, fstride, layer, smem_offset(&s.layer), next_tokens, next_parent, next_count};
+    const int call = __ldcg(&w.q_ctl[kQCall]);               // (every thread has it before any CTA can leave: see run_pipeline's barrier)
+    LayersSource src{w, p, logits, fstride, call};
+    LayersSink<LayerScratchT<NCAP>> sink{w, p, out, fstride, call, smem_offset(&s.layer), next_tokens, next_parent, next_count};
     run_pipeline<kAligned, kLong>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.B * fstride * p.V, w.status);
 }
 

@@ -32,12 +32,13 @@ struct SeqWork {
     double* T_phat;        // [D*n]
     int32_t* R;            // [2][n]   running top-n as gids in ascending order, double-buffered by layer parity
     double* E_prev;        // [1]      E of Algorithm 1
-    int32_t* st;           // [8]      1: rows finished since the build began, 2: |R|
+    int32_t* st;           // [8], 16-byte aligned   1: rows finished since the build began, 2: |R|
     int32_t* fmap;         // [n]      pruned draft: layer slot of the node behind each frontier row
 };
-enum { kStDone = 1, kStNR = 2, kStFront = 4, kStL1 = 6, kStQueue = 7 };   // 4, 5: layer-by-layer build: rows of an even / odd layer (0: finished)
-// 6: how the root's row was handled (top bit: decided; the rest: rows of layer 2 if its finisher grew layer 1 itself, else 0)
-// 7: layer-by-layer build: entry of the queue of sequences whose rows are all in (sequence + 1)
+enum { kStL1 = 0, kStDone = 1, kStNR = 2, kStQueue = 3, kStFront = 4 };
+// 0: how the root's row was handled (top bit: decided; the rest: rows of layer 2 if its finisher grew layer 1 itself, else 0)
+// 3: layer-by-layer build: entry of the queue of sequences whose rows are all in (sequence + 1)
+// 4 ... 7: layer-by-layer build: where the tree stands, two 64-bit words (see Front)
 
 struct TreeOut {           // mirrors opt_tree_out, pointers offset to the sequence
     int32_t *token, *parent, *depth;
