@@ -176,7 +176,9 @@ int opt_tree_build_pruned(opt_tree_ctx *ctx, const void *draft_logits_bf16, cons
  * `out` in that call.  The trees are those of opt_tree_build for the same logits.
  *   frontier_logits (dev) bf16 [B][frontier_stride][V]: row f of sequence b belongs to node f of the
  *                   layer returned by the previous step (the root for the first step); rows at or
- *                   beyond a sequence's count are read but ignored.  1 <= frontier_stride <= n
+ *                   beyond a sequence's count are not looked at.  1 <= frontier_stride <= n; a sequence with more
+ *                   nodes than frontier_stride is left as it is (next_count 0, OPT_TREE_ERR_INTERNAL in the status
+ *                   word) and goes on with the next step whose buffer is wide enough
  *   out             as in opt_tree_build; written for a sequence when it stops
  *   next_tokens     (dev) [B][n] int32  tokens of the new layer's nodes (to be expanded next)
  *   next_parent     (dev) [B][n] int32  for each, the index of its parent in the previous layer

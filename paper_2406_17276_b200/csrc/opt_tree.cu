@@ -789,13 +789,10 @@ struct LayersSink {
         const int lane = threadIdx.x & 31;
         // sequences that stopped at an earlier layer, or whose layer does not fit the buffer
         for (int b = (int)blockIdx.x + lane * (int)gridDim.x; b < p.B; b += 32 * (int)gridDim.x) {
-            const Front now = front_at(w, b, call);
-            if (now.rows >= 1 && now.rows <= fstride) continue;
+            const int fs = front_at(w, b, call).rows;
+            if (fs >= 1 && fs <= fstride) continue;
+            if (fs > fstride) set_status(w.status, kErrInternal);           // (a step with a wider buffer may follow)
             next_count[b] = 0;
-            if (now.rows > fstride) {
-                set_status(w.status, kErrInternal);
-                st_relaxed_u64(front_words(w, b) + ((now.layer + 1) & 1), front_word(call + 1, now.layer + 1, 0));
-            }
         }
         __syncwarp();
         const CtaCore& core = smem_at<CtaCore>(0);

@@ -62,3 +62,16 @@ def test_steps_of_fewer_sequences(calls, delta):
             break
     g.step(B)                                                # finished trees stay finished
     g.check()
+
+
+@pytest.mark.parametrize("delta", [-math.inf, 0.25])
+def test_a_buffer_too_narrow_for_a_layer_can_be_made_wider(delta):
+    g = _Driver(delta)
+    g.step(B)
+    assert all(len(t) == k for t in g.toks)                  # layer 1: k nodes each
+    assert g.step(B, stride=k - 1) == [0] * B                # no sequence can be grown from that
+    assert g.ot.device_status() == -5                        # OPT_TREE_ERR_INTERNAL
+    for _ in range(D):
+        if any(len(t) for t in g.toks):
+            g.step(B)
+    g.check()
