@@ -1178,9 +1178,10 @@ constexpr int kSegTokens = kSegVecs * 8;
 constexpr int kMaxSeg = 640;                 // rows of up to 327 680 logits take the one-pass path
 constexpr int kSampleExpLimit = 1 << 22;     // |exponent| beyond which the single-precision pass cannot scale
 struct alignas(8) SegPart { float sum; int E; };       // a segment's sum of 2^(x*c - E), E an integer
-template <int T>
+template <int T, bool kAligned>
 struct SampleSmem {
     union { SegPart part[kMaxSeg]; double cum[kMaxSeg]; };   // per segment: its partial sum, then the running sum up to and including it
+    int top[kAligned ? 1 : kMaxSeg];                         // unaligned rows: key of each segment's largest logit
     double wsum[T / 32];
     double S;
     float wmax[T / 32];
@@ -1188,11 +1189,11 @@ struct SampleSmem {
     int chosen, last_live, seg, live_seg;
 };
 
-// The plain way, for rows the one-pass path does not take (very long rows, extreme magnitudes): thread t owns the tokens [t*L, (t+1)*L); the row's maximum, then every thread's sum of
-// double-precision exponentials in token order, a scan over the threads, and the thread in whose stretch
-// u*S falls walks it once more.  Returns the drawn token to every thread.
-template <int T>
-__device__ __noinline__ int sample_row_plain(SampleSmem<T>& q, const uint16_t* row, int V, bool vec, double tau, double u) {
+// The plain way, for rows the one-pass path does not take (very long rows, extreme magnitudes): thread t owns the tokens
+// [t*L, (t+1)*L); the row's maximum, then every thread's sum of double-precision exponentials in token order, a scan over
+// the threads, and the thread in whose stretch u*S falls walks it once more.  Returns the drawn token to every thread.
+template <int T, bool kAligned>
+__device__ __noinline__ int sample_row_plain(SampleSmem<T, kAligned>& q, const uint16_t* row, int V, bool vec, double tau, double u) {
     const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
     const int L = (((V + T - 1) / T) + 7) & ~7;       // tokens per thread, a multiple of 8
     const int lo = min(tid * L, V), hi = min(lo + L, V);
@@ -1256,26 +1257,37 @@ __device__ __noinline__ int sample_row_plain(SampleSmem<T>& q, const uint16_t* r
     return y;
 }
 
-// Sum of the terms of the at most seven logits [t0, t1) at either end of a row, by one warp: a segment of its own.
-__device__ __noinline__ SegPart edge_part(const uint16_t* row, int t0, int t1, float c32, float c_hi, float c_lo) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t bits = t0 + lane < t1 ? (uint32_t)__ldg(row + t0 + lane) : 0xFF80u;
-    const uint32_t wkey = __reduce_max_sync(0xFFFFFFFFu, ord16(bits));
-    SegPart part;
-    part.sum = 0.0f; part.E = 0;
-    if (wkey > kOrdNegInf) {
-        const float Ef = rintf(fminf(fmaxf(fmaf(bf16_bits_to_float(ord16_inv(wkey)), c32, 1.0f), -1e9f), 1e9f));
-        const float x = fmaxf(bf16_bits_to_float(bits), -1e30f);
-        float sum = ex2_approx(fmaf(x, c_lo, fmaf(x, c_hi, -Ef)));
+// A segment of a row that does not lie on 16-byte boundaries, by one warp: the sum of e^((x - M) / tau), M its largest logit
+// (`key`: in ordered form), in double precision throughout.
+__device__ __forceinline__ double segment_f64(const uint16_t* row, int sg, int nv, int V, double c64, uint32_t& key) {
+    const int lane = threadIdx.x & 31, o = vec_offset(row);
+    auto vec_at = [&](int vi) -> uint4 {
+        if (vi >= 1 && vi * 8 + 16 <= V) {                   // the two granules that hold the vector lie within the row
+            const uint4* g = reinterpret_cast<const uint4*>(row + (size_t)vi * 8 - o);
+            return shift_halves(ld_nc_v4(g), ld_nc_v4(g + 1), o);
+        }
+        return vi < nv ? load_row_vec_unaligned(row, vi, V) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+    };
+    const uint4 a = vec_at(sg * kSegVecs + lane), b = vec_at(sg * kSegVecs + 32 + lane);
+    const uint32_t ww[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint32_t m2 = ww[0];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-        part.sum = sum; part.E = (int)Ef;
+    for (int i = 1; i < 8; ++i) m2 = max_bf16x2(m2, ww[i]);
+    key = __reduce_max_sync(0xFFFFFFFFu, max(ord16(m2 & 0xFFFFu), ord16(m2 >> 16)));
+    if (key <= kOrdNegInf) return 0.0;                       // (warp-uniform) no finite logit
+    const double M = (double)bf16_bits_to_float(ord16_inv(key));
+    double sum = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float lo = __uint_as_float(ww[i] << 16), hi = __uint_as_float(ww[i] & 0xFFFF0000u);
+        sum += lo == -INFINITY ? 0.0 : exp2(((double)lo - M) * c64);
+        sum += hi == -INFINITY ? 0.0 : exp2(((double)hi - M) * c64);
     }
-    return part;
+    return warp_sum(sum);
 }
 
-// CTA (j, b) as in verify_kernel.  One pass over the row's whole granules: warp w takes the segments w, w + T/32, ...
-// of them (an unaligned row has two more segments, its ends before and after them); a segment's terms 2^(x*c - E) (c = log2(e) / tau, E an integer just above the segment's largest exponent)
+// CTA (j, b) as in verify_kernel.  One pass over the row: warp w takes the segments w, w + T/32, ...; a
+// segment's terms 2^(x*c - E) (c = log2(e) / tau, E an integer just above the segment's largest exponent)
 // are summed in single precision with ex2.approx and kept per segment, so the running sum is known in
 // token order at segment granularity.  The exponent x*c is formed with c split into a 16-bit head and a
 // tail: x is bf16, so x * head is exact, and the rounding of c does not grow with |x*c| (low temperatures).
@@ -1283,14 +1295,18 @@ __device__ __noinline__ SegPart edge_part(const uint16_t* row, int t0, int t1, f
 // (512 logits, 512 / T per thread) double-precision exponentials and an exact scan.  What can differ from a
 // double-precision inverse CDF over the whole row is the placement of u*S relative to a segment's start, by
 // the rounding of the single-precision sums (a few 1e-7 of S).
-template <int T>
-__global__ void __launch_bounds__(T, T == kVerifyMany ? 16 : (T == kVerifySome ? 6 : 3))
+// Unaligned rows (kAligned false) take the same pass with segments counted from the row's first logit, whatever its address,
+// and double-precision terms and sums: their draws are those of a double-precision inverse CDF throughout.  The exponentials are
+// what bounds them: 784 rows of 32003 logits 80 us (284 by the plain way, 27 with single-precision sums, which moved draws),
+// 51 rows 27 us (129, 16), 130 rows of 128257 70 us (446, 27).  Eight, four and two CTAs per SM, for the registers these take.
+template <int T, bool kAligned>
+__global__ void __launch_bounds__(T, kAligned ? (T == kVerifyMany ? 16 : (T == kVerifySome ? 6 : 3)) : (T == kVerifyMany ? 8 : (T == kVerifySome ? 4 : 2)))
 verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const int32_t* __restrict__ root_token,
                       opt_tree_out tree, double tau, unsigned long long seed, unsigned long long step, int32_t* accept_len,
                       int32_t* accept_tokens, int32_t* accept_nodes, int32_t* next_root) {
     int* verify_walk = reinterpret_cast<int*>(ot_smem);
     __shared__ VerifySmem<T> s;
-    __shared__ SampleSmem<T> q;
+    __shared__ SampleSmem<T, kAligned> q;
     grid_dependency_wait();
     const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
     const int32_t* tok = tree.token + (size_t)b * p.n;
@@ -1302,28 +1318,29 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
     if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
     const uint16_t* row = target + (size_t)row_of(token, depth, p.H) * p.V;
     const double u = uniform53(seed, step, b, j);
-    const int h0 = min((8 - vec_offset(row)) & 7, p.V), nv = (p.V - h0) >> 3, h1 = h0 + nv * 8;
-    const int ngs = (nv + kSegVecs - 1) / kSegVecs, nseg = ngs + 2;    // segment 0: [0, h0); 1 ... ngs: 512 logits each; ngs + 1: [h1, V)
+    const int nv = (p.V + 7) >> 3, nseg = (nv + kSegVecs - 1) / kSegVecs;
     const double c64 = kLog2eD / tau;
     bool fast = nseg <= kMaxSeg && c64 < 1e30;
     int y = 0;
     if (fast) {
+        if (tid == 0) { q.chosen = -1; q.last_live = -1; q.seg = 0x7FFFFFFF; q.live_seg = -1; }
+        constexpr int kStep = T / 32;
+        if (!kAligned) {
+#pragma unroll 1
+            for (int sg = wp; sg < nseg; sg += kStep) {
+                uint32_t key;
+                const double sum = segment_f64(row, sg, nv, p.V, c64, key);
+                if (lane == 0) { q.cum[sg] = sum; q.top[sg] = (int)key; }
+            }
+        }
         const float c32 = (float)c64;
         const float c_hi = __uint_as_float(__float_as_uint(c32) & 0xFFFFFF00u);      // 16 significant bits
         const float c_lo = (float)(c64 - (double)c_hi);
-        const uint4* rv = reinterpret_cast<const uint4*>(row + h0);
-        if (tid == 0) { q.chosen = -1; q.last_live = -1; q.seg = 0x7FFFFFFF; q.live_seg = -1; }
+        const uint4* rv = reinterpret_cast<const uint4*>(row);
         // two segments per turn: four 16-byte loads in flight per lane
         const unsigned long long chi2 = pack2(c_hi, c_hi), clo2 = pack2(c_lo, c_lo);
-        constexpr int kStep = T / 32;
-        if (wp == 0) {                                        // the ends (empty for aligned rows)
-            const SegPart zero = {0.0f, 0};
-            const SegPart head = h0 > 0 ? edge_part(row, 0, h0, c32, c_hi, c_lo) : zero;
-            const SegPart tail = h1 < p.V ? edge_part(row, h1, p.V, c32, c_hi, c_lo) : zero;
-            if (lane == 0) { q.part[0] = head; q.part[ngs + 1] = tail; }
-        }
 #pragma unroll 1
-        for (int sg0 = wp; sg0 < ngs; sg0 += 2 * kStep) {
+        for (int sg0 = wp; kAligned && sg0 < nseg; sg0 += 2 * kStep) {
             const uint4 pad = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
             uint4 qq[2][2];
 #pragma unroll
@@ -1335,7 +1352,7 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int sg = sg0 + h * kStep;
-                if (sg >= ngs) break;                            // (warp-uniform)
+                if (sg >= nseg) break;                            // (warp-uniform)
                 const uint32_t ww[8] = {qq[h][0].x, qq[h][0].y, qq[h][0].z, qq[h][0].w, qq[h][1].x, qq[h][1].y, qq[h][1].z, qq[h][1].w};
                 uint32_t m2 = ww[0];
 #pragma unroll
@@ -1361,26 +1378,35 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
                 }
-                if (lane == 0) { q.part[sg + 1].sum = sum; q.part[sg + 1].E = (int)Ef; }
+                if (lane == 0) { q.part[sg].sum = sum; q.part[sg].E = (int)Ef; }
             }
         }
         __syncthreads();
         int e = -0x7FFFFFFF;
-        for (int sg = tid; sg < nseg; sg += T) if (q.part[sg].sum > 0.0f) e = max(e, q.part[sg].E);
+        for (int sg = tid; sg < nseg; sg += T) {
+            if (kAligned) { if (q.part[sg].sum > 0.0f) e = max(e, q.part[sg].E); }
+            else if (q.cum[sg] > 0.0) e = max(e, q.top[sg]);
+        }
         e = __reduce_max_sync(0xFFFFFFFFu, e);
         if (lane == 0) q.wE[wp] = e;
         __syncthreads();
         int Eg = q.wE[0];
 #pragma unroll
         for (int i = 1; i < T / 32; ++i) Eg = max(Eg, q.wE[i]);
-        fast = Eg > -kSampleExpLimit && Eg < kSampleExpLimit;                     // the same for every thread
+        fast = kAligned ? Eg > -kSampleExpLimit && Eg < kSampleExpLimit : Eg > 0;        // the same for every thread
+        const double Mg = kAligned ? 0.0 : (double)bf16_bits_to_float(ord16_inv((uint32_t)max(Eg, 0)));     // the row's largest logit
+        // term of logit x on the scale of the running sums
+        auto term = [&](float x) { return kAligned ? exp2((double)x * c64 - (double)Eg) : exp2(((double)x - Mg) * c64); };
         if (fast) {
             if (wp == 0) {                                    // running sums over the segments, in token order
                 double carry = 0.0;
                 for (int s0 = 0; s0 < nseg; s0 += 32) {
                     const int sg = s0 + lane;
                     double v = 0.0;
-                    if (sg < nseg) { const SegPart pt = q.part[sg]; v = pt.sum > 0.0f ? ldexp((double)pt.sum, pt.E - Eg) : 0.0; }
+                    if (sg < nseg) {
+                        if (kAligned) { const SegPart pt = q.part[sg]; v = pt.sum > 0.0f ? ldexp((double)pt.sum, pt.E - Eg) : 0.0; }
+                        else { v = q.cum[sg]; if (v > 0.0) v *= term(bf16_bits_to_float(ord16_inv((uint32_t)q.top[sg]))); }
+                    }
                     double incl = v;
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
@@ -1407,16 +1433,14 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
             const double before = sg > 0 ? q.cum[sg - 1] : 0.0;
             // inside the segment: kPer logits per thread, double precision
             constexpr int kPer = kSegTokens / T;
-            const int seg0 = sg == 0 ? 0 : min(h0 + (sg - 1) * kSegTokens, h1);
-            const int seg1 = sg == 0 ? h0 : (sg > ngs ? p.V : min(seg0 + kSegTokens, h1));
-            const int t0 = seg0 + kPer * tid;
+            const int t0 = sg * kSegTokens + kPer * tid;
             double ev[kPer];
             int live = -1;
 #pragma unroll
             for (int i = 0; i < kPer; ++i) {
                 const int tk = t0 + i;
-                const float xf = tk < seg1 ? bf16_bits_to_float(__ldg(row + tk)) : -INFINITY;
-                ev[i] = xf == -INFINITY ? 0.0 : exp2((double)xf * c64 - (double)Eg);
+                const float xf = tk < p.V ? bf16_bits_to_float(__ldg(row + tk)) : -INFINITY;
+                ev[i] = xf == -INFINITY ? 0.0 : term(xf);
                 if (ev[i] > 0.0) live = tk;
             }
             double mine = ev[0];
@@ -1448,10 +1472,10 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
             }
             __syncthreads();
             y = q.chosen;
-            if (y < 0) y = q.last_live < 0 ? min(seg0, p.V - 1) : q.last_live;   // the exact sums end just below u*S: the segment's last live token
+            if (y < 0) y = q.last_live < 0 ? min(sg * kSegTokens, p.V - 1) : q.last_live;   // the exact sums end just below u*S: the segment's last live token
         }
     }
-    if (!fast) y = sample_row_plain<T>(q, row, p.V, p.aligned != 0, tau, u);
+    if (!fast) y = sample_row_plain(q, row, p.V, kAligned, tau, u);
     verify_tail<T>(s, verify_walk, w, p, b, j, ns, y, tok, par, accept_len, accept_tokens, accept_nodes, next_root);
 }
 
@@ -1550,6 +1574,10 @@ void launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, 
 int verify_threads(int n, int B, int sms, int some) {
     const long long rows = (long long)(n + 1) * B;
     return rows <= 3ll * sms ? ot::kVerifyFew : (rows <= (long long)some * sms ? ot::kVerifySome : ot::kVerifyMany);
+}
+template <bool kAligned> auto sampled_variant(int threads) {
+    return threads == ot::kVerifyFew ? ot::verify_sampled_kernel<ot::kVerifyFew, kAligned>
+                                     : (threads == ot::kVerifySome ? ot::verify_sampled_kernel<ot::kVerifySome, kAligned> : ot::verify_sampled_kernel<ot::kVerifyMany, kAligned>);
 }
 size_t walk_smem(int n) { return (size_t)(3 * n + 1) * sizeof(int); }
 bool bad_tree(const opt_tree_out* t) {
@@ -1726,8 +1754,7 @@ int opt_tree_verify_sampled(opt_tree_ctx* ctx, const opt_tree_out* tree, const v
         return OPT_TREE_ERR_INVALID_ARG;
     const ot::Params p = make_params(ctx, target, 0.0f);
     const int threads = verify_threads(ctx->cfg.n, B, ctx->sms, 6);
-    launch_after(threads == ot::kVerifyFew ? ot::verify_sampled_kernel<ot::kVerifyFew>
-                                           : (threads == ot::kVerifySome ? ot::verify_sampled_kernel<ot::kVerifySome> : ot::verify_sampled_kernel<ot::kVerifyMany>),
+    launch_after(p.aligned ? sampled_variant<true>(threads) : sampled_variant<false>(threads),
                  dim3(ctx->cfg.n + 1, B), dim3(threads), walk_smem(ctx->cfg.n), static_cast<cudaStream_t>(stream),
                  ctx->ws, p, static_cast<const uint16_t*>(target), root_token, *tree, tau, (unsigned long long)seed,
                  (unsigned long long)step, accept_len, accept_tokens, accept_nodes, next_root);
