@@ -204,7 +204,8 @@ int opt_tree_layers_step(opt_tree_ctx *ctx, const void *frontier_logits_bf16, in
  * sum exceeds u * sum (the last token with e_v > 0 if rounding leaves none).  The row is read once: the
  * running sum is formed per segment of 512 logits in single precision (exponent arithmetic exact for
  * bf16 logits), and in double precision inside the segment where u * sum falls, so the token is that of
- * a double-precision inverse CDF unless u * sum lies within about 1e-6 * sum of a running sum.
+ * a double-precision inverse CDF unless u * sum lies within about 1e-6 * sum of a running sum.  (Rows that are
+ * not 16-byte aligned, or longer than 327 680 logits, are summed in double precision throughout.)
  * `step` is the caller's decoding step number, so that successive steps use fresh uniforms.
  * Errors as opt_tree_verify; tau <= 0 or NaN is OPT_TREE_ERR_INVALID_ARG. */
 int opt_tree_verify_sampled(opt_tree_ctx *ctx, const opt_tree_out *tree, const void *target_logits_bf16,
