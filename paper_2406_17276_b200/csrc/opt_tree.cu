@@ -1098,9 +1098,10 @@ verify_kernel(Workspace w, Params p, const uint16_t* __restrict__ target, const 
     const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x;
     const int32_t* tok = tree.token + (size_t)b * p.n;
     const int32_t* par = tree.parent + (size_t)b * p.n;
-    const int ns = tree.n_sel[b];                            // (all three loads at once: an unused slot's token is never looked at)
+    int ns = tree.n_sel[b];                                  // (all three loads at once: an unused slot's token is never looked at)
     int token = j == 0 ? root_token[b] : tok[j - 1];
     const int depth = j == 0 ? 0 : tree.depth[(size_t)b * p.n + j - 1];
+    if (ns > p.n) { set_status(w.status, kErrInternal); ns = p.n; }        // (the walk's shared memory is sized for n nodes)
     if (j > ns) return;
     if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
     const uint16_t* row = target + (size_t)row_of(token, depth, p.H) * p.V;
@@ -1311,9 +1312,10 @@ verify_sampled_kernel(Workspace w, Params p, const uint16_t* __restrict__ target
     const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
     const int32_t* tok = tree.token + (size_t)b * p.n;
     const int32_t* par = tree.parent + (size_t)b * p.n;
-    const int ns = tree.n_sel[b];                            // (all three loads at once: an unused slot's token is never looked at)
+    int ns = tree.n_sel[b];                                  // (all three loads at once: an unused slot's token is never looked at)
     int token = j == 0 ? root_token[b] : tok[j - 1];
     const int depth = j == 0 ? 0 : tree.depth[(size_t)b * p.n + j - 1];
+    if (ns > p.n) { set_status(w.status, kErrInternal); ns = p.n; }        // (the walk's shared memory is sized for n nodes)
     if (j > ns) return;
     if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
     const uint16_t* row = target + (size_t)row_of(token, depth, p.H) * p.V;
