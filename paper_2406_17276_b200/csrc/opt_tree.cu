@@ -33,8 +33,8 @@ __device__ __forceinline__ int row_of(int token, int depth, int H) {
 // ------------------------------------------------------------------------------------------------
 struct Workspace {
     // build
-    double* cand_phat;     // [B][cand_stride]
-    int32_t* cand_tok;     // [B][cand_stride]
+    double* cand_phat;     // [B][2][cand_stride]   even and odd layers
+    int32_t* cand_tok;     // [B][2][cand_stride]
     int32_t* T_tok;        // [B][D*n]
     int32_t* T_par;        // [B][D*n]
     double* T_phat;        // [B][D*n]
@@ -93,8 +93,8 @@ static size_t carve(const opt_tree_config& c, int grid, char* base, Workspace* w
     Layout L;
     size_t o;
 #define OT_TAKE(field, T, count) o = L.take<T>(count); if (w) w->field = reinterpret_cast<T*>(base + o);
-    OT_TAKE(cand_phat, double, B * cs)
-    OT_TAKE(cand_tok, int32_t, B * cs)
+    OT_TAKE(cand_phat, double, 2 * B * cs)
+    OT_TAKE(cand_tok, int32_t, 2 * B * cs)
     OT_TAKE(T_tok, int32_t, B * D * n)
     OT_TAKE(T_par, int32_t, B * D * n)
     OT_TAKE(T_phat, double, B * D * n)
@@ -136,10 +136,11 @@ struct Params {            // by-value kernel parameters
     int prune;             // draft only from layer nodes that are still among the n largest
 };
 
-__device__ __forceinline__ SeqWork seq_work(const Workspace& w, const Params& p, int b) {
+// d: the layer whose candidates are meant.
+__device__ __forceinline__ SeqWork seq_work(const Workspace& w, const Params& p, int b, int d) {
     SeqWork s;
-    s.cand_phat = w.cand_phat + (size_t)b * p.cstride;
-    s.cand_tok = w.cand_tok + (size_t)b * p.cstride;
+    s.cand_phat = w.cand_phat + ((size_t)b * 2 + (d & 1)) * p.cstride;
+    s.cand_tok = w.cand_tok + ((size_t)b * 2 + (d & 1)) * p.cstride;
     s.T_tok = w.T_tok + (size_t)b * p.max_depth * p.n;
     s.T_par = w.T_par + (size_t)b * p.max_depth * p.n;
     s.T_phat = w.T_phat + (size_t)b * p.max_depth * p.n;
@@ -204,7 +205,7 @@ __global__ void init_build_kernel(Workspace w, Params p, const int32_t* __restri
         w.mb_items[i] = item;
         w.mb_phat[i] = ph;
     }
-    for (long long j = i; j < (long long)p.B * p.cstride; j += (long long)gridDim.x * blockDim.x) {
+    for (long long j = i; j < 2ll * p.B * p.cstride; j += (long long)gridDim.x * blockDim.x) {
         reinterpret_cast<unsigned long long*>(w.cand_phat)[j] = 0ull;
         w.cand_tok[j] = 0;
     }
@@ -290,7 +291,7 @@ struct BuildSink {
     }
     __device__ void row_done(const RowDesc& d, const RowOut& r, FinScratch&) {
         const int lane = threadIdx.x & 31;
-        const SeqWork sw = seq_work(w, p, d.b);
+        const SeqWork sw = seq_work(w, p, d.b, d.d);
         if (d.d == 1) {                                                    // the root's row
             const bool direct = first_layer_direct(d, r, sw);
             __syncwarp();
@@ -410,6 +411,7 @@ struct BuildSink {
             __syncwarp();
             publish_layer(ls, b, d, cnt, g0, ls.gids, sw.fmap);
             void_entries(g0, cnt, reserve);
+            fence_gpu();                                    // the cleared candidate words before the rows of layer d + 2
             return cnt;
         }
         if (d < p.Dcap) void_entries(g0, 0, reserve);
@@ -496,7 +498,7 @@ struct BuildSink {
                 for (int q = 0; q < kOwn; ++q) {
                     if (cur_d[q] == 0) continue;
                     const int b = b0 + q * (int)gridDim.x;
-                    const SeqWork sw = seq_work(w, p, b);
+                    const SeqWork sw = seq_work(w, p, b, cur_d[q]);
                     int done = 0;
                     if (lane == 0) done = ld_acquire_s32(&sw.st[kStDone]);
                     done = __shfl_sync(0xFFFFFFFFu, done, 0);
@@ -564,7 +566,7 @@ struct BuildSink {
                         __syncwarp();
                         if (lane == 0) {
                             LayerJob& j = ls.job;
-                            j.kind = 3; j.fsize = nl; j.nR_old = nR_old; j.off = cached ? 1 : 0;
+                            j.kind = 3; j.ncand = fsize * p.k; j.fsize = nl; j.nR_old = nR_old; j.off = cached ? 1 : 0;
                             j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
                             ls.cache_b = b; ls.cache_d = d;
                         }
@@ -608,7 +610,10 @@ struct BuildSink {
                     } else if (more && !early) {
                         publish_layer(ls, b, d, nl, reserve_layer(nl));
                     }
-                    if (more) { cur_d[q] = d + 1; cur_f[q] = sent; cur_tot[q] += sent; }
+                    if (more) {
+                        cur_d[q] = d + 1; cur_f[q] = sent; cur_tot[q] += sent;
+                        fence_gpu();                          // the cleared candidate words before the rows of layer d + 2
+                    }
                     if (kPrune && lane == 0 && rows_read) rows_read[b] = cur_tot[q];
                     if (!more) {
                         cur_d[q] = 0; --live;
@@ -711,7 +716,7 @@ __device__ __forceinline__ Front front_at(const Workspace& w, int b, int call) {
 __global__ void layers_begin_kernel(Workspace w, Params p) {
     grid_dependency_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (long long j = i; j < (long long)p.B * p.cstride; j += (long long)gridDim.x * blockDim.x) {
+    for (long long j = i; j < 2ll * p.B * p.cstride; j += (long long)gridDim.x * blockDim.x) {
         reinterpret_cast<unsigned long long*>(w.cand_phat)[j] = 0ull;
         w.cand_tok[j] = 0;
     }
@@ -753,7 +758,7 @@ struct LayersSink {
     int32_t *next_tokens, *next_parent, *next_count;
     __device__ void row_done(const RowDesc& d, const RowOut& r, FinScratch&) {
         const int lane = threadIdx.x & 31;
-        const SeqWork sw = seq_work(w, p, d.b);
+        const SeqWork sw = seq_work(w, p, d.b, 0);
         if (lane < p.k) {
             unsigned long long* ph = reinterpret_cast<unsigned long long*>(sw.cand_phat) + d.slot * p.k + lane;
             unsigned int* tk = reinterpret_cast<unsigned int*>(sw.cand_tok) + d.slot * p.k + lane;
@@ -887,7 +892,7 @@ struct LayersSink {
     __device__ void step(LS& ls, int b) {
         const Front now = front_at(w, b, call);
         const int lane = threadIdx.x & 31, d = now.layer + 1, fsize = now.rows;
-        const SeqWork sw = seq_work(w, p, b);
+        const SeqWork sw = seq_work(w, p, b, 0);        // (a launch per layer: one candidate array will do)
         const int nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
         const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
         const int nvalid = fsize * p.kk, nl = nvalid < p.n ? nvalid : p.n;
@@ -901,7 +906,7 @@ struct LayersSink {
         }
         if (fsize * p.k <= kTeam) { stage_layer_candidates(ls, sw, fsize, p.k); cp_async_wait_all(); }
         do_job(ls, 1);
-        if (lane == 0) ls.job.fsize = nl;
+        if (lane == 0) { ls.job.ncand = fsize * p.k; ls.job.fsize = nl; }
         do_job(ls, 3);
         const int NR = nR_old + nl, nR = NR < p.n ? NR : p.n;
         const double esub = running_esub(ls, nR);

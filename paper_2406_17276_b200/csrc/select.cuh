@@ -25,7 +25,7 @@ __device__ __forceinline__ unsigned long long warp_and_u64(unsigned long long v)
 
 // Per-sequence state and arrays in the workspace (device pointers already offset to the sequence).
 struct SeqWork {
-    double* cand_phat;     // [n*k, padded to a multiple of 4, 16-byte aligned]  path values of this layer's candidates (Eq. 2), slot-major
+    double* cand_phat;     // [n*k, padded to a multiple of 4, 16-byte aligned]  path values of one layer's candidates (Eq. 2), slot-major
     int32_t* cand_tok;     // [n*k]
     int32_t* T_tok;        // [D*n]    drafted nodes, gid = (depth-1)*n + slot
     int32_t* T_par;        // [D*n]    slot of the parent in the previous layer
@@ -219,6 +219,19 @@ __device__ __forceinline__ void sweep_candidates(LS& s, const unsigned long long
     }
 }
 
+// A layer's candidate words, all of them read, are made zero for the rows of the next layer but one: a sequence's even and odd layers
+// have arrays of their own, so the clearing need not come before the next layer is sent out, and the layer warp's fence that
+// puts it before the rows of the layer after that (at the end of the job) costs nothing: a finisher on another SM cannot
+// store a word before its row has been sent out, so no clear can take a word away.  With one array the fence lay
+// between selection and publication, 3.7 % of a build of 32 sequences.  (A fence on the reading side as well, in the fetcher, costs a
+// step of one sequence 3 %; the finisher's store there depends on the mailbox word.)
+__device__ __forceinline__ void clear_candidates(double* cand_phat, int32_t* cand_tok, int N, int tt) {
+    #pragma unroll 1
+    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
+    #pragma unroll 1
+    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
+}
+
 // The team's part of a layer selection (N = fsize * k <= 1024; up to kTeam candidates were staged into s by the layer warp).  On return (after a last barrier) the new layer's nodes are in T and its
 // tokens and keys in s.ltok / s.lkeys.  Returns nl.
 template <bool kPrune, class LS>
@@ -255,11 +268,6 @@ __device__ __noinline__ int select_layer_team(int at, int tt, int* status) {
     ko = 0ull; ka = ~0ull;
 #pragma unroll
     for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
-    // every candidate has been read: the arrays are free for the next layer's rows once they are zero again
-    #pragma unroll 1
-    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
-    #pragma unroll 1
-    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
     unsigned long long thr = 0ull;                         // with no more candidates than wanted, all of them (key > 0) are taken
     int need_eq = 0, dirty = -1;
     auto staged = [&](int i) { return s.keys[i]; };
@@ -354,10 +362,7 @@ __device__ __noinline__ int select_running_team(int at, int tt, int* status) {
     ko = 0ull; ka = ~0ull;
 #pragma unroll
     for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
-    #pragma unroll 1
-    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
-    #pragma unroll 1
-    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
+    clear_candidates(cand_phat, cand_tok, N, tt);
     unsigned long long thr = 0ull;
     int need_eq = 0, dirty = -1;
     auto staged = [&](int i) { return s.keys[i]; };
@@ -713,11 +718,6 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
         }
     }
     if (total != nl) set_status(status, kErrInternal);
-    team_sync();                                           // everyone has read what it needs: the arrays can be cleared
-    #pragma unroll 1
-    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
-    #pragma unroll 1
-    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
     team_sync();
     return nl;
 }
@@ -774,6 +774,7 @@ template <class LS>
 __device__ __noinline__ int update_running_team(int at, int tt, int* status) {
     LS& s = smem_at<LS>(at);
     const LayerJob& j = s.job;
+    clear_candidates(j.cand_phat, j.cand_tok, j.ncand, tt);
     const bool cached = j.off != 0;
     const int32_t* const Rold = j.Rold;
     const double* const T_phat = j.T_phat;
