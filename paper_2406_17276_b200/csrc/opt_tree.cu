@@ -295,9 +295,15 @@ struct BuildSink {
         if (d.d == 1) {                                                    // the root's row
             const bool direct = first_layer_direct(d, r, sw);
             __syncwarp();
+            // Layer 1, the running top-n and E do not validate themselves: this word says, with release, that they are there.
+            // (Layer 2's rows are on their way already, so this is off the chain.)
             if (lane == 0) {
-                *reinterpret_cast<volatile unsigned int*>(&sw.st[kStL1]) = 0x80000000u | (direct ? (unsigned)r.kk : 0u);
-                if (direct) atom_add_relaxed_s32(&sw.st[kStDone], 1);
+                if (direct) {
+                    st_release_s32(&sw.st[kStL1], (int)(0x80000000u | (unsigned)r.kk));
+                    atom_add_relaxed_s32(&sw.st[kStDone], 1);
+                } else {
+                    *reinterpret_cast<volatile unsigned int*>(&sw.st[kStL1]) = 0x80000000u;
+                }
             }
             if (direct) return;
         }
@@ -507,7 +513,11 @@ struct BuildSink {
                     if (cur_d[q] == 1) {
                         // the finisher of the root's row says whether it grew layer 1 itself (then layer 2 is on its way)
                         unsigned int how = 0;
-                        if (lane == 0) how = poll_tok_word(reinterpret_cast<const unsigned int*>(&sw.st[kStL1]), w.status);
+                        if (lane == 0) {
+                            how = poll_tok_word(reinterpret_cast<const unsigned int*>(&sw.st[kStL1]), w.status);
+                            fence_gpu();                      // what the finisher wrote before that word
+                        }
+                        __syncwarp();
                         how = __shfl_sync(0xFFFFFFFFu, how, 0) & 0x7FFFFFFFu;
                         if (how != 0x7FFFFFFFu && how > 0) {
                             cur_d[q] = 2; cur_f[q] = (int)how; cur_tot[q] += (int)how;
