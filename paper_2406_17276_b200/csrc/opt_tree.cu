@@ -308,7 +308,9 @@ struct BuildSink {
             if (direct) return;
         }
         // Candidate words validate themselves (top bit; an absent child is all ones), so neither they nor
-        // the row count need a fence: the layer warp re-reads whatever it finds not yet written.
+        // the row count need a fence: the layer warp re-reads whatever it finds not yet written.  Except where layers can be
+        // large: their selection looks only at the tokens of the nodes it takes, so the count is what says that a row's words
+        // are all there and can be cleared (await_rows).
         if (lane < p.k) {
             unsigned long long* ph = reinterpret_cast<unsigned long long*>(sw.cand_phat) + d.slot * p.k + lane;
             unsigned int* tk = reinterpret_cast<unsigned int*>(sw.cand_tok) + d.slot * p.k + lane;
@@ -316,7 +318,10 @@ struct BuildSink {
             *tk = lane < r.kk ? (0x80000000u | (unsigned int)r.tok) : ~0u;
         }
         __syncwarp();
-        if (lane == 0) atom_add_relaxed_s32(&sw.st[kStDone], 1);     // the count runs on over the layers of a build
+        if (lane == 0) {                                             // the count runs on over the layers of a build
+            if (p.n * p.k > kStageCap) atom_add_release_s32(&sw.st[kStDone], 1);
+            else atom_add_relaxed_s32(&sw.st[kStDone], 1);
+        }
     }
     // The rows of a new layer take the next numbers of the build's running row count and with them
     // their CTAs (row g: CTA g % grid, mailbox entry g / grid).  Whatever the order in which the
@@ -449,6 +454,17 @@ struct BuildSink {
         if (!alone) team_sync();                            // the scratch may be written again
         __syncwarp();
     }
+    // A large layer's words may be cleared once all its rows have been counted: a token that came in later would pass for one of a
+    // later layer.  (Bounded.)  The path values have all been seen by then, so this hardly ever waits, and the next
+    // layer is on its way: two sequences of n = 512 431.8 us before, 432.0 with it.  (Waiting for the 8192 tokens: 443.)
+    __device__ void await_rows(const int32_t* done, int rows) {
+        if ((threadIdx.x & 31) == 0) {
+            int t = 0;
+            while (ld_acquire_s32(done) < rows && t < kWaitPolls) ++t;
+            if (t == kWaitPolls) set_status(w.status, kErrTimeout);
+        }
+        __syncwarp();
+    }
     // The layer warp follows its sequences (layer_follow); whenever a layer is complete it hands the
     // selection to the whole team: the job goes into shared memory, the team barrier starts it.  The
     // assistants wait at that barrier in between and leave when they find a job of kind 0.
@@ -572,6 +588,7 @@ struct BuildSink {
                     int nR;
                     {
                         const bool cached = ls.cache_b == b && ls.cache_d == d - 1;   // rsel / vals hold the top-n before this layer
+                        if (fsize * p.k > kStageCap) await_rows(&sw.st[kStDone], cur_tot[q]);
                         const int nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
                         __syncwarp();
                         if (lane == 0) {
@@ -778,7 +795,11 @@ struct LayersSink {
         __syncwarp();
         if (lane == 0) {
             LS& ls = smem_at<LS>(at);
-            if (atomicAdd(&sw.st[kStDone], 1) + 1 == d.fsize) {            // (the words validate themselves: no fence)
+            // (the words validate themselves: no fence, except for the tokens of large layers, see BuildSink::await_rows)
+            if (d.fsize * p.k > kStageCap) fence_gpu();
+            const bool complete = atomicAdd(&sw.st[kStDone], 1) + 1 == d.fsize;
+            if (d.fsize * p.k > kStageCap) fence_gpu();
+            if (complete) {
                 // this CTA's team, or, if that has a sequence already, the team that comes first
                 if (atomicCAS(const_cast<int*>(&ls.todo), 0, d.b + 1) != 0) {
                     const int pos = atomicAdd(&w.q_ctl[kQTail], 1);
