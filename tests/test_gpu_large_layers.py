@@ -1,5 +1,6 @@
-"""-m gpu: layers with more candidates than the layer team stages in shared memory (over 1024): around that size, with
-ties and narrow distributions that overflow the coarse bins of the selection's first sweep, and beyond them."""
+"""-m gpu: trees whose layers have more candidates than the layer team stages in shared memory (over 1024), against the oracle
+and the pruned build.  Deep layers hardly reach a tree of ties or narrow distributions; which nodes their selection keeps is
+checked in test_gpu_layer_selection.py."""
 import math
 
 import numpy as np
@@ -44,5 +45,4 @@ def test_large_layers(kind, n, k, D, B):
         torch.cuda.synchronize()
         for f in FIELDS:
             assert np.array_equal(g[f], getattr(tree, f).cpu().numpy()), f
-        assert np.all(np.diff(np.sort(g["phat"], axis=1)[:, ::-1]) <= 0)
     assert ot.device_status() == 0
