@@ -83,7 +83,7 @@ int opt_tree_create(opt_tree_ctx **ctx, const opt_tree_config *cfg);
 int opt_tree_destroy(opt_tree_ctx *ctx);
 
 /* Algorithm 1 (construction of an OPT-Tree) for B independent sequences.
- *   draft_logits_bf16 (dev) [H][V]   16-byte aligned base
+ *   draft_logits_bf16 (dev) [H][V]   any base a bf16 may have; fastest on a 16-byte boundary with V a multiple of 8
  *   root_token        (dev) [B]      last token x_l of each input sequence, 0 <= token < V
  *   delta                            threshold of the loop test (E_sub(T,n) - E > delta); pass
  *                                    -INFINITY to draft min(max_depth, n) layers unconditionally

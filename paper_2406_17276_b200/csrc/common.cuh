@@ -92,11 +92,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
@@ -125,10 +120,6 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
     unsigned long long d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
-}
-
-__device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
 // --- mbarrier + 1-D bulk async copy (global -> this CTA's shared memory, no multicast) ---
@@ -219,11 +210,6 @@ __device__ __forceinline__ void cp_async_wait_all() {
 }
 
 // --- global-memory flags and mailbox words (gpu scope) ---
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -239,9 +225,6 @@ __device__ __forceinline__ unsigned int ld_relaxed_u32(const unsigned int* p) {
     unsigned int v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-__device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 __device__ __forceinline__ int ld_acquire_s32(const int* p) {
     int v;
@@ -283,7 +266,6 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
     }
     return v;
 }
-__device__ __forceinline__ int warp_sum_i32(int v) { return __reduce_add_sync(0xFFFFFFFFu, v); }
 // Exclusive scan of one int per lane; total returned through `total`.
 __device__ __forceinline__ int warp_excl_scan(int v, int& total) {
     const int lane = threadIdx.x & 31;

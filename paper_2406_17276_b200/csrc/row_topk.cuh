@@ -516,16 +516,16 @@ __device__ __forceinline__ uint32_t ge_bf16x2(uint32_t a, uint32_t b) {
     return d;
 }
 
-// Ranks M <= 64 candidates (f.cand[0..M), distinct keys) and gives lane j < kk the j-th largest with
-// its probability.  S is the row's sum without the candidates unless `exact`.  Every row with kk near 32 comes here (up to 32
+// Ranks 32 < M <= 64 candidates (f.cand[0..M), distinct keys) and gives lane j < kk the j-th largest with
+// its probability.  S is the row's sum without the candidates.  Every row with kk near 32 comes here (up to 32
 // candidates finish_row_warp ranks itself).  By counting, two candidates per lane: a bitonic sort of 64 keys had as many
 // instructions, but 22 KB of them in a row, which a finisher had to fetch again for every row (20000 rows of 32000 logits, k = 32: 243 -> 235 us).
-__device__ __noinline__ void finish_many(FinScratch& f, int M, int kk, double m, double S, bool exact, RowOut& out) {
+__device__ __noinline__ void finish_many(FinScratch& f, int M, int kk, double m, double S, RowOut& out) {
     const int lane = threadIdx.x & 31;
     const unsigned long long x0 = f.cand[lane], x1 = lane + 32 < M ? f.cand[lane + 32] : 0ull;
     const double e0 = exp_f64((double)cand_logit(x0) - m);
     const double e1 = x1 ? exp_f64((double)cand_logit(x1) - m) : 0.0;
-    if (!exact) S += (double)warp_sum_u64(__double2ull_rn(e0 * kFixScale) + __double2ull_rn(e1 * kFixScale)) / kFixScale;
+    S += (double)warp_sum_u64(__double2ull_rn(e0 * kFixScale) + __double2ull_rn(e1 * kFixScale)) / kFixScale;
     int r0 = 0, r1 = 0;
 #pragma unroll 2
     for (int j = 0; j < M; ++j) {
@@ -790,7 +790,7 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
         }
         __syncwarp();
     } else {
-        finish_many(f, M, kk, m, S, exact, out);
+        finish_many(f, M, kk, m, S, out);                     // (never after the exact way, which leaves kk candidates)
     }
 }
 
