@@ -97,6 +97,11 @@ __device__ __forceinline__ int team_excl_scan(int v, int* wtot, int tw, int& tot
     return base + before;
 }
 
+// Key of a candidate's path-value word (0: no such child).
+__device__ __forceinline__ unsigned long long key_of_word(unsigned long long x) {
+    return x == ~0ull ? 0ull : (x & 0x7FFFFFFFFFFFFFFFull) + 1ull;
+}
+
 // Threshold of the `need` largest keys among keyf(0..N); key 0 means "not an element".  key_or / key_and
 // are the bitwise OR / AND over all non-zero keys (the caller folds them into the sweep that stages the keys): the
 // bits on which all keys agree need no pass, and a pass whose threshold bin holds exactly the elements still needed
@@ -105,9 +110,6 @@ __device__ __forceinline__ int team_excl_scan(int v, int* wtot, int tw, int& tot
 // arrays that are all zero on entry: pass p counts into array p % 3 and clears the one pass p-1
 // read, so one barrier per pass is enough.  Returns the array that is left non-zero (the caller
 // clears it after its next barrier), or -1.
-__device__ __forceinline__ unsigned long long key_of_word(unsigned long long x) {
-    return x == ~0ull ? 0ull : (x & 0x7FFFFFFFFFFFFFFFull) + 1ull;
-}
 template <class LS, class KeyFn>
 __device__ int team_radix_select(LS& s, KeyFn keyf, int N, int need, int tt, unsigned long long key_or, unsigned long long key_and,
                                  unsigned long long& thr, int& need_eq) {
