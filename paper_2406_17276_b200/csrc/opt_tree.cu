@@ -719,14 +719,16 @@ row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __
 // completes a sequence takes it / with the queue: 8 sequences of n = 50 354 / 268 / 237; 32 of n = 64 519 / 739 / 375; 64 of n = 24
 // 436 / 672 / 347; 8 of n = 256, k = 16 969 / 622 / 463.
 // ------------------------------------------------------------------------------------------------
-// Where a sequence's tree stands: `rows` nodes of layer `layer` are to be expanded next (0: the tree is finished).  A step may
+// Where a sequence's tree stands: `rows` nodes of layer `layer` are to be expanded next (0: the tree is finished); `before`: how many
+// were to get that layer.  A step may
 // be asked of fewer sequences than the one before, so every sequence counts its own layers.  While a step runs, its CTAs
 // must all see the state from before it: a sequence's even and odd layers have a word each, with the number of the
 // step from which on it holds, and the newest that holds already counts.
-struct Front { int layer, rows; };
+struct Front { int layer, rows, before; };
+static_assert(kMaxLayers < 512 && kMaxN < 2048, "fields of the word below");
 constexpr int kNever = 0x7FFFFFFF;
-__device__ __forceinline__ unsigned long long front_word(int call, int layer, int rows) {
-    return ((unsigned long long)(unsigned)call << 32) | ((unsigned)layer << 16) | (unsigned)rows;
+__device__ __forceinline__ unsigned long long front_word(int call, int layer, int rows, int before) {
+    return ((unsigned long long)(unsigned)call << 32) | ((unsigned)layer << 22) | ((unsigned)before << 11) | (unsigned)rows;
 }
 __device__ __forceinline__ unsigned long long* front_words(const Workspace& w, int b) {
     return reinterpret_cast<unsigned long long*>(w.st + (size_t)b * 8 + kStFront);
@@ -737,7 +739,7 @@ __device__ __forceinline__ Front front_at(const Workspace& w, int b, int call) {
     if ((int)(e >> 32) > call) e = 0ull;
     if ((int)(o >> 32) > call) o = 0ull;
     const unsigned long long v = (e >> 32) >= (o >> 32) ? e : o;
-    return Front{(int)((v >> 16) & 0xFFFFu), (int)(v & 0xFFFFu)};
+    return Front{(int)((v >> 22) & 511u), (int)(v & 2047u), (int)((v >> 11) & 2047u)};
 }
 
 __global__ void layers_begin_kernel(Workspace w, Params p) {
@@ -752,8 +754,8 @@ __global__ void layers_begin_kernel(Workspace w, Params p) {
     int32_t* st = w.st + (size_t)i * 8;
     st[kStQueue] = 0;
     st[kStDone] = 0; st[kStNR] = 0;
-    front_words(w, (int)i)[0] = front_word(0, 0, 1);               // the root
-    front_words(w, (int)i)[1] = front_word(kNever, 0, 0);
+    front_words(w, (int)i)[0] = front_word(0, 0, 1, 0);            // the root
+    front_words(w, (int)i)[1] = front_word(kNever, 0, 0, 0);
     w.E_prev[i] = 0.0;
     w.front_phat[(size_t)i * 2 * p.n] = 1.0;                       // the root counts as factor 1
 }
@@ -785,7 +787,7 @@ struct LayersSink {
     int32_t *next_tokens, *next_parent, *next_count;
     __device__ void row_done(const RowDesc& d, const RowOut& r, FinScratch&) {
         const int lane = threadIdx.x & 31;
-        const SeqWork sw = seq_work(w, p, d.b, 0);
+        const SeqWork sw = seq_work(w, p, d.b, d.d);
         if (lane < p.k) {
             unsigned long long* ph = reinterpret_cast<unsigned long long*>(sw.cand_phat) + d.slot * p.k + lane;
             unsigned int* tk = reinterpret_cast<unsigned int*>(sw.cand_tok) + d.slot * p.k + lane;
@@ -795,11 +797,7 @@ struct LayersSink {
         __syncwarp();
         if (lane == 0) {
             LS& ls = smem_at<LS>(at);
-            // (the words validate themselves: no fence, except for the tokens of large layers, see BuildSink::await_rows)
-            if (d.fsize * p.k > kStageCap) fence_gpu();
-            const bool complete = atomicAdd(&sw.st[kStDone], 1) + 1 == d.fsize;
-            if (d.fsize * p.k > kStageCap) fence_gpu();
-            if (complete) {
+            if (atomicAdd(&sw.st[kStDone], 1) + 1 == d.fsize) {            // (the words validate themselves: no fence)
                 // this CTA's team, or, if that has a sequence already, the team that comes first
                 if (atomicCAS(const_cast<int*>(&ls.todo), 0, d.b + 1) != 0) {
                     const int pos = atomicAdd(&w.q_ctl[kQTail], 1);
@@ -829,6 +827,15 @@ struct LayersSink {
             if (fs >= 1 && fs <= fstride) continue;
             if (fs > fstride) set_status(w.status, kErrInternal);           // (a step with a wider buffer may follow)
             next_count[b] = 0;
+        }
+        // The candidate words of the step before, in the array of the other layers' parity, are cleared for the next step while this
+        // one's rows stream.  (All of them were stored by the time that step's kernel ended.)
+        for (int b = (int)blockIdx.x; b < p.B; b += (int)gridDim.x) {
+            const Front now = front_at(w, b, call);
+            if (now.rows > 0) {
+                const SeqWork sw = seq_work(w, p, b, now.layer);
+                clear_candidates(sw.cand_phat, sw.cand_tok, now.before * p.k, lane, 32);
+            }
         }
         __syncwarp();
         const CtaCore& core = smem_at<CtaCore>(0);
@@ -921,11 +928,11 @@ struct LayersSink {
     }
     // One layer of one sequence.
     __device__ void step(LS& ls, int b) {
+        const int nR_old = __ldcg(&w.st[(size_t)b * 8 + kStNR]);       // (0 before the first layer, like E; one round trip for all three)
+        const double eprev = __ldcg(&w.E_prev[b]);
         const Front now = front_at(w, b, call);
         const int lane = threadIdx.x & 31, d = now.layer + 1, fsize = now.rows;
-        const SeqWork sw = seq_work(w, p, b, 0);        // (a launch per layer: one candidate array will do)
-        const int nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
-        const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
+        const SeqWork sw = seq_work(w, p, b, d);
         const int nvalid = fsize * p.kk, nl = nvalid < p.n ? nvalid : p.n;
         if (lane == 0) {
             LayerJob& j = ls.job;
@@ -937,7 +944,7 @@ struct LayersSink {
         }
         if (fsize * p.k <= kTeam) { stage_layer_candidates(ls, sw, fsize, p.k); cp_async_wait_all(); }
         do_job(ls, 1);
-        if (lane == 0) { ls.job.ncand = fsize * p.k; ls.job.fsize = nl; }
+        if (lane == 0) { ls.job.ncand = 0; ls.job.fsize = nl; }         // (the next step clears the candidates)
         do_job(ls, 3);
         const int NR = nR_old + nl, nR = NR < p.n ? NR : p.n;
         const double esub = running_esub(ls, nR);
@@ -948,7 +955,7 @@ struct LayersSink {
             if (to.esub_trace) to.esub_trace[d - 1] = esub;
             sw.st[kStNR] = nR; *sw.E_prev = esub;
             sw.st[kStDone] = 0;
-            st_relaxed_u64(front_words(w, b) + (d & 1), front_word(call + 1, d, more ? nl : 0));
+            st_relaxed_u64(front_words(w, b) + (d & 1), front_word(call + 1, d, more ? nl : 0, fsize));
             next_count[b] = more ? nl : 0;
             ls.job.nR_old = nR; ls.last_esub = esub;
         }

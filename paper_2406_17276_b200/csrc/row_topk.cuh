@@ -85,7 +85,7 @@ struct LayerJob {                  // what the layer warp hands its assistants (
     // kind 2 (pruned draft, one selection over the running top-n and the candidates together):
     int nR_old, off;               // old top-n in keys[0..nR_old), candidates from keys[off] (off even, >= nR_old)
     int32_t* Rnew;                 // the new top-n's gids, ascending
-    // kind 3 (running top-n after a layer of fsize nodes chosen from ncand candidates): off: the old one is still in rsel / vals, else in Rold
+    // kind 3 (running top-n after a layer of fsize nodes chosen from ncand candidates, which it clears): off: the old one is still in rsel / vals, else in Rold
     const int32_t* Rold;
     int ncand;
     // kind 4 (pack the running top-n in rsel / vals, nR_old nodes, as the tree of sequence b)

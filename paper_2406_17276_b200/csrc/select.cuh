@@ -227,11 +227,12 @@ __device__ __forceinline__ void sweep_candidates(LS& s, const unsigned long long
 // store a word before its row has been sent out, so no clear can take a word away.  With one array the fence lay
 // between selection and publication, 3.7 % of a build of 32 sequences.  (A fence on the reading side as well, in the fetcher, costs a
 // step of one sequence 3 %; the finisher's store there depends on the mailbox word.)
-__device__ __forceinline__ void clear_candidates(double* cand_phat, int32_t* cand_tok, int N, int tt) {
+// By `stride` threads, this one the tt-th.
+__device__ __forceinline__ void clear_candidates(double* cand_phat, int32_t* cand_tok, int N, int tt, int stride) {
     #pragma unroll 1
-    for (int i = tt * 2; i < N; i += 2 * kTeam) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
+    for (int i = tt * 2; i < N; i += 2 * stride) *reinterpret_cast<uint4*>(cand_phat + i) = make_uint4(0, 0, 0, 0);
     #pragma unroll 1
-    for (int i = tt * 4; i < N; i += 4 * kTeam) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
+    for (int i = tt * 4; i < N; i += 4 * stride) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
 }
 
 // The team's part of a layer selection (N = fsize * k <= 1024; up to kTeam candidates were staged into s by the layer warp).  On return (after a last barrier) the new layer's nodes are in T and its
@@ -364,7 +365,7 @@ __device__ __noinline__ int select_running_team(int at, int tt, int* status) {
     ko = 0ull; ka = ~0ull;
 #pragma unroll
     for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
-    clear_candidates(cand_phat, cand_tok, N, tt);
+    clear_candidates(cand_phat, cand_tok, N, tt, kTeam);
     unsigned long long thr = 0ull;
     int need_eq = 0, dirty = -1;
     auto staged = [&](int i) { return s.keys[i]; };
@@ -776,7 +777,7 @@ template <class LS>
 __device__ __noinline__ int update_running_team(int at, int tt, int* status) {
     LS& s = smem_at<LS>(at);
     const LayerJob& j = s.job;
-    clear_candidates(j.cand_phat, j.cand_tok, j.ncand, tt);
+    clear_candidates(j.cand_phat, j.cand_tok, j.ncand, tt, kTeam);
     const bool cached = j.off != 0;
     const int32_t* const Rold = j.Rold;
     const double* const T_phat = j.T_phat;
