@@ -55,6 +55,21 @@ constexpr int kWaitPolls = 1 << 22;                 // limit of the waits that c
 // build of ten layers, 32 sequences 225 -> 223; no pause gives no more.
 constexpr unsigned kPollPauseNs = 40;
 
+// Division by a number that is fixed for a launch: x / d = x * m >> (31 + s) with s = ceil(log2 d), m = floor(2^(31+s) / d) + 1, exact
+// for 0 <= x < 2^31 (Granlund and Montgomery 1994).
+struct FixedDiv {
+    unsigned d, m;
+    int s;
+    __host__ __device__ static FixedDiv by(unsigned d) {
+        FixedDiv f{d, 0u, 0};
+        while ((1ull << f.s) < d) ++f.s;
+        f.m = (unsigned)((1ull << (31 + f.s)) / d + 1ull);
+        return f;
+    }
+    __host__ __device__ __forceinline__ unsigned div(unsigned x) const { return (unsigned)(((unsigned long long)x * m) >> (31 + s)); }
+    __host__ __device__ __forceinline__ unsigned mod(unsigned x) const { return x - div(x) * d; }
+};
+
 // ---------------------------------------------------------------------------------------------
 // bf16 bit pattern -> 16-bit key whose unsigned order equals the numeric order of the values
 // (-0 is folded into +0 so that equal values have equal keys).
@@ -199,15 +214,6 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 
 // --- barrier of the layer team (named barrier 1; barrier 0 is the CTA's) ---
 __device__ __forceinline__ void team_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTeam) : "memory"); }
-
-// --- asynchronous global -> shared copies (16 bytes, L2 only: the data was written by other SMs;
-//     all copies of a sweep are in flight at once and need no registers) ---
-__device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gmem_src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
 
 // --- global-memory flags and mailbox words (gpu scope) ---
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {

@@ -13,7 +13,6 @@
 
 namespace ot {
 
-constexpr int kRowMul = 31;                 // row of (token t, depth d) = (t*31 + d) mod H
 constexpr int kSmallThreads = 256;          // block size of the mask / init kernels
 // Verify: one CTA per target row, a thread keeps eight 16-byte loads in flight.  With 128 threads sixteen CTAs fit an
 // SM, so the n + 1 rows of 32 sequences (c4: 2080 CTAs) are all resident at once instead of in two uneven waves.  Fewer
@@ -23,10 +22,6 @@ constexpr int kSmallThreads = 256;          // block size of the mask / init ker
 // greedy - / 9.4 / 8.6, sampled - / 13.4 / 12.3; 488 rows 12.2 / 10.5 / 13.1 and 20.2 / 17.0 / 18.7; 784 rows 14.0 / 12.1 / - and
 // 22.4 / 20.8 / -; 1026 rows 15.9 / 14.6 / - and 26.2 / 27.9 / -.
 constexpr int kVerifyMany = 128, kVerifySome = 256, kVerifyFew = 512;
-
-__device__ __forceinline__ int row_of(int token, int depth, int H) {
-    return (int)(((unsigned)token * (unsigned)kRowMul + (unsigned)depth) % (unsigned)H);     // below 2^31 (supported_cfg); in 64 bits this is 1 % of a build
-}
 
 // ------------------------------------------------------------------------------------------------
 // Workspace
@@ -133,8 +128,20 @@ struct Params {            // by-value kernel parameters
     float delta;
     int aligned;
     int mcap, grid, cstride;
+    FixedDiv by_grid, by_H, by_k;
     int prune;             // draft only from layer nodes that are still among the n largest
 };
+
+__device__ __forceinline__ RowQueue row_queue(const Workspace& w, const Params& p) {
+    return RowQueue{w.mb_items, w.mb_phat, p.by_grid, p.by_H, p.mcap, p.V};
+}
+
+// What is the same for all jobs of a launch.
+__device__ __forceinline__ void set_job_constants(LayerJob& j, const Workspace& w, const Params& p) {
+    j.n = p.n; j.k = p.k; j.kk = p.kk; j.max_depth = p.max_depth;
+    j.queue = row_queue(w, p);
+    j.by_k = p.by_k;
+}
 
 // d: the layer whose candidates are meant.
 __device__ __forceinline__ SeqWork seq_work(const Workspace& w, const Params& p, int b, int d) {
@@ -161,25 +168,6 @@ __device__ __forceinline__ TreeOut tree_out(const opt_tree_out& o, const Params&
     t.expected_len = o.expected_len + b;
     t.esub_trace = o.esub_trace ? o.esub_trace + (size_t)b * p.max_depth : nullptr;
     return t;
-}
-
-// Mailbox item: bit 63 valid | b (15 bits) | layer d (9) | void flag (1) | frontier slot (10, from bit 22) | table row of the node to
-// expand (22).  A second word at the same mailbox position carries the node's path value (bit 63
-// valid; a path value is never negative).  Both words validate themselves, so a row can be expanded
-// from them alone and the publisher needs no fence before writing them.
-constexpr int kMaxTableRows = 1 << 22;
-constexpr int kMaxLayers = 510;             // layers a build may draft: layer d+1 must fit the item's 9-bit field
-__device__ __forceinline__ unsigned long long item_encode(int b, int d, int slot, int row) {
-    return (1ull << 63) | ((unsigned long long)b << 48) | ((unsigned long long)d << 39) |
-           ((unsigned long long)slot << 22) | (unsigned long long)row;
-}
-
-// An entry that was handed out but is not needed after all (the pruned draft reserves a layer's entries
-// before it knows how many rows the layer will have): fetchers drop such a ticket.
-constexpr unsigned long long kItemVoid = 1ull << 38;
-
-__device__ __forceinline__ unsigned long long phat_word(double p) {
-    return (1ull << 63) | (unsigned long long)__double_as_longlong(p);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -269,18 +257,11 @@ struct BuildSink {
         g0 = __shfl_sync(0xFFFFFFFFu, g0, 0);
         if (lane < r.kk) {
             int token = r.tok;
-            if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
+            publish_node(row_queue(w, p), d.b, 1, g0, lane, token, phat_key(ph), w.status);
+            if (token < 0 || token >= p.V) token = 0;
             sw.T_tok[lane] = token; sw.T_par[lane] = 0; sw.T_phat[lane] = ph;
             sw.R[p.n + lane] = lane;                                       // the running top-n after layer 1 (buffer of odd layers)
             if (kPrune) sw.fmap[lane] = lane;
-            const unsigned g = g0 + (unsigned)lane, c = g % (unsigned)p.grid, e = g / (unsigned)p.grid;
-            if (e < (unsigned)p.mcap) {
-                const size_t pos = (size_t)c * p.mcap + e;
-                st_relaxed_u64(&w.mb_phat[pos], phat_word(ph));
-                st_relaxed_u64(&w.mb_items[pos], item_encode(d.b, 2, lane, row_of(token, 1, p.H)));
-            } else {
-                set_status(w.status, kErrInternal);
-            }
         }
         if (lane == 0) {
             if (to.esub_trace) to.esub_trace[0] = esub;
@@ -336,41 +317,28 @@ struct BuildSink {
     // pick != null (pruned draft): only the layer slots pick[0..nl) are sent out, as frontier rows 0..nl;
     // the map from frontier row to layer slot is left in fmap for the next selection.
     template <class LS>
-    __device__ void publish_layer(LS& ls, int b, int d, int nl, unsigned g0, const int* pick = nullptr,
-                                  int32_t* fmap = nullptr) {
-        const int lane = threadIdx.x & 31;
+    __device__ void publish_layer(LS& ls, int nl, unsigned g0, int32_t* fmap = nullptr, const int* pick = nullptr) {
         g0 = __shfl_sync(0xFFFFFFFFu, g0, 0);
-        for (int i = lane; i < nl; i += 32) {
+        for (int i = threadIdx.x & 31; i < nl; i += 32) {
             const int slot = pick ? pick[i] : i;
             if (fmap) fmap[i] = slot;
-            int token = ls.ltok[slot];
-            if (token < 0 || token >= p.V) { set_status(w.status, kErrInternal); token = 0; }
-            const unsigned g = g0 + (unsigned)i, c = g % (unsigned)p.grid, e = g / (unsigned)p.grid;
-            if (e < (unsigned)p.mcap) {
-                const size_t pos = (size_t)c * p.mcap + e;
-                st_relaxed_u64(&w.mb_phat[pos], (1ull << 63) | (ls.lkeys[slot] - 1ull));
-                st_relaxed_u64(&w.mb_items[pos], item_encode(b, d + 1, i, row_of(token, d, p.H)));
-            } else {
-                set_status(w.status, kErrInternal);
-            }
+            publish_node(ls.job.queue, ls.job.b, ls.job.d, g0, i, ls.ltok[slot], ls.lkeys[slot], w.status);
         }
         __syncwarp();
     }
     // Entries g0+from .. g0+to of a reservation are not needed.
-    __device__ void void_entries(unsigned g0, int from, int to) {
-        const int lane = threadIdx.x & 31;
+    template <class LS>
+    __device__ void void_entries(LS& ls, unsigned g0, int from, int to) {
         g0 = __shfl_sync(0xFFFFFFFFu, g0, 0);
-        for (int i = from + lane; i < to; i += 32) {
-            const unsigned g = g0 + (unsigned)i, c = g % (unsigned)p.grid, e = g / (unsigned)p.grid;
-            if (e < (unsigned)p.mcap) {
-                const size_t pos = (size_t)c * p.mcap + e;
-                st_relaxed_u64(&w.mb_phat[pos], 1ull << 63);
-                st_relaxed_u64(&w.mb_items[pos], (1ull << 63) | kItemVoid);
-            } else {
-                set_status(w.status, kErrInternal);
-            }
-        }
+        for (int i = from + (int)(threadIdx.x & 31); i < to; i += 32) void_entry(ls.job.queue, g0 + (unsigned)i, w.status);
         __syncwarp();
+    }
+    // What every selection job has in common (lane 0).
+    __device__ void set_job(LayerJob& j, int kind, const SeqWork& sw, int b, int d, int fsize) {
+        j.kind = kind; j.b = b; j.d = d; j.fsize = fsize;
+        j.cand_phat = sw.cand_phat; j.cand_tok = sw.cand_tok;
+        j.T_tok = sw.T_tok; j.T_par = sw.T_par; j.T_phat = sw.T_phat;
+        j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
     }
     // Pruned draft, a whole layer job with one selection (see select_running_team).  Returns the number
     // of rows of the next layer, or -1 if the sequence is finished.
@@ -378,34 +346,19 @@ struct BuildSink {
     __device__ int merged_layer_job(LS& ls, const SeqWork& sw, int b, int d, int fsize, int nR_old, int off) {
         const int lane = threadIdx.x & 31;
         const int nvalid = fsize * p.kk, reserve = nvalid < p.n ? nvalid : p.n;
-        stage_layer_candidates(ls, sw, fsize, p.k, off);
         const unsigned g0 = d < p.Dcap ? reserve_layer(reserve) : 0u;      // entries for the next layer, before its size is known
-        // the old top-n: still in the scratch if this warp's last job was this sequence's previous layer
-        const int32_t* Rold = sw.R + ((d - 1) & 1) * p.n;
-        const bool cached = ls.cache_b == b && ls.cache_d == d - 1;
-        for (int i = lane; i < nR_old; i += 32) {
-            int gid;
-            unsigned long long key;
-            if (cached) { gid = ls.rsel[i]; key = phat_key(ls.vals[i]); }
-            else { gid = __ldcg(&Rold[i]); key = phat_key(__ldcg(&sw.T_phat[gid])); }
-            ls.gids[i] = gid;
-            ls.keys[i] = key;
-        }
+        const bool early = d < p.Dcap && p.delta == -INFINITY;             // (the loop test only looks at the depth)
         if (lane == 0) {
             LayerJob& j = ls.job;
-            j.kind = 2; j.d = d; j.fsize = fsize; j.n = p.n; j.k = p.k; j.kk = p.kk;
-            j.cand_phat = sw.cand_phat; j.cand_tok = sw.cand_tok;
-            j.T_tok = sw.T_tok; j.T_par = sw.T_par; j.T_phat = sw.T_phat;
-            j.fmap = sw.fmap; j.nR_old = nR_old; j.off = off; j.Rnew = sw.R + (d & 1) * p.n;
+            set_job(j, 2, sw, b, d, fsize);
+            j.fmap = sw.fmap; j.nR_old = nR_old; j.off = off;
+            j.cached = ls.cache_b == b && ls.cache_d == d - 1;             // this warp's last job was this sequence's previous layer
+            j.publish = early;
         }
-        cp_async_wait_all();
         __syncwarp();
         team_sync();
-        const int nR = select_running_team<LS>(smem_offset(&ls), lane, w.status);
-        int kept_old = 0;
-#pragma unroll
-        for (int q = 0; q < kTeamWarps; ++q) kept_old += ls.scan_c[q];
-        const int cnt = nR - kept_old;                      // new members = the rows of the next layer
+        const int nR = running_job<LS>(smem_offset(&ls), lane, g0, w.status);
+        const int cnt = nR - ls.kept_old;                   // new members = the rows of the next layer
         const double esub = running_esub(ls, nR);
         const double eprev = d == 1 ? 0.0 : __ldcg(sw.E_prev);
         bool more = d < p.Dcap && (esub - eprev > (double)p.delta);
@@ -418,14 +371,14 @@ struct BuildSink {
         }
         __syncwarp();
         if (more && cnt > 0) {
-            for (int i = lane; i < cnt; i += 32) ls.gids[i] = i;       // members are sent out in slot order
-            __syncwarp();
-            publish_layer(ls, b, d, cnt, g0, ls.gids, sw.fmap);
-            void_entries(g0, cnt, reserve);
+            if (!early) {
+                publish_layer(ls, cnt, g0, sw.fmap);        // members are sent out in slot order
+                void_entries(ls, g0, cnt, reserve);
+            }
             fence_gpu();                                    // the cleared candidate words before the rows of layer d + 2
             return cnt;
         }
-        if (d < p.Dcap) void_entries(g0, 0, reserve);
+        if (d < p.Dcap && !early) void_entries(ls, g0, 0, reserve);
         int d_end = d;
         if (more) {                                         // nothing left to draft from: the loop would go on testing a gain of zero
             d_end = p.delta < 0.0f ? p.Dcap : d + 1;
@@ -443,7 +396,7 @@ struct BuildSink {
     __device__ void pack(LS& ls, const SeqWork& sw, const TreeOut& to, int b, int d, int nR, double esub) {
         if ((threadIdx.x & 31) == 0) {
             LayerJob& j = ls.job;
-            j.kind = 4; j.d = d; j.n = p.n; j.nR_old = nR; j.b = b; j.max_depth = p.max_depth;
+            j.kind = 4; j.d = d; j.nR_old = nR; j.b = b;
             j.T_tok = sw.T_tok; j.T_par = sw.T_par;
             ls.last_esub = esub;
         }
@@ -470,6 +423,8 @@ struct BuildSink {
     // assistants wait at that barrier in between and leave when they find a job of kind 0.
     template <class LS>
     __device__ void layer_loop(LS& ls) {
+        if ((threadIdx.x & 31) == 0) set_job_constants(ls.job, w, p);
+        __syncwarp();
         layer_follow(ls);
         if ((threadIdx.x & 31) == 0) ls.job.kind = 0;
         __syncwarp();
@@ -482,23 +437,22 @@ struct BuildSink {
             team_sync();
             const int kind = ls.job.kind, at = smem_offset(&ls);
             if (kind == 0) return;
-            if (kind == 2) select_running_team<LS>(at, tt, w.status);
-            else if (kind == 3) update_running_team<LS>(at, tt, w.status);
+            // (kinds 2 and 3 clear candidate words; the fence puts the clears before what this thread sends out in later jobs)
+            if (kind == 2) { running_job<LS>(at, tt, 0u, w.status); fence_gpu(); }
+            else if (kind == 3) { update_running_team<LS>(at, tt, w.status); fence_gpu(); }
             else if (kind == 4) { pack_tree<LS>(at, tree_out(out, p, ls.job.b), tt, kTeam, w.status); team_sync(); }
-            else if (ls.job.fsize * ls.job.k <= kStageCap) select_layer_team<kPrune, LS>(at, tt, w.status);
-            else select_layer_team_big<kPrune, LS>(at, tt, w.status);
+            else select_job<LS>(at, tt, 0u, w.status);
         }
     }
-    // Rows of layer d, of f rows, that may still be missing when the team starts on it.  Candidate words validate themselves,
-    // so the job's hand-over, the staging and most of the sweep go on while the last rows are finished, and only what
-    // is missing then is waited for.  As long as a layer's rows of all sequences take the SMs at most four times round, all
-    // but the first may be missing (see sweep_candidates); otherwise, and in the selections that stage their
-    // candidates (pruned draft, depth limit), sixteen rows or a quarter of a large layer: 32 sequences 221.5 us per build with
+    // Rows of a layer of f rows that may still be missing when the team starts on it.  Candidate words validate themselves, so the
+    // team can start at once and wait for the words.  It does as long as a layer's rows of all sequences take the SMs at most four
+    // times round; beyond that the polling would slow the rows down (a team reads every missing word again and again), and it
+    // starts when at most sixteen rows or a quarter of a large layer are missing: 32 sequences 221.5 us per build with
     // none, 219.7 with 16, 220.7 with half; n = 512 429 with none, 413 with a quarter or a half.
     // A warp that follows several sequences must not wait for one of them.
-    __device__ int rows_ahead(int f, int d) const {
-        const int a = !kPrune && d < p.Dcap && p.B * f <= 4 * (int)gridDim.x ? f - 1 : max(16, f >> 2);
-        return p.B <= (int)gridDim.x ? min(a, f - 1) : 0;
+    __device__ int rows_ahead(int f) const {
+        if (p.B > (int)gridDim.x) return 0;
+        return p.B * f <= 4 * (int)gridDim.x ? f : min(max(16, f >> 2), f - 1);
     }
     template <class LS>
     __device__ void layer_follow(LS& ls) {
@@ -521,10 +475,13 @@ struct BuildSink {
                     if (cur_d[q] == 0) continue;
                     const int b = b0 + q * (int)gridDim.x;
                     const SeqWork sw = seq_work(w, p, b, cur_d[q]);
-                    int done = 0;
-                    if (lane == 0) done = ld_acquire_s32(&sw.st[kStDone]);
-                    done = __shfl_sync(0xFFFFFFFFu, done, 0);
-                    if (done < cur_tot[q] - (cur_d[q] > 1 ? rows_ahead(cur_f[q], cur_d[q]) : 0)) continue;
+                    const int ahead = cur_d[q] > 1 ? rows_ahead(cur_f[q]) : 0;
+                    if (ahead < cur_f[q]) {
+                        int done = 0;
+                        if (lane == 0) done = ld_acquire_s32(&sw.st[kStDone]);
+                        done = __shfl_sync(0xFFFFFFFFu, done, 0);
+                        if (done < cur_tot[q] - ahead) continue;
+                    }
                     progressed = true;
                     if (cur_d[q] == 1) {
                         // the finisher of the root's row says whether it grew layer 1 itself (then layer 2 is on its way)
@@ -550,7 +507,7 @@ struct BuildSink {
                     // do not reach the running top-n need not be stored, and one selection does instead of two.
                     if (kPrune || d == p.Dcap) {
                         const int nR_old = d == 1 ? 0 : __ldcg(&sw.st[kStNR]);
-                        const int off = (nR_old + 1) & ~1;
+                        const int off = (nR_old + 31) & ~31;
                         if (off + fsize * p.k <= kStageCap) {
                             const int sent = merged_layer_job(ls, sw, b, d, fsize, nR_old, off);
                             if (sent > 0) { cur_d[q] = d + 1; cur_f[q] = sent; cur_tot[q] += sent; }
@@ -565,25 +522,19 @@ struct BuildSink {
                         }
                     }
                     const bool early = !kPrune && d < p.Dcap && p.delta == -INFINITY;
-                    if (fsize * p.k <= kTeam) stage_layer_candidates(ls, sw, fsize, p.k);
                     unsigned g0 = 0;
                     if (early) g0 = reserve_layer(nl);        // the rows' numbers, while the candidates load
-                    {
-                        const bool small = fsize * p.k <= kStageCap;    // the candidates fit the shared-memory staging
-                        if (lane == 0) {
-                            LayerJob& j = ls.job;
-                            j.kind = 1; j.d = d; j.fsize = fsize; j.n = p.n; j.k = p.k; j.kk = p.kk;
-                            j.cand_phat = sw.cand_phat; j.cand_tok = sw.cand_tok;
-                            j.T_tok = sw.T_tok; j.T_par = sw.T_par; j.T_phat = sw.T_phat;
-                            j.fmap = kPrune ? sw.fmap : nullptr;
-                        }
-                        if (fsize * p.k <= kTeam) cp_async_wait_all();       // the staged candidates are in shared memory
-                        __syncwarp();
-                        team_sync();                          // ... and, with the job, visible to the assistants
-                        if (small) select_layer_team<kPrune, LS>(smem_offset(&ls), lane, w.status);
-                        else select_layer_team_big<kPrune, LS>(smem_offset(&ls), lane, w.status);
+                    const bool small = fsize * p.k <= kStageCap;        // the team holds the candidates in registers
+                    if (lane == 0) {
+                        LayerJob& j = ls.job;
+                        set_job(j, 1, sw, b, d, fsize);
+                        j.fmap = kPrune ? sw.fmap : nullptr;
+                        j.publish = early && small;
                     }
-                    if (early) publish_layer(ls, b, d, nl, g0);
+                    __syncwarp();
+                    team_sync();
+                    select_job<LS>(smem_offset(&ls), lane, g0, w.status);
+                    if (early && !small) publish_layer(ls, nl, g0);
                     double esub;
                     int nR;
                     {
@@ -593,8 +544,7 @@ struct BuildSink {
                         __syncwarp();
                         if (lane == 0) {
                             LayerJob& j = ls.job;
-                            j.kind = 3; j.ncand = fsize * p.k; j.fsize = nl; j.nR_old = nR_old; j.off = cached ? 1 : 0;
-                            j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
+                            j.kind = 3; j.ncand = fsize * p.k; j.fsize = nl; j.nR_old = nR_old; j.cached = cached;
                             ls.cache_b = b; ls.cache_d = d;
                         }
                         __syncwarp();
@@ -623,7 +573,7 @@ struct BuildSink {
                         for (int i = lane; i < sent; i += 32) ls.gids[i] = ls.rsel[nR - sent + i] - gid0;
                         __syncwarp();
                         if (sent > 0) {
-                            publish_layer(ls, b, d, sent, reserve_layer(sent), ls.gids, sw.fmap);
+                            publish_layer(ls, sent, reserve_layer(sent), sw.fmap, ls.gids);
                         } else {
                             // Nothing left to draft from: further layers change neither T_opt nor E_sub.  The loop
                             // of Algorithm 1 would go on testing a gain of zero: to the depth limit if the
@@ -635,7 +585,7 @@ struct BuildSink {
                             more = false;
                         }
                     } else if (more && !early) {
-                        publish_layer(ls, b, d, nl, reserve_layer(nl));
+                        publish_layer(ls, nl, reserve_layer(nl));
                     }
                     if (more) {
                         cur_d[q] = d + 1; cur_f[q] = sent; cur_tot[q] += sent;
@@ -842,6 +792,7 @@ struct LayersSink {
             }
         }
         __syncwarp();
+        if (lane == 0) set_job_constants(ls.job, w, p);
         const CtaCore& core = smem_at<CtaCore>(0);
         int seen = 0;
         long long t0 = clock64();
@@ -910,8 +861,7 @@ struct LayersSink {
         if (kind == 3) update_running_team<LS>(at, tt, w.status);
         else if (kind == 4) { pack_tree<LS>(at, tree_out(out, p, ls.job.b), tt, kTeam, w.status); team_sync(); }
         else if (kind == 6) { hand_back(ls, tt); team_sync(); }
-        else if (ls.job.fsize * ls.job.k <= kStageCap) select_layer_team<false, LS>(at, tt, w.status);
-        else select_layer_team_big<false, LS>(at, tt, w.status);
+        else select_job<LS>(at, tt, 0u, w.status);
     }
     __device__ void hand_back(LS& ls, int tt) {
         const int b = ls.job.b, nl = ls.job.fsize, gid0 = (ls.job.d - 1) * p.n;
@@ -940,13 +890,12 @@ struct LayersSink {
         const int nvalid = fsize * p.kk, nl = nvalid < p.n ? nvalid : p.n;
         if (lane == 0) {
             LayerJob& j = ls.job;
-            j.b = b; j.d = d; j.fsize = fsize; j.n = p.n; j.k = p.k; j.kk = p.kk;
+            j.b = b; j.d = d; j.fsize = fsize;
             j.cand_phat = sw.cand_phat; j.cand_tok = sw.cand_tok;
             j.T_tok = sw.T_tok; j.T_par = sw.T_par; j.T_phat = sw.T_phat; j.fmap = nullptr;
-            j.nR_old = nR_old; j.off = 0; j.max_depth = p.max_depth;
+            j.nR_old = nR_old; j.cached = 0; j.publish = 0;
             j.Rold = sw.R + ((d - 1) & 1) * p.n; j.Rnew = sw.R + (d & 1) * p.n;
         }
-        if (fsize * p.k <= kTeam) { stage_layer_candidates(ls, sw, fsize, p.k); cp_async_wait_all(); }
         do_job(ls, 1);
         if (lane == 0) { ls.job.ncand = 0; ls.job.fsize = nl; }         // (the next step clears the candidates)
         do_job(ls, 3);
@@ -1603,6 +1552,7 @@ ot::Params make_params(const opt_tree_ctx* ctx, const void* table, float delta) 
     p.mcap = ctx->mcap;
     p.grid = ctx->grid;
     p.cstride = (int)ot::cand_stride(c.n, c.k);
+    p.by_grid = ot::FixedDiv::by((unsigned)ctx->grid); p.by_H = ot::FixedDiv::by((unsigned)c.H); p.by_k = ot::FixedDiv::by((unsigned)c.k);
     p.delta = delta;
     p.aligned = ((reinterpret_cast<uintptr_t>(table) & 15u) == 0 && (c.V % 8) == 0) ? 1 : 0;
     return p;

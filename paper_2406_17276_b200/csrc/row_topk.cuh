@@ -78,21 +78,33 @@ struct alignas(16) FinScratch {    // private to one finisher warp (hist is clea
     int cand_count;
 };
 
+struct RowQueue {                  // the row mailboxes of a build (see Workspace and Params)
+    unsigned long long *items, *phat;
+    FixedDiv by_grid, by_H;
+    int mcap, V;
+};
+
 struct LayerJob {                  // what the layer warp hands its assistants (kind 0: leave)
     int kind, d, fsize, n, k, kk;
     double* cand_phat; int32_t* cand_tok; int32_t* T_tok; int32_t* T_par; double* T_phat;
-    const int32_t* fmap;           // pruned draft: layer slot of the node behind each frontier row (null: the identity)
-    // kind 2 (pruned draft, one selection over the running top-n and the candidates together):
-    int nR_old, off;               // old top-n in keys[0..nR_old), candidates from keys[off] (off even, >= nR_old)
-    int32_t* Rnew;                 // the new top-n's gids, ascending
-    // kind 3 (running top-n after a layer of fsize nodes chosen from ncand candidates, which it clears): off: the old one is still in rsel / vals, else in Rold
+    int32_t* fmap;                 // pruned draft: layer slot of the node behind each frontier row (null: the identity)
+    // kinds 2 (pruned draft and depth limit: one selection over the running top-n and the candidates together) and 3 (running top-n
+    // after a layer of fsize nodes chosen from ncand candidates, which it clears):
+    int nR_old, off;               // members of the old top-n; kind 2: the candidates' first index (a multiple of 32)
+    int cached;                    // the old top-n is still in rsel / vals, else in Rold
     const int32_t* Rold;
+    int32_t* Rnew;                 // the new top-n's gids, ascending
     int ncand;
     // kind 4 (pack the running top-n in rsel / vals, nR_old nodes, as the tree of sequence b)
     int b, max_depth;
+    // kinds 1 and 2: publish the new nodes' rows straight away, numbered from g0 on
+    int publish;
+    unsigned g0;
+    RowQueue queue;
+    FixedDiv by_k;
 };
 
-constexpr int kStageCap = 1024;                    // candidates of a layer that the shared-memory staging holds
+constexpr int kStageCap = 1024;                    // candidates of a layer that the team holds in registers
 constexpr int kSmallN = 256;                       // node budgets up to this use the smaller of the two scratch layouts
 
 // Private to the layer team of a CTA.  NCAP is the largest node budget the layout serves: the kernels
@@ -100,13 +112,14 @@ constexpr int kSmallN = 256;                       // node budgets up to this us
 // CTA's shared memory (and with it the SM's L1) where it is best for them.
 template <int NCAP>
 struct alignas(16) LayerScratchT {
+    static constexpr int kBudget = NCAP;
     static constexpr int kSurvivors = 2 * NCAP > kStageCap ? 2 * NCAP : kStageCap;   // candidates that keys can hold
     static constexpr bool kWideGids = 2 * NCAP > kStageCap;    // gids holds as many as keys
     static constexpr int kKeys = kSurvivors + 2;
-    unsigned long long keys[kKeys];            // staged candidate keys, then the keys of R + layer
+    unsigned long long keys[kKeys];            // keys of a selection that does not fit the registers, or falls back on a radix select
     unsigned long long lkeys[NCAP];            // keys of the new layer, slot order
     double vals[NCAP];                         // path values of the new running top-n
-    int toks[kStageCap + 4];                   // staged candidate tokens
+    int toks[kStageCap];                       // large layers: candidate indexes
     int gids[2 * NCAP];
     int rsel[NCAP];                            // gids of the new running top-n, ascending
     int ltok[NCAP];                            // tokens of the new layer, slot order
@@ -115,7 +128,10 @@ struct alignas(16) LayerScratchT {
     int scan_a[kTeamWarps], scan_b[kTeamWarps];
     LayerJob job;
     static constexpr int kList = 64;
-    unsigned long long list[kList];            // large layers: keys of the threshold's bin
+    unsigned long long list[kList];            // keys of the threshold's bin
+    int listi[kList];                          // and their indexes
+    uint32_t pick[32];                         // ballots of a selection, in index order
+    int kept_old;
     int listn;
     volatile int todo;                         // layer-by-layer build: the sequence the team has (index + 1), 0: it is idle
     int rows_done;

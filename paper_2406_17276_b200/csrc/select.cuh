@@ -1,8 +1,8 @@
 // K2 / K3: layer selection (the n candidates of largest path value), running E_sub(T, n) and the
 // tree packer by the layer team.
 //
-// Selection never sorts: a radix select of at most 8 passes on the 64-bit keys finds the threshold of the
-// "need" largest, then an ordered compaction (ballot scans) emits the kept elements in index
+// Selection never sorts: one count into coarse bins (or, as the fallback, a radix select on the 64-bit keys) finds the
+// threshold of the "need" largest, then an ordered compaction (ballot scans) emits the kept elements in index
 // order, which is exactly the storage order the method wants (candidate-index order for a layer;
 // (depth, slot) order for the running top-n, which is also the packed order of the final tree).
 #pragma once
@@ -10,6 +10,30 @@
 #include "row_topk.cuh"
 
 namespace ot {
+
+constexpr int kRowMul = 31;                 // row of (token t, depth d) = (t*31 + d) mod H
+__device__ __forceinline__ int row_of(int token, int depth, int H) {
+    return (int)(((unsigned)token * (unsigned)kRowMul + (unsigned)depth) % (unsigned)H);     // below 2^31 (supported_cfg); in 64 bits this is 1 % of a build
+}
+
+// Mailbox item: bit 63 valid | b (15 bits) | layer d (9) | void flag (1) | frontier slot (10, from bit 22) | table row of the node to
+// expand (22).  A second word at the same mailbox position carries the node's path value (bit 63
+// valid; a path value is never negative).  Both words validate themselves, so a row can be expanded
+// from them alone and the publisher needs no fence before writing them.
+constexpr int kMaxTableRows = 1 << 22;
+constexpr int kMaxLayers = 510;             // layers a build may draft: layer d+1 must fit the item's 9-bit field
+__device__ __forceinline__ unsigned long long item_encode(int b, int d, int slot, int row) {
+    return (1ull << 63) | ((unsigned long long)b << 48) | ((unsigned long long)d << 39) |
+           ((unsigned long long)slot << 22) | (unsigned long long)row;
+}
+
+// An entry that was handed out but is not needed after all (the pruned draft reserves a layer's entries
+// before it knows how many rows the layer will have): fetchers drop such a ticket.
+constexpr unsigned long long kItemVoid = 1ull << 38;
+
+__device__ __forceinline__ unsigned long long phat_word(double p) {
+    return (1ull << 63) | (unsigned long long)__double_as_longlong(p);
+}
 
 // Positive doubles order like their bit patterns; +1 keeps every valid key above the "invalid" key 0.
 __device__ __forceinline__ unsigned long long phat_key(double p) { return (unsigned long long)__double_as_longlong(p) + 1ull; }
@@ -47,22 +71,6 @@ struct TreeOut {           // mirrors opt_tree_out, pointers offset to the seque
     double* expected_len;
     double* esub_trace;    // may be null
 };
-
-// Starts the asynchronous copies of a layer's candidates (path values and tokens) into the layer
-// warp's scratch; the layer warp waits for them before it starts the team.  Separate so that other round trips (the
-// mailbox reservations) can be in flight at the same time.
-template <class LS>
-__device__ __forceinline__ void stage_layer_candidates(LS& s, const SeqWork& w, int fsize, int k, int off = 0) {
-    const int lane = threadIdx.x & 31;
-    const int N = fsize * k;
-    if (off + N > kStageCap) return;                       // (off is even: the copies keep their 16-byte alignment)
-    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(w.cand_phat);
-    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(w.cand_tok);
-    #pragma unroll 1
-    for (int i = lane * 2; i < N; i += 64) cp_async_16(&s.keys[off + i], &gph[i]);
-    #pragma unroll 1
-    for (int i = lane * 4; i < N; i += 128) cp_async_16(&s.toks[i], &gtk[i]);
-}
 
 // A candidate word that was not there yet when it was looked at is read again until it is (bounded).
 // Rare, so out of line.
@@ -171,52 +179,33 @@ __device__ int team_radix_select(LS& s, KeyFn keyf, int N, int need, int tt, uns
     return (pass - 1) % 3;
 }
 
-// Sweep of the team over a layer's candidate words (gph, gtk): the keys and tokens go to shared memory, kW of them per thread
-// in flight.  Words that are not there yet are read again, all at once, until they are (bounded), with a short pause so that
-// the polling does not hold up the words themselves.  Together with starting the team when the layer's first row is in
-// (rows_ahead) this takes the staging by one warp and most of the hand-over off the chain: one sequence of n = 50 136.1 -> 131.5 us
-// per step, V = 128256 288.5 -> 277.7.  Four words per thread in flight.  Layers of at most
-// one candidate per thread keep the staging: n = 10 alone 75.2 us per step with it, 76.6 with a sweep.
-template <int kW, class LS>
-__device__ __forceinline__ void sweep_candidates(LS& s, const unsigned long long* gph, const unsigned int* gtk, int N, int tt, unsigned long long& ko,
-                                                 unsigned long long& ka, int* status) {
+// Candidate words i = u * kTeam + tt (u < kW) of a layer of N, into registers.  Words that are not there yet are read again, all
+// at once, until they are (bounded), with a short pause so that the polling does not hold up the words themselves.
+template <int kW>
+__device__ __forceinline__ void sweep_candidates(const unsigned long long* gph, const unsigned int* gtk, int N, int tt, unsigned long long (&x)[kW],
+                                                 unsigned int (&t32)[kW], int* status) {
+#pragma unroll
+    for (int u = 0; u < kW; ++u) {
+        const int i = u * kTeam + tt;
+        x[u] = i < N ? ld_relaxed_u64(&gph[i]) : ~0ull;
+        t32[u] = i < N ? ld_relaxed_u32(&gtk[i]) : ~0u;
+    }
     #pragma unroll 1
-    for (int i0 = tt; i0 - tt < N; i0 += kW * kTeam) {
-        unsigned long long x[kW];
-        unsigned int t32[kW];
+    for (int t = 0;; ++t) {
+        bool missing = false;
 #pragma unroll
         for (int u = 0; u < kW; ++u) {
-            const int i = i0 + u * kTeam;
-            x[u] = i < N ? ld_relaxed_u64(&gph[i]) : ~0ull;
-            t32[u] = i < N ? ld_relaxed_u32(&gtk[i]) : ~0u;
+            const int i = u * kTeam + tt;
+            if (!(x[u] >> 63)) { x[u] = ld_relaxed_u64(&gph[i]); missing = missing || !(x[u] >> 63); }
+            if (!(t32[u] >> 31)) { t32[u] = ld_relaxed_u32(&gtk[i]); missing = missing || !(t32[u] >> 31); }
         }
-        // words that are not there yet are read again, all at once, until they are (bounded)
-        #pragma unroll 1
-        for (int t = 0;; ++t) {
-            bool missing = false;
+        if (!__any_sync(0xFFFFFFFFu, missing)) break;
+        __nanosleep(20);
+        if (t >= kWaitPolls) {
+            set_status(status, kErrTimeout);
 #pragma unroll
-            for (int u = 0; u < kW; ++u) {
-                const int i = i0 + u * kTeam;
-                if (!(x[u] >> 63)) { x[u] = ld_relaxed_u64(&gph[i]); missing = missing || !(x[u] >> 63); }
-                if (!(t32[u] >> 31)) { t32[u] = ld_relaxed_u32(&gtk[i]); missing = missing || !(t32[u] >> 31); }
-            }
-            if (!__any_sync(0xFFFFFFFFu, missing)) break;
-            __nanosleep(20);
-            if (t >= kWaitPolls) {
-                set_status(status, kErrTimeout);
-#pragma unroll
-                for (int u = 0; u < kW; ++u) { if (!(x[u] >> 63)) x[u] = ~0ull; if (!(t32[u] >> 31)) t32[u] = ~0u; }
-                break;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kW; ++u) {
-            const int i = i0 + u * kTeam;
-            if (i >= N) break;
-            const unsigned long long key = key_of_word(x[u]);
-            s.keys[i] = key;
-            if (key) { ko |= key; ka &= key; }
-            s.toks[i] = (int)t32[u];
+            for (int u = 0; u < kW; ++u) { if (!(x[u] >> 63)) x[u] = ~0ull; if (!(t32[u] >> 31)) t32[u] = ~0u; }
+            break;
         }
     }
 }
@@ -235,203 +224,325 @@ __device__ __forceinline__ void clear_candidates(double* cand_phat, int32_t* can
     for (int i = tt * 4; i < N; i += 4 * stride) *reinterpret_cast<uint4*>(cand_tok + i) = make_uint4(0, 0, 0, 0);
 }
 
-// The team's part of a layer selection (N = fsize * k <= 1024; up to kTeam candidates were staged into s by the layer warp).  On return (after a last barrier) the new layer's nodes are in T and its
-// tokens and keys in s.ltok / s.lkeys.  Returns nl.
-template <bool kPrune, class LS>
-__device__ __noinline__ int select_layer_team(int at, int tt, int* status) {
+// The largest bin of the 1024 counts in s.thist at which at least `need` elements lie at or above; `at_or_above` is their
+// number (the elements must be that many).  Every warp for itself.
+template <class LS>
+__device__ __forceinline__ int warp_coarse_bin(const LS& s, int need, int& at_or_above) {
+    const int lane = threadIdx.x & 31;
+    const int* h = &s.thist[0][0];
+    int mine = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {                                               // (rotated: no bank conflicts)
+        const int4 v = reinterpret_cast<const int4*>(h)[lane * 8 + ((q + lane) & 7)];
+        mine += (v.x + v.y) + (v.z + v.w);
+    }
+    auto find = [&](int v, int want, int& above) -> int {                       // the lane in which the want-th from the top lies
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_down_sync(0xFFFFFFFFu, incl, o);
+            if (lane + o < 32) incl += u;
+        }
+        const unsigned hm = __ballot_sync(0xFFFFFFFFu, incl - v < want && want <= incl);
+        const int src = hm ? __ffs(hm) - 1 : 0;
+        above = __shfl_sync(0xFFFFFFFFu, incl - v, src);
+        return src;
+    };
+    int a0, a1;
+    const int l0 = find(mine, need, a0);
+    const int c = h[l0 * 32 + lane];
+    const int l1 = find(c, need - a0, a1);
+    at_or_above = a0 + a1 + __shfl_sync(0xFFFFFFFFu, c, l1);
+    return l0 * 32 + l1;
+}
+// Coarse bin of a path-value key: sixteen bins per factor of two, 1 at the top, everything below 2^-63 at the bottom.
+constexpr int kCoarseShift = 48, kCoarseBase = 16 * 0x3FF - 1023, kFineShift = kCoarseShift - 10;
+__device__ __forceinline__ int coarse_bin(unsigned long long key) {
+    const int e = (int)(key >> kCoarseShift) - kCoarseBase;
+    return e < 0 ? 0 : (e > 1023 ? 1023 : e);
+}
+
+// The fallback of team_pick: a radix select over the keys the team holds, key i of thread i % kTeam in s.keys[i] (N of them).
+// Returns this thread's taken keys as a mask (bit u: key u * kTeam + tt).
+template <class LS>
+__device__ __noinline__ unsigned pick_by_radix(int at, int N, int need, int tt) {
+    LS& s = smem_at<LS>(at);
+    const int lane = tt & 31, tw = tt >> 5;
+    team_sync();                                           // (keys written, the counts cleared)
+    unsigned long long thr;
+    int need_eq;
+    const int dirty = team_radix_select(s, [&](int i) { return s.keys[i]; }, N, need, tt, ~0ull, 0ull, thr, need_eq);
+    // ties at the threshold: lowest indices first
+    unsigned take = 0, tied = 0;
+    for (int u = 0; u * kTeam < N; ++u) {
+        const int i = u * kTeam + tt;
+        const unsigned long long key = i < N ? s.keys[i] : 0ull;
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, key == thr && key != 0ull);
+        if (lane == 0) s.pick[u * kTeamWarps + tw] = m;
+        take |= (key > thr ? 1u : 0u) << u;
+        tied |= ((m >> lane) & 1u) << u;
+    }
+    team_sync();
+    if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }
+    const int nm = (N + kTeam - 1) / kTeam * kTeamWarps;
+    int total;
+    const int base = warp_excl_scan(lane < nm ? __popc(s.pick[lane]) : 0, total);
+    for (int u = 0; u * kTeam < N; ++u) {
+        const int before = __shfl_sync(0xFFFFFFFFu, base, u * kTeamWarps + tw) + __popc(s.pick[u * kTeamWarps + tw] & ((1u << lane) - 1u));
+        if (((tied >> u) & 1u) && before < need_eq) take |= 1u << u;
+    }
+    team_sync();                                           // (s.pick may be written again)
+    return take;
+}
+
+// Selection among keys held in registers: thread tt of the team has key[u] of element i = u * kTeam + tt (0: not an element;
+// N <= kW * kTeam elements).  The `need` largest are taken, ties by lowest index (all of them when `all`).  Returns the mask of this
+// thread's taken keys; the elements taken before key[u] are picked_before(s, base, u, tt), all together `total`.
+// Bound by the latency of a chain of barriers, shared-memory accesses and shuffles, so there is one pass: the keys are counted into
+// coarse bins of their path values, the bin in which the threshold lies is listed (a
+// handful of keys) and the list is ranked.  A bin of more than kList keys (many equal path values, or values below 2^-63)
+// goes to a radix select over all.  A layer of 500 candidates takes 2.3 us from its last word to its last row sent out; with a radix
+// select over keys in shared memory and a compaction by contiguous stretches it took 3.9 to 9 (equal path values at the threshold).
+// Steps (B200, us, before / now): n = 50, V = 32000 132.9 / 118.0; n = 64, V = 128256 274.8 / 253.3; 32 sequences pruned 208.4 / 186.6.
+template <int kW, class LS>
+__device__ __forceinline__ unsigned team_pick(LS& s, const unsigned long long (&key)[kW], int N, int need, bool all, int tt, int& total, int& base) {
+    static_assert(kW * kTeamWarps <= 32, "one lane scans one ballot");
+    const int lane = tt & 31, tw = tt >> 5;
+    unsigned take = 0;
+    if (all) {
+#pragma unroll
+        for (int u = 0; u < kW; ++u) take |= (key[u] != 0ull ? 1u : 0u) << u;
+    } else {
+        int* coarse = &s.thist[0][0];
+        if (tt == 0) s.listn = 0;
+#pragma unroll
+        for (int u = 0; u < kW; ++u) if (key[u]) atomicAdd(&coarse[coarse_bin(key[u])], 1);
+        team_sync();
+        int S;
+        const int bin = warp_coarse_bin(s, need, S);
+        const int left = need - (S - coarse[bin]);         // of the bin's keys
+        const unsigned long long low = bin > 0 ? (unsigned long long)(bin + kCoarseBase) << kCoarseShift : 1ull;
+        const unsigned long long high = bin < 1023 ? (unsigned long long)(bin + 1 + kCoarseBase) << kCoarseShift : ~0ull;
+        unsigned mid = 0;
+        unsigned long long where = 0ull;                   // a byte per key: its place in the list
+#pragma unroll
+        for (int u = 0; u < kW; ++u) {
+            if (key[u] >= high) take |= 1u << u;
+            else if (key[u] >= low) {
+                const int q = atomicAdd(&s.listn, 1);
+                if (q < LS::kList) { s.list[q] = key[u]; s.listi[q] = u * kTeam + tt; where |= (unsigned long long)q << (8 * u); }
+                mid |= 1u << u;
+            }
+        }
+        team_sync();
+#pragma unroll
+        for (int q = 0; q < 1024 / (4 * kTeam); ++q) reinterpret_cast<int4*>(coarse)[q * kTeam + tt] = make_int4(0, 0, 0, 0);   // (every warp has its bin)
+        const int L = s.listn;
+        if (L <= left) {
+            take |= mid;
+        } else if (L <= LS::kList) {
+            const unsigned long long a = lane < L ? s.list[lane] : 0ull, b = lane + 32 < L ? s.list[lane + 32] : 0ull;
+            const int ia = lane < L ? s.listi[lane] : 0, ib = lane + 32 < L ? s.listi[lane + 32] : 0;
+            int ra = 0, rb = 0;                            // listed elements that come before this lane's two
+            #pragma unroll 2
+            for (int e = 0; e < L; ++e) {
+                const unsigned long long x = s.list[e];
+                const int xi = s.listi[e];
+                ra += x > a || (x == a && xi < ia) ? 1 : 0;
+                rb += x > b || (x == b && xi < ib) ? 1 : 0;
+            }
+            const unsigned ma = __ballot_sync(0xFFFFFFFFu, lane < L && ra < left), mb = __ballot_sync(0xFFFFFFFFu, lane + 32 < L && rb < left);
+#pragma unroll
+            for (int u = 0; u < kW; ++u) {
+                const int q = (int)(where >> (8 * u)) & 255;
+                if (((mid >> u) & 1u) && (((q < 32 ? ma : mb) >> (q & 31)) & 1u)) take |= 1u << u;
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < kW; ++u) { const int i = u * kTeam + tt; if (i < N) s.keys[i] = key[u]; }
+            take = pick_by_radix<LS>(smem_offset(&s), N, need, tt);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kW; ++u) {
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, (take >> u) & 1u);
+        if (lane == 0) s.pick[u * kTeamWarps + tw] = m;
+    }
+    team_sync();
+    base = warp_excl_scan(lane < kW * kTeamWarps ? __popc(s.pick[lane]) : 0, total);
+    return take;
+}
+template <class LS>
+__device__ __forceinline__ int picked_before(const LS& s, int base, int u, int tt) {       // (whole warp)
+    const int m = u * kTeamWarps + (tt >> 5);
+    return __shfl_sync(0xFFFFFFFFu, base, m) + __popc(s.pick[m] & ((1u << (tt & 31)) - 1u));
+}
+
+// Sends out a node of layer d of sequence b as frontier row `row` of layer d + 1 (row g0 + row of the build's running count).
+__device__ __forceinline__ void publish_node(const RowQueue& q, int b, int d, unsigned g0, int row, int token, unsigned long long key, int* status) {
+    if (token < 0 || token >= q.V) { set_status(status, kErrInternal); token = 0; }
+    const unsigned g = g0 + (unsigned)row, e = q.by_grid.div(g), c = g - e * q.by_grid.d;
+    if (e < (unsigned)q.mcap) {
+        const unsigned pos = c * (unsigned)q.mcap + e;     // (below 2^31: opt_tree_create)
+        st_relaxed_u64(&q.phat[pos], (1ull << 63) | (key - 1ull));
+        st_relaxed_u64(&q.items[pos], item_encode(b, d + 1, row, (int)q.by_H.mod((unsigned)token * (unsigned)kRowMul + (unsigned)d)));
+    } else {
+        set_status(status, kErrInternal);
+    }
+}
+
+// An entry of a reservation that is not needed.
+__device__ __forceinline__ void void_entry(const RowQueue& q, unsigned g, int* status) {
+    const unsigned e = q.by_grid.div(g), c = g - e * q.by_grid.d;
+    if (e < (unsigned)q.mcap) {
+        const unsigned pos = c * (unsigned)q.mcap + e;
+        st_relaxed_u64(&q.phat[pos], 1ull << 63);
+        st_relaxed_u64(&q.items[pos], (1ull << 63) | kItemVoid);
+    } else {
+        set_status(status, kErrInternal);
+    }
+}
+
+// The team's part of a layer selection (N = fsize * k <= kW * kTeam): the new layer's nodes go to T, their tokens and keys to
+// s.ltok / s.lkeys, and, when the job says so, their rows out (g0, the layer warp's, numbers them).  Returns nl after a last barrier.
+// It starts while the layer's rows are still being finished and waits for the candidate words themselves.
+template <int kW, class LS>
+__device__ __noinline__ int select_layer_team(int at, int tt, unsigned g0, int* status) {
     LS& s = smem_at<LS>(at);
     const LayerJob& j = s.job;
-    const int k = j.k;
-    int32_t *const T_tok = j.T_tok, *const T_par = j.T_par;
-    double* const T_phat = j.T_phat;
-    const int32_t* const fmap = j.fmap;
-    const int lane = threadIdx.x & 31, tw = tt >> 5;
-    const int N = j.fsize * k;
-    const int nvalid = j.fsize * j.kk;
-    const int nl = nvalid < j.n ? nvalid : j.n;
-    const int gid0 = (j.d - 1) * j.n;
-    double* const cand_phat = j.cand_phat;
-    int32_t* const cand_tok = j.cand_tok;
-    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(cand_phat);
-    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(cand_tok);
-    unsigned long long ko = 0ull, ka = ~0ull;
-    if (N > kTeam) sweep_candidates<4>(s, gph, gtk, N, tt, ko, ka, status);
-    else if (tt < N) {                                     // staged (see stage_layer_candidates); what was missing is read again (bounded)
-        unsigned long long x = s.keys[tt];
-        if (!(x >> 63)) x = poll_phat_word(&gph[tt], status);
-        unsigned int t32 = (unsigned int)s.toks[tt];
-        if (!(t32 >> 31)) { t32 = poll_tok_word(&gtk[tt], status); s.toks[tt] = (int)t32; }
-        const unsigned long long key = key_of_word(x);
-        s.keys[tt] = key;
-        if (key) ko = ka = key;
-    }
-    ko = warp_or_u64(ko); ka = warp_and_u64(ka);
-    if (lane == 0) { s.red_or[tw] = ko; s.red_and[tw] = ka; }
-    team_sync();
-    ko = 0ull; ka = ~0ull;
+    const int N = j.fsize * j.k, nvalid = j.fsize * j.kk, nl = nvalid < j.n ? nvalid : j.n, gid0 = (j.d - 1) * j.n;
+    unsigned long long x[kW];
+    unsigned int t32[kW];
+    sweep_candidates<kW>(reinterpret_cast<const unsigned long long*>(j.cand_phat), reinterpret_cast<const unsigned int*>(j.cand_tok), N, tt, x, t32, status);
 #pragma unroll
-    for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
-    unsigned long long thr = 0ull;                         // with no more candidates than wanted, all of them (key > 0) are taken
-    int need_eq = 0, dirty = -1;
-    auto staged = [&](int i) { return s.keys[i]; };
-    if (nl < nvalid) dirty = team_radix_select(s, staged, N, nl, tt, ko, ka, thr, need_eq);
-    // ordered compaction: thread tt owns a contiguous stretch of candidates
-    const int per = (N + kTeam - 1) / kTeam;
-    const int lo = min(tt * per, N), hi = min(lo + per, N);
-    int gt = 0, eq = 0;
-    #pragma unroll 1
-    for (int i = lo; i < hi; ++i) {
-        const unsigned long long key = s.keys[i];
-        gt += key > thr ? 1 : 0;
-        eq += key == thr ? 1 : 0;
-    }
-    int total_eq, total;
-    int eq_take = 0;
-    if (need_eq > 0) {                                     // (the same for all warps) ties at the threshold: lowest indices first
-        const int eq_before = team_excl_scan(eq, s.scan_a, tw, total_eq);
-        eq_take = need_eq - eq_before;
-        eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
-    }
-    int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
-    if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }     // everyone is past the last pass
-    int frow = lo / k, frank = lo - frow * k;          // frontier row and sibling rank of candidate i, carried along
-    #pragma unroll 1
-    for (int i = lo; i < hi; ++i) {
-        const unsigned long long key = s.keys[i];
-        bool take = key > thr;
-        if (key == thr && eq_take > 0) { take = true; --eq_take; }
-        if (take) {
-            const unsigned int t32 = (unsigned int)s.toks[i];
-            const int tok = t32 == ~0u ? -1 : (int)(t32 & 0x7FFFFFFFu);
-            T_tok[gid0 + pos] = tok;
-            s.ltok[pos] = tok;
-            T_par[gid0 + pos] = kPrune ? __ldcg(&fmap[frow]) : frow;
-            T_phat[gid0 + pos] = __longlong_as_double((long long)(key - 1ull));
-            s.lkeys[pos] = key;
-            ++pos;
+    for (int u = 0; u < kW; ++u) x[u] = key_of_word(x[u]);
+    if (tt == 0) s.job.g0 = g0;
+    int total, base;
+    const unsigned take = team_pick<kW>(s, x, N, nl, nl >= nvalid, tt, total, base);
+#pragma unroll
+    for (int u = 0; u < kW; ++u) {
+        if (u * kTeam >= N) break;
+        const int pos = picked_before(s, base, u, tt);
+        if ((take >> u) & 1u) {
+            s.ltok[pos] = t32[u] == ~0u ? -1 : (int)(t32[u] & 0x7FFFFFFFu);
+            s.lkeys[pos] = x[u];
+            s.toks[pos] = u * kTeam + tt;
         }
-        if (++frank == k) { frank = 0; ++frow; }
     }
-    if (total != nl) set_status(status, kErrInternal);
+    if (tt == 0 && total != nl) set_status(status, kErrInternal);
+    team_sync();
+    // (a node per thread from here on: with each taken candidate handled where it was found, up to kW of them one after the other
+    // in a warp, this took 2.1 us for 500 candidates and 4 for 1024)
+    g0 = s.job.g0;
+    #pragma unroll 1
+    for (int i = tt; i < nl; i += kTeam) {
+        const int tok = s.ltok[i], gid = gid0 + i;
+        const unsigned long long key = s.lkeys[i];
+        if (j.publish) publish_node(j.queue, j.b, j.d, g0, i, tok, key, status);
+        const int frow = (int)j.by_k.div((unsigned)s.toks[i]);
+        j.T_tok[gid] = tok;
+        j.T_par[gid] = j.fmap ? __ldcg(&j.fmap[frow]) : frow;
+        j.T_phat[gid] = __longlong_as_double((long long)(key - 1ull));
+    }
     team_sync();
     return nl;
 }
 
-// Pruned draft, both halves of a layer job in one selection: the new running top-n is the n largest
-// of the old one and the layer's candidates together (what a candidate outside them could add to T
-// can never matter, see opt_tree_build_pruned).  s.keys[0..nR_old) / s.gids[0..nR_old) hold the old
-// top-n (keys, gids ascending), s.keys[off..off+N) the staged candidate words (entries between are 0).
-// Array order is tie order (shallower first, then candidate index).  On return s.rsel / s.vals hold
-// the new top-n (gids ascending; also written to j.Rnew), its new members are T's nodes
-// gid0 .. gid0+cnt in candidate order with tokens and keys in s.ltok / s.lkeys, and s.scan_c sums
-// to the number of old members kept.  Returns |new top-n|.
+// Key of member i of the running top-n, and its gid.
 template <class LS>
-__device__ __noinline__ int select_running_team(int at, int tt, int* status) {
+__device__ __forceinline__ unsigned long long running_key(const LS& s, const LayerJob& j, int i, int& gid) {
+    if (j.cached) { gid = s.rsel[i]; return phat_key(s.vals[i]); }
+    gid = __ldcg(&j.Rold[i]);
+    return phat_key(__ldcg(&j.T_phat[gid]));
+}
+
+// Pruned draft, and the layer at the depth limit: both halves of a layer job in one selection: the new running top-n is the n largest
+// of the old one and the layer's candidates together (what a candidate outside them could add to T
+// can never matter, see opt_tree_build_pruned).  Elements 0 .. nR_old are the old top-n (gids ascending), off .. off+N the
+// candidate words.  Their order is tie order (shallower first, then candidate index).  On return s.rsel / s.vals hold
+// the new top-n (gids ascending; also written to j.Rnew), its new members are T's nodes
+// gid0 .. gid0+cnt in candidate order, and s.kept_old is the number of old members kept.  When the job says so the new members' rows
+// are sent out (as frontier rows 0 .. cnt, left in fmap) and the rest of the reservation voided.  Returns |new top-n|.
+template <int kW, class LS>
+__device__ __noinline__ int select_running_team(int at, int tt, unsigned g0, int* status) {
     LS& s = smem_at<LS>(at);
     const LayerJob& j = s.job;
-    const int k = j.k;
-    int32_t *const T_tok = j.T_tok, *const T_par = j.T_par, *const Rnew = j.Rnew;
-    double* const T_phat = j.T_phat;
-    const int32_t* const fmap = j.fmap;
-    const int lane = threadIdx.x & 31, tw = tt >> 5;
-    const int N = j.fsize * k, nRo = j.nR_old, off = j.off, M = off + N;
-    const int nvalid = j.fsize * j.kk;
-    const int need = nRo + nvalid < j.n ? nRo + nvalid : j.n;
-    const int gid0 = (j.d - 1) * j.n;
-    double* const cand_phat = j.cand_phat;
-    int32_t* const cand_tok = j.cand_tok;
-    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(cand_phat);
-    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(cand_tok);
-    unsigned long long ko = 0ull, ka = ~0ull;
-    #pragma unroll 1
-    for (int i = tt; i < M; i += kTeam) {
-        unsigned long long key;
-        if (i >= off) {
-            unsigned long long x = s.keys[i];
-            if (!(x >> 63)) x = poll_phat_word(&gph[i - off], status);
-            key = key_of_word(x);
-            s.keys[i] = key;
-            unsigned int t32 = (unsigned int)s.toks[i - off];
-            if (!(t32 >> 31)) { t32 = poll_tok_word(&gtk[i - off], status); s.toks[i - off] = (int)t32; }
-        } else {
-            key = i < nRo ? s.keys[i] : 0ull;
-            if (i >= nRo) s.keys[i] = 0ull;
-        }
-        if (key) { ko |= key; ka &= key; }
-    }
-    ko = warp_or_u64(ko); ka = warp_and_u64(ka);
-    if (lane == 0) { s.red_or[tw] = ko; s.red_and[tw] = ka; }
-    team_sync();
-    ko = 0ull; ka = ~0ull;
+    const int N = j.fsize * j.k, nRo = j.nR_old, off = j.off, M = off + N;
+    const int nvalid = j.fsize * j.kk, need = nRo + nvalid < j.n ? nRo + nvalid : j.n, gid0 = (j.d - 1) * j.n;
+    const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(j.cand_phat) - off;
+    const unsigned int* gtk = reinterpret_cast<const unsigned int*>(j.cand_tok) - off;
+    unsigned long long x[kW];
+    unsigned int t32[kW];                                  // candidates: token word; old members: gid
 #pragma unroll
-    for (int q = 0; q < kTeamWarps; ++q) { ko |= s.red_or[q]; ka &= s.red_and[q]; }
-    clear_candidates(cand_phat, cand_tok, N, tt, kTeam);
-    unsigned long long thr = 0ull;
-    int need_eq = 0, dirty = -1;
-    auto staged = [&](int i) { return s.keys[i]; };
-    if (need < nRo + nvalid) dirty = team_radix_select(s, staged, M, need, tt, ko, ka, thr, need_eq);
-    const int per = (M + kTeam - 1) / kTeam;
-    const int lo = min(tt * per, M), hi = min(lo + per, M);
-    int gt = 0, eq = 0;
+    for (int u = 0; u < kW; ++u) {
+        const int i = u * kTeam + tt;
+        x[u] = ~0ull; t32[u] = ~0u;
+        if (i >= off && i < M) { x[u] = ld_relaxed_u64(&gph[i]); t32[u] = ld_relaxed_u32(&gtk[i]); }
+    }
     #pragma unroll 1
-    for (int i = lo; i < hi; ++i) {
-        const unsigned long long key = s.keys[i];
-        gt += key > thr ? 1 : 0;
-        eq += (key == thr && key != 0ull) ? 1 : 0;
-    }
-    int total_eq, total;
-    int eq_take = 0;
-    if (need_eq > 0) {
-        const int eq_before = team_excl_scan(eq, s.scan_a, tw, total_eq);
-        eq_take = need_eq - eq_before;
-        eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
-    }
-    // old members kept: counted per thread, summed over the team along with the scan below
-    int kept_mine = 0;
-    {
-        int e = eq_take;
-        #pragma unroll 1
-        for (int i = lo; i < hi && i < nRo; ++i) {
-            const unsigned long long key = s.keys[i];
-            bool take = key > thr;
-            if (key == thr && key != 0ull && e > 0) { take = true; --e; }
-            kept_mine += take ? 1 : 0;
-        }
-    }
-    kept_mine = __reduce_add_sync(0xFFFFFFFFu, kept_mine);
-    if (lane == 0) s.scan_c[tw] = kept_mine;
-    int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);       // (its barrier also publishes scan_c)
-    if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }
-    int kept_old = 0;
+    for (int t = 0;; ++t) {
+        bool missing = false;
 #pragma unroll
-    for (int q = 0; q < kTeamWarps; ++q) kept_old += s.scan_c[q];
-    #pragma unroll 1
-    for (int i = lo; i < hi; ++i) {
-        const unsigned long long key = s.keys[i];
-        bool take = key > thr;
-        if (key == thr && key != 0ull && eq_take > 0) { take = true; --eq_take; }
-        if (!take) continue;
-        int gid;
-        if (i < nRo) {
-            gid = s.gids[i];
-        } else {
-            const int c = i - off, slot = pos - kept_old;
-            const unsigned int t32 = (unsigned int)s.toks[c];
-            const int tok = t32 == ~0u ? -1 : (int)(t32 & 0x7FFFFFFFu);
-            gid = gid0 + slot;
-            T_tok[gid] = tok;
-            T_par[gid] = __ldcg(&fmap[c / k]);      // layer slot of the node behind the candidate's frontier row
-            T_phat[gid] = __longlong_as_double((long long)(key - 1ull));
-            s.ltok[slot] = tok;
-            s.lkeys[slot] = key;
+        for (int u = 0; u < kW; ++u) {
+            const int i = u * kTeam + tt;
+            if (!(x[u] >> 63)) { x[u] = ld_relaxed_u64(&gph[i]); missing = missing || !(x[u] >> 63); }
+            if (!(t32[u] >> 31)) { t32[u] = ld_relaxed_u32(&gtk[i]); missing = missing || !(t32[u] >> 31); }
         }
-        s.rsel[pos] = gid;
-        s.vals[pos] = __longlong_as_double((long long)(key - 1ull));
-        Rnew[pos] = gid;
-        ++pos;
+        if (!__any_sync(0xFFFFFFFFu, missing)) break;
+        __nanosleep(20);
+        if (t >= kWaitPolls) {
+            set_status(status, kErrTimeout);
+#pragma unroll
+            for (int u = 0; u < kW; ++u) { if (!(x[u] >> 63)) x[u] = ~0ull; if (!(t32[u] >> 31)) t32[u] = ~0u; }
+            break;
+        }
     }
-    if (total != need) set_status(status, kErrInternal);
+#pragma unroll
+    for (int u = 0; u < kW; ++u) {
+        const int i = u * kTeam + tt;
+        x[u] = key_of_word(x[u]);
+        if (i < nRo) { int gid; x[u] = running_key(s, j, i, gid); t32[u] = (unsigned)gid; }
+    }
+    if (tt == 0) s.job.g0 = g0;
+    int total, base;
+    const unsigned take = team_pick<kW>(s, x, M, need, nRo + nvalid <= j.n, tt, total, base);
+    const int kept_old = __shfl_sync(0xFFFFFFFFu, base, off / 32);         // taken before element `off`
+    if (tt == 0) s.kept_old = kept_old;
+#pragma unroll
+    for (int u = 0; u < kW; ++u) {
+        const int i = u * kTeam + tt;
+        if (u * kTeam >= M) break;
+        const int pos = picked_before(s, base, u, tt);
+        if ((take >> u) & 1u) {
+            if (i >= off) {
+                const int slot = pos - kept_old;
+                s.ltok[slot] = t32[u] == ~0u ? -1 : (int)(t32[u] & 0x7FFFFFFFu);
+                s.lkeys[slot] = x[u];
+                s.toks[slot] = i - off;
+            }
+            s.rsel[pos] = i < off ? (int)t32[u] : gid0 + pos - kept_old;
+            s.vals[pos] = __longlong_as_double((long long)(x[u] - 1ull));
+        }
+    }
+    if (tt == 0 && total != need) set_status(status, kErrInternal);
     team_sync();
+    const int cnt = total - kept_old, reserve = j.publish ? (nvalid < j.n ? nvalid : j.n) : cnt;
+    g0 = s.job.g0;
+    #pragma unroll 1
+    for (int i = tt; i < reserve; i += kTeam) {
+        if (i >= cnt) { void_entry(j.queue, g0 + (unsigned)i, status); continue; }
+        const int tok = s.ltok[i], gid = gid0 + i;
+        const unsigned long long key = s.lkeys[i];
+        if (j.publish) publish_node(j.queue, j.b, j.d, g0, i, tok, key, status);
+        j.T_tok[gid] = tok;
+        j.T_par[gid] = __ldcg(&j.fmap[j.by_k.div((unsigned)s.toks[i])]);       // layer slot of the node behind the candidate's frontier row
+        j.T_phat[gid] = __longlong_as_double((long long)(key - 1ull));
+    }
+    #pragma unroll 1
+    for (int i = tt; i < need; i += kTeam) j.Rnew[i] = s.rsel[i];
+    clear_candidates(j.cand_phat, j.cand_tok, N, tt, kTeam);
+    team_sync();
+    if (j.publish) for (int i = tt; i < cnt; i += kTeam) j.fmap[i] = i;    // (read above)
     return need;
 }
 
@@ -483,41 +594,6 @@ __device__ __noinline__ int team_select_global(int at, const unsigned long long*
     return total;
 }
 
-// The largest bin of the 1024 counts in s.thist at which at least `need` elements lie at or above; `at_or_above` is their
-// number (the elements must be that many).  Every warp for itself.
-template <class LS>
-__device__ __forceinline__ int warp_coarse_bin(const LS& s, int need, int& at_or_above) {
-    const int lane = threadIdx.x & 31;
-    const int* h = &s.thist[0][0];
-    int mine = 0;
-#pragma unroll 8
-    for (int q = 0; q < 32; ++q) mine += h[lane * 32 + ((q + lane) & 31)];     // (rotated: no bank conflicts)
-    auto find = [&](int v, int want, int& above) -> int {                       // the lane in which the want-th from the top lies
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_down_sync(0xFFFFFFFFu, incl, o);
-            if (lane + o < 32) incl += u;
-        }
-        const unsigned hm = __ballot_sync(0xFFFFFFFFu, incl - v < want && want <= incl);
-        const int src = hm ? __ffs(hm) - 1 : 0;
-        above = __shfl_sync(0xFFFFFFFFu, incl - v, src);
-        return src;
-    };
-    int a0, a1;
-    const int l0 = find(mine, need, a0);
-    const int c = h[l0 * 32 + lane];
-    const int l1 = find(c, need - a0, a1);
-    at_or_above = a0 + a1 + __shfl_sync(0xFFFFFFFFu, c, l1);
-    return l0 * 32 + l1;
-}
-// Coarse bin of a path-value key: sixteen bins per factor of two, 1 at the top, everything below 2^-63 at the bottom.
-constexpr int kCoarseShift = 48, kCoarseBase = 16 * 0x3FF - 1023, kFineShift = kCoarseShift - 10;
-__device__ __forceinline__ int coarse_bin(unsigned long long key) {
-    const int e = (int)(key >> kCoarseShift) - kCoarseBase;
-    return e < 0 ? 0 : (e > 1023 ? 1023 : e);
-}
-
 // The team's selection for layers with more candidates than the shared-memory staging holds
 // (kStageCap < N <= n*k).  Bound by the round trips of 128 threads to the candidate words in L2 (8192 of them take 3 us,
 // 6 with their counting), so there are two sweeps and no more: the first counts the candidates into coarse bins of their path
@@ -527,7 +603,7 @@ __device__ __forceinline__ int coarse_bin(unsigned long long key) {
 // 2^-63 make that useless too, or a warp's segment overflows, further sweeps read global memory once per digit.)
 // Measured (two sequences, n = 512, k = 16, B200): 1059 us per step with a sweep per digit and tokens fetched one by one, 452
 // with bit marks, a gather and a radix select after the second sweep, 431 with the segments.
-template <bool kPrune, class LS>
+template <class LS>
 __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
     LS& s = smem_at<LS>(at);
     const LayerJob& j = s.job;
@@ -715,7 +791,7 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
             const int tok = t32[u] == ~0u ? -1 : (int)(t32[u] & 0x7FFFFFFFu);
             const int frow = c[u] / k;
             T_tok[gid0 + i] = tok;
-            T_par[gid0 + i] = kPrune ? __ldcg(&fmap[frow]) : frow;
+            T_par[gid0 + i] = fmap ? __ldcg(&fmap[frow]) : frow;
             T_phat[gid0 + i] = __longlong_as_double((long long)(s.lkeys[i] - 1ull));
             s.ltok[i] = tok;
         }
@@ -723,6 +799,21 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
     if (total != nl) set_status(status, kErrInternal);
     team_sync();
     return nl;
+}
+
+// A layer job's selection (kind 1) and the one over the running top-n and the candidates together (kind 2), by size.
+template <class LS>
+__device__ __forceinline__ void select_job(int at, int tt, unsigned g0, int* status) {
+    const LayerJob& j = smem_at<LS>(at).job;
+    const int N = j.fsize * j.k;
+    if (N <= 4 * kTeam) select_layer_team<4, LS>(at, tt, g0, status);
+    else if (N <= kStageCap) select_layer_team<8, LS>(at, tt, g0, status);
+    else select_layer_team_big<LS>(at, tt, status);
+}
+template <class LS>
+__device__ __forceinline__ int running_job(int at, int tt, unsigned g0, int* status) {
+    const LayerJob& j = smem_at<LS>(at).job;
+    return j.off + j.fsize * j.k <= 4 * kTeam ? select_running_team<4, LS>(at, tt, g0, status) : select_running_team<8, LS>(at, tt, g0, status);
 }
 
 // Once per sequence, when it is finished: T_opt = the running top-n (s.rsel / s.vals, already in
@@ -769,18 +860,47 @@ __device__ __forceinline__ double running_esub(const LS& s, int nR) {
     return warp_sum(part);
 }
 
-// Layer job, second half: the running top-n and E_sub(T, n) with the new layer (j.fsize nodes, left in s by the
-// selection), by the team: a radix select over the keys of the old top-n and the layer.  j.off: s.rsel / s.vals still
-// hold the old one (else it is read from j.Rold).  On return s.rsel / s.vals hold the new one (ascending gids; also
-// written to j.Rnew); returns |R|.
+// Layer job, second half: the running top-n with the new layer (j.fsize nodes, left in s by the selection): the n largest of the
+// old one and the layer.  j.cached: s.rsel / s.vals still hold the old one (else it is read from j.Rold).  On return s.rsel / s.vals
+// hold the new one (ascending gids; also written to j.Rnew); returns |R|.  Clears the layer's candidate words on the way.
+template <int kW, class LS>
+__device__ __forceinline__ int update_running(LS& s, int tt, int* status) {
+    const LayerJob& j = s.job;
+    clear_candidates(j.cand_phat, j.cand_tok, j.ncand, tt, kTeam);
+    const int nRo = j.nR_old, NR = nRo + j.fsize, need = NR < j.n ? NR : j.n, gid0 = (j.d - 1) * j.n;
+    unsigned long long key[kW];
+    int gid[kW];
+#pragma unroll
+    for (int u = 0; u < kW; ++u) {
+        const int i = u * kTeam + tt;
+        key[u] = 0ull; gid[u] = 0;
+        if (i >= NR) continue;
+        if (i < nRo) key[u] = running_key(s, j, i, gid[u]);
+        else { gid[u] = gid0 + (i - nRo); key[u] = s.lkeys[i - nRo]; }
+    }
+    int total, base;
+    const unsigned take = team_pick<kW>(s, key, NR, need, NR <= j.n, tt, total, base);
+#pragma unroll
+    for (int u = 0; u < kW; ++u) {
+        if (u * kTeam >= NR) break;
+        const int pos = picked_before(s, base, u, tt);
+        if ((take >> u) & 1u) {
+            j.Rnew[pos] = gid[u];
+            s.rsel[pos] = gid[u];
+            s.vals[pos] = __longlong_as_double((long long)(key[u] - 1ull));
+        }
+    }
+    if (tt == 0 && total != need) set_status(status, kErrInternal);
+    team_sync();
+    return need;
+}
+
+// The same with the keys in shared memory, for more of them than the team holds in registers (node budgets beyond 512).
 template <class LS>
-__device__ __noinline__ int update_running_team(int at, int tt, int* status) {
+__device__ __noinline__ int update_running_staged(int at, int tt, int* status) {
     LS& s = smem_at<LS>(at);
     const LayerJob& j = s.job;
     clear_candidates(j.cand_phat, j.cand_tok, j.ncand, tt, kTeam);
-    const bool cached = j.off != 0;
-    const int32_t* const Rold = j.Rold;
-    const double* const T_phat = j.T_phat;
     int32_t* const Rnew = j.Rnew;
     const int lane = tt & 31, tw = tt >> 5;
     const int nRo = j.nR_old, NR = nRo + j.fsize, need = NR < j.n ? NR : j.n, gid0 = (j.d - 1) * j.n;
@@ -790,8 +910,7 @@ __device__ __noinline__ int update_running_team(int at, int tt, int* status) {
         int gid;
         unsigned long long key;
         if (i >= nRo) { gid = gid0 + (i - nRo); key = s.lkeys[i - nRo]; }
-        else if (cached) { gid = s.rsel[i]; key = phat_key(s.vals[i]); }
-        else { gid = __ldcg(&Rold[i]); key = phat_key(__ldcg(&T_phat[gid])); }
+        else key = running_key(s, j, i, gid);
         s.gids[i] = gid;
         s.keys[i] = key;
         ko |= key; ka &= key;
@@ -832,6 +951,15 @@ __device__ __noinline__ int update_running_team(int at, int tt, int* status) {
     if (total != need) set_status(status, kErrInternal);
     team_sync();
     return need;
+}
+
+template <class LS>
+__device__ __noinline__ int update_running_team(int at, int tt, int* status) {
+    LS& s = smem_at<LS>(at);
+    const int NR = s.job.nR_old + s.job.fsize;
+    if (NR <= 4 * kTeam) return update_running<4>(s, tt, status);
+    if (LS::kBudget > 2 * kTeam && NR <= 8 * kTeam) return update_running<8>(s, tt, status);
+    return update_running_staged<LS>(at, tt, status);
 }
 
 }  // namespace ot
