@@ -43,7 +43,7 @@ constexpr int kDescRing = 16;                      // descriptors kept: a row's 
 // short rows do without (in one kernel for all, the row step on 32000 logits was 3 to 7 % slower, a build of 32
 // sequences 4 %).
 constexpr int kLongRow = 2 * kChunkElems;          // rows up to this many logits are short
-constexpr int kFinLoads = 8;                       // long rows: vectors a finisher lane has in flight
+constexpr int kFinLoads = 8;                       // long rows: vectors a finisher lane has in flight (unaligned: half as many, of two granules)
 constexpr int kLaneTauMaxK = 16;                   // largest k for which the finisher's threshold comes from the lane maxima
 constexpr int kPerLane = kConsumers / 32;          // per-thread results one finisher lane handles (16)
 
@@ -497,12 +497,14 @@ __device__ __noinline__ void row_exact_warp(FinScratch& f, const uint16_t* row, 
     S_out = warp_sum(acc);
 }
 
+// Whether the two granules that hold vector vi of an unaligned row lie within the row.
+__device__ __forceinline__ bool granules_inside(int vi, int V) { return vi >= 1 && vi * 8 + 16 <= V; }
 // One 16-byte vector of the row (8 logits starting at token 8*vi) as four packed words; logits at or
 // beyond V read as -inf.  Aligned rows take one vector load, others the two granules that hold the vector, or, at
 // either end of the row, where those may reach beyond the table, eight scalar loads.
 __device__ __noinline__ uint4 load_row_vec_unaligned(const uint16_t* row, int vi, int V) {
     const uint16_t* p = row + (size_t)vi * 8;
-    if (vi >= 1 && vi * 8 + 16 <= V) {
+    if (granules_inside(vi, V)) {
         const int o = vec_offset(p);
         const uint4* q = reinterpret_cast<const uint4*>(p - o);
         const uint4 a = __ldg(q), b = __ldg(q + 1);
@@ -511,6 +513,29 @@ __device__ __noinline__ uint4 load_row_vec_unaligned(const uint16_t* row, int vi
     uint32_t h[8];
     for (int e = 0; e < 8; ++e) h[e] = (vi * 8 + e < V) ? (uint32_t)__ldg(p + e) : 0xFF80u;
     return make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+}
+// The granules of vector vi (o: vec_offset(row)).
+__device__ __forceinline__ void load_granules(const uint16_t* row, int o, int vi, uint4& a, uint4& b) {
+    const uint4* q = reinterpret_cast<const uint4*>(row - o) + vi;
+    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "l"(q));
+    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(q + 1));
+}
+// The vectors vi[0 .. kN) of an unaligned row (negative: none, reads as -inf), all granules in flight together.  (One call of
+// load_row_vec after the other waits for each; steps of 16 sequences of n = 48, V = 32003, 154.0 us with calls, 148.5 now.)
+template <int kN>
+__device__ __forceinline__ void load_vecs_unaligned(uint4 (&w)[kN], const int (&vi)[kN], const uint16_t* row, int V) {
+    const int o = vec_offset(row);
+    uint4 b[kN];
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+        w[u] = b[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+        if (vi[u] >= 0 && granules_inside(vi[u], V)) load_granules(row, o, vi[u], w[u], b[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kN; ++u) w[u] = shift_halves(w[u], b[u], o);
+#pragma unroll
+    for (int u = 0; u < kN; ++u)
+        if (vi[u] >= 0 && !granules_inside(vi[u], V)) w[u] = load_row_vec_unaligned(row, vi[u], V);
 }
 template <bool kAligned>
 __device__ __forceinline__ uint4 load_row_vec(const uint16_t* row, int vi, int V) {
@@ -567,6 +592,7 @@ __device__ __noinline__ void finish_many(FinScratch& f, int M, int kk, double m,
 template <bool kAligned>
 __device__ __forceinline__ float find_candidates_long(FinScratch& f, const uint16_t* tkey, const uint16_t* row, int V, int kk, int nflag, float negE,
                                                       uint32_t& tau_key) {
+    constexpr int kLoads = kAligned ? kFinLoads : kFinLoads / 2;
     const int lane = threadIdx.x & 31;
     const int nvec = (V + 7) >> 3, nchunks = (V + kChunkElems - 1) / kChunkElems, vpt = nchunks * kVecPerThread;
     if (kk <= kLaneTauMaxK && nflag > kk) {
@@ -598,20 +624,23 @@ __device__ __forceinline__ float find_candidates_long(FinScratch& f, const uint1
     };
     float sub = 0.0f;
 #pragma unroll 1
-    for (int i0 = lane; i0 - lane < total; i0 += 32 * kFinLoads) {
-        uint4 w[kFinLoads];
+    for (int i0 = lane; i0 - lane < total; i0 += 32 * kLoads) {
+        uint4 w[kLoads];
+        int vis[kLoads];
 #pragma unroll
-        for (int u = 0; u < kFinLoads; ++u) {
+        for (int u = 0; u < kLoads; ++u) {
             const int idx = i0 + u * 32;
-            w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+            if (kAligned) w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+            vis[u] = -1;
             if (idx < total) {
                 const int vi = vector_of(idx);
-                if (vi < nvec) w[u] = load_row_vec<kAligned>(row, vi, V);
+                if (vi < nvec) { vis[u] = vi; if (kAligned) w[u] = load_row_vec<true>(row, vi, V); }
             }
         }
+        if (!kAligned) load_vecs_unaligned(w, vis, row, V);
         uint32_t hits = 0;                                  // bit u: vector u holds a candidate
 #pragma unroll
-        for (int u = 0; u < kFinLoads; ++u)
+        for (int u = 0; u < kLoads; ++u)
             hits |= (ge_bf16x2(max_bf16x2(max_bf16x2(w[u].x, w[u].y), max_bf16x2(w[u].z, w[u].w)), tau_b2) ? 1u : 0u) << u;
 #pragma unroll 1
         for (; hits; hits &= hits - 1) {
@@ -743,12 +772,13 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
                 const int idx = i0 + u * 32 + lane;
                 const int fi = idx & ((1 << lg) - 1), j = idx >> lg;
                 vis[u] = -1;
-                w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+                if (kAligned) w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
                 if (idx < total && fi < nflag) {
                     const int vi = (j / kVecPerThread) * kChunkVecs + (j % kVecPerThread) * kConsumers + f.flist[fi];
-                    if (vi < nvec) { vis[u] = vi; w[u] = load_row_vec<kAligned>(row, vi, V); }
+                    if (vi < nvec) { vis[u] = vi; if (kAligned) w[u] = load_row_vec<true>(row, vi, V); }
                 }
             }
+            if (!kAligned) load_vecs_unaligned(w, vis, row, V);
             if (i0 == 0) scale_factor();
             // bit 8u+e of m32: element e of vector u is a candidate (most vectors hold none)
             uint32_t m32 = 0;
