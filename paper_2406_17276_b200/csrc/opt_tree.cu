@@ -524,17 +524,15 @@ struct BuildSink {
                     const bool early = !kPrune && d < p.Dcap && p.delta == -INFINITY;
                     unsigned g0 = 0;
                     if (early) g0 = reserve_layer(nl);        // the rows' numbers, while the candidates load
-                    const bool small = fsize * p.k <= kStageCap;        // the team holds the candidates in registers
                     if (lane == 0) {
                         LayerJob& j = ls.job;
                         set_job(j, 1, sw, b, d, fsize);
                         j.fmap = kPrune ? sw.fmap : nullptr;
-                        j.publish = early && small;
+                        j.publish = early;
                     }
                     __syncwarp();
                     team_sync();
                     select_job<LS>(smem_offset(&ls), lane, g0, w.status);
-                    if (early && !small) publish_layer(ls, nl, g0);
                     double esub;
                     int nR;
                     {

@@ -602,9 +602,10 @@ __device__ __noinline__ int team_select_global(int at, const unsigned long long*
 // them.  (If the bin is too full one more sweep splits it in 1024; if over a thousand ties or a threshold below
 // 2^-63 make that useless too, or a warp's segment overflows, further sweeps read global memory once per digit.)
 // Measured (two sequences, n = 512, k = 16, B200): 1059 us per step with a sweep per digit and tokens fetched one by one, 452
-// with bit marks, a gather and a radix select after the second sweep, 431 with the segments.
+// with bit marks, a gather and a radix select after the second sweep, 431 with the segments; 401 then with the running top-n of
+// team_pick, 378 with the rows sent out by the team as their tokens come in instead of by one warp afterwards.
 template <class LS>
-__device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
+__device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, int* status) {
     LS& s = smem_at<LS>(at);
     const LayerJob& j = s.job;
     const int k = j.k;
@@ -621,7 +622,7 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
     const unsigned long long* gph = reinterpret_cast<const unsigned long long*>(cand_phat);
     const unsigned int* gtk = reinterpret_cast<const unsigned int*>(cand_tok);
     int* coarse = &s.thist[0][0];
-    if (tt == 0) s.listn = 0;
+    if (tt == 0) { s.listn = 0; s.job.g0 = g0; }
     #pragma unroll 1
     for (int i0 = tt; i0 - tt < N; i0 += 8 * kTeam) {
         unsigned long long x[8];
@@ -774,6 +775,7 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
         total = team_select_global<LS>(at, gph, N, nl, tt);
     }
     team_sync();                                           // s.ltok[i] is the candidate index of the new layer's node i, s.lkeys[i] its key
+    g0 = s.job.g0;
     #pragma unroll 1
     for (int i0 = tt; i0 < nl; i0 += 4 * kTeam) {
         int c[4];
@@ -789,7 +791,8 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, int* status) {
             if (i >= nl) break;
             if (!(t32[u] >> 31)) t32[u] = poll_tok_word(&gtk[c[u]], status);
             const int tok = t32[u] == ~0u ? -1 : (int)(t32[u] & 0x7FFFFFFFu);
-            const int frow = c[u] / k;
+            if (j.publish) publish_node(j.queue, j.b, j.d, g0, i, tok, s.lkeys[i], status);
+            const int frow = (int)j.by_k.div((unsigned)c[u]);
             T_tok[gid0 + i] = tok;
             T_par[gid0 + i] = fmap ? __ldcg(&fmap[frow]) : frow;
             T_phat[gid0 + i] = __longlong_as_double((long long)(s.lkeys[i] - 1ull));
@@ -808,7 +811,7 @@ __device__ __forceinline__ void select_job(int at, int tt, unsigned g0, int* sta
     const int N = j.fsize * j.k;
     if (N <= 4 * kTeam) select_layer_team<4, LS>(at, tt, g0, status);
     else if (N <= kStageCap) select_layer_team<8, LS>(at, tt, g0, status);
-    else select_layer_team_big<LS>(at, tt, status);
+    else select_layer_team_big<LS>(at, tt, g0, status);
 }
 template <class LS>
 __device__ __forceinline__ int running_job(int at, int tt, unsigned g0, int* status) {
