@@ -185,6 +185,7 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
     ThreadAcc acc;
     acc.reset();
     ChunkRegs ch;
+    uint32_t cm = 0;                                           // long rows: lane c keeps the warp's maximum of chunk c
     int off = 0;                                               // half of the stage at which the row in hand starts
     long long g = 0;
     for (int r = 0;; ++r) {
@@ -206,6 +207,7 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
             __syncwarp();
             if (lane == 0) mbar_arrive(&s.empty_bar[st]);          // the data is in registers: the stage is free
             chunk_chain(ch);
+            if (kLong) { const uint32_t key = chunk_key(ch); if (lane == c) cm = key; }
             const unsigned long long C2 = chunk_apply(acc, ch);
             chunk_exps<kLong>(acc, ch, C2, (ne + 7) >> 3);
         }
@@ -213,6 +215,7 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
         const int sl = r % kSlots;
         if (r >= kSlots && !mbar_wait_warp(&s.free_bar[sl], (uint32_t)((r / kSlots) - 1) & 1u, status)) return;
         store_thread_result(s.slot[sl], acc, tid);
+        if (kLong && lane < kTrackedChunks) s.slot[sl].cmax[lane][cwarp] = (uint16_t)cm;
         __syncwarp();
         if (lane == 0) mbar_arrive(&s.ready_bar[sl]);
         acc.reset();

@@ -43,7 +43,7 @@ constexpr int kDescRing = 16;                      // descriptors kept: a row's 
 // short rows do without (in one kernel for all, the row step on 32000 logits was 3 to 7 % slower, a build of 32
 // sequences 4 %).
 constexpr int kLongRow = 2 * kChunkElems;          // rows up to this many logits are short
-constexpr int kFinLoads = 8;                       // long rows: vectors a finisher lane has in flight (unaligned: half as many, of two granules)
+constexpr int kTrackedChunks = 10;                 // chunks whose maxima are kept (rows of up to 163840 logits)
 constexpr int kLaneTauMaxK = 16;                   // largest k for which the finisher's threshold comes from the lane maxima
 constexpr int kPerLane = kConsumers / 32;          // per-thread results one finisher lane handles (16)
 
@@ -69,6 +69,7 @@ struct alignas(16) RowSlot {
     float tsum[kConsumers];
     uint16_t tkey[kConsumers];     // per-thread maximum as an ordered key
     int warpE[kConsumerWarps];
+    uint16_t cmax[kTrackedChunks][kConsumerWarps];     // long rows: maximum of each warp's logits of a chunk, see chunk_key
 };
 
 struct alignas(16) FinScratch {    // private to one finisher warp (hist is cleared and read with 16-byte accesses)
@@ -119,7 +120,7 @@ struct alignas(16) LayerScratchT {
     unsigned long long keys[kKeys];            // keys of a selection that does not fit the registers, or falls back on a radix select
     unsigned long long lkeys[NCAP];            // keys of the new layer, slot order
     double vals[NCAP];                         // path values of the new running top-n
-    int toks[kStageCap];                       // large layers: candidate indexes
+    uint16_t index16[kWideGids ? 8 : kStageCap];   // large layers: candidate indexes (below 256 * 32; in gids where that is long enough)
     int gids[2 * NCAP];
     int rsel[NCAP];                            // gids of the new running top-n, ascending
     int ltok[NCAP];                            // tokens of the new layer, slot order
@@ -327,6 +328,13 @@ __device__ __forceinline__ void chunk_exps(ThreadAcc& a, const ChunkRegs& c, uns
         if (nv > kConsumers) vector_exps(a, c.w[1], C2);
         if (nv > 2 * kConsumers) vector_exps(a, c.w[2], C2);
     }
+}
+
+// Key of the maximum of a warp's logits of the chunk in hand: unsigned order is numeric order, and as ord16 but for -0, which comes just
+// below +0.
+__device__ __forceinline__ uint32_t chunk_key(const ChunkRegs& c) {
+    const int b = __float_as_int(fmaxf(__uint_as_float(c.m2 << 16), __uint_as_float(c.m2 & 0xFFFF0000u)));
+    return __reduce_max_sync(0xFFFFFFFFu, (uint32_t)b ^ ((uint32_t)(b >> 31) | 0x80000000u)) >> 16;
 }
 
 // End of a row: every thread's sum is brought to its warp's largest exponent and stored.
@@ -582,19 +590,49 @@ __device__ __noinline__ void finish_many(FinScratch& f, int M, int kk, double m,
     __syncwarp();
 }
 
-// The search of finish_row_warp in long rows: the flagged threads' vectors are read again for the logits >= tau.  The list is
-// first cut down to the threads at or above the exact kk-th largest per-thread maximum (for kk > kLaneTauMaxK tau is that
-// already), kFinLoads vectors per lane are in flight, and a vector that holds a candidate (few do) is read once more for
-// its logits.  Leaves the candidates in f.cand / f.cand_count, raises tau_key and returns the sum of the lane's candidates'
-// approximate terms.
-// Measured with the skipped padding (B200): one sequence, V = 128256, k = 16: 325 -> 297 us a step; row step on 128256
-// logits, k = 16: 5.5 -> 6.0 TB/s, on 152064, k = 10: 6.0 -> 6.15, 1999 unaligned rows of 50257: 71.6 -> 68.0 us.
+// Lists the logits >= tau of a lane's four vectors (number vis[u]; negative: none) in f and returns the sum of their approximate terms.
+__device__ __forceinline__ float take_candidates(FinScratch& f, const uint4 (&w)[4], const int (&vis)[4], uint32_t tau_b2, float negE) {
+    // bit 8u+e of m32: element e of vector u is a candidate (most vectors hold none)
+    uint32_t m32 = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const uint32_t gx = ge_bf16x2(w[u].x, tau_b2), gy = ge_bf16x2(w[u].y, tau_b2);
+        const uint32_t gz = ge_bf16x2(w[u].z, tau_b2), gw = ge_bf16x2(w[u].w, tau_b2);
+        const uint32_t m8 = ((gx & 1u) | ((gx >> 15) & 2u)) | (((gy & 1u) | ((gy >> 15) & 2u)) << 2) |
+                            (((gz & 1u) | ((gz >> 15) & 2u)) << 4) | (((gw & 1u) | ((gw >> 15) & 2u)) << 6);
+        m32 |= (vis[u] < 0 ? 0u : m8) << (8 * u);
+    }
+    float sub = 0.0f;
+#pragma unroll 1
+    while (m32) {
+        const int e = __ffs(m32) - 1;
+        m32 &= m32 - 1;
+        const int u = e >> 3, h = e & 7;
+        const uint4 wu = u < 2 ? (u == 0 ? w[0] : w[1]) : (u == 2 ? w[2] : w[3]);
+        const int vi = u < 2 ? (u == 0 ? vis[0] : vis[1]) : (u == 2 ? vis[2] : vis[3]);
+        const uint32_t word = h < 4 ? (h < 2 ? wu.x : wu.y) : (h < 6 ? wu.z : wu.w);
+        const uint32_t bits = (h & 1) ? (word >> 16) : (word & 0xFFFFu);
+        const int pos = atomicAdd(&f.cand_count, 1);
+        if (pos < kCandCap) f.cand[pos] = cand_key(bits, (uint32_t)(vi * 8 + h));
+        sub += ex2_approx(fmaf(bf16_bits_to_float(bits), kLog2e, negE));
+    }
+    return sub;
+}
+
+// The search of finish_row_warp in long rows: the flagged threads' vectors are read again for the logits >= tau.  The list of threads is
+// first cut down to those at or above the exact kk-th largest per-thread maximum (for kk > kLaneTauMaxK tau is that
+// already), and of a thread's chunks only those are read of which the consumers noted a maximum that high in the thread's warp: a dozen
+// or two of the hundred and more pairs of a thread and a chunk.  Leaves the candidates in f.cand / f.cand_count, raises tau_key and
+// returns the sum of the lane's candidates' approximate terms.
+// Measured (B200, us a step, with all of the threads' vectors read again, eight in flight per lane / now): one sequence, V = 128256, k = 16
+// 253.9 / 237.8; 64 sequences of n = 256, V = 152064, k = 32 17270 / 16060; 3 of n = 18, V = 92464 304.1 / 280.7; 13 of n = 143, V = 61120, k = 5,
+// four chunks, 627 / 647, the one shape seen to lose.  Up to 32 pairs take a lane each, without a list (3 sequences, n = 136, V = 46048: 579 / 568 us).
 template <bool kAligned>
-__device__ __forceinline__ float find_candidates_long(FinScratch& f, const uint16_t* tkey, const uint16_t* row, int V, int kk, int nflag, float negE,
+__device__ __forceinline__ float find_candidates_long(FinScratch& f, const RowSlot& slot, const uint16_t* row, int V, int kk, int nflag, float negE,
                                                       uint32_t& tau_key) {
-    constexpr int kLoads = kAligned ? kFinLoads : kFinLoads / 2;
     const int lane = threadIdx.x & 31;
-    const int nvec = (V + 7) >> 3, nchunks = (V + kChunkElems - 1) / kChunkElems, vpt = nchunks * kVecPerThread;
+    const int nvec = (V + 7) >> 3, nchunks = (V + kChunkElems - 1) / kChunkElems;
+    const uint16_t* tkey = slot.tkey;
     if (kk <= kLaneTauMaxK && nflag > kk) {
         const int t0 = lane < nflag ? f.flist[lane] : 0, t1 = lane + 32 < nflag ? f.flist[lane + 32] : 0;
         const uint32_t a = lane < nflag ? tkey[t0] : 0u, b = lane + 32 < nflag ? tkey[t1] : 0u;
@@ -615,52 +653,56 @@ __device__ __forceinline__ float find_candidates_long(FinScratch& f, const uint1
         __syncwarp();
     }
     const uint32_t tau_bits = ord16_inv(tau_key), tau_b2 = tau_bits | (tau_bits << 16);
-    // Work item i: flagged thread i mod nflag, vector i / nflag = umulhi(i, magic) (exact: i * nflag stays below 2^32).
-    const int total = vpt * nflag;
+    // Most pairs of a flagged thread and a chunk hold nothing: those whose warp's maximum of the chunk is below the threshold are left out.
+    // Pair i: flagged thread i mod nflag, chunk i / nflag = umulhi(i, magic) (exact: i * nflag stays below 2^32).
+    const int pairs = nchunks * nflag;
     const unsigned magic = 0xFFFFFFFFu / (unsigned)nflag + 1u;
-    auto vector_of = [&](int i) -> int {
-        const int j = nflag > 1 ? (int)__umulhi((unsigned)i, magic) : i;
-        return (j / kVecPerThread) * kChunkVecs + (j % kVecPerThread) * kConsumers + f.flist[i - j * nflag];
-    };
+    constexpr int kPairs = 256;                             // listed at a time
+    int* const list = f.hist;                               // (the histogram is done with)
     float sub = 0.0f;
+    int i = lane;
+    // Chunk and thread of pair i, or -1: left out.
+    auto pair_at = [&](int i) -> int {
+        if (i >= pairs) return -1;
+        const int c = nflag > 1 ? (int)__umulhi((unsigned)i, magic) : i, t = f.flist[i - c * nflag];
+        return nchunks > kTrackedChunks || slot.cmax[c][t >> 5] + 1u >= tau_key ? (c << 16) | t : -1;       // (+ 1: see chunk_key)
+    };
 #pragma unroll 1
-    for (int i0 = lane; i0 - lane < total; i0 += 32 * kLoads) {
-        uint4 w[kLoads];
-        int vis[kLoads];
-#pragma unroll
-        for (int u = 0; u < kLoads; ++u) {
-            const int idx = i0 + u * 32;
-            if (kAligned) w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
-            vis[u] = -1;
-            if (idx < total) {
-                const int vi = vector_of(idx);
-                if (vi < nvec) { vis[u] = vi; if (kAligned) w[u] = load_row_vec<true>(row, vi, V); }
+    do {
+        int e = -1, listed = 32;
+        if (pairs <= 32) {                                  // one for each lane, no list
+            e = pair_at(i);
+            i += 32;
+        } else {
+            listed = 0;
+#pragma unroll 1
+            for (; i - lane < pairs && listed <= kPairs - 32; i += 32) {
+                e = pair_at(i);
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, e >= 0);
+                if (e >= 0) list[listed + __popc(m & ((1u << lane) - 1u))] = e;
+                listed += __popc(m);
             }
+            __syncwarp();
         }
-        if (!kAligned) load_vecs_unaligned(w, vis, row, V);
-        uint32_t hits = 0;                                  // bit u: vector u holds a candidate
+#pragma unroll 1
+        for (int i0 = lane; i0 - lane < listed; i0 += 32) {
+            if (pairs > 32) e = i0 < listed ? list[i0] : -1;
+            uint4 w[4];
+            int vis[4];
 #pragma unroll
-        for (int u = 0; u < kLoads; ++u)
-            hits |= (ge_bf16x2(max_bf16x2(max_bf16x2(w[u].x, w[u].y), max_bf16x2(w[u].z, w[u].w)), tau_b2) ? 1u : 0u) << u;
-#pragma unroll 1
-        for (; hits; hits &= hits - 1) {
-            const int vi = vector_of(i0 + (__ffs(hits) - 1) * 32);
-            const uint4 x = load_row_vec<kAligned>(row, vi, V);
-            const uint32_t gx = ge_bf16x2(x.x, tau_b2), gy = ge_bf16x2(x.y, tau_b2);
-            const uint32_t gz = ge_bf16x2(x.z, tau_b2), gw = ge_bf16x2(x.w, tau_b2);
-            uint32_t m8 = ((gx & 1u) | ((gx >> 15) & 2u)) | (((gy & 1u) | ((gy >> 15) & 2u)) << 2) |
-                          (((gz & 1u) | ((gz >> 15) & 2u)) << 4) | (((gw & 1u) | ((gw >> 15) & 2u)) << 6);
-#pragma unroll 1
-            for (; m8; m8 &= m8 - 1) {
-                const int h = __ffs(m8) - 1;
-                const uint32_t word = h < 4 ? (h < 2 ? x.x : x.y) : (h < 6 ? x.z : x.w);
-                const uint32_t bits = (h & 1) ? (word >> 16) : (word & 0xFFFFu);
-                const int pos = atomicAdd(&f.cand_count, 1);
-                if (pos < kCandCap) f.cand[pos] = cand_key(bits, (uint32_t)(vi * 8 + h));
-                sub += ex2_approx(fmaf(bf16_bits_to_float(bits), kLog2e, negE));
+            for (int u = 0; u < 4; ++u) {
+                const int vi = (e >> 16) * kChunkVecs + u * kConsumers + (e & 0xFFFF);
+                vis[u] = e >= 0 && vi < nvec ? vi : -1;
+                if (kAligned) {
+                    w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+                    if (vis[u] >= 0) w[u] = load_row_vec<true>(row, vi, V);
+                }
             }
+            if (!kAligned) load_vecs_unaligned(w, vis, row, V);
+            sub += take_candidates(f, w, vis, tau_b2, negE);
         }
-    }
+        __syncwarp();
+    } while (i - lane < pairs);
     return sub;
 }
 
@@ -747,7 +789,7 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
         // Work item i: flagged thread i mod P (P = nflag rounded up to a power of two), vector i / P.
         const float negE = -(float)emax;
         float sub = 0.0f;
-        if (kLong) sub = find_candidates_long<kAligned>(f, slot.tkey, row, V, kk, nflag, negE, tau_key);
+        if (kLong) sub = find_candidates_long<kAligned>(f, slot, row, V, kk, nflag, negE, tau_key);
         const uint32_t tau_bits = ord16_inv(tau_key);
         const float tau_f = bf16_bits_to_float(tau_bits);
         const uint32_t tau_b2 = tau_bits | (tau_bits << 16);
@@ -780,29 +822,7 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
             }
             if (!kAligned) load_vecs_unaligned(w, vis, row, V);
             if (i0 == 0) scale_factor();
-            // bit 8u+e of m32: element e of vector u is a candidate (most vectors hold none)
-            uint32_t m32 = 0;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t gx = ge_bf16x2(w[u].x, tau_b2), gy = ge_bf16x2(w[u].y, tau_b2);
-                const uint32_t gz = ge_bf16x2(w[u].z, tau_b2), gw = ge_bf16x2(w[u].w, tau_b2);
-                const uint32_t m8 = ((gx & 1u) | ((gx >> 15) & 2u)) | (((gy & 1u) | ((gy >> 15) & 2u)) << 2) |
-                                    (((gz & 1u) | ((gz >> 15) & 2u)) << 4) | (((gw & 1u) | ((gw >> 15) & 2u)) << 6);
-                m32 |= (vis[u] < 0 ? 0u : m8) << (8 * u);
-            }
-#pragma unroll 1
-            while (m32) {
-                const int e = __ffs(m32) - 1;
-                m32 &= m32 - 1;
-                const int u = e >> 3, h = e & 7;
-                const uint4 wu = u < 2 ? (u == 0 ? w[0] : w[1]) : (u == 2 ? w[2] : w[3]);
-                const int vi = u < 2 ? (u == 0 ? vis[0] : vis[1]) : (u == 2 ? vis[2] : vis[3]);
-                const uint32_t word = h < 4 ? (h < 2 ? wu.x : wu.y) : (h < 6 ? wu.z : wu.w);
-                const uint32_t bits = (h & 1) ? (word >> 16) : (word & 0xFFFFu);
-                const int pos = atomicAdd(&f.cand_count, 1);
-                if (pos < kCandCap) f.cand[pos] = cand_key(bits, (uint32_t)(vi * 8 + h));
-                sub += ex2_approx(fmaf(bf16_bits_to_float(bits), kLog2e, negE));
-            }
+            sub += take_candidates(f, w, vis, tau_b2, negE);
         }
         __syncwarp();
         M = f.cand_count;

@@ -426,7 +426,7 @@ __device__ __noinline__ int select_layer_team(int at, int tt, unsigned g0, int* 
         if ((take >> u) & 1u) {
             s.ltok[pos] = t32[u] == ~0u ? -1 : (int)(t32[u] & 0x7FFFFFFFu);
             s.lkeys[pos] = x[u];
-            s.toks[pos] = u * kTeam + tt;
+            s.gids[pos] = u * kTeam + tt;
         }
     }
     if (tt == 0 && total != nl) set_status(status, kErrInternal);
@@ -439,7 +439,7 @@ __device__ __noinline__ int select_layer_team(int at, int tt, unsigned g0, int* 
         const int tok = s.ltok[i], gid = gid0 + i;
         const unsigned long long key = s.lkeys[i];
         if (j.publish) publish_node(j.queue, j.b, j.d, g0, i, tok, key, status);
-        const int frow = (int)j.by_k.div((unsigned)s.toks[i]);
+        const int frow = (int)j.by_k.div((unsigned)s.gids[i]);
         j.T_tok[gid] = tok;
         j.T_par[gid] = j.fmap ? __ldcg(&j.fmap[frow]) : frow;
         j.T_phat[gid] = __longlong_as_double((long long)(key - 1ull));
@@ -518,7 +518,7 @@ __device__ __noinline__ int select_running_team(int at, int tt, unsigned g0, int
                 const int slot = pos - kept_old;
                 s.ltok[slot] = t32[u] == ~0u ? -1 : (int)(t32[u] & 0x7FFFFFFFu);
                 s.lkeys[slot] = x[u];
-                s.toks[slot] = i - off;
+                s.gids[slot] = i - off;
             }
             s.rsel[pos] = i < off ? (int)t32[u] : gid0 + pos - kept_old;
             s.vals[pos] = __longlong_as_double((long long)(x[u] - 1ull));
@@ -535,7 +535,7 @@ __device__ __noinline__ int select_running_team(int at, int tt, unsigned g0, int
         const unsigned long long key = s.lkeys[i];
         if (j.publish) publish_node(j.queue, j.b, j.d, g0, i, tok, key, status);
         j.T_tok[gid] = tok;
-        j.T_par[gid] = __ldcg(&j.fmap[j.by_k.div((unsigned)s.toks[i])]);       // layer slot of the node behind the candidate's frontier row
+        j.T_par[gid] = __ldcg(&j.fmap[j.by_k.div((unsigned)s.gids[i])]);       // layer slot of the node behind the candidate's frontier row
         j.T_phat[gid] = __longlong_as_double((long long)(key - 1ull));
     }
     #pragma unroll 1
@@ -680,7 +680,8 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
     }
     // second sweep
     constexpr int kSeg = LS::kSurvivors / kTeamWarps;
-    int* idx = LS::kWideGids ? s.gids : s.toks;
+    auto put_index = [&](int at_v, int i) { if (LS::kWideGids) s.gids[at_v] = i; else s.index16[at_v] = (uint16_t)i; };
+    auto index_at = [&](int at_v) -> int { return LS::kWideGids ? s.gids[at_v] : (int)s.index16[at_v]; };
     const unsigned below = (1u << lane) - 1u;
     const int per = (((N + kTeamWarps - 1) / kTeamWarps) + 255) & ~255;        // candidates per warp
     const int lo = min(tw * per, N), hi = min(lo + per, N);
@@ -697,7 +698,7 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
             const int pos = mine + __popc(m & below);
             if (key >= low && pos < kSeg) {
                 s.keys[tw * kSeg + pos] = key;
-                idx[tw * kSeg + pos] = i0 + u * 32 + lane;
+                put_index(tw * kSeg + pos, i0 + u * 32 + lane);
             }
             mine += __popc(m);
         }
@@ -769,7 +770,7 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
             const unsigned long long key = s.keys[at_v];
             bool take = key > thr;
             if (key == thr && eq_take > 0) { take = true; --eq_take; }
-            if (take) { s.lkeys[pos] = key; s.ltok[pos] = idx[at_v]; ++pos; }
+            if (take) { s.lkeys[pos] = key; s.ltok[pos] = index_at(at_v); ++pos; }
         }
     } else {
         total = team_select_global<LS>(at, gph, N, nl, tt);
