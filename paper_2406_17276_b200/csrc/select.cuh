@@ -211,8 +211,8 @@ __device__ __forceinline__ void sweep_candidates(const unsigned long long* gph, 
 }
 
 // A layer's candidate words, all of them read, are made zero for the rows of the next layer but one: a sequence's even and odd layers
-// have arrays of their own, so the clearing need not come before the next layer is sent out, and the layer warp's fence that
-// puts it before the rows of the layer after that (at the end of the job) costs nothing: a finisher on another SM cannot
+// have arrays of their own, so the clearing need not come before the next layer is sent out, and the fence of every thread of the team
+// that puts it before the rows of the layer after that (at the end of the job, after its last barrier) costs nothing: a finisher on another SM cannot
 // store a word before its row has been sent out, so no clear can take a word away.  With one array the fence lay
 // between selection and publication, 3.7 % of a build of 32 sequences.  (A fence on the reading side as well, in the fetcher, costs a
 // step of one sequence 3 %; the finisher's store there depends on the mailbox word.)
