@@ -541,8 +541,10 @@ __device__ __noinline__ int select_running_team(int at, int tt, unsigned g0, int
     #pragma unroll 1
     for (int i = tt; i < need; i += kTeam) j.Rnew[i] = s.rsel[i];
     clear_candidates(j.cand_phat, j.cand_tok, N, tt, kTeam);
+    const bool renumber = j.publish != 0;                  // (the layer warp may set up its next job once the last barrier is past)
+    int32_t* const fmap = j.fmap;
     team_sync();
-    if (j.publish) for (int i = tt; i < cnt; i += kTeam) j.fmap[i] = i;    // (read above)
+    if (renumber) for (int i = tt; i < cnt; i += kTeam) fmap[i] = i;       // (read above; the next job's first barrier puts it before its reads)
     return need;
 }
 
