@@ -264,6 +264,17 @@ int opt_tree_step_host(opt_tree_ctx *ctx, const void *draft_logits_bf16, const v
 #define OPT_TREE_SELFTEST_WAITS 5
 int opt_tree_selftest_waits(opt_tree_ctx *ctx, int32_t *result, void *stream);
 
+/* Self-test of a layer selection whose candidates never come (not a step of the paper's method).  One small kernel selects layer 2 of
+ * a tree from `rows` frontier rows, of which only the first `written` have their k candidates (candidate i: path value 1/2, 1/4
+ * or 1/8 by i mod 3, token i mod V); the wait for the others is given up after 2^10 polls.  joint: the selection over the running
+ * top-n (one node of path value 1) and the candidates together (32 + rows * k <= 1024).
+ *   result (dev) [1] int32: OPT_TREE_ERR_TIMEOUT if any row is missing, else OPT_TREE_OK
+ *   token, parent (dev) [n] int32, phat (dev) [n] double: the nodes selected; a missing candidate counts as token 0 of path
+ *                value 0; beyond the layer's nodes -1
+ * Needs max_depth >= 2.  Uses the context's workspace as a build does. */
+int opt_tree_selftest_selection(opt_tree_ctx *ctx, int32_t rows, int32_t written, int32_t joint, int32_t *result, int32_t *token,
+                                int32_t *parent, double *phat, void *stream);
+
 /* Reads (and clears) the device status word; synchronises the device.  *status_host is
  * OPT_TREE_OK or the first device-side error recorded since the last call. */
 int opt_tree_last_device_status(opt_tree_ctx *ctx, int32_t *status_host);

@@ -20,7 +20,7 @@ OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_CUDA, ERR_TIMEOUT, ERR_INTERNAL = 0, -
 EXPORTS = ["opt_tree_workspace_bytes", "opt_tree_create", "opt_tree_destroy", "opt_tree_build", "opt_tree_mask",
            "opt_tree_verify", "opt_tree_row_softmax_topk", "opt_tree_step_host", "opt_tree_last_device_status",
            "opt_tree_launch_count", "opt_tree_strerror", "opt_tree_verify_static", "opt_tree_post_verify", "opt_tree_build_pruned", "opt_tree_layers_begin",
-           "opt_tree_layers_step", "opt_tree_verify_sampled", "opt_tree_selftest_waits"]
+           "opt_tree_layers_step", "opt_tree_verify_sampled", "opt_tree_selftest_waits", "opt_tree_selftest_selection"]
 
 
 class Config(C.Structure):
@@ -76,6 +76,7 @@ def lib():
         L.opt_tree_post_verify.argtypes = [C.c_void_p, C.POINTER(Out), C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32,
                                            C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
         L.opt_tree_selftest_waits.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p]
+        L.opt_tree_selftest_selection.argtypes = [C.c_void_p, C.c_int32, C.c_int32, C.c_int32] + [C.c_void_p] * 5
         L.opt_tree_strerror.restype = C.c_char_p
         L.opt_tree_strerror.argtypes = [C.c_int]
         _lib = L
@@ -269,6 +270,15 @@ class OptTree:
         res = torch.full((5,), 77, dtype=torch.int32, device=self.device)
         _check(lib().opt_tree_selftest_waits(self._ctx, _ptr(res), _stream()), "opt_tree_selftest_waits")
         return res
+
+    def selftest_selection(self, rows: int, written: int, joint: bool):
+        """opt_tree_selftest_selection: (status, tokens, parents, path values) of a selection of which `rows - written` rows never come."""
+        res = torch.full((1,), 77, dtype=torch.int32, device=self.device)
+        tok, par = (torch.full((self.cfg.n,), 77, dtype=torch.int32, device=self.device) for _ in range(2))
+        ph = torch.full((self.cfg.n,), 77.0, dtype=torch.float64, device=self.device)
+        _check(lib().opt_tree_selftest_selection(self._ctx, rows, written, int(joint), _ptr(res), _ptr(tok), _ptr(par), _ptr(ph), _stream()),
+               "opt_tree_selftest_selection")
+        return res, tok, par, ph
 
     def device_status(self) -> int:
         st = C.c_int32(0)

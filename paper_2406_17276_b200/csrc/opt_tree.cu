@@ -138,7 +138,7 @@ __device__ __forceinline__ RowQueue row_queue(const Workspace& w, const Params& 
 
 // What is the same for all jobs of a launch.
 __device__ __forceinline__ void set_job_constants(LayerJob& j, const Workspace& w, const Params& p) {
-    j.n = p.n; j.k = p.k; j.kk = p.kk; j.max_depth = p.max_depth;
+    j.n = p.n; j.k = p.k; j.kk = p.kk; j.max_depth = p.max_depth; j.polls = kWaitPolls;
     j.queue = row_queue(w, p);
     j.by_k = p.by_k;
 }
@@ -1505,6 +1505,48 @@ wait_probe_kernel(int* result, const unsigned long long* zero_words, long long l
     }
 }
 
+// Self-test of a layer selection whose candidate words never come: one CTA, of which only the layer team works.  It selects layer 2 of
+// sequence 0 from `rows` frontier rows, of which only the first `written` have their words, and leaves the selection's nodes in the caller's
+// arrays.  joint: the selection over the running top-n (one node of layer 1) and the candidates together.
+template <int NCAP>
+__global__ void __launch_bounds__(kThreads)
+selection_probe_kernel(Workspace w, Params p, int rows, int written, int joint, int polls, int* status, int32_t* tok, int32_t* par, double* phat) {
+    using LS = LayerScratchT<NCAP>;
+    CtaSmemT<NCAP>& s = *reinterpret_cast<CtaSmemT<NCAP>*>(ot_smem);
+    LS& ls = s.layer;
+    pipeline_init(s.core, ls);
+    const int tt = (int)threadIdx.x - (kConsumerWarps + kHelperLayer) * 32;
+    if (tt < 0 || tt >= kTeam) return;
+    const SeqWork sw = seq_work(w, p, 0, 2);
+    for (int i = tt; i < rows * p.k; i += kTeam) {         // path values 1/2, 1/4, 1/8, 1/2 ...: ties as well
+        const bool there = i < written * p.k;
+        sw.cand_phat[i] = there ? __longlong_as_double((long long)phat_word(1.0 / (2 << (i % 3)))) : 0.0;
+        sw.cand_tok[i] = there ? (int)(0x80000000u | (unsigned)(i % p.V)) : 0;
+    }
+    for (int i = tt; i < p.n; i += kTeam) sw.fmap[i] = i;
+    if (tt == 0) {
+        LayerJob& j = ls.job;
+        set_job_constants(j, w, p);
+        j.polls = polls;
+        j.kind = joint ? 2 : 1; j.b = 0; j.d = 2; j.fsize = rows; j.ncand = 0;
+        j.cand_phat = sw.cand_phat; j.cand_tok = sw.cand_tok;
+        j.T_tok = sw.T_tok; j.T_par = sw.T_par; j.T_phat = sw.T_phat;
+        j.fmap = sw.fmap; j.nR_old = 1; j.off = 32; j.cached = 0; j.publish = 1;
+        j.Rold = sw.R + p.n; j.Rnew = sw.R;
+        sw.R[p.n] = 0; sw.T_tok[0] = 0; sw.T_par[0] = 0; sw.T_phat[0] = 1.0;
+    }
+    __threadfence();
+    team_sync();
+    const int at = smem_offset(&ls), nvalid = rows * p.kk;
+    int nl = nvalid < p.n ? nvalid : p.n;
+    if (joint) nl = running_job<LS>(at, tt, 0u, status) - ls.kept_old;
+    else select_job<LS>(at, tt, 0u, status);
+    for (int i = tt; i < p.n; i += kTeam) {
+        tok[i] = i < nl ? __ldcg(&sw.T_tok[p.n + i]) : -1; par[i] = i < nl ? __ldcg(&sw.T_par[p.n + i]) : -1;
+        phat[i] = i < nl ? __ldcg(&sw.T_phat[p.n + i]) : -1.0;
+    }
+}
+
 }  // namespace ot
 
 // ------------------------------------------------------------------------------------------------
@@ -1854,6 +1896,25 @@ int opt_tree_selftest_waits(opt_tree_ctx* ctx, int32_t* result, void* stream) {
     }
     ot::wait_probe_kernel<<<1, ot::kThreads, sizeof(ot::CtaSmem), st>>>(
         result, reinterpret_cast<const unsigned long long*>(ctx->ws.o_mask), 1ll << 16, 1 << 10);
+    ctx->launches++;
+    return check_launch();
+}
+
+int opt_tree_selftest_selection(opt_tree_ctx* ctx, int32_t rows, int32_t written, int32_t joint, int32_t* result, int32_t* token,
+                                int32_t* parent, double* phat, void* stream) {
+    if (!ctx || !result || !token || !parent || !phat || rows < 1 || rows > ctx->cfg.n || written < 0 || written > rows || ctx->cfg.max_depth < 2)
+        return OPT_TREE_ERR_INVALID_ARG;
+    if (joint && 32 + rows * ctx->cfg.k > ot::kStageCap) return OPT_TREE_ERR_INVALID_ARG;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    ot::Params p = make_params(ctx, nullptr, 0.0f);
+    p.B = 1;
+    const bool small = small_n(ctx->cfg.n);
+    auto* kernel = small ? ot::selection_probe_kernel<ot::kSmallN> : ot::selection_probe_kernel<ot::kMaxN>;
+    if (!allow_smem(kernel, ctx->smem) || cudaMemsetAsync(result, 0, sizeof(int32_t), st) != cudaSuccess) {
+        cudaGetLastError();
+        return OPT_TREE_ERR_CUDA;
+    }
+    kernel<<<1, ot::kThreads, ctx->smem, st>>>(ctx->ws, p, rows, written, joint, 1 << 10, result, token, parent, phat);
     ctx->launches++;
     return check_launch();
 }

@@ -101,6 +101,7 @@ struct LayerJob {                  // what the layer warp hands its assistants (
     // kinds 1 and 2: publish the new nodes' rows straight away, numbered from g0 on
     int publish;
     unsigned g0;
+    int polls;                     // limit of the waits for candidate words (kWaitPolls; 0 once one has run out)
     RowQueue queue;
     FixedDiv by_k;
 };

@@ -179,16 +179,28 @@ __device__ int team_radix_select(LS& s, KeyFn keyf, int N, int need, int tt, uns
     return (pass - 1) % 3;
 }
 
-// Candidate words i = u * kTeam + tt (u < kW) of a layer of N, into registers.  Words that are not there yet are read again, all
-// at once, until they are (bounded), with a short pause so that the polling does not hold up the words themselves.
+// The words of a candidate that never came (see sweep_candidates): token 0, path value 0.
+constexpr unsigned long long kLostPhat = 1ull << 63;
+constexpr unsigned kLostTok = 1u << 31;
+// Once a wait of a team has run out the team waits no more: the build comes to its end, with the status set.
+__device__ __forceinline__ void wait_ran_out(LayerJob& job, int* status) {
+    set_status(status, kErrTimeout);
+    atomicExch(&job.polls, 0);
+}
+
+// Candidate words i = u * kTeam + tt (u < kW) of [first, end), into registers (all ones elsewhere); gph and gtk are the words' arrays
+// shifted by `first`.  Words that are not there yet are read again, all at once, until they are (at most job.polls times), with a short
+// pause so that the polling does not hold up the words themselves.  A word that never came reads as token 0 of path value 0: the layer
+// has as many nodes as it was to get, and all that follows works on nodes that exist, with the status set.
 template <int kW>
-__device__ __forceinline__ void sweep_candidates(const unsigned long long* gph, const unsigned int* gtk, int N, int tt, unsigned long long (&x)[kW],
-                                                 unsigned int (&t32)[kW], int* status) {
+__device__ __forceinline__ void sweep_candidates(const unsigned long long* gph, const unsigned int* gtk, int first, int end, int tt, unsigned long long (&x)[kW],
+                                                 unsigned int (&t32)[kW], LayerJob& job, int* status) {
 #pragma unroll
     for (int u = 0; u < kW; ++u) {
         const int i = u * kTeam + tt;
-        x[u] = i < N ? ld_relaxed_u64(&gph[i]) : ~0ull;
-        t32[u] = i < N ? ld_relaxed_u32(&gtk[i]) : ~0u;
+        const bool word = i >= first && i < end;
+        x[u] = word ? ld_relaxed_u64(&gph[i]) : ~0ull;
+        t32[u] = word ? ld_relaxed_u32(&gtk[i]) : ~0u;
     }
     #pragma unroll 1
     for (int t = 0;; ++t) {
@@ -201,10 +213,10 @@ __device__ __forceinline__ void sweep_candidates(const unsigned long long* gph, 
         }
         if (!__any_sync(0xFFFFFFFFu, missing)) break;
         __nanosleep(20);
-        if (t >= kWaitPolls) {
-            set_status(status, kErrTimeout);
+        if (t >= job.polls) {
+            wait_ran_out(job, status);
 #pragma unroll
-            for (int u = 0; u < kW; ++u) { if (!(x[u] >> 63)) x[u] = ~0ull; if (!(t32[u] >> 31)) t32[u] = ~0u; }
+            for (int u = 0; u < kW; ++u) { if (!(x[u] >> 63)) x[u] = kLostPhat; if (!(t32[u] >> 31)) t32[u] = kLostTok; }
             break;
         }
     }
@@ -413,7 +425,7 @@ __device__ __noinline__ int select_layer_team(int at, int tt, unsigned g0, int* 
     const int N = j.fsize * j.k, nvalid = j.fsize * j.kk, nl = nvalid < j.n ? nvalid : j.n, gid0 = (j.d - 1) * j.n;
     unsigned long long x[kW];
     unsigned int t32[kW];
-    sweep_candidates<kW>(reinterpret_cast<const unsigned long long*>(j.cand_phat), reinterpret_cast<const unsigned int*>(j.cand_tok), N, tt, x, t32, status);
+    sweep_candidates<kW>(reinterpret_cast<const unsigned long long*>(j.cand_phat), reinterpret_cast<const unsigned int*>(j.cand_tok), 0, N, tt, x, t32, s.job, status);
 #pragma unroll
     for (int u = 0; u < kW; ++u) x[u] = key_of_word(x[u]);
     if (tt == 0) s.job.g0 = g0;
@@ -473,30 +485,7 @@ __device__ __noinline__ int select_running_team(int at, int tt, unsigned g0, int
     const unsigned int* gtk = reinterpret_cast<const unsigned int*>(j.cand_tok) - off;
     unsigned long long x[kW];
     unsigned int t32[kW];                                  // candidates: token word; old members: gid
-#pragma unroll
-    for (int u = 0; u < kW; ++u) {
-        const int i = u * kTeam + tt;
-        x[u] = ~0ull; t32[u] = ~0u;
-        if (i >= off && i < M) { x[u] = ld_relaxed_u64(&gph[i]); t32[u] = ld_relaxed_u32(&gtk[i]); }
-    }
-    #pragma unroll 1
-    for (int t = 0;; ++t) {
-        bool missing = false;
-#pragma unroll
-        for (int u = 0; u < kW; ++u) {
-            const int i = u * kTeam + tt;
-            if (!(x[u] >> 63)) { x[u] = ld_relaxed_u64(&gph[i]); missing = missing || !(x[u] >> 63); }
-            if (!(t32[u] >> 31)) { t32[u] = ld_relaxed_u32(&gtk[i]); missing = missing || !(t32[u] >> 31); }
-        }
-        if (!__any_sync(0xFFFFFFFFu, missing)) break;
-        __nanosleep(20);
-        if (t >= kWaitPolls) {
-            set_status(status, kErrTimeout);
-#pragma unroll
-            for (int u = 0; u < kW; ++u) { if (!(x[u] >> 63)) x[u] = ~0ull; if (!(t32[u] >> 31)) t32[u] = ~0u; }
-            break;
-        }
-    }
+    sweep_candidates<kW>(gph, gtk, off, M, tt, x, t32, s.job, status);
 #pragma unroll
     for (int u = 0; u < kW; ++u) {
         const int i = u * kTeam + tt;
@@ -587,7 +576,7 @@ __device__ __noinline__ int team_select_global(int at, const unsigned long long*
     eq_take = eq_take < 0 ? 0 : (eq_take > eq ? eq : eq_take);
     int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
     #pragma unroll 1
-    for (int i = lo; i < hi; ++i) {
+    for (int i = lo; total == need && i < hi; ++i) {
         const unsigned long long key = key_of_word(ld_relaxed_u64(&gph[i]));
         bool take = key > thr;
         if (key == thr && key != 0ull && eq_take > 0) { take = true; --eq_take; }
@@ -638,10 +627,10 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
             for (int u = 0; u < 8; ++u)
                 if (!(x[u] >> 63)) { x[u] = ld_relaxed_u64(&gph[i0 + u * kTeam]); missing = missing || !(x[u] >> 63); }
             if (!__any_sync(0xFFFFFFFFu, missing)) break;
-            if (t >= kWaitPolls) {
-                set_status(status, kErrTimeout);
+            if (t >= j.polls) {
+                wait_ran_out(s.job, status);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) if (!(x[u] >> 63)) x[u] = ~0ull;
+                for (int u = 0; u < 8; ++u) if (!(x[u] >> 63)) x[u] = kLostPhat;
                 break;
             }
         }
@@ -767,7 +756,7 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
         int pos = team_excl_scan(gt + eq_take, s.scan_b, tw, total);
         if (dirty >= 0) { s.thist[dirty][tt] = 0; s.thist[dirty][tt + kTeam] = 0; }
         #pragma unroll 1
-        for (int v = v0; v < v1; ++v) {
+        for (int v = v0; total == nl && v < v1; ++v) {
             const int at_v = at_of(v);
             const unsigned long long key = s.keys[at_v];
             bool take = key > thr;
@@ -777,7 +766,12 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
     } else {
         total = team_select_global<LS>(at, gph, N, nl, tt);
     }
-    team_sync();                                           // s.ltok[i] is the candidate index of the new layer's node i, s.lkeys[i] its key
+    // s.ltok[i] is the candidate index of the new layer's node i, s.lkeys[i] its key
+    if (total != nl) {                                     // (words that came between the sweeps, after a wait that ran out: nothing was taken)
+        for (int i = tt; i < nl; i += kTeam) { s.ltok[i] = 0; s.lkeys[i] = phat_key(0.0); }
+        if (tt == 0) set_status(status, kErrInternal);
+    }
+    team_sync();
     g0 = s.job.g0;
     #pragma unroll 1
     for (int i0 = tt; i0 < nl; i0 += 4 * kTeam) {
@@ -792,8 +786,8 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
         for (int u = 0; u < 4; ++u) {
             const int i = i0 + u * kTeam;
             if (i >= nl) break;
-            if (!(t32[u] >> 31)) t32[u] = poll_tok_word(&gtk[c[u]], status);
-            const int tok = t32[u] == ~0u ? -1 : (int)(t32[u] & 0x7FFFFFFFu);
+            if (!(t32[u] >> 31)) t32[u] = poll_tok_word(&gtk[c[u]], status, j.polls);
+            const int tok = t32[u] == ~0u ? 0 : (int)(t32[u] & 0x7FFFFFFFu);        // (all ones: it never came)
             if (j.publish) publish_node(j.queue, j.b, j.d, g0, i, tok, s.lkeys[i], status);
             const int frow = (int)j.by_k.div((unsigned)c[u]);
             T_tok[gid0 + i] = tok;
@@ -802,7 +796,6 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
             s.ltok[i] = tok;
         }
     }
-    if (total != nl) set_status(status, kErrInternal);
     team_sync();
     return nl;
 }
