@@ -609,13 +609,13 @@ struct BuildSink {
 
 // Algorithm 1 for a whole batch in one launch: persistent CTAs take rows from their mailboxes; layers
 // of different sequences overlap freely because sequences never exchange data.
-template <bool kPrune, int NCAP, bool kAligned, bool kLong>
+template <bool kPrune, int NCAP, int kForm>
 __global__ void __launch_bounds__(kThreads)
 build_kernel(Workspace w, Params p, const uint16_t* __restrict__ draft, opt_tree_out out, int32_t* rows_read) {
     CtaSmemT<NCAP>& s = *reinterpret_cast<CtaSmemT<NCAP>*>(ot_smem);
     BuildSource<kPrune> src{w, p, draft};
     BuildSink<kPrune> sink{w, p, out, rows_read};
-    run_pipeline<kAligned, kLong>(s, src, sink, p.V, p.k, draft, draft + (size_t)p.H * p.V, w.status);
+    run_pipeline<kForm>(s, src, sink, p.V, p.k, draft, draft + (size_t)p.H * p.V, w.status);
 }
 
 // The row step alone over a list of rows (static round-robin over the CTAs).
@@ -645,14 +645,14 @@ struct ListSink {
         }
     }
 };
-template <bool kAligned, bool kLong>
+template <int kForm>
 __global__ void __launch_bounds__(kThreads)
 row_topk_kernel(Params p, const uint16_t* __restrict__ logits, const int32_t* __restrict__ rows, int nrows,
                 int32_t* tok_out, double* prob_out, int* status) {
     CtaSmem& s = *reinterpret_cast<CtaSmem*>(ot_smem);
     ListSource src{logits, rows, nrows, p.V, p.H, (int)blockIdx.x, (int)gridDim.x, status};
     ListSink sink{tok_out, prob_out, p.k};
-    run_pipeline<kAligned, kLong>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.H * p.V, status);
+    run_pipeline<kForm>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.H * p.V, status);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -913,7 +913,7 @@ struct LayersSink {
         do_job(ls, more ? 6 : 4);
     }
 };
-template <int NCAP, bool kAligned, bool kLong>
+template <int NCAP, int kForm>
 __global__ void __launch_bounds__(kThreads)
 layers_kernel(Workspace w, Params p, const uint16_t* __restrict__ logits, int fstride, opt_tree_out out, int32_t* next_tokens,
               int32_t* next_parent, int32_t* next_count) {
@@ -922,7 +922,7 @@ layers_kernel(Workspace w, Params p, const uint16_t* __restrict__ logits, int fs
     const int call = __ldcg(&w.q_ctl[kQCall]);               // (every thread has it before any CTA can leave: see run_pipeline's barrier)
     LayersSource src{w, p, logits, fstride, call};
     LayersSink<LayerScratchT<NCAP>> sink{w, p, out, fstride, call, smem_offset(&s.layer), next_tokens, next_parent, next_count};
-    run_pipeline<kAligned, kLong>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.B * fstride * p.V, w.status);
+    run_pipeline<kForm>(s, src, sink, p.V, p.k, logits, logits + (size_t)p.B * fstride * p.V, w.status);
 }
 
 // Tree attention mask + position ids: one CTA per sequence, a thread per node (in rounds of the block
@@ -1630,27 +1630,27 @@ size_t cta_smem_bytes(int n) { return small_n(n) ? sizeof(ot::CtaSmemT<ot::kSmal
 
 using BuildKernel = void (*)(ot::Workspace, ot::Params, const uint16_t*, opt_tree_out, int32_t*);
 using RowKernel = void (*)(ot::Params, const uint16_t*, const int32_t*, int, int32_t*, double*, int*);
-// Variants: bit 0 pruned draft, bit 1 aligned rows, bit 2 long rows.
-constexpr int kPrunedBit = 1, kAlignedBit = 2, kLongBit = 4, kVariants = 8;
-template <int NCAP> BuildKernel build_variant(int v) {
-    static const BuildKernel kernels[kVariants] = {
-        ot::build_kernel<false, NCAP, false, false>, ot::build_kernel<true, NCAP, false, false>,
-        ot::build_kernel<false, NCAP, true, false>,  ot::build_kernel<true, NCAP, true, false>,
-        ot::build_kernel<false, NCAP, false, true>,  ot::build_kernel<true, NCAP, false, true>,
-        ot::build_kernel<false, NCAP, true, true>,   ot::build_kernel<true, NCAP, true, true>};
-    return kernels[v];
+// Variants: a form of row each (RowForm), the build's also pruned or not.
+constexpr int kForms = ot::kRowForms;
+template <int NCAP> BuildKernel build_variant(int form, bool prune) {
+    static const BuildKernel kernels[kForms][2] = {
+        {ot::build_kernel<false, NCAP, 0>, ot::build_kernel<true, NCAP, 0>}, {ot::build_kernel<false, NCAP, 1>, ot::build_kernel<true, NCAP, 1>},
+        {ot::build_kernel<false, NCAP, 2>, ot::build_kernel<true, NCAP, 2>}, {ot::build_kernel<false, NCAP, 3>, ot::build_kernel<true, NCAP, 3>},
+        {ot::build_kernel<false, NCAP, 4>, ot::build_kernel<true, NCAP, 4>}};
+    return kernels[form][prune ? 1 : 0];
 }
-BuildKernel build_kernel_for(int n, int v) { return small_n(n) ? build_variant<ot::kSmallN>(v) : build_variant<ot::kMaxN>(v); }
-RowKernel row_variant(int v) {
-    return (v & kLongBit) ? ((v & kAlignedBit) ? ot::row_topk_kernel<true, true> : ot::row_topk_kernel<false, true>)
-                          : ((v & kAlignedBit) ? ot::row_topk_kernel<true, false> : ot::row_topk_kernel<false, false>);
+BuildKernel build_kernel_for(int n, int form, bool prune) { return small_n(n) ? build_variant<ot::kSmallN>(form, prune) : build_variant<ot::kMaxN>(form, prune); }
+RowKernel row_variant(int form) {
+    static const RowKernel kernels[kForms] = {ot::row_topk_kernel<0>, ot::row_topk_kernel<1>, ot::row_topk_kernel<2>, ot::row_topk_kernel<3>, ot::row_topk_kernel<4>};
+    return kernels[form];
 }
 using LayersKernel = void (*)(ot::Workspace, ot::Params, const uint16_t*, int, opt_tree_out, int32_t*, int32_t*, int32_t*);
-template <int NCAP> LayersKernel layers_variant(int v) {
-    return (v & kLongBit) ? ((v & kAlignedBit) ? ot::layers_kernel<NCAP, true, true> : ot::layers_kernel<NCAP, false, true>)
-                          : ((v & kAlignedBit) ? ot::layers_kernel<NCAP, true, false> : ot::layers_kernel<NCAP, false, false>);
+template <int NCAP> LayersKernel layers_variant(int form) {
+    static const LayersKernel kernels[kForms] = {ot::layers_kernel<NCAP, 0>, ot::layers_kernel<NCAP, 1>, ot::layers_kernel<NCAP, 2>,
+                                                 ot::layers_kernel<NCAP, 3>, ot::layers_kernel<NCAP, 4>};
+    return kernels[form];
 }
-int variant_of(const ot::Params& p) { return (p.prune ? kPrunedBit : 0) | (p.aligned ? kAlignedBit : 0) | (p.V > ot::kLongRow ? kLongBit : 0); }
+int form_of(const ot::Params& p) { return ot::row_form(p.aligned != 0, p.V, p.kk); }
 template <class F> bool allow_smem(F* kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
 }
@@ -1662,15 +1662,18 @@ int persistent_grid(int n) {
     constexpr int S = ot::kSmallN, L = ot::kMaxN;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
     bool ok = true;
-    for (int v = 0; v < kVariants; ++v)
-        ok = ok && allow_smem(build_variant<S>(v), sizeof(ot::CtaSmemT<S>)) && allow_smem(build_variant<L>(v), sizeof(ot::CtaSmemT<L>)) &&
-             allow_smem(row_variant(v), sizeof(ot::CtaSmem)) && allow_smem(layers_variant<S>(v), sizeof(ot::CtaSmemT<S>)) &&
-             allow_smem(layers_variant<L>(v), sizeof(ot::CtaSmemT<L>));
-    int least = 1 << 30;                             // the variants share one grid: the smallest occupancy counts
-    for (int v = 0; v < kVariants && ok; ++v) {
-        ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_kernel_for(n, v), ot::kThreads, cta_smem_bytes(n)) == cudaSuccess;
-        least = per_sm < least ? per_sm : least;
+    for (int f = 0; f < kForms; ++f) {
+        for (int prune = 0; prune < 2; ++prune)
+            ok = ok && allow_smem(build_variant<S>(f, prune), sizeof(ot::CtaSmemT<S>)) && allow_smem(build_variant<L>(f, prune), sizeof(ot::CtaSmemT<L>));
+        ok = ok && allow_smem(row_variant(f), sizeof(ot::CtaSmem)) && allow_smem(layers_variant<S>(f), sizeof(ot::CtaSmemT<S>)) &&
+             allow_smem(layers_variant<L>(f), sizeof(ot::CtaSmemT<L>));
     }
+    int least = 1 << 30;                             // the variants share one grid: the smallest occupancy counts
+    for (int f = 0; f < kForms && ok; ++f)
+        for (int prune = 0; prune < 2 && ok; ++prune) {
+            ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_kernel_for(n, f, prune), ot::kThreads, cta_smem_bytes(n)) == cudaSuccess;
+            least = per_sm < least ? per_sm : least;
+        }
     if (!ok || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -1746,7 +1749,7 @@ static int build_common(opt_tree_ctx* ctx, const void* draft, const int32_t* roo
     p.prune = prune;
     const long long init_threads = (long long)ctx->grid * ctx->mcap > B ? (long long)ctx->grid * ctx->mcap : B;
     launch_after(ot::init_build_kernel, dim3((unsigned)((init_threads + 255) / 256)), dim3(256), 0, st, ctx->ws, p, root_token);
-    launch_after(build_kernel_for(ctx->cfg.n, variant_of(p)), dim3(ctx->grid), dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(draft), *out, rows_read);
+    launch_after(build_kernel_for(ctx->cfg.n, form_of(p), prune != 0), dim3(ctx->grid), dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(draft), *out, rows_read);
     ctx->launches += 2;
     return check_launch();
 }
@@ -1832,8 +1835,8 @@ int opt_tree_layers_step(opt_tree_ctx* ctx, const void* frontier_logits, int32_t
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     ot::Params p = make_params(ctx, frontier_logits, delta);
     p.B = B;
-    const int nrows = B * frontier_stride, v = variant_of(p);
-    launch_after(small_n(ctx->cfg.n) ? layers_variant<ot::kSmallN>(v) : layers_variant<ot::kMaxN>(v), dim3(nrows < ctx->grid ? nrows : ctx->grid),
+    const int nrows = B * frontier_stride, form = form_of(p);
+    launch_after(small_n(ctx->cfg.n) ? layers_variant<ot::kSmallN>(form) : layers_variant<ot::kMaxN>(form), dim3(nrows < ctx->grid ? nrows : ctx->grid),
                  dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(frontier_logits), frontier_stride, *out,
                  next_tokens, next_parent, next_count);
     ctx->launches++;
@@ -1846,7 +1849,7 @@ int opt_tree_row_softmax_topk(opt_tree_ctx* ctx, const void* logits, const int32
     if (nrows == 0) return OPT_TREE_OK;
     const ot::Params p = make_params(ctx, logits, 0.0f);
     const int grid = nrows < ctx->grid ? nrows : ctx->grid;
-    launch_after(row_variant(variant_of(p)), dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem),
+    launch_after(row_variant(form_of(p)), dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem),
         static_cast<cudaStream_t>(stream), p, static_cast<const uint16_t*>(logits), rows, nrows, tok_out, prob_out, ctx->ws.status);
     ctx->launches++;
     return check_launch();

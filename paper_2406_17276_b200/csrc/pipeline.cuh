@@ -178,14 +178,15 @@ __device__ void issuer_role(CtaCore& s, int V, const uint16_t* lo, const uint16_
 // A warp takes its share of a chunk out of the ring into registers and hands the stage back at once
 // (so the issuer can refill it while the exponentials run); a row's descriptor is only looked at for
 // its stop flag.
-template <bool kAligned, bool kLong>
+template <int kForm>
 __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
+    constexpr bool kAligned = form_aligned(kForm), kLong = form_long(kForm), kTracked = form_tracked(kForm);
     const int lane = threadIdx.x & 31, tid = cwarp * 32 + lane;     // index among the consumer threads
     const int nchunks = (V + kChunkElems - 1) / kChunkElems;
     ThreadAcc acc;
     acc.reset();
     ChunkRegs ch;
-    uint32_t cm = 0;                                           // long rows: lane c keeps the warp's maximum of chunk c
+    uint32_t cm = 0;                                           // tracked rows: lane c keeps the warp's maximum of chunk c
     int off = 0;                                               // half of the stage at which the row in hand starts
     long long g = 0;
     for (int r = 0;; ++r) {
@@ -207,7 +208,7 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
             __syncwarp();
             if (lane == 0) mbar_arrive(&s.empty_bar[st]);          // the data is in registers: the stage is free
             chunk_chain(ch);
-            if (kLong) { const uint32_t key = chunk_key(ch); if (lane == c) cm = key; }
+            if (kTracked) { const uint32_t key = chunk_key(ch); if (lane == c) cm = key; }
             const unsigned long long C2 = chunk_apply(acc, ch);
             chunk_exps<kLong>(acc, ch, C2, (ne + 7) >> 3);
         }
@@ -215,7 +216,17 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
         const int sl = r % kSlots;
         if (r >= kSlots && !mbar_wait_warp(&s.free_bar[sl], (uint32_t)((r / kSlots) - 1) & 1u, status)) return;
         store_thread_result(s.slot[sl], acc, tid);
-        if (kLong && lane < kTrackedChunks) s.slot[sl].cmax[lane][cwarp] = (uint16_t)cm;
+        if (kTracked) {
+            uint32_t gm = cm;
+            if (nchunks > kChunkGroups) {                          // (lanes beyond the row's chunks hold 0)
+#pragma unroll
+                for (int o = kChunkGroups; o < kMaxTracked; o += kChunkGroups) {
+                    const uint32_t u = __shfl_down_sync(0xFFFFFFFFu, cm, o);
+                    if (lane + o < kMaxTracked) gm = max(gm, u);
+                }
+            }
+            if (lane < kChunkGroups) s.slot[sl].cmax[lane][cwarp] = (uint16_t)gm;
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(&s.ready_bar[sl]);
         acc.reset();
@@ -224,7 +235,7 @@ __device__ void consumer_role(CtaCore& s, int cwarp, int V, int* status) {
 
 // ---- finisher warps ----------------------------------------------------------------------------
 // Sink::row_done(const RowDesc&, const RowOut&, FinScratch&) is called by the whole warp.
-template <bool kAligned, bool kLong, class Sink>
+template <int kForm, class Sink>
 __device__ void finisher_role(CtaCore& s, Sink& sink, int fidx, int V, int k, int* status) {
     const int lane = threadIdx.x & 31;
     FinScratch& f = s.fin[fidx];
@@ -248,28 +259,27 @@ __device__ void finisher_role(CtaCore& s, Sink& sink, int fidx, int V, int k, in
         const RowSlot& slot = s.slot[sl];
         const RowDesc dsc = s.desc[r % kDescRing];
         RowOut out;
-        finish_row_warp<kAligned, kLong>(f, slot, dsc.row, V, k, out);
+        finish_row_warp<kForm>(f, slot, dsc.row, V, k, out);
         __syncwarp();
         if (lane == 0) mbar_arrive(&s.free_bar[sl]);                              // the slot can be refilled
         sink.row_done(dsc, out, f);
     }
 }
 
-// kAligned: the table's base and row pitch are multiples of 16 bytes (a compile-time choice, so that the code of the
-// common case carries nothing of the other); kLong: more than kLongRow logits.  lo / hi bound the table.
-template <bool kAligned, bool kLong, class Smem, class Source, class Sink>
+// kForm: see RowForm.  lo / hi bound the table.
+template <int kForm, class Smem, class Source, class Sink>
 __device__ __forceinline__ void run_pipeline(Smem& sm, Source& src, Sink& sink, int V, int k, const uint16_t* lo, const uint16_t* hi, int* status) {
     CtaCore& s = sm.core;
     pipeline_init(s, sm.layer);
     grid_dependency_wait();                                // shared memory is set up; global memory from here on
     const int warp = threadIdx.x >> 5;
-    if (warp < kConsumerWarps) { consumer_role<kAligned, kLong>(s, warp, V, status); return; }
+    if (warp < kConsumerWarps) { consumer_role<kForm>(s, warp, V, status); return; }
     const int helper = warp - kConsumerWarps;
-    if (helper == kHelperIssuer) issuer_role<kAligned>(s, V, lo, hi, status);
+    if (helper == kHelperIssuer) issuer_role<form_aligned(kForm)>(s, V, lo, hi, status);
     else if (helper == kHelperFetcher) fetcher_role(s, src, status);
     else if (helper == kHelperLayer) sink.layer_loop(sm.layer);
     else if (helper < kHelperFirstFinisher) sink.layer_assist(sm.layer, helper - kHelperLayer);
-    else finisher_role<kAligned, kLong>(s, sink, helper - kHelperFirstFinisher, V, k, status);
+    else finisher_role<kForm>(s, sink, helper - kHelperFirstFinisher, V, k, status);
 }
 
 }  // namespace ot

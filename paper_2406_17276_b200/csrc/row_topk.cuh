@@ -38,12 +38,30 @@ constexpr int kCandCap = 128;                      // candidate list capacity pe
 constexpr int kMaxFlag = 64;                       // flagged threads the fast finisher accepts
 constexpr int kDesc = 4;                           // rows a CTA may hold between ticket and descriptor read
 constexpr int kDescRing = 16;                      // descriptors kept: a row's lives until its finisher has copied it
-// Rows of more than two chunks take kernels of their own (kLong): their last chunk may be mostly padding, and a finisher
-// has many vectors to look at again per flagged thread.  Both cost code in the two hottest loops, which the kernels for
-// short rows do without (in one kernel for all, the row step on 32000 logits was 3 to 7 % slower, a build of 32
-// sequences 4 %).
+// The forms of a row, each with kernels of its own, so that the two hottest loops carry no other form's code.
+//   Aligned: the table's base and row pitch are multiples of 16 bytes.
+//   Long: more than two chunks.  The last chunk may be mostly padding, and a finisher has many vectors to look at again per flagged thread
+//   (in one kernel for all, the row step on 32000 logits was 3 to 7 % slower, a build of 32 sequences 4 %).
+//   Tracked: long, and the consumers note each warp's maximum of a chunk, from which the finisher knows which chunks to read again (see
+//   find_candidates_long).  That is ten instructions per warp and chunk, 2 to 4 % of the consumer loop whether they are run or
+//   branched around, so rows with few chunks or few winners do without: aligned ones of up to four chunks, and those with up to 64 pairs
+//   of a chunk and a winner.  Rows off a 16-byte boundary, whose vectors take two loads each, are all tracked.
+//   Measured (B200, us, tracked / not): row step, 4000 rows of 40000 logits, k = 5, 73.7 / 71.3; 2617 of 61120, k = 16, 68.7 / 67.3, k = 32 71.0 / 70.2;
+//   1249 of 128256, k = 5 65.0 / 64.3, k = 16 66.0 / 69.5; 1628 of 98304, k = 32 65.8 / 73.6; a step of one sequence of n = 50, k = 16, V = 98304
+//   138.8 / 145.0, V = 61120 124.7 / 125.2; unaligned: 3183 rows of 50257, k = 16, 89.4 / 92.7, k = 5 86.3 / 84.2.
+enum RowForm { kShortUnaligned, kLongUnaligned, kShortAligned, kLongAligned, kTrackedAligned, kRowForms };
+__host__ __device__ constexpr bool form_aligned(int f) { return f >= kShortAligned; }
+__host__ __device__ constexpr bool form_long(int f) { return f != kShortUnaligned && f != kShortAligned; }
+__host__ __device__ constexpr bool form_tracked(int f) { return f == kLongUnaligned || f == kTrackedAligned; }
 constexpr int kLongRow = 2 * kChunkElems;          // rows up to this many logits are short
-constexpr int kTrackedChunks = 10;                 // chunks whose maxima are kept (rows of up to 163840 logits)
+constexpr int kChunkGroups = 10;                   // chunk maxima kept per warp: those of the chunks c mod kChunkGroups together
+constexpr int kMaxTracked = 32;                    // chunks of a row that are tracked (a lane each while the row streams); longer rows are not
+inline int row_form(bool aligned, int V, int k) {
+    const int chunks = (V + kChunkElems - 1) / kChunkElems;
+    if (V <= kLongRow) return aligned ? kShortAligned : kShortUnaligned;
+    if (!aligned) return kLongUnaligned;
+    return chunks > 4 && chunks <= kMaxTracked && chunks * k > 64 ? kTrackedAligned : kLongAligned;
+}
 constexpr int kLaneTauMaxK = 16;                   // largest k for which the finisher's threshold comes from the lane maxima
 constexpr int kPerLane = kConsumers / 32;          // per-thread results one finisher lane handles (16)
 
@@ -69,7 +87,7 @@ struct alignas(16) RowSlot {
     float tsum[kConsumers];
     uint16_t tkey[kConsumers];     // per-thread maximum as an ordered key
     int warpE[kConsumerWarps];
-    uint16_t cmax[kTrackedChunks][kConsumerWarps];     // long rows: maximum of each warp's logits of a chunk, see chunk_key
+    uint16_t cmax[kChunkGroups][kConsumerWarps];       // tracked rows: maximum of each warp's logits of a group of chunks, see chunk_key
 };
 
 struct alignas(16) FinScratch {    // private to one finisher warp (hist is cleared and read with 16-byte accesses)
@@ -628,7 +646,7 @@ __device__ __forceinline__ float take_candidates(FinScratch& f, const uint4 (&w)
 // Measured (B200, us a step, with all of the threads' vectors read again, eight in flight per lane / now): one sequence, V = 128256, k = 16
 // 253.9 / 237.8; 64 sequences of n = 256, V = 152064, k = 32 17270 / 16060; 3 of n = 18, V = 92464 304.1 / 280.7; 13 of n = 143, V = 61120, k = 5,
 // four chunks, 627 / 647, the one shape seen to lose.  Up to 32 pairs take a lane each, without a list (3 sequences, n = 136, V = 46048: 579 / 568 us).
-template <bool kAligned>
+template <bool kAligned, bool kTracked>
 __device__ __forceinline__ float find_candidates_long(FinScratch& f, const RowSlot& slot, const uint16_t* row, int V, int kk, int nflag, float negE,
                                                       uint32_t& tau_key) {
     const int lane = threadIdx.x & 31;
@@ -666,7 +684,8 @@ __device__ __forceinline__ float find_candidates_long(FinScratch& f, const RowSl
     auto pair_at = [&](int i) -> int {
         if (i >= pairs) return -1;
         const int c = nflag > 1 ? (int)__umulhi((unsigned)i, magic) : i, t = f.flist[i - c * nflag];
-        return nchunks > kTrackedChunks || slot.cmax[c][t >> 5] + 1u >= tau_key ? (c << 16) | t : -1;       // (+ 1: see chunk_key)
+        const bool all = !kTracked || (!kAligned && nchunks > kMaxTracked);
+        return all || slot.cmax[c % kChunkGroups][t >> 5] + 1u >= tau_key ? (c << 16) | t : -1;       // (+ 1: see chunk_key)
     };
 #pragma unroll 1
     do {
@@ -708,8 +727,9 @@ __device__ __forceinline__ float find_candidates_long(FinScratch& f, const RowSl
 }
 
 // Turns a finished slot into the row's k winners.  Whole finisher warp; f is its private scratch.
-template <bool kAligned, bool kLong>
+template <int kForm>
 __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& slot, const uint16_t* row, int V, int k, RowOut& out) {
+    constexpr bool kAligned = form_aligned(kForm), kLong = form_long(kForm);
     const int lane = threadIdx.x & 31;
     const int kk = k < V ? k : V;
     const int nvec = (V + 7) >> 3;
@@ -790,7 +810,7 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
         // Work item i: flagged thread i mod P (P = nflag rounded up to a power of two), vector i / P.
         const float negE = -(float)emax;
         float sub = 0.0f;
-        if (kLong) sub = find_candidates_long<kAligned>(f, slot, row, V, kk, nflag, negE, tau_key);
+        if (kLong) sub = find_candidates_long<kAligned, form_tracked(kForm)>(f, slot, row, V, kk, nflag, negE, tau_key);
         const uint32_t tau_bits = ord16_inv(tau_key);
         const float tau_f = bf16_bits_to_float(tau_bits);
         const uint32_t tau_b2 = tau_bits | (tau_bits << 16);

@@ -1,6 +1,6 @@
 """-m gpu: the search for a long row's candidates (rows of more than two chunks of 16384 logits), which reads only the chunks in which
-the consumers noted a maximum at or above the threshold: at the numbers of chunks and of pairs (flagged thread, chunk) where its way
-changes, on winners placed by hand, against a softmax and a sort in double precision."""
+the consumers noted a maximum at or above the threshold, or, in rows with few chunks or few winners, all of a flagged thread's: at the
+numbers of chunks and of pairs (flagged thread, chunk) where its way changes, on winners placed by hand, against a softmax and a sort in double precision."""
 import numpy as np
 import pytest
 import torch
@@ -32,7 +32,10 @@ def _place(kind, V, k, rng):
     return x
 
 
-@pytest.mark.parametrize("V,k", [(32776, 10), (49152, 2), (49153, 16), (81920, 5), (81928, 17), (128256, 16), (152063, 10), (163840, 32), (163848, 9), (180225, 32)])
+@pytest.mark.parametrize("V,k", [(32776, 10), (49152, 2), (49153, 16), (81920, 5), (81928, 17), (128256, 16), (152063, 10), (163840, 32), (163848, 9), (180225, 32),
+                                 (65536, 32), (65544, 12), (65544, 13), (81920, 12), (81920, 13),       # five chunks, 64 pairs of a chunk and a winner
+                                 (200003, 10), (262144, 10), (262152, 3), (327688, 16),                 # maxima of several chunks kept together
+                                 (524288, 5), (524296, 5), (524295, 4)])                                # 32 chunks, and one more
 @pytest.mark.parametrize("kind", ["normal", "one_warp", "zeros", "last"])
 def test_winners_of_long_rows(kind, V, k):
     H, rng = 3, np.random.default_rng(V + k)
