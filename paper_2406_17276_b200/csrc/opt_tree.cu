@@ -307,8 +307,9 @@ struct BuildSink {
     // The rows of a new layer take the next numbers of the build's running row count and with them
     // their CTAs (row g: CTA g % grid, mailbox entry g / grid).  Whatever the order in which the
     // sequences publish, every CTA is sent the same number of rows to within one, and a layer spreads
-    // over as many SMs as it has rows.  reserve_layer only starts the atomic (lane 0 keeps the result
-    // in a register; nothing waits for it until publish_layer writes the entries).
+    // over as many SMs as it has rows.  reserve_layer only starts the atomic: lane 0 keeps the result
+    // in a register, and nothing waits for it until the team has its candidates (threshold off: it goes to the job) or publish_layer
+    // writes the entries.
     __device__ unsigned reserve_layer(int nl) {
         unsigned g0 = 0;
         if ((threadIdx.x & 31) == 0) g0 = atomicAdd(reinterpret_cast<unsigned int*>(&w.q_ctl[kQCursor]), (unsigned)nl);

@@ -526,9 +526,9 @@ __device__ __noinline__ void row_exact_warp(FinScratch& f, const uint16_t* row, 
 
 // Whether the two granules that hold vector vi of an unaligned row lie within the row.
 __device__ __forceinline__ bool granules_inside(int vi, int V) { return vi >= 1 && vi * 8 + 16 <= V; }
-// One 16-byte vector of the row (8 logits starting at token 8*vi) as four packed words; logits at or
-// beyond V read as -inf.  Aligned rows take one vector load, others the two granules that hold the vector, or, at
-// either end of the row, where those may reach beyond the table, eight scalar loads.
+// One vector of an unaligned row (8 logits starting at token 8*vi) as four packed words; logits at or
+// beyond V read as -inf.  Two granules hold it; at either end of the row, where those may reach beyond the table, it takes eight scalar
+// loads.
 __device__ __noinline__ uint4 load_row_vec_unaligned(const uint16_t* row, int vi, int V) {
     const uint16_t* p = row + (size_t)vi * 8;
     if (granules_inside(vi, V)) {
@@ -548,7 +548,7 @@ __device__ __forceinline__ void load_granules(const uint16_t* row, int o, int vi
     asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(q + 1));
 }
 // The vectors vi[0 .. kN) of an unaligned row (negative: none, reads as -inf), all granules in flight together.  (One call of
-// load_row_vec after the other waits for each; steps of 16 sequences of n = 48, V = 32003, 154.0 us with calls, 148.5 now.)
+// load_row_vec_unaligned after the other waits for each; steps of 16 sequences of n = 48, V = 32003, 154.0 us with calls, 148.5 now.)
 template <int kN>
 __device__ __forceinline__ void load_vecs_unaligned(uint4 (&w)[kN], const int (&vi)[kN], const uint16_t* row, int V) {
     const int o = vec_offset(row);
@@ -564,15 +564,12 @@ __device__ __forceinline__ void load_vecs_unaligned(uint4 (&w)[kN], const int (&
     for (int u = 0; u < kN; ++u)
         if (vi[u] >= 0 && !granules_inside(vi[u], V)) w[u] = load_row_vec_unaligned(row, vi[u], V);
 }
-template <bool kAligned>
-__device__ __forceinline__ uint4 load_row_vec(const uint16_t* row, int vi, int V) {
-    if (kAligned) {
-        uint4 v;
-        asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
-                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(reinterpret_cast<const uint4*>(row) + vi));
-        return v;
-    }
-    return load_row_vec_unaligned(row, vi, V);
+// Vector vi of an aligned row.
+__device__ __forceinline__ uint4 load_row_vec(const uint16_t* row, int vi) {
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(reinterpret_cast<const uint4*>(row) + vi));
+    return v;
 }
 
 __device__ __noinline__ double exp_f64(double x) { return exp(x); }    // one copy of the routine for all its callers
@@ -640,12 +637,12 @@ __device__ __forceinline__ float take_candidates(FinScratch& f, const uint4 (&w)
 
 // The search of finish_row_warp in long rows: the flagged threads' vectors are read again for the logits >= tau.  The list of threads is
 // first cut down to those at or above the exact kk-th largest per-thread maximum (for kk > kLaneTauMaxK tau is that
-// already), and of a thread's chunks only those are read of which the consumers noted a maximum that high in the thread's warp: a dozen
-// or two of the hundred and more pairs of a thread and a chunk.  Leaves the candidates in f.cand / f.cand_count, raises tau_key and
+// already), and in tracked rows (see RowForm) of a thread's chunks only those are read of which the consumers noted a maximum that high in
+// the thread's warp: a dozen or two of the hundred and more pairs of a thread and a chunk.  Leaves the candidates in f.cand / f.cand_count, raises tau_key and
 // returns the sum of the lane's candidates' approximate terms.
 // Measured (B200, us a step, with all of the threads' vectors read again, eight in flight per lane / now): one sequence, V = 128256, k = 16
-// 253.9 / 237.8; 64 sequences of n = 256, V = 152064, k = 32 17270 / 16060; 3 of n = 18, V = 92464 304.1 / 280.7; 13 of n = 143, V = 61120, k = 5,
-// four chunks, 627 / 647, the one shape seen to lose.  Up to 32 pairs take a lane each, without a list (3 sequences, n = 136, V = 46048: 579 / 568 us).
+// 253.9 / 237.8; 64 sequences of n = 256, V = 152064, k = 32 17270 / 16060; 3 of n = 18, V = 92464 304.1 / 280.7; 8 of n = 60, V = 200064, k = 10
+// 371 / 339; 13 of n = 143, V = 61120, k = 5, four chunks, not tracked, 636 / 628.  Up to 32 pairs take a lane each, without a list (3 sequences, n = 136, V = 46048: 579 / 568 us).
 template <bool kAligned, bool kTracked>
 __device__ __forceinline__ float find_candidates_long(FinScratch& f, const RowSlot& slot, const uint16_t* row, int V, int kk, int nflag, float negE,
                                                       uint32_t& tau_key) {
@@ -672,7 +669,7 @@ __device__ __forceinline__ float find_candidates_long(FinScratch& f, const RowSl
         __syncwarp();
     }
     const uint32_t tau_bits = ord16_inv(tau_key), tau_b2 = tau_bits | (tau_bits << 16);
-    // Most pairs of a flagged thread and a chunk hold nothing: those whose warp's maximum of the chunk is below the threshold are left out.
+    // Most pairs of a flagged thread and a chunk hold nothing: in tracked rows those whose warp's maximum of the chunk is below the threshold are left out.
     // Pair i: flagged thread i mod nflag, chunk i / nflag = umulhi(i, magic) (exact: i * nflag stays below 2^32).
     const int pairs = nchunks * nflag;
     const unsigned magic = 0xFFFFFFFFu / (unsigned)nflag + 1u;
@@ -715,7 +712,7 @@ __device__ __forceinline__ float find_candidates_long(FinScratch& f, const RowSl
                 vis[u] = e >= 0 && vi < nvec ? vi : -1;
                 if (kAligned) {
                     w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
-                    if (vis[u] >= 0) w[u] = load_row_vec<true>(row, vi, V);
+                    if (vis[u] >= 0) w[u] = load_row_vec(row, vi);
                 }
             }
             if (!kAligned) load_vecs_unaligned(w, vis, row, V);
@@ -838,7 +835,7 @@ __device__ __forceinline__ void finish_row_warp(FinScratch& f, const RowSlot& sl
                 if (kAligned) w[u] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
                 if (idx < total && fi < nflag) {
                     const int vi = (j / kVecPerThread) * kChunkVecs + (j % kVecPerThread) * kConsumers + f.flist[fi];
-                    if (vi < nvec) { vis[u] = vi; if (kAligned) w[u] = load_row_vec<true>(row, vi, V); }
+                    if (vi < nvec) { vis[u] = vi; if (kAligned) w[u] = load_row_vec(row, vi); }
                 }
             }
             if (!kAligned) load_vecs_unaligned(w, vis, row, V);

@@ -88,7 +88,7 @@ __device__ __noinline__ unsigned int poll_tok_word(const unsigned int* p, int* s
 }
 
 // ------------------------------------------------------------------------------------------------
-// The same layer selection by the layer team (kTeam threads: the layer warp and its assistants;
+// What the layer team's selections are made of (kTeam threads: the layer warp and its assistants;
 // thread tt of the team).  Every step that loops over the candidates is split over the team;
 // the decisions in between are computed by each warp for itself from the same shared-memory
 // counts, so all warps take the same path and meet at the same barriers.
@@ -182,10 +182,10 @@ __device__ int team_radix_select(LS& s, KeyFn keyf, int N, int need, int tt, uns
 // The words of a candidate that never came (see sweep_candidates): token 0, path value 0.
 constexpr unsigned long long kLostPhat = 1ull << 63;
 constexpr unsigned kLostTok = 1u << 31;
-// Once a wait of a team has run out the team waits no more: the build comes to its end, with the status set.
-__device__ __forceinline__ void wait_ran_out(LayerJob& job, int* status) {
+// Once a wait of a team has run out the team waits no more: the build comes to its end, with the status set.  (Inlined, n = 1024 takes 3 % more.)
+__device__ __noinline__ void wait_ran_out(int job_at, int* status) {
     set_status(status, kErrTimeout);
-    atomicExch(&job.polls, 0);
+    atomicExch(&smem_at<LayerJob>(job_at).polls, 0);
 }
 
 // Candidate words i = u * kTeam + tt (u < kW) of [first, end), into registers (all ones elsewhere); gph and gtk are the words' arrays
@@ -214,7 +214,7 @@ __device__ __forceinline__ void sweep_candidates(const unsigned long long* gph, 
         if (!__any_sync(0xFFFFFFFFu, missing)) break;
         __nanosleep(20);
         if (t >= job.polls) {
-            wait_ran_out(job, status);
+            wait_ran_out(smem_offset(&job), status);
 #pragma unroll
             for (int u = 0; u < kW; ++u) { if (!(x[u] >> 63)) x[u] = kLostPhat; if (!(t32[u] >> 31)) t32[u] = kLostTok; }
             break;
@@ -267,7 +267,7 @@ __device__ __forceinline__ int warp_coarse_bin(const LS& s, int need, int& at_or
     at_or_above = a0 + a1 + __shfl_sync(0xFFFFFFFFu, c, l1);
     return l0 * 32 + l1;
 }
-// Coarse bin of a path-value key: sixteen bins per factor of two, 1 at the top, everything below 2^-63 at the bottom.
+// Coarse bin of a path-value key: sixteen bins per factor of two, 1 at the top, everything below 1.125 * 2^-64 at the bottom.
 constexpr int kCoarseShift = 48, kCoarseBase = 16 * 0x3FF - 1023, kFineShift = kCoarseShift - 10;
 __device__ __forceinline__ int coarse_bin(unsigned long long key) {
     const int e = (int)(key >> kCoarseShift) - kCoarseBase;
@@ -312,7 +312,7 @@ __device__ __noinline__ unsigned pick_by_radix(int at, int N, int need, int tt) 
 // thread's taken keys; the elements taken before key[u] are picked_before(s, base, u, tt), all together `total`.
 // Bound by the latency of a chain of barriers, shared-memory accesses and shuffles, so there is one pass: the keys are counted into
 // coarse bins of their path values, the bin in which the threshold lies is listed (a
-// handful of keys) and the list is ranked.  A bin of more than kList keys (many equal path values, or values below 2^-63)
+// handful of keys) and the list is ranked.  A bin of more than kList keys (many equal path values, or values below 2^-64)
 // goes to a radix select over all.  A layer of 500 candidates takes 2.3 us from its last word to its last row sent out; with a radix
 // select over keys in shared memory and a compaction by contiguous stretches it took 3.9 to 9 (equal path values at the threshold).
 // Steps (B200, us, before / now): n = 50, V = 32000 132.9 / 118.0; n = 64, V = 128256 274.8 / 253.3; 32 sequences pruned 208.4 / 186.6.
@@ -585,13 +585,13 @@ __device__ __noinline__ int team_select_global(int at, const unsigned long long*
     return total;
 }
 
-// The team's selection for layers with more candidates than the shared-memory staging holds
+// The team's selection for layers with more candidates than it holds in registers
 // (kStageCap < N <= n*k).  Bound by the round trips of 128 threads to the candidate words in L2 (8192 of them take 3 us,
 // 6 with their counting), so there are two sweeps and no more: the first counts the candidates into coarse bins of their path
 // values, the second brings those at or above the bin in which the threshold lies, usually few more than n, into shared
 // memory, each warp into a segment of its own; the keys of that bin are listed and the threshold is found by ranking
 // them.  (If the bin is too full one more sweep splits it in 1024; if over a thousand ties or a threshold below
-// 2^-63 make that useless too, or a warp's segment overflows, further sweeps read global memory once per digit.)
+// 2^-64 make that useless too, or a warp's segment overflows, further sweeps read global memory once per digit.)
 // Measured (two sequences, n = 512, k = 16, B200): 1059 us per step with a sweep per digit and tokens fetched one by one, 452
 // with bit marks, a gather and a radix select after the second sweep, 431 with the segments; 401 then with the running top-n of
 // team_pick, 378 with the rows sent out by the team as their tokens come in instead of by one warp afterwards.
@@ -628,7 +628,7 @@ __device__ __noinline__ int select_layer_team_big(int at, int tt, unsigned g0, i
                 if (!(x[u] >> 63)) { x[u] = ld_relaxed_u64(&gph[i0 + u * kTeam]); missing = missing || !(x[u] >> 63); }
             if (!__any_sync(0xFFFFFFFFu, missing)) break;
             if (t >= j.polls) {
-                wait_ran_out(s.job, status);
+                wait_ran_out(smem_offset(&s.job), status);
 #pragma unroll
                 for (int u = 0; u < 8; ++u) if (!(x[u] >> 63)) x[u] = kLostPhat;
                 break;

@@ -11,7 +11,7 @@ import torch
 from paper_2406_17276_b200 import binding
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-PARITY_LOG = os.path.join(ROOT, "gpurun_out", "parity_counts.json")
+PARITY_LOG = os.environ.get("OPT_TREE_PARITY_LOG", os.path.join(ROOT, "build", "parity_counts.json"))
 
 
 def dev_table(tab: np.ndarray) -> torch.Tensor:
