@@ -448,8 +448,9 @@ struct BuildSink {
     // Rows of a layer of f rows that may still be missing when the team starts on it.  Candidate words validate themselves, so the
     // team can start at once and wait for the words.  It does as long as a layer's rows of all sequences take the SMs at most four
     // times round; beyond that the polling would slow the rows down (a team reads every missing word again and again), and it
-    // starts when at most sixteen rows or a quarter of a large layer are missing: 32 sequences 221.5 us per build with
-    // none, 219.7 with 16, 220.7 with half; n = 512 429 with none, 413 with a quarter or a half.
+    // starts when at most sixteen rows or a quarter of a large layer are missing.  Steps (B200, us) with none ahead / always sixteen or a
+    // quarter / always all / this rule: one sequence, n = 50 123.1 / 120.5 / 115.4 / 115.5; 2 of n = 512 399 / 385 / 373 / 380; 32 of n = 64
+    // 250.3 / 246.6 / 261.2 / 245.1; 64 of n = 256, V = 152064 16190 / 16190 / 16830 / 16230; 32 pruned 200.6 / 190.1 / 192.9 / 188.6.
     // A warp that follows several sequences must not wait for one of them.
     __device__ int rows_ahead(int f) const {
         if (p.B > (int)gridDim.x) return 0;
@@ -1651,7 +1652,7 @@ template <int NCAP> LayersKernel layers_variant(int form) {
                                                  ot::layers_kernel<NCAP, 3>, ot::layers_kernel<NCAP, 4>};
     return kernels[form];
 }
-int form_of(const ot::Params& p) { return ot::row_form(p.aligned != 0, p.V, p.kk); }
+int form_of(const ot::Params& p, bool build) { return ot::row_form(p.aligned != 0, p.V, p.kk, build); }
 template <class F> bool allow_smem(F* kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
 }
@@ -1750,7 +1751,7 @@ static int build_common(opt_tree_ctx* ctx, const void* draft, const int32_t* roo
     p.prune = prune;
     const long long init_threads = (long long)ctx->grid * ctx->mcap > B ? (long long)ctx->grid * ctx->mcap : B;
     launch_after(ot::init_build_kernel, dim3((unsigned)((init_threads + 255) / 256)), dim3(256), 0, st, ctx->ws, p, root_token);
-    launch_after(build_kernel_for(ctx->cfg.n, form_of(p), prune != 0), dim3(ctx->grid), dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(draft), *out, rows_read);
+    launch_after(build_kernel_for(ctx->cfg.n, form_of(p, true), prune != 0), dim3(ctx->grid), dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(draft), *out, rows_read);
     ctx->launches += 2;
     return check_launch();
 }
@@ -1836,7 +1837,7 @@ int opt_tree_layers_step(opt_tree_ctx* ctx, const void* frontier_logits, int32_t
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     ot::Params p = make_params(ctx, frontier_logits, delta);
     p.B = B;
-    const int nrows = B * frontier_stride, form = form_of(p);
+    const int nrows = B * frontier_stride, form = form_of(p, true);
     launch_after(small_n(ctx->cfg.n) ? layers_variant<ot::kSmallN>(form) : layers_variant<ot::kMaxN>(form), dim3(nrows < ctx->grid ? nrows : ctx->grid),
                  dim3(ot::kThreads), ctx->smem, st, ctx->ws, p, static_cast<const uint16_t*>(frontier_logits), frontier_stride, *out,
                  next_tokens, next_parent, next_count);
@@ -1850,7 +1851,7 @@ int opt_tree_row_softmax_topk(opt_tree_ctx* ctx, const void* logits, const int32
     if (nrows == 0) return OPT_TREE_OK;
     const ot::Params p = make_params(ctx, logits, 0.0f);
     const int grid = nrows < ctx->grid ? nrows : ctx->grid;
-    launch_after(row_variant(form_of(p)), dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem),
+    launch_after(row_variant(form_of(p, false)), dim3(grid), dim3(ot::kThreads), sizeof(ot::CtaSmem),
         static_cast<cudaStream_t>(stream), p, static_cast<const uint16_t*>(logits), rows, nrows, tok_out, prob_out, ctx->ws.status);
     ctx->launches++;
     return check_launch();

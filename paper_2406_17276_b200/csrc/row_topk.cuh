@@ -44,11 +44,15 @@ constexpr int kDescRing = 16;                      // descriptors kept: a row's 
 //   (in one kernel for all, the row step on 32000 logits was 3 to 7 % slower, a build of 32 sequences 4 %).
 //   Tracked: long, and the consumers note each warp's maximum of a chunk, from which the finisher knows which chunks to read again (see
 //   find_candidates_long).  That is ten instructions per warp and chunk, 2 to 4 % of the consumer loop whether they are run or
-//   branched around, so rows with few chunks or few winners do without: aligned ones of up to four chunks, and those with up to 64 pairs
-//   of a chunk and a winner.  Rows off a 16-byte boundary, whose vectors take two loads each, are all tracked.
+//   branched around, so rows with few chunks or few winners do without.  In the builds, whose layers wait for their last row, aligned rows
+//   are tracked from more than 32 pairs of a chunk and a winner on (up to 32 a finisher's lanes look at one pair each); in the row step,
+//   where finishers work beside the consumers, from five chunks and more than 64 pairs on.  Rows off a 16-byte boundary, whose vectors
+//   take two loads each, are all tracked.
 //   Measured (B200, us, tracked / not): row step, 4000 rows of 40000 logits, k = 5, 73.7 / 71.3; 2617 of 61120, k = 16, 68.7 / 67.3, k = 32 71.0 / 70.2;
-//   1249 of 128256, k = 5 65.0 / 64.3, k = 16 66.0 / 69.5; 1628 of 98304, k = 32 65.8 / 73.6; a step of one sequence of n = 50, k = 16, V = 98304
-//   138.8 / 145.0, V = 61120 124.7 / 125.2; unaligned: 3183 rows of 50257, k = 16, 89.4 / 92.7, k = 5 86.3 / 84.2.
+//   1249 of 128256, k = 5 65.0 / 64.3, k = 16 66.0 / 69.5; 1628 of 98304, k = 32 65.8 / 73.6; steps: one sequence of n = 50, V = 61120, k = 16
+//   123.5 / 127.5, k = 32 146.3 / 153.6, V = 98304, k = 5 (30 pairs) 120.2 / 123.0; 4 of n = 187, V = 99744, k = 6 (42) 481 / 491; 13 of n = 143,
+//   V = 61120, k = 5 (20) 648 / 627; 32 of n = 64, V = 50000, k = 12 (48) 389 / 384; unaligned: 3183 rows of 50257, k = 16, 89.4 / 92.7, k = 5
+//   86.3 / 84.2.
 enum RowForm { kShortUnaligned, kLongUnaligned, kShortAligned, kLongAligned, kTrackedAligned, kRowForms };
 __host__ __device__ constexpr bool form_aligned(int f) { return f >= kShortAligned; }
 __host__ __device__ constexpr bool form_long(int f) { return f != kShortUnaligned && f != kShortAligned; }
@@ -56,11 +60,12 @@ __host__ __device__ constexpr bool form_tracked(int f) { return f == kLongUnalig
 constexpr int kLongRow = 2 * kChunkElems;          // rows up to this many logits are short
 constexpr int kChunkGroups = 10;                   // chunk maxima kept per warp: those of the chunks c mod kChunkGroups together
 constexpr int kMaxTracked = 32;                    // chunks of a row that are tracked (a lane each while the row streams); longer rows are not
-inline int row_form(bool aligned, int V, int k) {
-    const int chunks = (V + kChunkElems - 1) / kChunkElems;
+inline int row_form(bool aligned, int V, int k, bool build) {
+    const int chunks = (V + kChunkElems - 1) / kChunkElems, pairs = chunks * k;
     if (V <= kLongRow) return aligned ? kShortAligned : kShortUnaligned;
     if (!aligned) return kLongUnaligned;
-    return chunks > 4 && chunks <= kMaxTracked && chunks * k > 64 ? kTrackedAligned : kLongAligned;
+    const bool tracked = chunks <= kMaxTracked && (build ? pairs > 32 : chunks > 4 && pairs > 64);
+    return tracked ? kTrackedAligned : kLongAligned;
 }
 constexpr int kLaneTauMaxK = 16;                   // largest k for which the finisher's threshold comes from the lane maxima
 constexpr int kPerLane = kConsumers / 32;          // per-thread results one finisher lane handles (16)
